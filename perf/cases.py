@@ -17,6 +17,8 @@ PITCH = 0.5             # metres between actuators
 R0, L0 = 1.0, 25.0      # Fried parameter and outer scale of the turbulence, metres
 FRAME = 1e-3            # seconds per frame
 N_SLOPES = 4            # frames of slopes that a state holds; passes take them in turn
+RESTART = 16            # passes after which a loop goes back to its checkpoint: filters of few members drift off
+                        # over hundreds of frames, and what is timed is a loop that follows the truth
 
 
 def _case(name, kind, n_sub, m, precision, path, sigma=0.2, a=0.995, a2=0.0, obstruction=0.0, dom_sub=4, halo=2,
@@ -229,15 +231,16 @@ def prepare(case, seed):
     systems = _inputs(case, seed)
     if case["kind"] == "serve":
         srv = Server(max_pending=8)
-        ids, outs, hosts, states = [], [], [], []
+        ids, outs, hosts, start = [], [], [], []
         for kw, X, ys in systems:
             sid = srv.admit(**{k: v for k, v in kw.items() if k != "path"})
-            _lib.letkf_set_state(_lib.letkf_server_context(srv.srv, sid), X.data_ptr(), 0)
             outs.append(srv.set_output(sid, 2))
             hosts.append(ys.cpu().numpy())
             ids.append(sid)
-        torch.cuda.synchronize()
-        return {"kind": "serve", "srv": srv, "ids": ids, "outs": outs, "ys": hosts, "k": 0}
+            start.append(X)
+        s = {"kind": "serve", "srv": srv, "ids": ids, "outs": outs, "ys": hosts, "start": start, "k": 0}
+        _restore(s)
+        return s
     kw, X, ys = systems[0]
     if case["kind"] == "pair":
         f = LETKFPair(**{k: v for k, v in kw.items() if k not in ("path", "piston")})
@@ -245,15 +248,28 @@ def prepare(case, seed):
     else:
         f = LETKF(**kw)
         filters, X = [f], [X]
-    for g, x in zip(filters, X):
-        g.set_state(x, 0)
+    s = {"kind": case["kind"], "f": f, "filters": filters, "ys": [y.contiguous() for y in ys], "start": X, "k": 0,
+         "out": torch.empty(f.info.n_act, dtype=f.dtype, device=f.device), "state": [torch.empty_like(x) for x in X]}
+    _restore(s)
     torch.cuda.synchronize()
-    return {"kind": case["kind"], "f": f, "filters": filters, "ys": [y.contiguous() for y in ys], "k": 0,
-            "out": torch.empty(f.info.n_act, dtype=f.dtype, device=f.device), "state": [torch.empty_like(x) for x in X]}
+    return s
+
+
+def _restore(s):
+    """The checkpoint's ensembles, the frame counters going on."""
+    if s["kind"] == "serve":
+        for sid, x in zip(s["ids"], s["start"]):
+            _lib.letkf_set_state(_lib.letkf_server_context(s["srv"].srv, sid), x.data_ptr(), 2 * s["k"])
+        torch.cuda.synchronize()    # a server's streams are its own
+    else:
+        for g, x in zip(s["filters"], s["start"]):
+            g.set_state(x, s["k"])
 
 
 def run(s):
     k = s["k"]
+    if k and k % RESTART == 0:
+        _restore(s)
     s["k"] = k + 1
     if s["kind"] == "serve":
         srv = s["srv"]
