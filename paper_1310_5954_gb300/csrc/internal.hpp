@@ -16,7 +16,7 @@ namespace letkf {
 // Bits of the device status word (latched until letkf_sync reads them).
 enum : int {
     ST_NONFINITE = 1,   // a frame's slopes held a NaN or Inf; the frame was rejected
-    ST_NOCONV = 2,      // an eigensolve hit its sweep limit
+    ST_NOCONV = 2,      // an inverse square root hit its step limit
     ST_TIMEOUT = 4,     // a bounded wait on an mbarrier gave up
 };
 
