@@ -2557,7 +2557,7 @@ int fused_prepare(letkf_ctx* c) {
     if (cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, prio_least) != cudaSuccess) return LETKF_ECUDA;
     const size_t vbytes = (size_t)c->n_act * c->m_pad * 4;
     const size_t xbytes = c->precision == LETKF_PREC_MIXED ? noise_xi_bytes(c->n_act, c->m)
-                                                           : vbytes;
+                                                           : rg_xi_bytes(c->n_act, c->m, 4);
     for (int b = 0; b < 2; ++b) {
         if (cudaEventCreateWithFlags(&c->ev_v_ready[b], cudaEventDisableTiming) != cudaSuccess) return LETKF_ECUDA;
         if (cudaEventCreateWithFlags(&c->ev_v_used[b], cudaEventDisableTiming) != cudaSuccess) return LETKF_ECUDA;

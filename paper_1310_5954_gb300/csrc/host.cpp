@@ -247,7 +247,7 @@ void free_all(letkf_ctx* c) {
     }
     if (c->Xi_side) cudaFree(c->Xi_side);
     if (c->pair_pred) cudaFree(c->pair_pred);
-    for (void* q : {c->rg_items, c->rg_tiles, static_cast<void*>(c->rg_count), c->rg_part})
+    for (void* q : {c->rg_items, c->rg_tiles, c->rg_part})
         if (q) cudaFree(q);
     if (c->scratch) cudaFree(c->scratch);
     letkf::fused_graph_reset(c);
@@ -305,7 +305,7 @@ size_t footprint_bytes(const letkf_params* p, const HostModel& h) {
     } else {
         const size_t vbytes = na * m_pad * 4;
         b += 2 * vbytes + (p->precision == LETKF_PREC_MIXED ? letkf::noise_xi_bytes(h.n_act, p->m)
-                                                             : vbytes);
+                                                             : letkf::rg_xi_bytes(h.n_act, p->m, eb));
         b += na * 4;            // the second filter's prediction of letkf_step_pair
         if (p->m + 1 > 128) {   // dual form: per-CTA halo anomalies
             int sms = 0;
@@ -317,9 +317,9 @@ size_t footprint_bytes(const letkf_params* p, const HostModel& h) {
         b += letkf::noise_plan(h.n_act, p->m, letkf::lower_triangular(p->q_sqrt, h.n_act)).bytes;
         b += letkf::noise_xi_bytes(h.n_act, p->m);
     } else if (p->q_sqrt) {
-        b += na * na * eb + na * row;
-        if (p->path != LETKF_PATH_GLOBAL)
-            b += letkf::rg_bytes(h.n_act, p->m, letkf::lower_triangular(p->q_sqrt, h.n_act), eb);
+        b += p->path == LETKF_PATH_GLOBAL
+                 ? na * na * eb
+                 : letkf::rg_bytes(h.n_act, p->m, letkf::lower_triangular(p->q_sqrt, h.n_act), eb);
     }
     if (p->piston != LETKF_PISTON_OFF) b += letkf::piston_bytes(h, (int)nd, (int)eb);
     if (p->path == LETKF_PATH_GLOBAL) {

@@ -68,8 +68,10 @@ struct letkf_ctx {
     int phase = 0;                  // 0: forecast phase, 1: analysis phase
     unsigned long long frame = 0;
     // process noise
-    void* Lq = nullptr;             // FP64 / FP32: device L, n_act x n_act row-major
-    void* Xi = nullptr;             // normals: n_act x m_pad (FP64 / FP32) or 64-row BF16 tiles (mixed)
+    void* Lq = nullptr;             // FP64 / FP32: device L, in the draw kernel's chunks (global path:
+                                    // n_act x n_act row-major)
+    void* Xi = nullptr;             // normals, in the layout of the draw (FP64 / FP32) or as 64-row BF16
+                                    // tiles (mixed)
     // mixed precision: L as BF16 128 x 64 operand tiles (lower-triangle tiles only when L is lower
     // triangular) and the work items of the noise kernel
     void* Lt = nullptr;
@@ -134,11 +136,10 @@ struct letkf_ctx {
     int cap_dom = -1;
     // fused path: this context's prediction when it is the second filter of letkf_step_pair
     void* pair_pred = nullptr;
-    // FP32 / FP64 dense process noise: work items and tiles (int4), per-tile counters and partial
-    // tiles of the split-K draw V = L xi
+    // FP32 / FP64 dense process noise: work items and tiles (int4) and partial tiles of the draw
+    // V = L xi
     void* rg_items = nullptr;
     void* rg_tiles = nullptr;
-    int* rg_count = nullptr;
     void* rg_part = nullptr;
     int rg_n_items = 0;
     // stage timing
@@ -170,14 +171,16 @@ int draw_perturbations(letkf_ctx* c, unsigned long long frame);
 // Normals of `frame` into xi, then V = L xi into v_out, on `stream`.
 int draw_perturbations_on(letkf_ctx* c, unsigned long long frame, void* xi, void* v_out, cudaStream_t stream);
 int init_ensemble(letkf_ctx* c, const double* L_host, const double* P0_host);
-// Split-K work plan of the per-frame draw V = L xi (n x n factor, m members): items and tiles
-// (4 ints each, filled when not null), partial-tile slots; rg_bytes: its device bytes.
+// Work plan of the FP32 / FP64 per-frame draw V = L xi (n x n factor, m members, eb bytes per
+// element): items and tiles (4 ints each, filled when not null), elements of the factor's and the
+// normals' layouts and of the partial tiles; rg_bytes: its device bytes; rg_xi_bytes: the normals'.
 struct RowGemmPlan {
     int n_items = 0, n_tiles = 0, n_slots = 0;
-    size_t part_elems = 0;
+    size_t part_elems = 0, l_elems = 0, xi_elems = 0;
 };
-RowGemmPlan rg_plan(int n, int m, bool lower, int* items, int* tiles);
+RowGemmPlan rg_plan(int n, int m, bool lower, size_t eb, int* items, int* tiles);
 size_t rg_bytes(int n, int m, bool lower, size_t eb);
+size_t rg_xi_bytes(int n, int m, size_t eb);
 // Node parameters of the normals kernel draw_perturbations_on launches (arguments held in *nn).
 struct NormalsNode {
     cudaKernelNodeParams params;

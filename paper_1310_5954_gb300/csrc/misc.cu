@@ -9,11 +9,13 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
 #include "common.cuh"
 #include "internal.hpp"
+#include "umma.cuh"
 
 namespace letkf {
 namespace {
@@ -207,108 +209,238 @@ __global__ void __launch_bounds__(RG_THREADS) row_gemm_kernel(const T* __restric
     }
 }
 
-// The per-frame draw V = L Xi with split K: a work item is a 64 x 128 tile of V over one piece of
-// at most RK_KC values of k (with a lower-triangular L, a row block's k stops at its last row), so
-// that the long row blocks of a triangular factor spread over many CTAs.  256 threads, each a
-// 4 x 8 register block (rows ty + 16 i, columns tx + 16 j), K steps of 16 staged in shared memory
-// with a register prefetch.  A tile of one piece writes V; otherwise each piece writes its partial
-// tile to the scratch and the CTA that finishes last (per-tile counter) sums the pieces in piece
-// order, so the result does not depend on which CTA ran first, and resets the counter.
-constexpr int RK_BM = 64, RK_BN = 128, RK_BK = 16, RK_KC = 512, RK_THREADS = 256;
+// The per-frame draw V = L Xi in the state type on the CUDA cores.  Both operands are laid out for
+// bulk copies: L once, at creation, as chunks of 16 values of k by BM rows (k-major, so that a
+// thread's rows are adjacent; a lower-triangular factor keeps the chunks up to each row block's last
+// row only), Xi by its generator as 16 rows of BN columns.  A work item is a BM x BN tile of V over a
+// run of chunks: one thread refills a ring of four chunk pairs, 256 threads compute TM x TN register
+// blocks (TM adjacent rows, columns tx + CX j).  A row block's chunks are split into runs of equal
+// length so that all items together fill two CTAs per SM once; a split tile's runs go to the scratch
+// and rg_reduce_kernel adds them in order, so the result does not depend on scheduling.
+//
+// What bounds it: the FMA pipe (an 8 x 7 block does 56 multiply-adds per 9 shared-memory reads), in
+// FP64 the two FP64 lanes of an SM: there the tiles are 32 rows by 8 TN columns, so that few of the
+// multiply-adds are padding.  Measured, normals and product (before: 64 x 128 tiles of K pieces of
+// 512, scalar loads, the last CTA of a tile summing its pieces): 69 actuators, m = 20, FP64 180 -> 21 us;
+// 1 353, m = 50, FP32 93 -> 22 us; 4 836, m = 100, FP32 frame 242 -> 192 us (the draw runs beside it).
+constexpr int RK_KC = 16, RK_STAGES = 4, RK_THREADS = 256, RK_ITEMS = 2 * 152;
+constexpr long long RK_WAIT = 4000000000LL;
 
-template <typename T>
-__global__ void __launch_bounds__(RK_THREADS) rg_splitk_kernel(const T* __restrict__ L, const T* __restrict__ Xi,
-                                                               T* __restrict__ V, int n, int m, int ldx, int ldv,
-                                                               const int4* __restrict__ items,
-                                                               const int4* __restrict__ tiles, T* __restrict__ part,
-                                                               int* __restrict__ count) {
-    __shared__ T As[RK_BK][RK_BM + 1];   // As[k][row]: L tile, transposed
-    __shared__ T Bs[RK_BK][RK_BN];       // Bs[k][col]: Xi tile
-    __shared__ int last;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int4 it = items[blockIdx.x];   // tile, k0, k1, piece
-    const int4 tl = tiles[it.x];         // row block, column block, pieces, first scratch slot
-    const int r0 = tl.x * RK_BM, c0 = tl.y * RK_BN, k0 = it.y, k1 = it.z;
-    // loads: A, 64 rows x 16 k, thread -> row tid / 4, k 4 (tid % 4) .. + 3;
-    //        B, 16 k x 128 columns, thread -> k tid / 16, columns 8 (tid % 16) .. + 7
-    const int ar = tid >> 2, ak = 4 * (tid & 3);
-    const int bk = tid >> 4, bc = 8 * (tid & 15);
-    T ra[4], rb[8];
-    auto fetch = [&](int kb) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int r = r0 + ar, k = kb + ak + u;
-            ra[u] = (r < n && k < k1) ? L[(size_t)r * n + k] : T(0);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int k = kb + bk, cc = c0 + bc + u;
-            rb[u] = (k < k1 && cc < m) ? Xi[(size_t)k * ldx + cc] : T(0);
-        }
+// Chunks before row block rb (nk: chunks of a full row).
+__host__ __device__ inline size_t rk_prefix(int rb, int bm, int nk, int lower) {
+    return lower ? (size_t)(bm / RK_KC) * rb * (rb + 1) / 2 : (size_t)rb * nk;
+}
+
+template <typename T, int CX, int TM, int TN>
+__global__ void __launch_bounds__(RK_THREADS, 2) rg_kernel(const T* __restrict__ Lt, const T* __restrict__ Xi,
+                                                           T* __restrict__ V, int n, int m, int ldv, int lower,
+                                                           const int4* __restrict__ items,
+                                                           const int4* __restrict__ tiles, T* __restrict__ part,
+                                                           int* __restrict__ status) {
+    constexpr int RX = RK_THREADS / CX, BM = RX * TM, BN = CX * TN;
+    constexpr uint32_t A_B = RK_KC * BM * sizeof(T), B_B = RK_KC * BN * sizeof(T);
+    extern __shared__ __align__(128) unsigned char rk_smem[];
+    __shared__ __align__(8) uint64_t full[RK_STAGES];
+    const int tid = threadIdx.x, tx = tid % CX, ty = tid / CX;
+    const int4 it = items[blockIdx.x];   // tile, first chunk, end chunk, run
+    const int4 tl = tiles[it.x];         // row block, column block, runs, first scratch slot
+    const int nk = (n + RK_KC - 1) / RK_KC, nc = it.z - it.y;
+    const unsigned char* ga = reinterpret_cast<const unsigned char*>(Lt) + (rk_prefix(tl.x, BM, nk, lower) + it.y) * A_B;
+    const unsigned char* gb = reinterpret_cast<const unsigned char*>(Xi) + ((size_t)tl.y * nk + it.y) * B_B;
+    auto load = [&](int c) {
+        const int s = c % RK_STAGES;
+        unsigned char* st = rk_smem + s * (A_B + B_B);
+        umma::mbar_arrive_expect_tx(&full[s], A_B + B_B);
+        umma::bulk_g2s(st, ga + (size_t)c * A_B, A_B, &full[s]);
+        umma::bulk_g2s(st + A_B, gb + (size_t)c * B_B, B_B, &full[s]);
     };
-    T acc[4][8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = T(0);
-    if (k0 < k1) fetch(k0);
-    for (int kb = k0; kb < k1; kb += RK_BK) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) As[ak + u][ar] = ra[u];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) Bs[bk][bc + u] = rb[u];
-        __syncthreads();
-        if (kb + RK_BK < k1) fetch(kb + RK_BK);
-#pragma unroll
-        for (int k = 0; k < RK_BK; ++k) {
-            T a[4], b[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) b[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
+    if (tid == 0) {
+        for (int s = 0; s < RK_STAGES; ++s) umma::mbar_init(&full[s], 1);
+        umma::fence_mbar_init();
     }
-    if (tl.z == 1) {
+    __syncthreads();
+    if (tid == 0)
+        for (int c = 0; c < nc && c < RK_STAGES; ++c) load(c);
+    T acc[TM][TN];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + ty + 16 * i;
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int cc = c0 + tx + 16 * j;
-                if (r < n && cc < m) V[(size_t)r * ldv + cc] = acc[i][j];
+        for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
+    int issued = min(nc, RK_STAGES), done = 0;
+    bool ok = true;
+    for (int c = 0; c < nc; ++c) {
+        const int s = c % RK_STAGES;
+        ok = umma::mbar_wait_bounded(&full[s], (uint32_t)((c / RK_STAGES) & 1), RK_WAIT);
+        if (ok) {
+            const T* As = reinterpret_cast<const T*>(rk_smem + s * (A_B + B_B));
+            const T* Bs = As + RK_KC * BM;
+#pragma unroll
+            for (int k = 0; k < RK_KC; ++k) {
+                T a[TM], b[TN];
+                if constexpr (TM % 4 == 0 && sizeof(T) == 4) {
+#pragma unroll
+                    for (int i = 0; i < TM; i += 4) {
+                        const float4 v = *reinterpret_cast<const float4*>(As + k * BM + ty * TM + i);
+                        a[i] = v.x; a[i + 1] = v.y; a[i + 2] = v.z; a[i + 3] = v.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) a[i] = As[k * BM + ty * TM + i];
+                }
+#pragma unroll
+                for (int j = 0; j < TN; ++j) b[j] = Bs[k * BN + tx + CX * j];
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
             }
+        }
+        done = c + 1;
+        if (__syncthreads_or(!ok)) break;          // the stage is read by every warp: it can be refilled
+        if (tid == 0 && c + RK_STAGES < nc) {
+            load(c + RK_STAGES);
+            issued = c + RK_STAGES + 1;
+        }
+    }
+    if (done < nc || !ok) {
+        // a copy did not land in time: the ones in flight get a bounded time before the CTA leaves
+        if (tid == 0) {
+            atomicOr(status, ST_TIMEOUT);
+            for (int c = done; c < issued; ++c)
+                umma::mbar_wait_bounded(&full[c % RK_STAGES], (uint32_t)((c / RK_STAGES) & 1), RK_WAIT / 8);
         }
         return;
     }
-    T* mine = part + (size_t)(tl.w + it.w) * RK_BM * RK_BN;
+    const int r0 = tl.x * BM + ty * TM, c0 = tl.y * BN + tx;
+    if (tl.z == 1) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) mine[(ty + 16 * i) * RK_BN + tx + 16 * j] = acc[i][j];
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(&count[it.x], 1) == tl.z - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
+            for (int j = 0; j < TN; ++j)
+                if (r0 + i < n && c0 + CX * j < m) V[(size_t)(r0 + i) * ldv + c0 + CX * j] = acc[i][j];
+        return;
+    }
+    T* mine = part + (size_t)(tl.w + it.w) * BM * BN + (size_t)ty * TM * BN + tx;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = r0 + ty + 16 * i;
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int cc = c0 + tx + 16 * j;
-            const size_t off = (size_t)(ty + 16 * i) * RK_BN + tx + 16 * j;
-            T s = T(0);
-            for (int p = 0; p < tl.z; ++p) s += part[(size_t)(tl.w + p) * RK_BM * RK_BN + off];
-            if (r < n && cc < m) V[(size_t)r * ldv + cc] = s;
+        for (int j = 0; j < TN; ++j) mine[i * BN + CX * j] = acc[i][j];
+}
+
+// Tiles split into runs: V = the sum of the runs' partial tiles, in order.  blockIdx.y: the tile;
+// four columns per thread.
+template <typename T>
+__global__ void rg_reduce_kernel(const T* __restrict__ part, const int4* __restrict__ tiles, int bm, int bn,
+                                 T* __restrict__ V, int n, int m, int ldv) {
+    const int4 tl = tiles[blockIdx.y];
+    const int e = blockIdx.x * blockDim.x + threadIdx.x, c4 = bn >> 2;
+    if (tl.z == 1 || e >= bm * c4) return;
+    const int r = e / c4, c = 4 * (e - r * c4), row = tl.x * bm + r, col = tl.y * bn + c;
+    if (row >= n || col >= m) return;
+    const T* p = part + (size_t)tl.w * bm * bn + (size_t)r * bn + c;
+    T s[4] = {T(0), T(0), T(0), T(0)};
+    for (int q = 0; q < tl.z; ++q, p += (size_t)bm * bn) {
+        if constexpr (sizeof(T) == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(p);
+            s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
+        } else {
+            const double2 v = *reinterpret_cast<const double2*>(p), w = *reinterpret_cast<const double2*>(p + 2);
+            s[0] += v.x; s[1] += v.y; s[2] += w.x; s[3] += w.y;
         }
     }
-    if (tid == 0) count[it.x] = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (col + u < m) V[(size_t)row * ldv + col + u] = s[u];
+}
+
+// The normals of a draw in rg_kernel's layout: column block i / bn, then 16-row chunks of bn columns,
+// which is row k of bn columns throughout.  Rows and columns past n_act and m keep the zeros the
+// buffer was made with.
+template <typename O>
+__global__ void rg_normals_kernel(O* __restrict__ out, int bn, int n_act, int m, unsigned long long seed,
+                                  uint32_t stream, uint32_t frame) {
+    const int nq = (n_act + 3) / 4, total = nq * m;
+    const size_t krows = (size_t)(n_act + RK_KC - 1) / RK_KC * RK_KC;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const int q = t / m, i = t - q * m;
+        O z[4];
+        normals4<O>(seed, stream, frame, (uint32_t)i, (uint32_t)q, z);
+        O* o = out + ((size_t)(i / bn) * krows + 4 * q) * bn + i % bn;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (4 * q + r < n_act) o[(size_t)r * bn] = z[r];
+    }
+}
+
+// L (FP64, row-major) into rg_kernel's chunks: element (row block, chunk, k, row).
+template <typename T>
+__global__ void rg_pack_kernel(const double* __restrict__ L, T* __restrict__ Lt, int n, int bm, int lower) {
+    const int rb = blockIdx.y, nk = (n + RK_KC - 1) / RK_KC;
+    const int kend = lower ? min(n, (rb + 1) * bm) : n, chunks = (kend + RK_KC - 1) / RK_KC;
+    T* out = Lt + rk_prefix(rb, bm, nk, lower) * RK_KC * bm;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < chunks * RK_KC * bm; e += gridDim.x * blockDim.x) {
+        const int k = e / bm, row = rb * bm + e - k * bm;
+        out[e] = (row < n && k < kend) ? (T)L[(size_t)row * n + k] : T(0);
+    }
+}
+
+// Tile shape of a draw: FP32 rows by the size of the system (large tiles where there are enough of
+// them to fill the SMs), FP64 always 32; the columns split evenly into blocks of at most 128 (FP64:
+// 64), each rounded up to a width rg_launch has.
+struct RkShape {
+    int cx, tm, tn, bm, bn, ncb, nrb, nk;
+};
+RkShape rk_shape(int n, int m, size_t eb) {
+    RkShape s;
+    const int most = eb == 8 ? 64 : 128;
+    s.cx = eb == 8 ? 8 : 16;
+    s.tm = eb == 8 ? 1 : (n >= 2048 ? 8 : n >= 512 ? 4 : 2);
+    s.ncb = (m + most - 1) / most;
+    const int w = (m + s.ncb - 1) / s.ncb;
+    static const int w4[] = {2, 4, 6, 7, 8}, w8[] = {3, 5, 8};
+    const int* ws = eb == 8 ? w8 : w4;
+    while (*ws * s.cx < w) ++ws;
+    s.tn = *ws;
+    s.bm = RK_THREADS / s.cx * s.tm;
+    s.bn = s.cx * s.tn;
+    s.nrb = (n + s.bm - 1) / s.bm;
+    s.nk = (n + RK_KC - 1) / RK_KC;
+    return s;
+}
+
+template <typename T, typename F>
+int rk_with(const RkShape& s, F&& f) {     // f(kernel of this shape)
+#define RK_CASE(CX, TM, TN) \
+    if (s.cx == CX && s.tm == TM && s.tn == TN) return f(rg_kernel<T, CX, TM, TN>)
+    if constexpr (sizeof(T) == 8) {
+        RK_CASE(8, 1, 3);
+        RK_CASE(8, 1, 5);
+        RK_CASE(8, 1, 8);
+    } else {
+        RK_CASE(16, 2, 2); RK_CASE(16, 2, 4); RK_CASE(16, 2, 6); RK_CASE(16, 2, 7); RK_CASE(16, 2, 8);
+        RK_CASE(16, 4, 2); RK_CASE(16, 4, 4); RK_CASE(16, 4, 6); RK_CASE(16, 4, 7); RK_CASE(16, 4, 8);
+        RK_CASE(16, 8, 2); RK_CASE(16, 8, 4); RK_CASE(16, 8, 6); RK_CASE(16, 8, 7); RK_CASE(16, 8, 8);
+    }
+#undef RK_CASE
+    return LETKF_EINVAL;
+}
+
+int rk_smem_bytes(const RkShape& s, size_t eb) { return RK_STAGES * RK_KC * (s.bm + s.bn) * (int)eb; }
+
+template <typename T>
+int rg_product(letkf_ctx* c, const void* xi, void* V, cudaStream_t stream) {
+    const int n = c->n_act, m = c->m;
+    const RkShape s = rk_shape(n, m, sizeof(T));
+    const int rc = rk_with<T>(s, [&](auto* k) -> int {
+        k<<<c->rg_n_items, RK_THREADS, rk_smem_bytes(s, sizeof(T)), stream>>>(
+            (const T*)c->Lq, (const T*)xi, (T*)V, n, m, c->m_pad, c->lq_lower, (const int4*)c->rg_items,
+            (const int4*)c->rg_tiles, (T*)c->rg_part, c->d_status);
+        return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
+    });
+    if (rc || !c->rg_part) return rc;
+    rg_reduce_kernel<T><<<dim3((s.bm * (s.bn >> 2) + 255) / 256, s.nrb * s.ncb), 256, 0, stream>>>(
+        (const T*)c->rg_part, (const int4*)c->rg_tiles, s.bm, s.bn, (T*)V, n, m, c->m_pad);
+    return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
 
 // FP64 / FP32: V (n_act x m, ld m_pad) = L (n_act x n_act, row-major) * Xi (n_act x m, ld xld) on
@@ -360,41 +492,24 @@ int draw_perturbations_impl(letkf_ctx* c, unsigned long long frame) {
     return draw_perturbations_on(c, frame, c->Xi, c->V, c->stream);
 }
 
-// The per-frame product with the split-K kernel (work tables made by rg_prepare).
-int noise_gemm_split(letkf_ctx* c, const void* Xi, int gemm_type, void* V, cudaStream_t stream) {
+// The per-frame product (factor and work tables made by rg_prepare).
+int rg_draw_product(letkf_ctx* c, const void* Xi, void* V, cudaStream_t stream) {
     if (c->rg_n_items < 1) return LETKF_EINVAL;
-    const int m = c->m, na = c->n_act;
-    if (gemm_type == 0)
-        rg_splitk_kernel<double><<<c->rg_n_items, RK_THREADS, 0, stream>>>(
-            (const double*)c->Lq, (const double*)Xi, (double*)V, na, m, c->m_pad, c->m_pad, (const int4*)c->rg_items,
-            (const int4*)c->rg_tiles, (double*)c->rg_part, c->rg_count);
-    else if (gemm_type == 1)
-        rg_splitk_kernel<float><<<c->rg_n_items, RK_THREADS, 0, stream>>>(
-            (const float*)c->Lq, (const float*)Xi, (float*)V, na, m, c->m_pad, c->m_pad, (const int4*)c->rg_items,
-            (const int4*)c->rg_tiles, (float*)c->rg_part, c->rg_count);
-    else
-        return LETKF_EINVAL;
-    return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
+    return c->precision == LETKF_PREC_FP64 ? rg_product<double>(c, Xi, V, stream) : rg_product<float>(c, Xi, V, stream);
 }
 
 int draw_perturbations_on(letkf_ctx* c, unsigned long long frame, void* xi, void* v_out, cudaStream_t stream) {
     if (c->Lt) return noise_draw(c, frame, xi, v_out, stream);
-    const int gt = gemm_type_of(c);
-    const int nq = (c->n_act + 3) / 4;
-    const int g = grid_for((size_t)nq * c->m, 256);
-    if (gt == 0)
-        normals_kernel<double><<<g, 256, 0, stream>>>((double*)xi, c->m_pad, c->n_act, c->m, c->seed, 1u,
-                                                      (uint32_t)frame);
-    else
-        normals_kernel<float><<<g, 256, 0, stream>>>((float*)xi, c->m_pad, c->n_act, c->m, c->seed, 1u,
-                                                     (uint32_t)frame);
-    if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
-    return noise_gemm_split(c, xi, gt, v_out, stream);
+    NormalsNode nn;
+    normals_node_params(c, frame, xi, &nn);
+    if (cudaLaunchKernel(nn.params.func, nn.params.gridDim, nn.params.blockDim, nn.args, 0, stream) != cudaSuccess)
+        return LETKF_ECUDA;
+    return rg_draw_product(c, xi, v_out, stream);
 }
 
 int draw_product_on(letkf_ctx* c, const void* xi, void* v_out, cudaStream_t stream) {
     if (c->Lt) return noise_product(c, xi, v_out, stream);
-    return noise_gemm_split(c, xi, gemm_type_of(c), v_out, stream);
+    return rg_draw_product(c, xi, v_out, stream);
 }
 
 // Kernel-node parameters of the normals launch draw_perturbations_on makes for `frame` into xi
@@ -404,7 +519,7 @@ int normals_node_params(letkf_ctx* c, unsigned long long frame, void* xi, Normal
     const int gt = gemm_type_of(c);
     const int nq = (c->n_act + 3) / 4;
     nn->out = xi;
-    nn->ld = c->m_pad;
+    nn->ld = rk_shape(c->n_act, c->m, gt == 0 ? 8 : 4).bn;
     nn->n_act = c->n_act;
     nn->m = c->m;
     nn->seed = c->seed;
@@ -418,9 +533,9 @@ int normals_node_params(letkf_ctx* c, unsigned long long frame, void* xi, Normal
     nn->args[5] = &nn->stream_id;
     nn->args[6] = &nn->frame;
     cudaKernelNodeParams& kp = nn->params;
-    kp.func = gt == 0 ? (void*)normals_kernel<double> : (void*)normals_kernel<float>;
-    kp.gridDim = dim3(grid_for((size_t)nq * c->m, 256));
-    kp.blockDim = dim3(256);
+    kp.func = gt == 0 ? (void*)rg_normals_kernel<double> : (void*)rg_normals_kernel<float>;
+    kp.gridDim = dim3(grid_for((size_t)nq * c->m, 128));
+    kp.blockDim = dim3(128);
     kp.sharedMemBytes = 0;
     kp.kernelParams = nn->args;
     kp.extra = nullptr;
@@ -462,16 +577,23 @@ int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
     return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
 
-// Initial ensemble (Sect. 2.2): second instant = P0 xi0, first = a * second + L xi1, with
-// xi0, xi1 the Philox draws (stream 0, frames 0 and 1).  P0 defaults to L times the stationary
-// standard deviation of the AR model (1 / sqrt(1 - a^2) for AR(1)).
-RowGemmPlan rg_plan(int n, int m, bool lower, int* items, int* tiles) {
+RowGemmPlan rg_plan(int n, int m, bool lower, size_t eb, int* items, int* tiles) {
+    const RkShape s = rk_shape(n, m, eb);
+    auto chunks = [&](int rb) { return ((lower ? std::min(n, (rb + 1) * s.bm) : n) + RK_KC - 1) / RK_KC; };
+    // the shortest run with which all items fit on the chip at once
+    int run = 1;
+    for (;; ++run) {
+        long long n_items = 0;
+        for (int rb = 0; rb < s.nrb; ++rb) n_items += (chunks(rb) + run - 1) / run;
+        if (n_items * s.ncb <= RK_ITEMS || run >= s.nk) break;
+    }
     RowGemmPlan P;
-    const int nrb = (n + RK_BM - 1) / RK_BM, ncb = (m + RK_BN - 1) / RK_BN;
-    for (int rb = 0; rb < nrb; ++rb)
-        for (int cb = 0; cb < ncb; ++cb) {
-            const int kend = lower ? std::min(n, (rb + 1) * RK_BM) : n;
-            const int np = std::max(1, (kend + RK_KC - 1) / RK_KC);
+    P.l_elems = (rk_prefix(s.nrb - 1, s.bm, s.nk, lower) + chunks(s.nrb - 1)) * RK_KC * s.bm;
+    P.xi_elems = (size_t)s.ncb * s.nk * RK_KC * s.bn;
+    // the longest row blocks first
+    for (int rb = s.nrb - 1; rb >= 0; --rb)
+        for (int cb = 0; cb < s.ncb; ++cb) {
+            const int ch = chunks(rb), np = (ch + run - 1) / run;
             if (tiles) {
                 int* t = tiles + 4 * P.n_tiles;
                 t[0] = rb; t[1] = cb; t[2] = np; t[3] = np > 1 ? P.n_slots : 0;
@@ -479,41 +601,63 @@ RowGemmPlan rg_plan(int n, int m, bool lower, int* items, int* tiles) {
             for (int p = 0; p < np; ++p) {
                 if (items) {
                     int* it = items + 4 * P.n_items;
-                    it[0] = P.n_tiles; it[1] = p * RK_KC; it[2] = std::min(kend, (p + 1) * RK_KC); it[3] = p;
+                    it[0] = P.n_tiles; it[1] = (int)((long long)p * ch / np); it[2] = (int)((long long)(p + 1) * ch / np);
+                    it[3] = p;
                 }
                 ++P.n_items;
             }
             if (np > 1) P.n_slots += np;
             ++P.n_tiles;
         }
-    P.part_elems = (size_t)P.n_slots * RK_BM * RK_BN;
+    P.part_elems = (size_t)P.n_slots * s.bm * s.bn;
     return P;
 }
 
 size_t rg_bytes(int n, int m, bool lower, size_t eb) {
-    const RowGemmPlan P = rg_plan(n, m, lower, nullptr, nullptr);
-    return 16 * (size_t)P.n_items + 16 * (size_t)P.n_tiles + 4 * (size_t)P.n_tiles + eb * P.part_elems;
+    const RowGemmPlan P = rg_plan(n, m, lower, eb, nullptr, nullptr);
+    return 16 * (size_t)P.n_items + 16 * (size_t)P.n_tiles + eb * (P.part_elems + P.l_elems + P.xi_elems);
 }
 
-// Work tables, counters and scratch of the per-frame split-K draw.
-int rg_prepare(letkf_ctx* c, size_t eb) {
-    const RowGemmPlan P = rg_plan(c->n_act, c->m, c->lq_lower != 0, nullptr, nullptr);
+size_t rg_xi_bytes(int n, int m, size_t eb) {
+    const RkShape s = rk_shape(n, m, eb);
+    return eb * (size_t)s.ncb * s.nk * RK_KC * s.bn;
+}
+
+// The factor in rg_kernel's layout (L64: FP64 row-major, on the device), normals buffer, work tables
+// and scratch of the per-frame draw.
+template <typename T>
+int rg_prepare(letkf_ctx* c, const double* L64) {
+    const int n = c->n_act, m = c->m;
+    const bool lower = c->lq_lower != 0;
+    const RkShape s = rk_shape(n, m, sizeof(T));
+    const RowGemmPlan P = rg_plan(n, m, lower, sizeof(T), nullptr, nullptr);
     std::vector<int> items(4 * (size_t)P.n_items), tiles(4 * (size_t)P.n_tiles);
-    rg_plan(c->n_act, c->m, c->lq_lower != 0, items.data(), tiles.data());
-    if (cudaMalloc(&c->rg_items, items.size() * 4) != cudaSuccess ||
-        cudaMalloc(&c->rg_tiles, tiles.size() * 4) != cudaSuccess ||
-        cudaMalloc((void**)&c->rg_count, (size_t)P.n_tiles * 4) != cudaSuccess)
+    rg_plan(n, m, lower, sizeof(T), items.data(), tiles.data());
+    if (cudaMalloc(&c->Lq, P.l_elems * sizeof(T)) != cudaSuccess ||
+        cudaMalloc(&c->Xi, P.xi_elems * sizeof(T)) != cudaSuccess ||
+        cudaMalloc(&c->rg_items, items.size() * 4) != cudaSuccess ||
+        cudaMalloc(&c->rg_tiles, tiles.size() * 4) != cudaSuccess)
         return LETKF_ENOMEM;
-    if (P.part_elems && cudaMalloc(&c->rg_part, P.part_elems * eb) != cudaSuccess) return LETKF_ENOMEM;
-    if (cudaMemcpy(c->rg_items, items.data(), items.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(c->rg_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(c->rg_count, 0, (size_t)P.n_tiles * 4) != cudaSuccess)
+    if (P.part_elems && cudaMalloc(&c->rg_part, P.part_elems * sizeof(T)) != cudaSuccess) return LETKF_ENOMEM;
+    if (cudaMemset(c->Xi, 0, P.xi_elems * sizeof(T)) != cudaSuccess ||
+        cudaMemcpy(c->rg_items, items.data(), items.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(c->rg_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
         return LETKF_ECUDA;
+    rg_pack_kernel<T><<<dim3(64, s.nrb), 256, 0, c->stream>>>(L64, (T*)c->Lq, n, s.bm, lower ? 1 : 0);
+    if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     c->rg_n_items = P.n_items;
-    c->device_bytes += rg_bytes(c->n_act, c->m, c->lq_lower != 0, eb);
-    return LETKF_OK;
+    c->device_bytes += rg_bytes(n, m, lower, sizeof(T));
+    // (the attribute belongs to the kernel: every context with this shape sets the same value)
+    return rk_with<T>(s, [&](auto* k) -> int {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, rk_smem_bytes(s, sizeof(T))) == cudaSuccess
+                   ? LETKF_OK
+                   : LETKF_ECUDA;
+    });
 }
 
+// Initial ensemble (Sect. 2.2): second instant = P0 xi0, first = a * second + L xi1, with
+// xi0, xi1 the Philox draws (stream 0, frames 0 and 1).  P0 defaults to L times the stationary
+// standard deviation of the AR model (1 / sqrt(1 - a^2) for AR(1)).
 int init_ensemble(letkf_ctx* c, const double* L_host, const double* P0_host) {
     const int na = c->n_act, m = c->m;
     const bool f64 = c->precision == LETKF_PREC_FP64;
@@ -532,24 +676,20 @@ int init_ensemble(letkf_ctx* c, const double* L_host, const double* P0_host) {
         void* tmp = nullptr;
         if (cudaMalloc(&tmp, nn * 8) != cudaSuccess) return LETKF_ENOMEM;
         cudaMemcpy(tmp, L_host, nn * 8, cudaMemcpyHostToDevice);
-        const size_t lbytes = nn * eb;
-        if (cudaMalloc(&c->Lq, lbytes) != cudaSuccess) { cudaFree(tmp); return LETKF_ENOMEM; }
-        c->device_bytes += lbytes;
-        const int g = grid_for(nn, 256);
-        if (f64)
-            cudaMemcpyAsync(c->Lq, tmp, nn * 8, cudaMemcpyDeviceToDevice, c->stream);
-        else
-            f64_to_f32<<<g, 256, 0, c->stream>>>((const double*)tmp, (float*)c->Lq, nn);
+        int rc = LETKF_OK;
+        if (c->path == LETKF_PATH_GLOBAL) {   // draws with its tiled GEMM, from tiles of the FP32 factor
+            if (cudaMalloc(&c->Lq, nn * eb) != cudaSuccess) {
+                rc = LETKF_ENOMEM;
+            } else {
+                c->device_bytes += nn * eb;
+                f64_to_f32<<<grid_for(nn, 256), 256, 0, c->stream>>>((const double*)tmp, (float*)c->Lq, nn);
+            }
+        } else {
+            rc = f64 ? rg_prepare<double>(c, (const double*)tmp) : rg_prepare<float>(c, (const double*)tmp);
+        }
         cudaStreamSynchronize(c->stream);
         cudaFree(tmp);
-        const size_t xib = (size_t)na * row;
-        if (cudaMalloc(&c->Xi, xib) != cudaSuccess) return LETKF_ENOMEM;
-        cudaMemset(c->Xi, 0, xib);
-        c->device_bytes += xib;
-        if (c->path != LETKF_PATH_GLOBAL) {   // the global path draws with its tiled GEMM
-            const int rc = rg_prepare(c, eb);
-            if (rc) return rc;
-        }
+        if (rc) return rc;
     }
     // the initial ensemble itself is formed at full state precision (FP64 or FP32 GEMMs)
     const int gt = f64 ? 0 : 1;
