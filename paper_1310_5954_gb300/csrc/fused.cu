@@ -178,14 +178,18 @@ __device__ __forceinline__ void issue_product(uint32_t d_tmem, const unsigned ch
     const uint32_t w_lbo = w_mn ? (uint32_t)(N >> 3) * 128u : 128u;
     const uint32_t w_sbo = w_mn ? 128u : x_sbo;
     const uint32_t w_step = 2u * w_lbo;
-    const unsigned char* xs[3] = {xh, xh, xl};
-    const unsigned char* ws[3] = {wh, wl, wh};
-    uint32_t acc = first_term > 0 ? 1u : 0u;
     // consecutive K steps differ only in the start-address field (bits 0-13, in 16-byte units)
     const uint64_t x_inc = 256u >> 4, w_inc = w_step >> 4;
-    for (int t = first_term; t < nterms; ++t) {
-        uint64_t xd = sdesc(smem_u32(xs[t]), 128u, x_sbo), wd = sdesc(smem_u32(ws[t]), w_lbo, w_sbo);
-        for (int ks = 0; ks < (K >> 4); ++ks) {
+    const uint64_t xdh = sdesc(smem_u32(xh), 128u, x_sbo), xdl = sdesc(smem_u32(xl), 128u, x_sbo);
+    const uint64_t wdh = sdesc(smem_u32(wh), w_lbo, w_sbo), wdl = sdesc(smem_u32(wl), w_lbo, w_sbo);
+    const int nk = K >> 4;
+    uint32_t acc = first_term > 0 ? 1u : 0u;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        if (t < first_term || t >= nterms) continue;
+        uint64_t xd = t == 2 ? xdl : xdh, wd = t == 1 ? wdl : wdh;
+#pragma unroll 1
+        for (int ks = 0; ks < nk; ++ks) {
             mma_bf16(d_tmem, xd, wd, idesc, acc);
             acc = 1;
             xd += x_inc;
@@ -475,6 +479,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     const SysDesc A = ctl->sd;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int row = 32 * (warp & 3) + lane, hh = warp >> 2;
+    const int uwarp = uniform_warp();
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
     uint32_t ph_mma = *ph_mma_io;
     float* vec = reinterpret_cast<float*>(smem + A.off_vec);
@@ -532,7 +537,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     // Y T (unless with_y is false) and T Z, committed together
     auto yt_tz = [&](unsigned char* Yh_, unsigned char* Yl_, unsigned char* Th_, unsigned char* Tl_,
                      unsigned char* Zh_, unsigned char* Zl_, bool with_y) -> bool {
-        if (tid == 0) {
+        if (uwarp == 0 && elect_one()) {
             tc_fence_after();
             if (with_y) issue_product(tbase + TM_Y, Yh_, Yl_, Th_, Tl_, NP, NP, 3, 1);
             issue_product(tbase + TM_Z, Th_, Tl_, Zh_, Zl_, NP, NP, 3, 1);
@@ -656,7 +661,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     unsigned char* Sg_l = big + A.sz_opg;
     write_S(Sg_h, Sg_l, Hs4 ? Hs4 : Xs4);
     to_mma();
-    if (tid == 0) {
+    if (uwarp == 0 && elect_one()) {
         tc_fence_after();
         issue_product(tbase + TM_G, Sg_h, Sg_l, Sg_h, Sg_l, MP, NP, A.gram_terms, 0);   // K = S S^T
         mma_commit(&ctl->bar_mma);
@@ -678,7 +683,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     if (A.gram_terms < 3 && 1.f + sqrtf(fro) / c > A.s_split) {
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) {
+        if (uwarp == 0 && elect_one()) {
             tc_fence_after();
             issue_product(tbase + TM_G, Sg_h, Sg_l, Sg_h, Sg_l, MP, NP, 3, 0, 1);
             mma_commit(&ctl->bar_mma);
@@ -732,7 +737,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     }
     if (more)
     for (; it < A.max_it; ++it) {
-        if (tid == 0) {
+        if (uwarp == 0 && elect_one()) {
             tc_fence_after();
             issue_product(tbase + TM_P, Zh, Zl, Yh, Yl, NP, NP, 3, 1);
             mma_commit(&ctl->bar_mma);
@@ -953,7 +958,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     }
     to_mma();
     for (int k = 0; k < 6; ++k) {
-        if (tid == 0) {
+        if (uwarp == 0 && elect_one()) {
             tc_fence_after();
             issue_product(tbase + TM_P, Yh, Yl, Th, Tl, NP, NP, 3, 1);     // Q = M X
             mma_commit(&ctl->bar_mma);
@@ -978,7 +983,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         if (k > 0 && sqrtf(r2) < 1e-6f * (float)P) break;
         const bool last = r2 < 1e-6f * (float)P;     // the update lands ||R||_F under the bound
         to_mma();
-        if (tid == 0) {
+        if (uwarp == 0 && elect_one()) {
             tc_fence_after();
             issue_product(tbase + TM_G, Th, Tl, Zh, Zl, NP, NP, 3, 1);     // X R
             mma_commit(&ctl->bar_mma);
@@ -1019,7 +1024,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     }
     if (!A.hs_w) write_S(Wh, Wl, Xs4);
     to_mma();
-    if (tid == 0) {
+    if (uwarp == 0 && elect_one()) {
         tc_fence_after();
         issue_product(tbase + TM_Y, Zt_h, Zt_l, Wh, Wl, NP, MP, 3, 1);    // W = (Z / sqrt(c)) S
         mma_commit(&ctl->bar_mma);
@@ -1086,7 +1091,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         store8(A1h, A1l, e, kc * 8, MP, v, A.tr_terms > 1);
     }
     to_mma();
-    if (tid == 0) {
+    if (uwarp == 0 && elect_one()) {
         tc_fence_after();
         issue_product(tbase + TM_P, A1h, A1l, Wh, Wl, MP, NP, A.tr_terms, 0);   // P1 = X'_E W^T
         mma_commit(&ctl->bar_mma);
@@ -1103,7 +1108,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         if (row < NP) store8(Xh_op, Xl_op, row, col0 + 8 * q8, NP, xv, true);
     }
     to_mma();
-    if (tid == 0) {
+    if (uwarp == 0 && elect_one()) {
         tc_fence_after();
         issue_product(tbase + TM_Y, Xh_op, Xl_op, Wh, Wl, NP, MP, 3, 1);   // XW = (I + Z)^-1 W
         mma_commit(&ctl->bar_mma);
@@ -1132,7 +1137,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
                 if (mcol0 + 8 * q8 + u < m) A.cap[CAP_HDR + m + (P + row) * m + mcol0 + 8 * q8 + u] = wv[u];
     }
     to_mma();
-    if (tid == 0) {
+    if (uwarp == 0 && elect_one()) {
         tc_fence_after();
         issue_product(tbase + TM_Y, A2h, A2l, Wh, Wl, NP, MP, A.tr_terms, 1);   // P3 = P1 (XW)
         mma_commit(&ctl->bar_mma);
@@ -1547,6 +1552,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
     extern __shared__ __align__(1024) unsigned char smem[];
     Ctrl* ctl = reinterpret_cast<Ctrl*>(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int uwarp = uniform_warp();
     const int row = 32 * (warp & 3) + lane;          // TMEM lane / matrix row of this thread
     const int hh = warp >> 2;                        // column half of this thread
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
@@ -1758,7 +1764,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             // here, filled under the Gram product (each subaperture writes its own four slots)
             for (int j = tid; j < n_h; j += FT) inc4[j] = make_uchar4(0xFF, 0xFF, 0xFF, 0xFF);
             __syncthreads();
-            if (tid == 0) {
+            if (uwarp == 0 && elect_one()) {
                 tc_fence_after();
                 issue_product(tbase + TM_G, opg_h, opg_l, opg_h, opg_l, KP, NP, A.gram_terms, 0);
                 mma_commit(&ctl->bar_mma);
@@ -1792,7 +1798,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 // conditioning bound too large for single BF16 operands: add the high/low cross terms
                 tc_fence_before();
                 __syncthreads();
-                if (tid == 0) {
+                if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
                     issue_product(tbase + TM_G, opg_h, opg_l, opg_h, opg_l, KP, NP, 3, 0, 1);
                     mma_commit(&ctl->bar_mma);
@@ -1846,7 +1852,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 fence_async_smem();
                 tc_fence_before();
                 __syncthreads();
-                if (tid == 0) {
+                if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
                     issue_product(tbase + TM_Y, Yh, Yl, Zh, Zl, NP, NP, 3, 1);     // Y_1 = Y_0 T_0
                     mma_commit(&ctl->bar_mma);
@@ -1863,7 +1869,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             }
             if (z_state != 0)
             for (; it < A.max_it; ++it) {
-                if (tid == 0) {
+                if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
                     issue_product(tbase + TM_P, Zh, Zl, Yh, Yl, NP, NP, 3, 1);
                     mma_commit(&ctl->bar_mma);
@@ -1916,7 +1922,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 // are skipped
                 const bool last = rn < ns_last;
                 if (last) {
-                    if (tid == 32) {
+                    if (uwarp == 1 && elect_one()) {
                         tc_fence_after();
                         issue_product(tbase + TM_Z, Th, Tl, Zh, Zl, NP, NP, 3, 1);     // T Z
                         mma_commit(&ctl->bar_mma2);
@@ -1929,11 +1935,11 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 }
                 // the two products are issued by threads of different warps, so their issue loops
                 // (one tcgen05.mma per K step and BF16 term) overlap
-                if (tid == 0) {
+                if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
                     issue_product(tbase + TM_Y, Yh, Yl, Th, Tl, NP, NP, 3, 1);     // Y T
                     mma_commit(&ctl->bar_mma);
-                } else if (tid == 32) {
+                } else if (uwarp == 1 && elect_one()) {
                     tc_fence_after();
                     issue_product(tbase + TM_Z, Th, Tl, Zh, Zl, NP, NP, 3, 1);     // T Z
                     mma_commit(&ctl->bar_mma2);
@@ -2162,7 +2168,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             __syncthreads();
             // the product is issued from warp 1, so that its issue loop (one tcgen05.mma per K step
             // and term, ~2.7 k cycles) overlaps warp 0's fetch of the next item
-            if (tid == 32) {
+            if (uwarp == 1 && elect_one()) {
                 tc_fence_after();
                 issue_product(tbase + TM_P, Ah, Al, Bh, Bl, NP, NP, A.tr_terms, 1);   // X'_E T
                 mma_commit(&ctl->bar_mma);
@@ -2386,7 +2392,7 @@ __global__ void __launch_bounds__(FT, 1) umma_selftest_kernel(const float* __res
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = ctl->tmem_base;
-    if (tid == 0) {
+    if (uniform_warp() == 0 && elect_one()) {
         issue_product(tbase, a_h, a_l, b_h, b_l, K, N, terms, b_mn);
         mma_commit(&ctl->bar_mma);
     }

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const GemmArgs g) {
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) uint64_t full[L::STAGES], empty[L::STAGES], done;
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, issued;        // issued: stages the producer filled (for the drain on abort)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (g.next_flag && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
         // this launch decides whether the next step runs (see GemmArgs), also when it does
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const GemmArgs g) {
             mbar_init(&empty[s], 1);
         }
         mbar_init(&done, 1);
-        abort_flag = 0;
+        abort_flag = issued = 0;
         fence_mbar_init();
     }
     if (warp == 0) {
@@ -121,8 +121,8 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const GemmArgs g) {
     const size_t b_next = (size_t)g.b_nkb * TILE_B;   // the second 128-row tile of a 256-row block
     const uint8_t* b_hi = g.b_hi + b_row_tile + b_half;
     const uint8_t* b_lo = g.b_lo ? g.b_lo + b_row_tile + b_half : nullptr;
-    int issued = 0;   // stages the producer filled (for the drain on abort)
-    if (warp == 0 && lane == 0) {
+    const int uwarp = uniform_warp();
+    if (uwarp == 0 && elect_one()) {
         for (int kb = 0; kb < nkb; ++kb) {
             const int s = kb % L::STAGES;
             if (kb >= L::STAGES && !mbar_wait_bounded(&empty[s], ((kb / L::STAGES) - 1) & 1, GEMM_WAIT)) {
@@ -152,9 +152,9 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const GemmArgs g) {
                     bulk_g2s(st + 2 * TILE_B + L::B_BYTES, b_lo + boff, L::B_BYTES, &full[s]);
                 }
             }
-            issued = kb + 1;
+            *reinterpret_cast<volatile int*>(&issued) = kb + 1;
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (uwarp == 1 && elect_one()) {
         const uint32_t idesc = idesc_bf16(128, BN, g.b_mn);
         // K-major B: K-adjacent core matrices 128 B apart, row-adjacent 1024 B, a K step 256 B;
         // MN-major B: N-adjacent core matrices 128 B apart, K-adjacent 1024 B, a K step 2048 B

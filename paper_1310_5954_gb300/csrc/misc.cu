@@ -259,7 +259,8 @@ __global__ void __launch_bounds__(RK_THREADS, 2) rg_kernel(const T* __restrict__
         umma::fence_mbar_init();
     }
     __syncthreads();
-    if (tid == 0)
+    const int uwarp = umma::uniform_warp();
+    if (uwarp == 0 && umma::elect_one())
         for (int c = 0; c < nc && c < RK_STAGES; ++c) load(c);
     T acc[TM][TN];
 #pragma unroll
@@ -297,8 +298,8 @@ __global__ void __launch_bounds__(RK_THREADS, 2) rg_kernel(const T* __restrict__
         }
         done = c + 1;
         if (__syncthreads_or(!ok)) break;          // the stage is read by every warp: it can be refilled
-        if (tid == 0 && c + RK_STAGES < nc) {
-            load(c + RK_STAGES);
+        if (c + RK_STAGES < nc) {
+            if (uwarp == 0 && umma::elect_one()) load(c + RK_STAGES);
             issued = c + RK_STAGES + 1;
         }
     }

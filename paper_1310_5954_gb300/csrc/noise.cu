@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(NT) noise_kernel(const __grid_constant__ Noise
     Ctl* ctl = reinterpret_cast<Ctl*>(smem);
     unsigned char* stage0 = smem + 1024;
     const int stage_b = TILE_A + a.tile_b;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, uwarp = uniform_warp();
     const uint32_t ncols = a.np <= 128 ? 128u : 256u;
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(NT) noise_kernel(const __grid_constant__ Noise
     for (int it = blockIdx.x; it < a.n_items; it += gridDim.x) {
         const int4 item = a.items[it];
         const int J = item.x, kc0 = item.y, nch = item.z - item.y, slot = item.w;
-        if (tid == 0) {                       // producer
+        if (uwarp == 0 && elect_one()) {      // producer
             const unsigned char* lrow = a.Lt + (size_t)(a.prefix[J] + kc0) * TILE_A;
             for (int t = 0; t < nch; ++t) {
                 const int g = g0 + t, s = g % STAGES;
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(NT) noise_kernel(const __grid_constant__ Noise
                 bulk_g2s(st, lrow + (size_t)t * TILE_A, TILE_A, &ctl->bl[s]);
                 bulk_g2s(st + TILE_A, a.Xi + (size_t)(kc0 + t) * a.tile_b, (uint32_t)a.tile_b, &ctl->bl[s]);
             }
-        } else if (tid == 32) {               // tensor-core issue
+        } else if (uwarp == 1 && elect_one()) {   // tensor-core issue
             for (int t = 0; t < nch; ++t) {
                 const int g = g0 + t, s = g % STAGES;
                 if (!mbar_wait_bounded(&ctl->bl[s], (uint32_t)((g / STAGES) & 1), WAIT_CYCLES)) {

@@ -55,6 +55,24 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     return true;
 }
 
+// One lane of a converged warp.  Asynchronous instructions whose operands live in uniform registers
+// (tcgen05.mma, tcgen05.commit, bulk copies) are issued under `warp-uniform condition && elect_one()`:
+// the compiler then knows that a single thread is active.  Under `threadIdx.x == 0` it does not, and
+// wraps each of them in a loop over the active lanes: measured back to back, a 128 x N x 16
+// tcgen05.mma then takes 250 cycles whatever N is, against 61 (N = 112), 65 (N = 128) and 129 (N = 256)
+// when elected, which is the tensor pipe's own rate.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+// This thread's warp index, known to be the same in all its lanes.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 // ---------------------------------------------------------------- bulk copy
 // Global -> shared 1-D bulk copy; bytes a multiple of 16, both addresses 16-byte aligned.
 // Completion is counted in bytes on the mbarrier.
