@@ -27,6 +27,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -94,6 +95,9 @@ struct SysDesc {
     int off_hs;          // dual form: the halo anomalies' rows in the big region beside the Gram operand, or -1
     int off_hs2;         // dual form: the same rows beside Z's FP32 rows for the mean weights, or -1
     int hs_w;            // dual form: the same rows fit below the W operand (at the big region's start)
+    int off_pst;         // m x m form: FP32 rows of the transform's product for the epilogue (big region)
+    int off_xh3;         // two CTAs per SM: the halo rows once more, for the mean weights (big region)
+    int off_sxe, off_sxh;   // two CTAs per SM: own and halo rows of a SIMT domain (big region)
     // test instrument: when cap is set, the analysis of domain cap_dom writes what it computed
     // (header, mean weights, transform or its factors; layout in letkf_set_capture) to cap
     float* cap;
@@ -150,9 +154,7 @@ struct FusedBatch {
 
 // Write 8 consecutive K-values of row `row` into the hi (and optionally lo) operand: hi is the
 // BF16 rounding of v, lo the BF16 rounding of v - hi.
-__device__ __forceinline__ void store8(unsigned char* hi_base, unsigned char* lo_base, int row, int k0, int K,
-                                       const float* v, bool with_lo) {
-    uint32_t h[4], l[4];
+__device__ __forceinline__ void split8(const float* v, uint32_t (&h)[4], uint32_t (&l)[4]) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const __nv_bfloat162 hv = __floats2bfloat162_rn(v[2 * u], v[2 * u + 1]);
@@ -161,9 +163,17 @@ __device__ __forceinline__ void store8(unsigned char* hi_base, unsigned char* lo
         const __nv_bfloat162 lv = __floats2bfloat162_rn(v[2 * u] - f.x, v[2 * u + 1] - f.y);
         l[u] = *reinterpret_cast<const uint32_t*>(&lv);
     }
-    const uint32_t off = op_offset(row, k0, K);
+}
+__device__ __forceinline__ void store8_at(unsigned char* hi_base, unsigned char* lo_base, uint32_t off, const float* v,
+                                          bool with_lo) {
+    uint32_t h[4], l[4];
+    split8(v, h, l);
     *reinterpret_cast<uint4*>(hi_base + off) = make_uint4(h[0], h[1], h[2], h[3]);
     if (with_lo) *reinterpret_cast<uint4*>(lo_base + off) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+__device__ __forceinline__ void store8(unsigned char* hi_base, unsigned char* lo_base, int row, int k0, int K,
+                                       const float* v, bool with_lo) {
+    store8_at(hi_base, lo_base, op_offset(row, k0, K), v, with_lo);
 }
 
 // Issue D = sum over terms of X_t * op(W_t) on a (MT x N) tile with K columns (no commit).
@@ -193,6 +203,30 @@ __device__ __forceinline__ void issue_product(uint32_t d_tmem, const unsigned ch
             mma_bf16(d_tmem, xd, wd, idesc, acc);
             acc = 1;
             xd += x_inc;
+            wd += w_inc;
+        }
+    }
+}
+
+// The three-term product with X in tensor memory (high parts from column xh, low parts from xl) and W
+// K rows x N columns: the same terms in the same order.
+__device__ __forceinline__ void issue_product_ta(uint32_t d_tmem, uint32_t xh, uint32_t xl, const unsigned char* wh,
+                                                 const unsigned char* wl, int K, int N) {
+    const uint32_t idesc = idesc_bf16(MT, N, 1);
+    const uint32_t w_lbo = (uint32_t)(N >> 3) * 128u;
+    const uint64_t w_inc = (2u * w_lbo) >> 4;
+    const uint64_t wdh = sdesc(smem_u32(wh), w_lbo, 128u), wdl = sdesc(smem_u32(wl), w_lbo, 128u);
+    const int nk = K >> 4;
+    uint32_t acc = 0u;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        uint64_t wd = t == 1 ? wdl : wdh;
+        uint32_t xa = t == 2 ? xl : xh;
+#pragma unroll 1
+        for (int ks = 0; ks < nk; ++ks) {
+            mma_bf16_ta(d_tmem, xa, wd, idesc, acc);
+            acc = 1;
+            xa += 8;
             wd += w_inc;
         }
     }
@@ -382,10 +416,8 @@ __device__ __forceinline__ void simt_rows(const SysDesc& A, int e0, int n_own) {
 // Warp 0, all 32 lanes: bulk copies of domain d's halo rows (observed instant) and own rows, lane
 // l issuing rows l, l + 32, ... once lane 0 has announced the bytes on the barrier (one thread
 // issuing them all, with a table read per row, held the CTA ~10 k cycles per domain).
-__device__ __forceinline__ void issue_loads(const SysDesc& A, int d, unsigned char* smem, uint64_t* bar) {
+__device__ __forceinline__ void issue_loads(const SysDesc& A, int d, float* Xh, float* XE, uint64_t* bar) {
     const int lane = threadIdx.x & 31;
-    float* Xh = reinterpret_cast<float*>(smem + A.off_xh);
-    float* XE = reinterpret_cast<float*>(smem + A.off_xe);
     const int e0 = A.tab.own_off[d], n_own = A.tab.own_off[d + 1] - e0;
     const int h0 = A.tab.halo_off[d], n_h = A.tab.halo_off[d + 1] - h0;
     const int n_e = (A.with_forecast && A.a2 == 0.f) ? n_own : 2 * n_own;   // AR(2) needs both instants
@@ -421,7 +453,8 @@ __device__ void fetch_item(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, 
         ctl->dom = d;
     }
     if (!A.dual && A.tab.obs_off[d + 1] > A.tab.obs_off[d] && A.off_big <= busy_from) {
-        issue_loads(A, d, smem, &ctl->bar_load);
+        issue_loads(A, d, reinterpret_cast<float*>(smem + A.off_xh), reinterpret_cast<float*>(smem + A.off_xe),
+                    &ctl->bar_load);
         if (lane == 0) ctl->loaded = 1;
     }
 }
@@ -1339,9 +1372,10 @@ __device__ __forceinline__ void own_row_means(const SysDesc& A, const float* XE,
 // w_bar, xe_mean and uvec like the tensor-core form, fetches the next work item once the halo and
 // own rows are consumed, and returns the n_e x m rows of X'_E T (row stride *ld_out) in shared
 // memory.
+template <bool TWO>
 __device__ __noinline__ const float* analyse_simt(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, int d,
                                                   int* ld_out) {
-    const SysDesc& A = ctl->sd;
+    const SysDesc& A = TWO ? B.sys[ctl->sys] : ctl->sd;
     const int tid = threadIdx.x;
     const int m = A.m;
     const float c = (float)(m - 1);
@@ -1356,8 +1390,8 @@ __device__ __noinline__ const float* analyse_simt(const FusedBatch& B, Ctrl* ctl
     float* uvec = vec + 1152;
     float* dtv = vec + 1280;
     float* tvv = vec + 1408;
-    const float* XE = reinterpret_cast<const float*>(smem + A.off_xe);
-    const float* Xh = reinterpret_cast<const float*>(smem + A.off_xh);
+    const float* XE = reinterpret_cast<const float*>(smem + (TWO ? A.off_big + A.off_sxe : A.off_xe));
+    const float* Xh = reinterpret_cast<const float*>(smem + (TWO ? A.off_big + A.off_sxh : A.off_xh));
     float* ws = reinterpret_cast<float*>(smem + A.off_big);
     const int e0 = A.tab.own_off[d], n_own = A.tab.own_off[d + 1] - e0;
     const int o0 = A.tab.obs_off[d], n_obs = A.tab.obs_off[d + 1] - o0;
@@ -1507,7 +1541,7 @@ __device__ __noinline__ const float* analyse_simt(const FusedBatch& B, Ctrl* ctl
         E[e * lm + i] = XE[(size_t)e * A.m_pad + i] - xe_mean[e];
     }
     __syncthreads();
-    if ((tid >> 5) == 0) fetch_item(B, ctl, smem, A.off_big);
+    if (!TWO && (tid >> 5) == 0) fetch_item(B, ctl, smem, A.off_big);
     // ---- transform
     const float rs = rsqrtf(s_ns);    // T = Z / sqrt(s_ns) (m x m form); Z / sqrt(s_ns) = (I + K/c)^(-1/2)
     *ld_out = lm;
@@ -1548,7 +1582,22 @@ __device__ __noinline__ const float* analyse_simt(const FusedBatch& B, Ctrl* ctl
     return E;
 }
 
-__global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ FusedBatch B) {
+// TWO: two CTAs per SM (half the shared memory and tensor memory each), for m x m systems that fit
+// (fused_layout2) and launches of more domains than SMs.  A domain is a chain of dependent products,
+// read-outs and barriers that leaves an SM's issue slots 72 % idle, so two chains side by side take
+// little longer than one.  The arithmetic is the same, bit for bit; what differs is where things live:
+//   - Y's left operand of Y T is kept in tensor memory, so that T's operand takes the place of Y's in
+//     shared memory: two operand pairs instead of three;
+//   - P and Y T share an accumulator, T Z goes over Y's left operand once Y T is done;
+//   - rows are read by all warps when they are needed (the halo rows centred on the way in) instead of
+//     by bulk copies under the previous domain; where the halo rows have to give way to the iteration's
+//     operands they are read once more for the mean weights.
+// Measured, 332 domains of m = 100: 118 k cycles for two domains side by side (92 k for one before), the
+// frame 156 -> 130 us; two such systems in one launch 294 -> 229 us.
+template <bool TWO>
+__global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_constant__ FusedBatch B) {
+    constexpr int tG = TM_G, tP = TWO ? 0 : TM_P, tY = TWO ? 0 : TM_Y, tZ = TWO ? 128 : TM_Z;
+    constexpr uint32_t tmem_cols = TWO ? TM_COLS / 2 : TM_COLS;
     extern __shared__ __align__(1024) unsigned char smem[];
     Ctrl* ctl = reinterpret_cast<Ctrl*>(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1565,7 +1614,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc(&ctl->tmem_base, TM_COLS);
+        tmem_alloc(&ctl->tmem_base, tmem_cols);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -1577,17 +1626,20 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
     // read what this kernel writes)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    if (warp == 0) fetch_item(B, ctl, smem, 1 << 30);
+    constexpr int fetch_all = TWO ? -1 : 1 << 30;    // TWO: an item's rows are copied when its turn comes
+    if (warp == 0) fetch_item(B, ctl, smem, fetch_all);
     __syncthreads();
 
     while (ctl->item < B.n_items && !ctl->abort) {
-        {
+        if constexpr (!TWO) {
             const uint32_t* src = reinterpret_cast<const uint32_t*>(&B.sys[ctl->sys]);
             uint32_t* dst = reinterpret_cast<uint32_t*>(&ctl->sd);
             for (int t = tid; t < (int)(sizeof(SysDesc) / 4); t += FT) dst[t] = src[t];
             __syncthreads();
         }
-        const SysDesc A = ctl->sd;   // by value: fields stay in registers across barriers
+        // by value: fields stay in registers across barriers; TWO, with half the registers, reads the
+        // constant bank where it needs them
+        typename std::conditional<TWO, const SysDesc&, const SysDesc>::type A = TWO ? B.sys[ctl->sys] : ctl->sd;
         const int d = ctl->dom;
         float* vec = reinterpret_cast<float*>(smem + A.off_vec);
         float* xh_mean = vec;            // 256 (halo actuators)
@@ -1600,8 +1652,9 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
         float* uvec = vec + 1152;        // 128 (mean update of each own row)
         float* dtv = vec + 1280;         // 128 (innovation d / sigma of each observed slope)
         float* tvv = vec + 1408;         // 128 (slope-space residual)
-        float* XE = reinterpret_cast<float*>(smem + A.off_xe);
-        float* Xh = reinterpret_cast<float*>(smem + A.off_xh);   // halo anomalies, kept for the refinement
+        float* XE = reinterpret_cast<float*>(smem + (TWO ? A.off_big + A.off_xe : A.off_xe));
+        float* Xh = reinterpret_cast<float*>(smem + (TWO ? A.off_big + A.off_xh : A.off_xh));   // halo anomalies, kept
+                                                                                                // for the refinement
         // Operand buffers hold only the rows that can be non-zero (NP, or RA for the transform's A);
         // a 128-row MMA reads the rows beyond them from whatever follows, which only feeds output
         // rows that are never used.
@@ -1612,12 +1665,13 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
         unsigned char* Yl = big + A.sz_op;
         unsigned char* Zh = big + 2 * A.sz_op;
         unsigned char* Zl = big + 3 * A.sz_op;
-        unsigned char* Th = big + 4 * A.sz_op;
-        unsigned char* Tl = big + 5 * A.sz_op;
-        unsigned char* Ah = big;                 // transform operands reuse the NS region
-        unsigned char* Al = big + A.sz_a;
-        unsigned char* Bh = big + 2 * A.sz_a;
-        unsigned char* Bl = big + 2 * A.sz_a + A.sz_op;
+        unsigned char* Th = TWO ? Yh : big + 4 * A.sz_op;
+        unsigned char* Tl = TWO ? Yl : big + 5 * A.sz_op;
+        // transform operands reuse the NS region (TWO: B first, which leaves the own rows alone)
+        unsigned char* Ah = TWO ? big + 2 * A.sz_op : big;
+        unsigned char* Al = Ah + A.sz_a;
+        unsigned char* Bh = TWO ? big : big + 2 * A.sz_a;
+        unsigned char* Bl = Bh + A.sz_op;
         const int m = A.m, NP = A.NP, KP = A.KP, half = NP / 2, nq = half / 8;
         const int col0 = hh * half;                      // first column of this thread's half-row
         const float c = (float)(m - 1);
@@ -1631,11 +1685,55 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
         if (n_obs == 0) {
             simt_rows(A, e0, n_own);
             __syncthreads();
-            if (warp == 0) fetch_item(B, ctl, smem, 1 << 30);
+            if (warp == 0) fetch_item(B, ctl, smem, fetch_all);
             __syncthreads();
             continue;
         }
-        if (warp == 0 && !A.dual && !ctl->loaded) issue_loads(A, d, smem, &ctl->bar_load);
+        const bool simt = A.simt_q > 0 && min(p_loc, m) <= A.simt_q;
+        // TWO: the rows of the own actuators, 16 bytes per thread and copy
+        auto copy_own = [&]() {
+            const int q4 = A.m_pad >> 2;
+            for (int e = warp; e < n_e; e += FT / 32) {
+                const int r = e < n_own ? A.tab.own[e0 + e] : A.n_act + A.tab.own[e0 + e - n_own];
+                if (lane < q4) cp_async16(XE + (size_t)e * A.m_pad + 4 * lane, A.X + (size_t)r * A.m_pad + 4 * lane);
+            }
+            cp_async_commit();
+        };
+        // TWO: f(j, u, member, value) over the halo rows of this warp, four rows' loads in flight (a
+        // lane's values are members lane + 32 u); done(j, sum) once per row before its f calls
+        auto halo_rows = [&](auto&& done, auto&& f) {
+            const int* hal = A.tab.halo + h0;
+            const int jl = warp + (FT / 32) * lane;
+            const int hrow = jl < n_h ? hal[jl] : 0;             // n_h <= 255: at most 32 rows per warp
+            for (int i0 = 0; warp + (FT / 32) * i0 < n_h; i0 += 4) {
+                float v[4][4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int j = warp + (FT / 32) * (i0 + q);
+                    const float* x = A.X + (size_t)(A.row_obs + __shfl_sync(0xffffffffu, hrow, (i0 + q) & 31)) * A.m_pad;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[q][u] = (j < n_h && lane + 32 * u < m) ? x[lane + 32 * u] : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int j = warp + (FT / 32) * (i0 + q);
+                    const float mu = done(j, v[q]);
+                    if (j < n_h)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (lane + 32 * u < m) f(j, lane + 32 * u, v[q][u] - mu);
+                }
+            }
+        };
+        if constexpr (TWO) {
+            if (simt) {
+                Xh = reinterpret_cast<float*>(big + A.off_sxh);
+                XE = reinterpret_cast<float*>(big + A.off_sxe);
+                copy_own();
+            }
+        } else if (warp == 0 && !A.dual && !ctl->loaded) {
+            issue_loads(A, d, Xh, XE, &ctl->bar_load);
+        }
         // ---- frame ingest: a non-finite slope in this domain's observation region rejects the
         //      system's frame (its state is restored when the launch ends)
         // (the m x m forms keep the region's slopes in shared memory for the innovation row)
@@ -1651,6 +1749,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             }
         }
         const bool dom_bad = __syncthreads_or(nonfinite) != 0;
+        if constexpr (!TWO)
         if (A.dual) {
             if (dom_bad) {
                 if (tid == 0) {
@@ -1666,14 +1765,20 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             continue;
         }
         // ---- 1. the halo rows of the observed instant and the own rows
-        if (!wait_all(ctl, &ctl->bar_load, ph_load, A.status)) break;
-        ph_load ^= 1;
+        if constexpr (!TWO) {
+            if (!wait_all(ctl, &ctl->bar_load, ph_load, A.status)) break;
+            ph_load ^= 1;
+        }
         if (dom_bad) {
+            if constexpr (TWO) {
+                cp_async_wait_all();
+                __syncthreads();      // every thread has read this item's number and system
+            }
             if (tid == 0) {
                 atomicExch(A.dom_bad, 1);
                 atomicOr(A.status, ST_NONFINITE);
             }
-            if (warp == 0) fetch_item(B, ctl, smem, 1 << 30);
+            if (warp == 0) fetch_item(B, ctl, smem, fetch_all);
             __syncthreads();
             continue;
         }
@@ -1681,6 +1786,17 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
         //        k = 2 s + direction) and the innovation row as the Gram operand
         // two rows per warp at a time, the values kept in registers between the sum and the
         // subtraction (m <= 127 here: four values per lane and row)
+        if constexpr (TWO) {
+            // straight from global memory: the same sums, two rows' reductions and more in flight
+            halo_rows(
+                [&](int j, const float (&v)[4]) {
+                    const float mu = warp_sum(((v[0] + v[1]) + v[2]) + v[3]) / (float)m;
+                    if (lane == 0 && j < n_h) xh_mean[j] = mu;
+                    return mu;
+                },
+                [&](int j, int i, float x) { Xh[(size_t)j * A.m_pad + i] = x; });
+            if (simt) cp_async_wait_all();
+        } else
         for (int j0 = warp; j0 < n_h; j0 += 2 * (FT / 32)) {
             const int j1 = j0 + FT / 32;
             float v0[4], v1[4], s0 = 0.f, s1 = 0.f;
@@ -1711,51 +1827,65 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
         }
         int* pcs = reinterpret_cast<int*>(vec + 1792);   // 64: the domain's packed corners
         int* owns = reinterpret_cast<int*>(vec + 1984);  // 64: its own actuators
-        uchar4* inc4 = reinterpret_cast<uchar4*>(xh_mean);   // over the halo means once they are used
-        for (int t = tid; t < n_obs; t += FT) pcs[t] = A.tab.obs_corner[o0 + t];
+        // over the halo means once they are used (TWO needs them again, and has room past the vectors)
+        uchar4* inc4 = reinterpret_cast<uchar4*>(TWO ? vec + 2048 : xh_mean);
+        int4* poff = reinterpret_cast<int4*>(vec + 1536);    // 64: their rows' offsets in Xh (over hv, unused yet)
+        for (int t = tid; t < n_obs; t += FT) {
+            const int pc = A.tab.obs_corner[o0 + t];
+            pcs[t] = pc;
+            poff[t] = make_int4((pc & 0xFF) * A.m_pad, ((pc >> 8) & 0xFF) * A.m_pad, ((pc >> 16) & 0xFF) * A.m_pad,
+                                ((pc >> 24) & 0xFF) * A.m_pad);
+        }
         for (int t = tid; t < n_own; t += FT) owns[t] = A.tab.own[e0 + t];
         __syncthreads();
         // ---- small domains: the FP32 SIMT analysis leaves X'_E T in shared memory
-        const bool simt = A.simt_q > 0 && min(p_loc, m) <= A.simt_q;
         const float* sout = nullptr;
         int sld = 0;
         if (simt) {
-            sout = analyse_simt(B, ctl, smem, d, &sld);
+            sout = analyse_simt<TWO>(B, ctl, smem, d, &sld);
         } else {
             // thread (i = tid mod 128, kc = tid / 128 + 2 k): row i of the operand, 8 K-values per task
-            for (int kc = tid >> 7, i = tid & 127; i < NP && kc < (KP >> 3); kc += 2) {
-                float v[8];
+            // (row m, the innovation, is written after it: as a branch here its warps ran both sides)
+            {
+                const int i = tid & 127;
+                const float* xi = Xh + i;
+                uint32_t off = op_offset(i, (tid >> 7) * 8, KP);
+                if (i < NP && i != m)
+                    for (int kc = tid >> 7; kc < (KP >> 3); kc += 2, off += 256) {
+                        float v[8];
     #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int sidx = 4 * kc + u;
-                    float sx = 0.f, sy = 0.f;
-                    if (i <= m && sidx < n_obs) {
-                        const int pc = pcs[sidx];
-                        const int c00 = pc & 0xFF, c01 = (pc >> 8) & 0xFF, c10 = (pc >> 16) & 0xFF, c11 = (pc >> 24) & 0xFF;
-                        float a00, a01, a10, a11;
-                        if (i < m) {
-                            a00 = Xh[(size_t)c00 * A.m_pad + i]; a01 = Xh[(size_t)c01 * A.m_pad + i];
-                            a10 = Xh[(size_t)c10 * A.m_pad + i]; a11 = Xh[(size_t)c11 * A.m_pad + i];
-                        } else {
-                            a00 = xh_mean[c00]; a01 = xh_mean[c01]; a10 = xh_mean[c10]; a11 = xh_mean[c11];
+                        for (int u = 0; u < 4; ++u) {
+                            const int sidx = 4 * kc + u;
+                            float sx = 0.f, sy = 0.f;
+                            if (i < m && sidx < n_obs) {
+                                const int4 po = poff[sidx];
+                                const float a00 = xi[po.x], a01 = xi[po.y], a10 = xi[po.z], a11 = xi[po.w];
+                                sx = 0.5f * ((a01 + a11) - (a00 + a10)) * A.inv_sigma;
+                                sy = 0.5f * ((a10 + a11) - (a00 + a01)) * A.inv_sigma;
+                            }
+                            v[2 * u] = sx;
+                            v[2 * u + 1] = sy;
                         }
-                        sx = 0.5f * ((a01 + a11) - (a00 + a10));
-                        sy = 0.5f * ((a10 + a11) - (a00 + a01));
-                        if (i < m) {
-                            sx *= A.inv_sigma;
-                            sy *= A.inv_sigma;
-                        } else {
-                            sx = (ys[2 * sidx] - sx) * A.inv_sigma;
-                            sy = (ys[2 * sidx + 1] - sy) * A.inv_sigma;
-                            dtv[2 * sidx] = sx;
-                            dtv[2 * sidx + 1] = sy;
-                        }
+                        store8_at(opg_h, opg_l, off, v, true);
                     }
-                    v[2 * u] = sx;
-                    v[2 * u + 1] = sy;
-                }
-                store8(opg_h, opg_l, i, kc * 8, KP, v, true);
             }
+            for (int k = tid; k < KP; k += FT) {      // d / sigma: slope k of the innovation
+                float dk = 0.f;
+                if (k < p_loc) {
+                    const int pc = pcs[k >> 1];
+                    const float a00 = xh_mean[pc & 0xFF], a01 = xh_mean[(pc >> 8) & 0xFF];
+                    const float a10 = xh_mean[(pc >> 16) & 0xFF], a11 = xh_mean[(pc >> 24) & 0xFF];
+                    const float sl =
+                        (k & 1) == 0 ? 0.5f * ((a01 + a11) - (a00 + a10)) : 0.5f * ((a10 + a11) - (a00 + a01));
+                    dk = (ys[k] - sl) * A.inv_sigma;
+                    dtv[k] = dk;
+                }
+                const __nv_bfloat16 dh = __float2bfloat16_rn(dk), dl = __float2bfloat16_rn(dk - __bfloat162float(dh));
+                const uint32_t off = op_offset(m, k, KP);
+                *reinterpret_cast<__nv_bfloat16*>(opg_h + off) = dh;
+                *reinterpret_cast<__nv_bfloat16*>(opg_l + off) = dl;
+            }
+            if (tid >= m && tid < 128) bvec[tid] = 0.f;   // past b's end: read as zeros with Z's padding
             fence_async_smem();
             __syncthreads();
             // the incidence of the halo actuators in the observed subapertures, for the refinement's
@@ -1766,7 +1896,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             __syncthreads();
             if (uwarp == 0 && elect_one()) {
                 tc_fence_after();
-                issue_product(tbase + TM_G, opg_h, opg_l, opg_h, opg_l, KP, NP, A.gram_terms, 0);
+                issue_product(tbase + tG, opg_h, opg_l, opg_h, opg_l, KP, NP, A.gram_terms, 0);
                 mma_commit(&ctl->bar_mma);
             }
             for (int s2 = tid; s2 < n_obs; s2 += FT) {
@@ -1783,15 +1913,20 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             // ---- 3a. G and b; scale s = 1 + ||G||_F / c, an upper bound of cond((m-1)I + G)
             auto read_gram = [&]() -> float {
                 float fr = 0.f;
-                tmem_rows(tl + TM_G, nq, [&](int q8, const float (&g)[8]) {
+                tmem_rows(tl + tG, nq, [&](int q8, const float (&g)[8]) {
+                    if (col0 + 8 * q8 + 8 <= m) {
     #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int j = col0 + 8 * q8 + u;
-                        if (row < m && j < m) fr += g[u] * g[u];
-                        if (row < m && j == m) bvec[row] = g[u];
+                        for (int u = 0; u < 8; ++u) fr += g[u] * g[u];
+                    } else {
+    #pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            const int j = col0 + 8 * q8 + u;
+                            if (j < m) fr += g[u] * g[u];
+                            if (row < m && j == m) bvec[row] = g[u];
+                        }
                     }
                 });
-                return block_sum(ctl, fr);
+                return block_sum(ctl, row < m ? fr : 0.f);
             };
             float fro = read_gram();
             if (A.gram_terms < 3 && 1.f + sqrtf(fro) / c > A.s_split) {
@@ -1800,7 +1935,7 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 __syncthreads();
                 if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
-                    issue_product(tbase + TM_G, opg_h, opg_l, opg_h, opg_l, KP, NP, 3, 0, 1);
+                    issue_product(tbase + tG, opg_h, opg_l, opg_h, opg_l, KP, NP, 3, 0, 1);
                     mma_commit(&ctl->bar_mma);
                 }
                 if (!wait_all(ctl, &ctl->bar_mma, ph_mma, A.status)) break;
@@ -1820,27 +1955,58 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             //      Z_1 = T_0: one pass over G writes Y_0, T_0 as Z_1 and the residual; Y_1 = Y_0 T_0
             //      reads T_0 from Z's buffer (T_0 is symmetric: its K-major and MN-major operand
             //      layouts hold the same bytes).
-            int z_state = 1;     // where Z is: 0 identity, 1 shared memory only (Z_1 = T_0), 2 also TMEM
+            // 8 columns of this thread's half-row of Y into its operand (TWO: also Y's left operand in
+            // tensor memory, at the columns of T Z's accumulator: high parts, then low parts)
+            const uint32_t off0 = op_offset(row, col0, NP);      // this thread's half-row; a chunk is 128 bytes on
+            auto put_y = [&](int q8, const float (&yv)[8]) {
+                uint32_t h[4], l[4];
+                split8(yv, h, l);
+                if (row < NP) {
+                    const uint32_t off = off0 + 128u * q8;
+                    *reinterpret_cast<uint4*>(Yh + off) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4*>(Yl + off) = make_uint4(l[0], l[1], l[2], l[3]);
+                }
+                if constexpr (TWO) {
+                    const uint32_t ta = tbase + lane_off + tZ + (uint32_t)((col0 + 8 * q8) >> 1);
+                    tmem_st4(ta, h);
+                    tmem_st4(ta + (uint32_t)(NP >> 1), l);
+                }
+            };
+            int z_state = 1;     // where Z ends: 0 identity, 1 its operands (step limit hit), 2 tensor memory
             int it = 1;
             bool ok = true;
             float rn_prev;
+            // Whether chunk q8 meets the diagonal in this warp's rows, or (edge) the end of the m x m
+            // block: elsewhere the identity and the bounds drop out of the element's arithmetic (what
+            // lies past m is zero in every iterate; the passes are bound by their instructions)
+            const int rw0 = 32 * (warp & 3);
+            auto on_diag = [&](int q8) { return col0 + 8 * q8 < rw0 + 32 && col0 + 8 * q8 + 8 > rw0; };
             {
                 float r2 = 0.f;
-                tmem_rows(tl + TM_G, nq, [&](int q8, const float (&g)[8]) {
+                tmem_rows(tl + tG, nq, [&](int q8, const float (&g)[8]) {
                     float yv[8], tv[8];
+                    if (!on_diag(q8) && rw0 + 32 <= m && col0 + 8 * q8 + 8 <= m) {
     #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int j = col0 + 8 * q8 + u;
-                        const bool in = row < m && j < m;
-                        const float id = (row == j) ? 1.f : 0.f;
-                        yv[u] = in ? fmaf(g[u], inv_cs, id * id_scale) : 0.f;
-                        const float rr = id - yv[u];
-                        if (in) r2 += rr * rr;
-                        tv[u] = in ? 1.5f * id - 0.5f * yv[u] : 0.f;
+                        for (int u = 0; u < 8; ++u) {
+                            yv[u] = g[u] * inv_cs;
+                            r2 += yv[u] * yv[u];
+                            tv[u] = -0.5f * yv[u];
+                        }
+                    } else {
+    #pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            const int j = col0 + 8 * q8 + u;
+                            const bool in = row < m && j < m;
+                            const float id = (row == j) ? 1.f : 0.f;
+                            yv[u] = in ? fmaf(g[u], inv_cs, id * id_scale) : 0.f;
+                            const float rr = id - yv[u];
+                            if (in) r2 += rr * rr;
+                            tv[u] = in ? 1.5f * id - 0.5f * yv[u] : 0.f;
+                        }
                     }
                     if (row < NP) {
-                        store8(Yh, Yl, row, col0 + 8 * q8, NP, yv, true);
-                        store8(Zh, Zl, row, col0 + 8 * q8, NP, tv, true);
+                        store8_at(Yh, Yl, off0 + 128u * q8, yv, true);
+                        store8_at(Zh, Zl, off0 + 128u * q8, tv, true);
                     }
                 });
                 rn_prev = sqrtf(block_sum_open(ctl, r2));   // a barrier follows on either branch
@@ -1854,15 +2020,14 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 __syncthreads();
                 if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
-                    issue_product(tbase + TM_Y, Yh, Yl, Zh, Zl, NP, NP, 3, 1);     // Y_1 = Y_0 T_0
+                    issue_product(tbase + tY, Yh, Yl, Zh, Zl, NP, NP, 3, 1);     // Y_1 = Y_0 T_0
                     mma_commit(&ctl->bar_mma);
                 }
                 if (!wait_all(ctl, &ctl->bar_mma, ph_mma, A.status)) break;
                 ph_mma ^= 1;
                 tc_fence_after();
-                tmem_rows(tl + TM_Y, nq, [&](int q8, const float (&yv)[8]) {
-                    if (row < NP) store8(Yh, Yl, row, col0 + 8 * q8, NP, yv, true);
-                });
+                tmem_rows(tl + tY, nq, [&](int q8, const float (&yv)[8]) { put_y(q8, yv); });
+                if constexpr (TWO) tmem_wait_st();
                 fence_async_smem();
                 tc_fence_before();
                 __syncthreads();
@@ -1871,39 +2036,33 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             for (; it < A.max_it; ++it) {
                 if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
-                    issue_product(tbase + TM_P, Zh, Zl, Yh, Yl, NP, NP, 3, 1);
+                    issue_product(tbase + tP, Zh, Zl, Yh, Yl, NP, NP, 3, 1);
                     mma_commit(&ctl->bar_mma);
                 }
                 if (!wait_all(ctl, &ctl->bar_mma, ph_mma, A.status)) { ok = false; break; }
                 ph_mma ^= 1;
                 tc_fence_after();
                 float r2 = 0.f;
-                {   // the next chunk's TMEM load is in flight while this one is processed
-                    uint32_t rc[8], rn[8];
-                    tmem_ld8_async(tl + TM_P, rc);
-                    tmem_wait_ld(rc);
-    #pragma unroll 1
-                    for (int q8 = 0; q8 < nq; ++q8) {
-                        if (q8 + 1 < nq) tmem_ld8_async(tl + TM_P + 8 * (q8 + 1), rn);
-                        float tv[8];
+                tmem_rows(tl + tP, nq, [&](int q8, const float (&pv)[8]) {
+                    float tv[8];
+                    if (!on_diag(q8)) {
     #pragma unroll
                         for (int u = 0; u < 8; ++u) {
-                            const int j = col0 + 8 * q8 + u;
-                            const bool in = row < m && j < m;
-                            const float id = (row == j) ? 1.f : 0.f;
-                            const float pv = __uint_as_float(rc[u]);
-                            const float rr = id - pv;
-                            if (in) r2 += rr * rr;
-                            tv[u] = in ? 1.5f * id - 0.5f * pv : 0.f;
+                            r2 += pv[u] * pv[u];
+                            tv[u] = -0.5f * pv[u];
                         }
-                        if (row < NP) store8(Th, Tl, row, col0 + 8 * q8, NP, tv, true);
-                        if (q8 + 1 < nq) {
-                            tmem_wait_ld(rn);
+                    } else {
     #pragma unroll
-                            for (int u = 0; u < 8; ++u) rc[u] = rn[u];
+                        for (int u = 0; u < 8; ++u) {
+                            const float id = (row == col0 + 8 * q8 + u && row < m) ? 1.f : 0.f;
+                            const float rr = id - pv[u];
+                            r2 += rr * rr;
+                            tv[u] = 1.5f * id - 0.5f * pv[u];
                         }
                     }
-                }
+                    if (row < NP) store8_at(Th, Tl, off0 + 128u * q8, tv, true);
+                });
+                if (row >= m) r2 = 0.f;
                 // one barrier for the residual's block sum and T's stores (to the tensor core)
                 r2 = warp_sum(r2);
                 if (lane == 0) ctl->red[warp] = r2;
@@ -1916,15 +2075,14 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 const float rn = sqrtf(r2);
                 const bool conv = rn < 2e-6f * (float)m || (rn < 2e-2f && rn > 0.6f * rn_prev);
                 rn_prev = rn;
-                if (conv) break;
-                // the update after which ||I - P|| lands at the rounding floor is the last: only its
-                // T Z is used afterwards (read from tensor memory), so Y T and the operand stores
-                // are skipped
-                const bool last = rn < ns_last;
+                // the update after which ||I - P|| lands at the rounding floor is the last (also one
+                // that starts there): only its T Z is used afterwards (read from tensor memory), so
+                // Y T and the operand stores are skipped
+                const bool last = conv || rn < ns_last;
                 if (last) {
                     if (uwarp == 1 && elect_one()) {
                         tc_fence_after();
-                        issue_product(tbase + TM_Z, Th, Tl, Zh, Zl, NP, NP, 3, 1);     // T Z
+                        issue_product(tbase + tZ, Th, Tl, Zh, Zl, NP, NP, 3, 1);     // T Z
                         mma_commit(&ctl->bar_mma2);
                     }
                     if (!wait_all(ctl, &ctl->bar_mma2, ph_mma2, A.status)) { ok = false; break; }
@@ -1935,24 +2093,47 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 }
                 // the two products are issued by threads of different warps, so their issue loops
                 // (one tcgen05.mma per K step and BF16 term) overlap
-                if (uwarp == 0 && elect_one()) {
+                if constexpr (TWO) {
+                    // T Z's accumulator lies over Y's left operand: its product waits for Y T
+                    if (uwarp == 0 && elect_one()) {
+                        tc_fence_after();
+                        issue_product_ta(tbase + tY, tbase + tZ, tbase + tZ + (uint32_t)(NP >> 1), Th, Tl, NP, NP);   // Y T
+                        mma_commit(&ctl->bar_mma);
+                        if (mbar_wait_bounded(&ctl->bar_mma, ph_mma, WAIT_CYCLES)) {
+                            tc_fence_after();
+                            issue_product(tbase + tZ, Th, Tl, Zh, Zl, NP, NP, 3, 1);                                 // T Z
+                            mma_commit(&ctl->bar_mma2);
+                        }
+                    }
+                } else if (uwarp == 0 && elect_one()) {
                     tc_fence_after();
-                    issue_product(tbase + TM_Y, Yh, Yl, Th, Tl, NP, NP, 3, 1);     // Y T
+                    issue_product(tbase + tY, Yh, Yl, Th, Tl, NP, NP, 3, 1);     // Y T
                     mma_commit(&ctl->bar_mma);
                 } else if (uwarp == 1 && elect_one()) {
                     tc_fence_after();
-                    issue_product(tbase + TM_Z, Th, Tl, Zh, Zl, NP, NP, 3, 1);     // T Z
+                    issue_product(tbase + tZ, Th, Tl, Zh, Zl, NP, NP, 3, 1);     // T Z
                     mma_commit(&ctl->bar_mma2);
                 }
                 if (!wait_all2(ctl, ph_mma, ph_mma2, A.status)) { ok = false; break; }
                 ph_mma ^= 1;
                 ph_mma2 ^= 1;
                 tc_fence_after();
+                if constexpr (TWO) {
+                    tmem_rows(tl + tZ, nq, [&](int q8, const float (&zv)[8]) {
+                        if (row < NP) store8_at(Zh, Zl, off0 + 128u * q8, zv, true);
+                    });
+                    // Y's left operand goes over Z's accumulator: both warps of these lanes have read it
+                    tc_fence_before();
+                    asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 3)) : "memory");
+                    tc_fence_after();
+                    tmem_rows(tl + tY, nq, [&](int q8, const float (&yv)[8]) { put_y(q8, yv); });
+                    tmem_wait_st();
+                } else {
     #pragma unroll 1
                 for (int q8 = 0; q8 < nq; ++q8) {
                     uint32_t ry[8], rz[8];
-                    tmem_ld8_async(tl + TM_Y + 8 * q8, ry);
-                    tmem_ld8_async(tl + TM_Z + 8 * q8, rz);
+                    tmem_ld8_async(tl + tY + 8 * q8, ry);
+                    tmem_ld8_async(tl + tZ + 8 * q8, rz);
                     tmem_wait_ld(ry, rz);
                     float yv[8], zv[8];
     #pragma unroll
@@ -1961,23 +2142,65 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                         zv[u] = __uint_as_float(rz[u]);
                     }
                     if (row < NP) {
-                        store8(Yh, Yl, row, col0 + 8 * q8, NP, yv, true);
-                        store8(Zh, Zl, row, col0 + 8 * q8, NP, zv, true);
+                        store8_at(Yh, Yl, off0 + 128u * q8, yv, true);
+                        store8_at(Zh, Zl, off0 + 128u * q8, zv, true);
                     }
                 }
-                z_state = 2;
+                }
                 fence_async_smem();
                 tc_fence_before();
                 __syncthreads();
             }
             if (!ok) break;
             if (it == A.max_it && tid == 0) atomicOr(A.status, ST_NOCONV);
+            if constexpr (TWO) {
+                // Z goes to tensor memory where it is not there yet: its operands' place is needed
+                if (z_state != 2) {
+                    __syncthreads();       // the last reads of Z's columns (Y's left operand) are done
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int q8 = 0; q8 < nq; ++q8) {
+                        float zv[8];
+                        if (z_state == 1) {
+                            const uint32_t off = op_offset(row < NP ? row : 0, col0 + 8 * q8, NP);
+                            const uint4 h = *reinterpret_cast<const uint4*>(Zh + off);
+                            const uint4 l = *reinterpret_cast<const uint4*>(Zl + off);
+                            const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const float2 fh = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[u]));
+                                const float2 fl = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&lw[u]));
+                                zv[2 * u] = fh.x + fl.x;
+                                zv[2 * u + 1] = fh.y + fl.y;
+                            }
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) zv[u] = (row == col0 + 8 * q8 + u && row < m) ? 1.f : 0.f;
+                        }
+                        tmem_st8(tl + tZ + 8 * q8, zv);
+                    }
+                    tmem_wait_st();
+                    z_state = 2;
+                }
+                fence_async_smem();
+            }
             tc_fence_before();
             __syncthreads();
             tc_fence_after();
+            if constexpr (TWO) {
+                // the own rows, and (where they had to give way) the halo anomalies once more: the same
+                // rows less the same means
+                copy_own();
+                if (A.off_xh3 != A.off_xh) {
+                    Xh = reinterpret_cast<float*>(big + A.off_xh3);
+                    halo_rows([&](int j, const float (&)[4]) { return xh_mean[j < n_h ? j : 0]; },
+                              [&](int j, int i, float x) { Xh[(size_t)j * A.m_pad + i] = x; });
+                }
+                cp_async_wait_all();      // (published by the barrier below)
+            }
             // the domain's rows of the process noise V, copied to shared memory now for the epilogue
             // (its global rows may sit in the other die's memory: a latency the analysis hides)
-            const bool vstage = A.with_forecast && A.vmode == 0 && A.off_vs >= 0;
+            const bool vstage = !TWO && A.with_forecast && A.vmode == 0 && A.off_vs >= 0;
             float* vs = reinterpret_cast<float*>(big + (A.off_vs >= 0 ? A.off_vs : 0));
             if (vstage) {
                 const int q4 = A.m_pad >> 2;
@@ -1990,8 +2213,8 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             // ---- 4. mean weights w_bar = Z (Z b) / (c s), refined against the exact operator
             // 8 columns of this thread's half-row of Z = A_s^(-1/2)
             auto zrow = [&](int q8, float (&zv)[8]) {
-                if (z_state == 2) {
-                    tmem_ld8(tl + TM_Z + 8 * q8, zv);
+                if (TWO || z_state == 2) {
+                    tmem_ld8(tl + tZ + 8 * q8, zv);
                 } else if (z_state == 1) {     // high + low BF16 parts of the shared-memory operand
                     const uint32_t off = op_offset(row < NP ? row : 0, col0 + 8 * q8, NP);
                     const uint4 h = *reinterpret_cast<const uint4*>(Zh + off);
@@ -2016,15 +2239,12 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             const int zld = NP + 4;
             auto zf_put = [&](int q8, const float (&zv)[8]) {
                 if (row >= NP) return;
-                float w8[8];
-    #pragma unroll
-                for (int u = 0; u < 8; ++u) w8[u] = (row < m && col0 + 8 * q8 + u < m) ? zv[u] : 0.f;
                 float4* dst = reinterpret_cast<float4*>(zf + row * zld + col0 + 8 * q8);
-                dst[0] = make_float4(w8[0], w8[1], w8[2], w8[3]);
-                dst[1] = make_float4(w8[4], w8[5], w8[6], w8[7]);
+                dst[0] = make_float4(zv[0], zv[1], zv[2], zv[3]);
+                dst[1] = make_float4(zv[4], zv[5], zv[6], zv[7]);
             };
-            if (z_state == 2) {
-                tmem_rows(tl + TM_Z, nq, zf_put);
+            if (TWO || z_state == 2) {
+                tmem_rows(tl + tZ, nq, zf_put);
             } else {
     #pragma unroll 1
                 for (int q8 = 0; q8 < nq; ++q8) {
@@ -2042,11 +2262,10 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                 for (int q4 = 0; q4 < half / 4; ++q4) {
                     const float4 z4 = *reinterpret_cast<const float4*>(zr + 4 * q4);
                     const float4 x4 = *reinterpret_cast<const float4*>(x_in + col0 + 4 * q4);
-                    const int j = col0 + 4 * q4;
-                    if (j < m) part += z4.x * x4.x;
-                    if (j + 1 < m) part += z4.y * x4.y;
-                    if (j + 2 < m) part += z4.z * x4.z;
-                    if (j + 3 < m) part += z4.w * x4.w;
+                    part += z4.x * x4.x;           // (Z and x are zero past m)
+                    part += z4.y * x4.y;
+                    part += z4.z * x4.z;
+                    part += z4.w * x4.w;
                 }
                 vtmp[hh * 128 + row] = part;
                 __syncthreads();
@@ -2137,7 +2356,9 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
     #pragma unroll 1
             for (int q8 = 0; q8 < nq; ++q8) {
                 float zv[8], bv[8];
-                {
+                if constexpr (TWO) {    // (B's operand goes over the FP32 rows)
+                    tmem_ld8(tl + tZ + 8 * q8, zv);
+                } else {
                     const float4* zr = reinterpret_cast<const float4*>(zf + (row < NP ? row : 0) * zld + col0 + 8 * q8);
                     const float4 a0 = zr[0], a1 = zr[1];
                     zv[0] = a0.x; zv[1] = a0.y; zv[2] = a0.z; zv[3] = a0.w;
@@ -2146,22 +2367,27 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
     #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int j = col0 + 8 * q8 + u;
-                    bv[u] = (row < m && j < m) ? zv[u] * rs : 0.f;
+                    bv[u] = zv[u] * rs;
                     if (cap && row < m && j < m) A.cap[CAP_HDR + m + row * m + j] = bv[u];
                 }
-                if (row < NP) store8(Bh, Bl, row, col0 + 8 * q8, NP, bv, A.tr_terms > 1);
+                if (row < NP) store8_at(Bh, Bl, off0 + 128u * q8, bv, A.tr_terms > 1);
             }
             own_row_means(A, XE, n_e, wbar, xe_mean, uvec);   // member means, mean update X'_E w_bar
-            const int RA = A.RA;
-            for (int t = tid; t < RA * (NP >> 3); t += FT) {
-                const int e = t % RA, kc = t / RA;
-                float v[8];
+            // X'_E's operand, its own n_e rows (what the rows past them hold only reaches rows of the product
+            // that are not read): sixteen lanes per row, a chunk of 8 members each
+            for (int er = 2 * warp; er < n_e; er += FT / 16) {
+                const int e = er + (lane >> 4), kc = lane & 15;
+                if (e < n_e && kc < (NP >> 3)) {
+                    const float* xr = XE + (size_t)e * A.m_pad + kc * 8;
+                    const float mu = xe_mean[e];
+                    float v[8];
     #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int k = kc * 8 + u;
-                    v[u] = (e < n_e && k < m) ? XE[(size_t)e * A.m_pad + k] - xe_mean[e] : 0.f;
+                    for (int u = 0; u < 8; ++u) v[u] = 0.f;
+                    if (kc * 8 < m) get8(xr, v, min(8, A.m_pad - kc * 8));
+    #pragma unroll
+                    for (int u = 0; u < 8; ++u) v[u] = kc * 8 + u < m ? v[u] - mu : 0.f;
+                    store8(Ah, Al, e, kc * 8, NP, v, A.tr_terms > 1);
                 }
-                store8(Ah, Al, e, kc * 8, NP, v, A.tr_terms > 1);
             }
             fence_async_smem();
             tc_fence_before();
@@ -2170,11 +2396,11 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
             // and term, ~2.7 k cycles) overlaps warp 0's fetch of the next item
             if (uwarp == 1 && elect_one()) {
                 tc_fence_after();
-                issue_product(tbase + TM_P, Ah, Al, Bh, Bl, NP, NP, A.tr_terms, 1);   // X'_E T
+                issue_product(tbase + tP, Ah, Al, Bh, Bl, NP, NP, A.tr_terms, 1);   // X'_E T
                 mma_commit(&ctl->bar_mma);
             }
             // the halo and own-row tiles are free now: fetch the next domain's under this product
-            if (warp == 0) fetch_item(B, ctl, smem, A.off_big);
+            if (!TWO && warp == 0) fetch_item(B, ctl, smem, A.off_big);
             if (!wait_all(ctl, &ctl->bar_mma, ph_mma, A.status)) break;
             ph_mma ^= 1;
             tc_fence_after();
@@ -2195,16 +2421,16 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
                     f(q8, dv);
                 }
             } else {
-                tmem_rows(tl + TM_P, nq, f);
+                tmem_rows(tl + tP, nq, f);
             }
         };
         const bool mine = row < n_e;
         // the tensor-core product is read from tensor memory once: its rows go to shared memory
         // (FP32, row stride NP + 4, over Z's rows, which the transform no longer needs) for the
         // passes below
-        float* pst = reinterpret_cast<float*>(big + A.off_zf);
+        float* pst = reinterpret_cast<float*>(big + A.off_pst);
         const int pld = NP + 4;
-        const bool vsm = !simt && A.with_forecast && A.vmode == 0 && A.off_vs >= 0;   // V rows staged
+        const bool vsm = !TWO && !simt && A.with_forecast && A.vmode == 0 && A.off_vs >= 0;   // V rows staged
         if (vsm) cp_async_wait_all();   // this thread's copies; the barrier below publishes them all
         {   // member mean of this row of X'_E T (two column halves)
             float part = 0.f;
@@ -2323,14 +2549,19 @@ __global__ void __launch_bounds__(FT, 1) fused_kernel(const __grid_constant__ Fu
         }
         tc_fence_before();
         __syncthreads();
+        if constexpr (TWO) {
+            // every thread has read this item's number and system: take the next one
+            if (warp == 0) fetch_item(B, ctl, smem, fetch_all);
+            __syncthreads();
+        }
         tc_fence_after();
     }
     // a wait that ran out may leave bulk copies in flight: give them a bounded time to land
-    if (ctl->abort && tid == 0) mbar_wait_bounded(&ctl->bar_load, ph_load, WAIT_CYCLES);
+    if (!TWO && ctl->abort && tid == 0) mbar_wait_bounded(&ctl->bar_load, ph_load, WAIT_CYCLES);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) tmem_dealloc(tbase, TM_COLS);
+    if (warp == 0) tmem_dealloc(tbase, tmem_cols);
     // the last CTA to finish (all work items taken and done) closes the launch
     if (tid == 0) {
         __threadfence();
@@ -2436,6 +2667,7 @@ int round_up(int v, int a) { return (v + a - 1) / a * a; }
 struct FusedLayout {
     int NP, KP, RA, sz_op, sz_opg, sz_a, off_vec, off_xe, off_xh, off_big, off_zf = 0, off_vs = -1, total;
     int off_hs = -1, off_hs2 = -1, hs_w = 0;
+    int off_pst = 0, off_xh3 = 0, off_sxe = 0, off_sxh = 0;
 };
 
 // Ensembles of m >= 128 members do not fit one 128-row MMA tile: they take the dual form.
@@ -2504,8 +2736,66 @@ FusedLayout fused_layout(const letkf_ctx* c) {
         L.off_vs = off_vs;
         big = std::max(big, off_vs + vs_bytes);
     }
+    L.off_pst = L.off_zf;
     L.total = L.off_big + round_up(big, 1024);
     if (c->simt_q > 0) L.total = std::max(L.total, L.off_big + round_up(c->simt_ws, 1024));
+    return L;
+}
+
+// Shared memory of a CTA when two share an SM (228 KB per SM, 1 KB of it reserved per CTA).
+constexpr int TWO_SMEM = 113 * 1024;
+
+// The layout of fused_kernel<true> (offsets within the big region unless they are off_vec or
+// off_big); total = 0 when the system does not fit or takes the dual form.
+FusedLayout fused_layout2(const letkf_ctx* c) {
+    const HostModel& h = c->host;
+    FusedLayout L;
+    L.total = 0;
+    if (uses_dual(c->m)) return L;
+    L.NP = round_up(c->m + 1, 16);
+    L.KP = std::max(16, round_up(h.p_loc_max, 16));
+    L.RA = round_up(std::max(h.n_loc_max, 1), 16);
+    L.sz_op = L.NP * L.NP * 2;
+    L.sz_opg = L.NP * L.KP * 2;
+    L.sz_a = L.RA * L.NP * 2;
+    L.off_vec = 1024;
+    L.off_big = L.off_vec + 8192 + 1024;
+    const int xh = std::max(h.n_h_max, 1) * c->m_pad * 4, xe = std::max(h.n_loc_max, 1) * c->m_pad * 4;
+    // slopes: the Gram's operand pair; iteration: Y (then T) and Z; mean weights: Z's FP32 rows;
+    // transform: Z's operand, X'_E's; epilogue: the AR(2) hand-over rows, the product's rows; each
+    // operand pair with the rows a 128-row MMA reads past it
+    const int zf = L.NP * (L.NP + 4) * 4;
+    const int ops = std::max(std::max(2 * L.sz_opg, 4 * L.sz_op), std::max(zf, 2 * L.sz_op + 2 * L.sz_a));
+    const int past = std::max(std::max(L.sz_opg + MT * L.KP * 2, 3 * L.sz_op + MT * L.NP * 2),
+                              2 * L.sz_op + L.sz_a + MT * L.NP * 2);
+    L.off_zf = 0;
+    L.off_pst = round_up(xe / 2 + 16, 128);
+    const int epi = L.off_pst + std::max(h.n_loc_max, 1) * (L.NP + 4) * 4;
+    // the halo rows past all of them when that fits, else past the Gram's operands, and again past Z's
+    // FP32 rows; the own rows past those and the transform's operands
+    L.off_xh = L.off_xh3 = round_up(ops, 128);
+    L.off_xe = round_up(L.off_xh + xh, 128);
+    if (L.off_big + L.off_xe + xe > TWO_SMEM) {
+        L.off_xh = 2 * L.sz_opg;
+        L.off_xh3 = round_up(zf, 128);
+        L.off_xe = round_up(std::max(L.off_xh3 + xh, 2 * L.sz_op + 2 * L.sz_a), 128);
+    }
+    int big = std::max(std::max(ops, past), std::max(epi, std::max(L.off_xh + xh, L.off_xe + xe)));
+    if (c->simt_q > 0) {   // SIMT domains: the workspace, then their own and halo rows
+        int ne = 1, nh = 1;
+        for (int d = 0; d < c->n_dom; ++d) {
+            const int p = 2 * (h.obs_off[d + 1] - h.obs_off[d]);
+            if (p > 0 && std::min(p, c->m) <= c->simt_q) {
+                ne = std::max(ne, 2 * (h.own_off[d + 1] - h.own_off[d]));
+                nh = std::max(nh, h.halo_off[d + 1] - h.halo_off[d]);
+            }
+        }
+        L.off_sxe = round_up(c->simt_ws, 128);
+        L.off_sxh = L.off_sxe + round_up(ne * c->m_pad * 4, 128);
+        big = std::max(big, L.off_sxh + nh * c->m_pad * 4);
+    }
+    const int total = L.off_big + round_up(big, 128);
+    if (total <= TWO_SMEM && 2 * L.NP <= TM_COLS / 2 && L.RA <= MT) L.total = total;
     return L;
 }
 
@@ -2538,6 +2828,7 @@ int fused_plan(letkf_ctx* c) {
     if (L.total > 227 * 1024) return LETKF_EINVAL;
     if (h.n_h_max > 255 || h.n_loc_max > MT) return LETKF_EINVAL;
     c->fused_smem = L.total;
+    c->fused_smem2 = fused_layout2(c).total;
     return LETKF_OK;
 }
 
@@ -2552,7 +2843,11 @@ int fused_prepare(letkf_ctx* c) {
         c->device_bytes += sb;
     }
     static_assert(sizeof(FusedBatch) < 32000, "kernel parameters too large");
-    if (cudaFuncSetAttribute(fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+    if (cudaFuncSetAttribute(fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TWO_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(fused_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared) != cudaSuccess)
         return LETKF_ECUDA;
     // One CTA per SM pulling domains from the work queue: domains differ in cost (edge domains
     // see fewer subapertures), so the full grid balances better than fewer, evenly loaded CTAs.
@@ -2616,7 +2911,7 @@ int noise_prefetch(letkf_ctx* c, unsigned long long frame, cudaStream_t stream) 
 }
 
 // Descriptor of system c's next frame, with the process-noise block V (dense noise) given.
-void fill_desc(const FusedFrame& f, const float* V, SysDesc* S) {
+void fill_desc(const FusedFrame& f, const float* V, bool two, SysDesc* S) {
     letkf_ctx* c = f.c;
     if (f.sigma > 0) c->sigma = f.sigma;
     S->X = static_cast<const float*>(c->X[c->cur]);
@@ -2644,7 +2939,7 @@ void fill_desc(const FusedFrame& f, const float* V, SysDesc* S) {
     S->n_subv = c->n_subv;
     S->n_dom = c->n_dom;
     S->row_obs = c->obs_block == 1 ? c->n_act : 0;
-    const FusedLayout L = fused_layout(c);
+    const FusedLayout L = two ? fused_layout2(c) : fused_layout(c);
     S->NP = L.NP;
     S->KP = L.KP;
     S->RA = L.RA;
@@ -2675,38 +2970,69 @@ void fill_desc(const FusedFrame& f, const float* V, SysDesc* S) {
     S->off_hs = L.off_hs;
     S->off_hs2 = L.off_hs2;
     S->hs_w = L.hs_w;
+    S->off_pst = L.off_pst;
+    S->off_xh3 = L.off_xh3;
+    S->off_sxe = L.off_sxe;
+    S->off_sxh = L.off_sxh;
     S->cap = c->cap_dev;
     S->cap_dom = c->cap_dom;
 }
 
 // Descriptor of system c's next frame; `stream` (the kernel's) waits for its noise block.
-int make_desc(const FusedFrame& f, cudaStream_t stream, SysDesc* S) {
+int make_desc(const FusedFrame& f, cudaStream_t stream, bool two, SysDesc* S) {
     const float* V = nullptr;
     if (f.with_forecast && (f.c->Lq || f.c->Lt)) {
         const int rc = noise_ready(f.c, f.c->frame, stream, &V);
         if (rc) return rc;
     }
-    fill_desc(f, V, S);
+    fill_desc(f, V, two, S);
     return LETKF_OK;
+}
+
+// How a launch over n systems' frames runs: two CTAs per SM when every system fits them and there are
+// more domains than SMs, else one (a lone domain per SM is faster with the SM's registers and shared
+// memory to itself).  One system alone runs on its tuned grid (letkf_set_tuning); a batch fills every SM.
+struct FusedLaunch {
+    bool two;
+    int grid, smem;
+    const void* fn;
+};
+FusedLaunch fused_launch(const FusedFrame* f, int n, int sms) {
+    FusedLaunch l{true, 0, 0, nullptr};
+    int items = 0, smem1 = 0, smem2 = 0;
+    for (int k = 0; k < n; ++k) {
+        const letkf_ctx* c = f[k].c;
+        items += c->n_dom;
+        smem1 = std::max(smem1, c->fused_smem);
+        smem2 = std::max(smem2, c->fused_smem2);
+        l.two = l.two && c->fused_smem2 > 0;
+    }
+    const int per_sm = n == 1 && f[0].c->fused_grid > 0 ? f[0].c->fused_grid : sms;
+    l.two = l.two && items > sms;
+    l.grid = std::min(l.two ? 2 * per_sm : per_sm, items);
+    l.smem = l.two ? smem2 : smem1;
+    l.fn = l.two ? reinterpret_cast<const void*>(fused_kernel<true>) : reinterpret_cast<const void*>(fused_kernel<false>);
+    return l;
 }
 
 int launch_batch(const FusedFrame* f, const int* order, int n, int* queue, cudaStream_t stream, int sms) {
     thread_local FusedBatch B;   // host staging of the kernel parameters
-    int items = 0, smem = 0;
+    const FusedLaunch L = fused_launch(f, n, sms);
+    int items = 0;
     for (int k = 0; k < n; ++k) {
         SysDesc& S = B.sys[k];
-        const int rc = make_desc(f[order[k]], stream, &S);
+        const int rc = make_desc(f[order[k]], stream, L.two, &S);
         if (rc) return rc;
         S.item0 = items;
         items += S.n_dom;
-        smem = std::max(smem, f[order[k]].c->fused_smem);
     }
     B.n_sys = n;
     B.n_items = items;
     B.queue = queue;
-    // one system alone runs on its tuned grid (letkf_set_tuning); a batch fills every SM
-    const int grid = n == 1 && f[order[0]].c->fused_grid > 0 ? f[order[0]].c->fused_grid : sms;
-    fused_kernel<<<std::min(grid, items), FT, smem, stream>>>(B);
+    if (L.two)
+        fused_kernel<true><<<L.grid, FT, L.smem, stream>>>(B);
+    else
+        fused_kernel<false><<<L.grid, FT, L.smem, stream>>>(B);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     for (int k = 0; k < n; ++k) {
         letkf_ctx* c = f[order[k]].c;
@@ -2761,7 +3087,8 @@ int graph_capture(letkf_ctx* c, int p) {
     const bool dense = c->Lq != nullptr || c->Lt != nullptr;
     thread_local FusedBatch B;
     FusedFrame f{c, nullptr, 0.0, nullptr, 1};
-    fill_desc(f, dense ? static_cast<const float*>(c->Vbuf[p]) : nullptr, &B.sys[0]);
+    const FusedLaunch L = fused_launch(&f, 1, c->sms);
+    fill_desc(f, dense ? static_cast<const float*>(c->Vbuf[p]) : nullptr, L.two, &B.sys[0]);
     B.sys[0].item0 = 0;
     B.n_sys = 1;
     B.n_items = c->n_dom;
@@ -2773,7 +3100,8 @@ int graph_capture(letkf_ctx* c, int p) {
     // them for SMs at launch, and it reads nothing the kernel writes.
     cudaStream_t cs = c->cap_stream;
     if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LETKF_ECUDA;
-    fused_kernel<<<std::min(c->fused_grid > 0 ? c->fused_grid : c->sms, c->n_dom), FT, c->fused_smem, cs>>>(B);
+    void* fargs[1] = {&B};
+    cudaLaunchKernel(L.fn, dim3(L.grid), dim3(FT), fargs, L.smem, cs);
     bool ok = cudaGetLastError() == cudaSuccess;
     if (ok && dense) {
         NormalsNode nn;
@@ -2812,7 +3140,7 @@ int graph_capture(letkf_ctx* c, int p) {
         if (cudaGraphNodeGetType(nd, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
         cudaKernelNodeParams kp;
         if (cudaGraphKernelNodeGetParams(nd, &kp) != cudaSuccess) continue;
-        if (kp.func == reinterpret_cast<void*>(fused_kernel)) c->gnode_fused[p] = nd;
+        if (kp.func == L.fn) c->gnode_fused[p] = nd;
         else if (kp.func == nn.params.func) c->gnode_normals[p] = nd;
     }
     if (!c->gnode_fused[p] || (dense && !c->gnode_normals[p])) return LETKF_ECUDA;
@@ -2847,17 +3175,18 @@ int graph_step(letkf_ctx* c, const void* y, double sigma, void* xpred) {
     }
     thread_local FusedBatch B;
     FusedFrame f{c, y, sigma, xpred, 1};
-    fill_desc(f, V, &B.sys[0]);
+    const FusedLaunch L = fused_launch(&f, 1, c->sms);
+    fill_desc(f, V, L.two, &B.sys[0]);
     B.sys[0].item0 = 0;
     B.n_sys = 1;
     B.n_items = c->n_dom;
     B.queue = c->d_queue;
     void* args[1] = {&B};
     cudaKernelNodeParams kp;
-    kp.func = reinterpret_cast<void*>(fused_kernel);
-    kp.gridDim = dim3(std::min(c->fused_grid > 0 ? c->fused_grid : c->sms, c->n_dom));
+    kp.func = const_cast<void*>(L.fn);
+    kp.gridDim = dim3(L.grid);
     kp.blockDim = dim3(FT);
-    kp.sharedMemBytes = c->fused_smem;
+    kp.sharedMemBytes = L.smem;
     kp.kernelParams = args;
     kp.extra = nullptr;
     if (cudaGraphExecKernelNodeSetParams(c->gexec[p], c->gnode_fused[p], &kp) != cudaSuccess) return LETKF_ECUDA;

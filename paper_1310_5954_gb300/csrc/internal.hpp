@@ -94,6 +94,7 @@ struct letkf_ctx {
     int* d_queue = nullptr;         // fused kernel: [0] work queue, [1] CTAs done, [2] non-finite slope seen
     size_t device_bytes = 0;
     int fused_smem = 0;             // dynamic shared memory of the fused kernel
+    int fused_smem2 = 0;            // the same with two CTAs per SM (0: does not fit)
     int fused_grid = 0;
     int dual = 0;                   // fused analysis in observation space (m >= 128)
     void* scratch = nullptr;        // dual form: per-CTA halo anomalies, SMs x scratch_stride floats
