@@ -40,6 +40,10 @@ namespace {
 using namespace umma;
 
 constexpr int FT = 256;                  // threads per CTA
+// Threads per CTA of the dual form's kernel: its CTA has the SM to itself, and the elementwise passes
+// between its products are short chains per thread (ELT, m = 200: 267 -> 235 us with the leaner passes; the
+// m x m form gained nothing from the same).
+constexpr int FTD = 512;
 constexpr int MT = 128;                  // MMA rows
 constexpr long long WAIT_CYCLES = 4000000000LL;  // ~2 s at 2 GHz: a wait that long means a fault
 // ||I - P||_F below which the next Newton-Schulz update is the last: the update squares it
@@ -137,10 +141,11 @@ struct Ctrl {
     int flag;
     float s;
     float rn;
-    float red[FT / 32];
-    SysDesc sd;          // the current item's system (copied from the kernel parameters)
+    float red[FTD / 32];
 };
 static_assert(sizeof(Ctrl) <= 1024, "control block overlaps the vector area");
+// Dual form: offset of Z's FP32 rows in the big region, past the partial sums and the incidence of S^T u.
+constexpr int DUAL_ZF = FTD * 16 + 1024;
 
 // Kernel parameters of one launch (read through the constant bank).  One launch of one
 // system and one launch of many run the same code, so a system's results do not depend on
@@ -174,6 +179,19 @@ __device__ __forceinline__ void store8_at(unsigned char* hi_base, unsigned char*
 __device__ __forceinline__ void store8(unsigned char* hi_base, unsigned char* lo_base, int row, int k0, int K,
                                        const float* v, bool with_lo) {
     store8_at(hi_base, lo_base, op_offset(row, k0, K), v, with_lo);
+}
+
+// Eight consecutive values of a split operand: high + low BF16 parts.
+__device__ __forceinline__ void op_row8(const unsigned char* hi, const unsigned char* lo, uint32_t off, float (&v)[8]) {
+    const uint4 h = *reinterpret_cast<const uint4*>(hi + off), l = *reinterpret_cast<const uint4*>(lo + off);
+    const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const float2 fh = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw[u]));
+        const float2 fl = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&lw[u]));
+        v[2 * u] = fh.x + fl.x;
+        v[2 * u + 1] = fh.y + fl.y;
+    }
 }
 
 // Issue D = sum over terms of X_t * op(W_t) on a (MT x N) tile with K columns (no commit).
@@ -268,13 +286,14 @@ __device__ bool wait_all2(Ctrl* ctl, uint32_t p1, uint32_t p2, int* status) {
     return true;
 }
 
+template <int NT = FT>
 __device__ __forceinline__ float block_sum(Ctrl* ctl, float v) {
     v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) ctl->red[threadIdx.x >> 5] = v;
     __syncthreads();
     float s = 0.f;
 #pragma unroll
-    for (int w = 0; w < FT / 32; ++w) s += ctl->red[w];
+    for (int w = 0; w < NT / 32; ++w) s += ctl->red[w];
     __syncthreads();
     return s;
 }
@@ -378,6 +397,7 @@ __device__ __forceinline__ float block_sum_open(Ctrl* ctl, float v) {
 }
 
 // Domains with no observation: rows copied exactly, and the forecast applied.
+template <int FT>
 __device__ __forceinline__ void simt_rows(const SysDesc& A, int e0, int n_own) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int e = warp; e < n_own; e += FT / 32) {
@@ -462,6 +482,7 @@ __device__ void fetch_item(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, 
 // The last CTA of the launch: systems whose frame met a non-finite slope get their state back
 // unchanged (and the prediction of that state); every system's frame flag is published and the
 // per-launch counters are reset for the next launch.
+template <int FT>
 __device__ void finish_batch(const FusedBatch& B) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int si = 0; si < B.n_sys; ++si) {
@@ -507,11 +528,11 @@ __device__ void finish_batch(const FusedBatch& B) {
 // eigenvalues of I + Z lie in (1, 2]), and u is refined against the exact operator.  Halo
 // anomalies stay in a per-CTA global scratch (L2-resident), so shared memory holds only the
 // operands of one product at a time.
-__device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32_t tbase, uint32_t* ph_mma_io,
-                                          int d) {
-    const SysDesc A = ctl->sd;
+__device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsigned char* smem, uint32_t tbase,
+                                             uint32_t* ph_mma_io, int d) {
+    constexpr int FT = FTD;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row = 32 * (warp & 3) + lane, hh = warp >> 2;
+    const int row = 32 * (warp & 3) + lane, hh = warp >> 2;      // TMEM lane; column group
     const int uwarp = uniform_warp();
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
     uint32_t ph_mma = *ph_mma_io;
@@ -534,8 +555,11 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     const int h0 = A.tab.halo_off[d], n_h = A.tab.halo_off[d + 1] - h0;
     const int P = 2 * n_obs;
     const int n_e = (A.with_forecast && A.a2 == 0.f) ? n_own : 2 * n_own;   // AR(2) needs both instants
-    // p-space matrices: NP x NP, this thread's TMEM lane `row`, columns col0 .. col0 + NP/2
-    const int half = NP / 2, nq = half / 8, col0 = hh * half;
+    // p-space matrices: NP x NP, this thread's TMEM lane `row`, the 8-column chunks of column group hh of four
+    const int c0 = ((NP >> 3) * hh >> 2), nq = ((NP >> 3) * (hh + 1) >> 2) - c0, col0 = 8 * c0;
+    const uint32_t off0 = op_offset(row, col0, NP);             // its operand bytes; a chunk is 128 on
+    const int rw0 = 32 * (warp & 3);
+    auto on_diag = [&](int q8) { return col0 + 8 * q8 < rw0 + 32 && col0 + 8 * q8 + 8 > rw0; };
     const uint32_t tl = tbase + lane_off + (uint32_t)col0;
     unsigned char* Yh = big;
     unsigned char* Yl = big + A.sz_op;
@@ -595,8 +619,8 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
                 zv[u] = __uint_as_float(rz[u]);
             }
             if (row < NP) {
-                store8(Yh, Yl, row, col0 + 8 * q8, NP, yv, true);
-                store8(Zh, Zl, row, col0 + 8 * q8, NP, zv, true);
+                store8_at(Yh, Yl, off0 + 128u * q8, yv, true);
+                store8_at(Zh, Zl, off0 + 128u * q8, zv, true);
             }
         }
     };
@@ -640,7 +664,6 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
             if (l16 == 0) xh_mean[j] = mu;
         }
     }
-    float* hv = vec + 1536;                          // 256: halo-actuator vector
     int* pcs = reinterpret_cast<int*>(vec + 1792);   // 64: the domain's packed corners
     for (int s = tid; s < n_obs; s += FT) pcs[s] = A.tab.obs_corner[o0 + s];
     __syncthreads();
@@ -653,6 +676,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         const float yv = (k & 1) == 0 ? A.y[sub] : A.y[A.n_subv + sub];
         dvec[k] = (yv - sl) * A.inv_sigma;
     }
+    if (tid >= P && tid < 128) dvec[tid] = 0.f;      // past its end: read as zeros with Z's padding
     // S as an NP x MP operand (rows: slopes, K: members): both slopes of a subaperture from one
     //      read of its four corners' anomalies, eight members at a time
     auto restage = [&](float4* dst4) {    // the halo anomalies' rows from the scratch (L2) into shared memory
@@ -707,10 +731,9 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
             float g[8];
             tmem_ld8(tl + TM_G + 8 * q8, g);
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (row < P && col0 + 8 * q8 + u < P) fr += g[u] * g[u];
+            for (int u = 0; u < 8; ++u) fr += g[u] * g[u];    // (K is zero past P)
         }
-        return block_sum(ctl, fr);
+        return block_sum<FT>(ctl, row < P ? fr : 0.f);
     };
     float fro = read_fro();
     if (A.gram_terms < 3 && 1.f + sqrtf(fro) / c > A.s_split) {
@@ -730,41 +753,55 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     const float ns_last = ns_stop(A.ns_last, A.gram_terms, s_scale, A.s_split);
     const float id_scale = 1.f / s_ns;   // A_s = I / s_ns + K / (c s_ns) by multiplications
     // ---- Z = ((I + K/c)/s)^(-1/2) by the coupled Newton-Schulz iteration (dimension P), from
-    //      Y_0 = A_s, Z_0 = I: the first step's P_0 = Z_0 Y_0 is Y_0 itself, so one pass over G
-    //      writes Y_0, T_0 = (3I - Y_0)/2, Z_0 and the residual, and the step's two products follow
+    //      Y_0 = A_s, Z_0 = I: the first step's P_0 = Z_0 Y_0 is Y_0 itself and Z_1 is T_0, so one
+    //      pass over G writes Y_0, T_0 = (3I - Y_0)/2 as Z_1 and the residual; Y_1 = Y_0 T_0 reads T_0
+    //      from Z's buffer (symmetric: both operand layouts hold the same bytes).  All iterates are
+    //      zero past P, so the passes need the identity only in chunks that meet the diagonal.
     float r2_0 = 0.f;
 #pragma unroll 1
     for (int q8 = 0; q8 < nq; ++q8) {
-        float g[8], yv[8], zv[8], tv[8];
+        float g[8], yv[8], tv[8];
         tmem_ld8(tl + TM_G + 8 * q8, g);
+        if (!on_diag(q8)) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int j = col0 + 8 * q8 + u;
-            const bool in = row < P && j < P;
-            const float id = (row == j) ? 1.f : 0.f;
-            yv[u] = in ? fmaf(g[u], inv_cs, id * id_scale) : 0.f;
-            zv[u] = in ? id : 0.f;
-            tv[u] = in ? 1.5f * id - 0.5f * yv[u] : 0.f;
-            if (in) r2_0 += (id - yv[u]) * (id - yv[u]);
+            for (int u = 0; u < 8; ++u) {
+                yv[u] = g[u] * inv_cs;
+                r2_0 += yv[u] * yv[u];
+                tv[u] = -0.5f * yv[u];
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float id = (row == col0 + 8 * q8 + u && row < P) ? 1.f : 0.f;
+                yv[u] = fmaf(g[u], inv_cs, id * id_scale);
+                r2_0 += (id - yv[u]) * (id - yv[u]);
+                tv[u] = 1.5f * id - 0.5f * yv[u];
+            }
         }
         if (row < NP) {
-            store8(Yh, Yl, row, col0 + 8 * q8, NP, yv, true);
-            store8(Zh, Zl, row, col0 + 8 * q8, NP, zv, true);
-            store8(Th, Tl, row, col0 + 8 * q8, NP, tv, true);
+            store8_at(Yh, Yl, off0 + 128u * q8, yv, true);
+            store8_at(Zh, Zl, off0 + 128u * q8, tv, true);
         }
     }
-    float rn_prev = sqrtf(block_sum(ctl, r2_0));
-    bool z_in_tmem = false, more = false;
+    float rn_prev = sqrtf(block_sum<FT>(ctl, row < P ? r2_0 : 0.f));
+    int z_state = 0;       // where Z ends: 0 identity, 1 its operands, 2 tensor memory
+    bool more = false;
     int it = 0;
     if (rn_prev >= 2e-6f * (float)P) {   // else converged at once: Z = I
-        to_mma();
-        const bool last0 = rn_prev < ns_last;
-        if (!yt_tz(Yh, Yl, Th, Tl, Zh, Zl, !last0)) return false;    // Y_1 = Y_0 T_0, Z_1 = T_0 Z_0
-        z_in_tmem = true;
-        if (!last0) {                    // else the update was the last: Z_1 = T_0
+        z_state = 1;                     // Z_1 = T_0
+        if (rn_prev >= ns_last) {        // else that update was the last
+            to_mma();
+            if (uwarp == 0 && elect_one()) {
+                tc_fence_after();
+                issue_product(tbase + TM_Y, Yh, Yl, Zh, Zl, NP, NP, 3, 1);     // Y_1 = Y_0 T_0
+                mma_commit(&ctl->bar_mma);
+            }
+            if (!mma_wait()) return false;
             it = 1;
             more = true;
-            read_yz();
+            tmem_rows(tl + TM_Y, nq, [&](int q8, const float (&yv)[8]) {
+                if (row < NP) store8_at(Yh, Yl, off0 + 128u * q8, yv, true);
+            });
             to_mma();
         }
     }
@@ -779,26 +816,31 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         float r2 = 0.f;
         tmem_rows(tl + TM_P, nq, [&](int q8, const float (&pv)[8]) {
             float tv[8];
+            if (!on_diag(q8)) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int j = col0 + 8 * q8 + u;
-                const bool in = row < P && j < P;
-                const float id = (row == j) ? 1.f : 0.f;
-                const float rr = id - pv[u];
-                if (in) r2 += rr * rr;
-                tv[u] = in ? 1.5f * id - 0.5f * pv[u] : 0.f;
+                for (int u = 0; u < 8; ++u) {
+                    r2 += pv[u] * pv[u];
+                    tv[u] = -0.5f * pv[u];
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const float id = (row == col0 + 8 * q8 + u && row < P) ? 1.f : 0.f;
+                    const float rr = id - pv[u];
+                    r2 += rr * rr;
+                    tv[u] = 1.5f * id - 0.5f * pv[u];
+                }
             }
-            if (row < NP) store8(Th, Tl, row, col0 + 8 * q8, NP, tv, true);
+            if (row < NP) store8_at(Th, Tl, off0 + 128u * q8, tv, true);
         });
-        r2 = sum_to_mma(r2);              // one barrier: the residual and T to the tensor core
+        r2 = sum_to_mma(row < P ? r2 : 0.f);   // one barrier: the residual and T to the tensor core
         const float rn = sqrtf(r2);
         const bool conv = rn < 2e-6f * (float)P || (rn < 2e-2f && rn > 0.6f * rn_prev);
         rn_prev = rn;
-        if (conv) break;
         // the last update (see the m x m form): only T Z is used afterwards
-        const bool last = rn < ns_last;
+        const bool last = conv || rn < ns_last;
         if (!yt_tz(Yh, Yl, Th, Tl, Zh, Zl, !last)) return false;
-        z_in_tmem = true;
+        z_state = 2;
         if (last) break;
         read_yz();
         to_mma();
@@ -807,17 +849,32 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    auto zrow = [&](int q8, float (&zv)[8]) {       // 8 columns of this thread's half-row of Z_ns
-        if (z_in_tmem) {
+    auto zrow = [&](int q8, float (&zv)[8]) {       // 8 columns of this thread's part of Z_ns
+        if (z_state == 2) {
             tmem_ld8(tl + TM_Z + 8 * q8, zv);
+        } else if (z_state == 1) {
+            op_row8(Zh, Zl, row < NP ? off0 + 128u * q8 : 0u, zv);
         } else {
 #pragma unroll
             for (int u = 0; u < 8; ++u) zv[u] = (row == col0 + 8 * q8 + u && row < P) ? 1.f : 0.f;
         }
     };
+    if (z_state != 2) {    // its operands' place is needed: into tensor memory first
+#pragma unroll 1
+        for (int q8 = 0; q8 < nq; ++q8) {
+            float zv[8];
+            zrow(q8, zv);
+            tmem_st8(tl + TM_Z + 8 * q8, zv);
+        }
+        tmem_wait_st();
+        z_state = 2;
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+    }
     // Z_ns's rows in FP32 in the big region for the mean weights (free between the iterations);
     // each thread writes and reads only its own half-row
-    float* zf = reinterpret_cast<float*>(big + 8192);
+    float* zf = reinterpret_cast<float*>(big + DUAL_ZF);
     const int zld = NP + 4;
 #pragma unroll 1
     for (int q8 = 0; q8 < nq; ++q8) {
@@ -829,24 +886,27 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
             d4[1] = make_float4(zv[4], zv[5], zv[6], zv[7]);
         }
     }
+    float* hv = vec + 1536;                          // 256: halo-actuator vector
+    // the column groups' partial sums (0, 1 in vtmp, 2, 3 in hv, which holds nothing then)
+    auto vpart = [&](int g) { return g < 2 ? vtmp + 128 * g : hv + 128 * (g - 2); };
+    auto vsum = [&](int r) { return (vpart(0)[r] + vpart(1)[r]) + (vpart(2)[r] + vpart(3)[r]); };
     auto zmatvec = [&](const float* x_in, float* y_out) {   // y = Z_ns x over the first P entries
         float part = 0.f;
         if (row < NP) {
             const float4* z4 = reinterpret_cast<const float4*>(zf + row * zld + col0);
             const float4* x4 = reinterpret_cast<const float4*>(x_in + col0);
 #pragma unroll 2
-            for (int q = 0; q < 2 * nq; ++q) {
+            for (int q = 0; q < 2 * nq; ++q) {      // (Z and x are zero past P)
                 const float4 z = z4[q], x = x4[q];
-                const int j = col0 + 4 * q;
-                if (j + 0 < P) part += z.x * x.x;
-                if (j + 1 < P) part += z.y * x.y;
-                if (j + 2 < P) part += z.z * x.z;
-                if (j + 3 < P) part += z.w * x.w;
+                part += z.x * x.x;
+                part += z.y * x.y;
+                part += z.z * x.z;
+                part += z.w * x.w;
             }
         }
-        vtmp[hh * 128 + row] = part;
+        vpart(hh)[row] = part;
         __syncthreads();
-        if (hh == 0) y_out[row] = (row < P) ? vtmp[row] + vtmp[128 + row] : 0.f;
+        if (hh == 0) y_out[row] = (row < P) ? vsum(row) : 0.f;
         __syncthreads();
     };
     // the halo anomalies' rows for the mean weights: in shared memory past Z's rows when they fit
@@ -942,6 +1002,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     for (int ref = 0; ref < n_ref; ++ref) {
         st_times(uvp, wbar);                                   // S^T u
         xh_times(wbar, hv);                                    // h = X'_h (S^T u)
+        if (tid >= P && tid < 128) vr[tid] = 0.f;
         for (int k = tid; k < P; k += FT) {                    // rho = d - c u - S (S^T u)
             const int pc = pcs[k >> 1];
             const float a00 = hv[pc & 0xFF], a01 = hv[(pc >> 8) & 0xFF];
@@ -976,17 +1037,23 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     for (int q8 = 0; q8 < nq; ++q8) {               // M = I + Z into Y's buffers, X_1 into T's
         float zv[8], mv[8], xv[8];
         zrow(q8, zv);
+        if (!on_diag(q8)) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int j = col0 + 8 * q8 + u;
-            const bool in = row < P && j < P;
-            const float id = (row == j) ? 1.f : 0.f;
-            mv[u] = in ? id + zv[u] * rs : 0.f;
-            xv[u] = in ? 2.f * alpha * id - alpha * alpha * mv[u] : 0.f;
+            for (int u = 0; u < 8; ++u) {
+                mv[u] = zv[u] * rs;
+                xv[u] = -(alpha * alpha) * mv[u];
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float id = (row == col0 + 8 * q8 + u && row < P) ? 1.f : 0.f;
+                mv[u] = id + zv[u] * rs;
+                xv[u] = 2.f * alpha * id - alpha * alpha * mv[u];
+            }
         }
         if (row < NP) {
-            store8(Yh, Yl, row, col0 + 8 * q8, NP, mv, true);
-            store8(Th, Tl, row, col0 + 8 * q8, NP, xv, true);
+            store8_at(Yh, Yl, off0 + 128u * q8, mv, true);
+            store8_at(Th, Tl, off0 + 128u * q8, xv, true);
         }
     }
     to_mma();
@@ -998,21 +1065,25 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         }
         if (!mma_wait()) return false;
         float r2 = 0.f;
-#pragma unroll 1
-        for (int q8 = 0; q8 < nq; ++q8) {
-            float qv[8], rv[8];
-            tmem_ld8(tl + TM_P + 8 * q8, qv);
+        tmem_rows(tl + TM_P, nq, [&](int q8, const float (&qv)[8]) {
+            float rv[8];
+            if (!on_diag(q8)) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int j = col0 + 8 * q8 + u;
-                const bool in = row < P && j < P;
-                const float id = (row == j) ? 1.f : 0.f;
-                if (in) r2 += (id - qv[u]) * (id - qv[u]);
-                rv[u] = in ? 2.f * id - qv[u] : 0.f;
+                for (int u = 0; u < 8; ++u) {
+                    r2 += qv[u] * qv[u];
+                    rv[u] = -qv[u];
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const float id = (row == col0 + 8 * q8 + u && row < P) ? 1.f : 0.f;
+                    r2 += (id - qv[u]) * (id - qv[u]);
+                    rv[u] = 2.f * id - qv[u];
+                }
             }
-            if (row < NP) store8(Zh, Zl, row, col0 + 8 * q8, NP, rv, true);   // Z's operand is not needed
-        }
-        r2 = block_sum(ctl, r2);
+            if (row < NP) store8_at(Zh, Zl, off0 + 128u * q8, rv, true);   // Z's operand is not needed
+        });
+        r2 = block_sum<FT>(ctl, row < P ? r2 : 0.f);
         if (k > 0 && sqrtf(r2) < 1e-6f * (float)P) break;
         const bool last = r2 < 1e-6f * (float)P;     // the update lands ||R||_F under the bound
         to_mma();
@@ -1023,12 +1094,9 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         }
         if (!mma_wait()) return false;
         if (last) break;                            // X stays in tensor memory
-#pragma unroll 1
-        for (int q8 = 0; q8 < nq; ++q8) {
-            float xv[8];
-            tmem_ld8(tl + TM_G + 8 * q8, xv);
-            if (row < NP) store8(Th, Tl, row, col0 + 8 * q8, NP, xv, true);
-        }
+        tmem_rows(tl + TM_G, nq, [&](int q8, const float (&xv)[8]) {
+            if (row < NP) store8_at(Th, Tl, off0 + 128u * q8, xv, true);
+        });
         to_mma();
     }
     tc_fence_before();
@@ -1052,8 +1120,8 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         float zv[8];
         zrow(q8, zv);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) zv[u] = (row < P && col0 + 8 * q8 + u < P) ? zv[u] * zscale : 0.f;
-        if (row < NP) store8(Zt_h, Zt_l, row, col0 + 8 * q8, NP, zv, true);
+        for (int u = 0; u < 8; ++u) zv[u] *= zscale;
+        if (row < NP) store8_at(Zt_h, Zt_l, off0 + 128u * q8, zv, true);
     }
     if (!A.hs_w) write_S(Wh, Wl, Xs4);
     to_mma();
@@ -1093,35 +1161,32 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         }
     }
     if (!mma_wait()) return false;
-    const int mhalf = MP / 2, mq = mhalf / 8, mcol0 = hh * mhalf;
+    const int mc0 = ((MP >> 3) * hh >> 2), mq = ((MP >> 3) * (hh + 1) >> 2) - mc0, mcol0 = 8 * mc0;
+    const uint32_t moff0 = op_offset(row, mcol0, MP);
     const uint32_t tlm = tbase + lane_off + (uint32_t)mcol0;
-#pragma unroll 1
-    for (int q8 = 0; q8 < mq; ++q8) {               // W -> operand over S
-        float wv[8];
-        tmem_ld8(tlm + TM_Y + 8 * q8, wv);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) wv[u] = (row < P && mcol0 + 8 * q8 + u < m) ? wv[u] : 0.f;
-        if (row < NP) store8(Wh, Wl, row, mcol0 + 8 * q8, MP, wv, true);
+    tmem_rows(tlm + TM_Y, mq, [&](int q8, const float (&wv)[8]) {   // W -> operand over S (zero past P and m)
+        if (row < NP) store8_at(Wh, Wl, moff0 + 128u * q8, wv, true);
         if (cap && row < P)
 #pragma unroll
             for (int u = 0; u < 8; ++u)
                 if (mcol0 + 8 * q8 + u < m) A.cap[CAP_HDR + m + row * m + mcol0 + 8 * q8 + u] = wv[u];
-    }
+    });
     unsigned char* A1h = big;                       // X'_E (RA x MP) over Z's operand
     unsigned char* A1l = big + RA * MP * 2;
-    for (int t = tid; t < RA * (MP >> 3); t += FT) {
-        const int e = t % RA, kc = t / RA;
-        float v[8];
+    // its own n_e rows (what the rows past them hold only reaches rows of the products that are not
+    // read): a warp per row, a chunk of 8 members per lane
+    for (int e = warp; e < n_e; e += FT / 32) {
+        const int r = e < n_own ? A.tab.own[e0 + e] : A.n_act + A.tab.own[e0 + e - n_own];
+        const float mu = xe_mean[e];
+        for (int kc = lane; kc < (MP >> 3); kc += 32) {
+            float v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = 0.f;
-        if (e < n_e) {
-            const int r = e < n_own ? A.tab.own[e0 + e] : A.n_act + A.tab.own[e0 + e - n_own];
-            get8(A.X + (size_t)r * A.m_pad + kc * 8, v, min(8, A.m_pad - kc * 8));
-            const float mu = xe_mean[e];
+            for (int u = 0; u < 8; ++u) v[u] = 0.f;
+            if (kc * 8 < m) get8(A.X + (size_t)r * A.m_pad + kc * 8, v, min(8, A.m_pad - kc * 8));
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = kc * 8 + u < m ? v[u] - mu : 0.f;
+            store8(A1h, A1l, e, kc * 8, MP, v, A.tr_terms > 1);
         }
-        store8(A1h, A1l, e, kc * 8, MP, v, A.tr_terms > 1);
     }
     to_mma();
     if (uwarp == 0 && elect_one()) {
@@ -1132,14 +1197,9 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     if (!mma_wait()) return false;
     unsigned char* Xh_op = big;                     // (I + Z)^-1 operand over A1
     unsigned char* Xl_op = big + A.sz_op;
-#pragma unroll 1
-    for (int q8 = 0; q8 < nq; ++q8) {
-        float xv[8];
-        tmem_ld8(tl + TM_G + 8 * q8, xv);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) xv[u] = (row < P && col0 + 8 * q8 + u < P) ? xv[u] : 0.f;
-        if (row < NP) store8(Xh_op, Xl_op, row, col0 + 8 * q8, NP, xv, true);
-    }
+    tmem_rows(tl + TM_G, nq, [&](int q8, const float (&xv)[8]) {    // (zero past P)
+        if (row < NP) store8_at(Xh_op, Xl_op, off0 + 128u * q8, xv, true);
+    });
     to_mma();
     if (uwarp == 0 && elect_one()) {
         tc_fence_after();
@@ -1149,26 +1209,16 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
     if (!mma_wait()) return false;
     unsigned char* A2h = big;                       // P1 (RA x NP) over X's operand
     unsigned char* A2l = big + RA * NP * 2;
-#pragma unroll 1
-    for (int q8 = 0; q8 < nq; ++q8) {
-        float pv[8];
-        tmem_ld8(tl + TM_P + 8 * q8, pv);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) pv[u] = (row < n_e && col0 + 8 * q8 + u < P) ? pv[u] : 0.f;
-        if (row < RA) store8(A2h, A2l, row, col0 + 8 * q8, NP, pv, A.tr_terms > 1);
-    }
-#pragma unroll 1
-    for (int q8 = 0; q8 < mq; ++q8) {               // XW -> operand over W
-        float wv[8];
-        tmem_ld8(tlm + TM_Y + 8 * q8, wv);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) wv[u] = (row < P && mcol0 + 8 * q8 + u < m) ? wv[u] : 0.f;
-        if (row < NP) store8(Wh, Wl, row, mcol0 + 8 * q8, MP, wv, true);
+    tmem_rows(tl + TM_P, nq, [&](int q8, const float (&pv)[8]) {    // (columns past P are zero: W's rows are)
+        if (row < n_e) store8_at(A2h, A2l, off0 + 128u * q8, pv, A.tr_terms > 1);
+    });
+    tmem_rows(tlm + TM_Y, mq, [&](int q8, const float (&wv)[8]) {   // XW -> operand over W (zero past P and m)
+        if (row < NP) store8_at(Wh, Wl, moff0 + 128u * q8, wv, true);
         if (cap && row < P)
 #pragma unroll
             for (int u = 0; u < 8; ++u)
                 if (mcol0 + 8 * q8 + u < m) A.cap[CAP_HDR + m + (P + row) * m + mcol0 + 8 * q8 + u] = wv[u];
-    }
+    });
     to_mma();
     if (uwarp == 0 && elect_one()) {
         tc_fence_after();
@@ -1187,15 +1237,14 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         float part = 0.f;
         tmem_rows(tlm + TM_Y, mq, [&](int q8, const float (&dv)[8]) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (mcol0 + 8 * q8 + u < m) part += dv[u];
+            for (int u = 0; u < 8; ++u) part += dv[u];          // (zero past m)
             if (mine) {
                 float4* dst = reinterpret_cast<float4*>(p3s + row * pld + mcol0 + 8 * q8);
                 dst[0] = make_float4(dv[0], dv[1], dv[2], dv[3]);
                 dst[1] = make_float4(dv[4], dv[5], dv[6], dv[7]);
             }
         });
-        vtmp[hh * 128 + row] = part;
+        vpart(hh)[row] = part;
         __syncthreads();
     }
     // AR(2) forecast: second-instant rows hand their analysis to the first-instant rows
@@ -1205,7 +1254,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         for (int t = tid; t < (n_e - n_own) * m; t += FT) {
             const int r = n_own + t / m, j = t - (t / m) * m;
             const int ja = A.tab.own[e0 + r - n_own];
-            const float p3mean = (vtmp[r] + vtmp[128 + r]) / (float)m;
+            const float p3mean = vsum(r) / (float)m;
             x2buf[(r - n_own) * A.m_pad + j] =
                 A.X[(size_t)(A.n_act + ja) * A.m_pad + j] + uvec[r] - (p3s[r * pld + j] - p3mean);
         }
@@ -1217,7 +1266,7 @@ __device__ __noinline__ bool analyse_dual(Ctrl* ctl, unsigned char* smem, uint32
         const bool row_w = !(ar2 && e >= n_own);
         const int ja = e < n_own ? A.tab.own[e0 + e] : A.tab.own[e0 + e - n_own];
         const int gr = e < n_own ? ja : A.n_act + ja;
-        const float p3mean = (vtmp[e] + vtmp[128 + e]) / (float)m;
+        const float p3mean = vsum(e) / (float)m;
         const float shift = uvec[e];
         float n1s = 0.f;
         for (int ck = lane; ck < nck && row_w; ck += 32) {
@@ -1375,7 +1424,7 @@ __device__ __forceinline__ void own_row_means(const SysDesc& A, const float* XE,
 template <bool TWO>
 __device__ __noinline__ const float* analyse_simt(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, int d,
                                                   int* ld_out) {
-    const SysDesc& A = TWO ? B.sys[ctl->sys] : ctl->sd;
+    const SysDesc& A = B.sys[ctl->sys];
     const int tid = threadIdx.x;
     const int m = A.m;
     const float c = (float)(m - 1);
@@ -1594,8 +1643,15 @@ __device__ __noinline__ const float* analyse_simt(const FusedBatch& B, Ctrl* ctl
 //     operands they are read once more for the mean weights.
 // Measured, 332 domains of m = 100: 118 k cycles for two domains side by side (92 k for one before), the
 // frame 156 -> 130 us; two such systems in one launch 294 -> 229 us.
-template <bool TWO>
-__global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_constant__ FusedBatch B) {
+//
+// DUAL: systems of the observation-space form, one CTA of twice the threads per SM (a kernel of its own:
+// its registers and code are not the m x m form's).
+enum FusedMode { MODE_ONE, MODE_TWO, MODE_DUAL };
+template <FusedMode MODE>
+__global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO ? 2 : 1)
+    fused_kernel(const __grid_constant__ FusedBatch B) {
+    constexpr bool TWO = MODE == MODE_TWO, DUAL = MODE == MODE_DUAL;
+    constexpr int NT = DUAL ? FTD : FT;
     constexpr int tG = TM_G, tP = TWO ? 0 : TM_P, tY = TWO ? 0 : TM_Y, tZ = TWO ? 128 : TM_Z;
     constexpr uint32_t tmem_cols = TWO ? TM_COLS / 2 : TM_COLS;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -1631,15 +1687,9 @@ __global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_con
     __syncthreads();
 
     while (ctl->item < B.n_items && !ctl->abort) {
-        if constexpr (!TWO) {
-            const uint32_t* src = reinterpret_cast<const uint32_t*>(&B.sys[ctl->sys]);
-            uint32_t* dst = reinterpret_cast<uint32_t*>(&ctl->sd);
-            for (int t = tid; t < (int)(sizeof(SysDesc) / 4); t += FT) dst[t] = src[t];
-            __syncthreads();
-        }
-        // by value: fields stay in registers across barriers; TWO, with half the registers, reads the
-        // constant bank where it needs them
-        typename std::conditional<TWO, const SysDesc&, const SysDesc>::type A = TWO ? B.sys[ctl->sys] : ctl->sd;
+        // ONE: by value, fields stay in registers across barriers; the others, with half the registers per
+        // thread, read the constant bank where they need them
+        typename std::conditional<MODE == MODE_ONE, const SysDesc, const SysDesc&>::type A = B.sys[ctl->sys];
         const int d = ctl->dom;
         float* vec = reinterpret_cast<float*>(smem + A.off_vec);
         float* xh_mean = vec;            // 256 (halo actuators)
@@ -1683,7 +1733,7 @@ __global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_con
         const int p_loc = 2 * n_obs;
         const int n_e = (A.with_forecast && A.a2 == 0.f) ? n_own : 2 * n_own;   // AR(2) needs both instants
         if (n_obs == 0) {
-            simt_rows(A, e0, n_own);
+            simt_rows<NT>(A, e0, n_own);
             __syncthreads();
             if (warp == 0) fetch_item(B, ctl, smem, fetch_all);
             __syncthreads();
@@ -1731,7 +1781,7 @@ __global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_con
                 XE = reinterpret_cast<float*>(big + A.off_sxe);
                 copy_own();
             }
-        } else if (warp == 0 && !A.dual && !ctl->loaded) {
+        } else if (!DUAL && warp == 0 && !ctl->loaded) {
             issue_loads(A, d, Xh, XE, &ctl->bar_load);
         }
         // ---- frame ingest: a non-finite slope in this domain's observation region rejects the
@@ -1739,31 +1789,29 @@ __global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_con
         // (the m x m forms keep the region's slopes in shared memory for the innovation row)
         float* ys = vec + 1856;          // 128: x and y slope of each observed subaperture
         int nonfinite = 0;
-        for (int t = tid; t < n_obs; t += FT) {
+        for (int t = tid; t < n_obs; t += NT) {
             const int sub = A.tab.obs_sub[o0 + t];
             const float yx = A.y[sub], yy = A.y[A.n_subv + sub];
             if (!isfinite(yx) || !isfinite(yy)) nonfinite = 1;
-            if (!A.dual) {
+            if (!DUAL) {
                 ys[2 * t] = yx;
                 ys[2 * t + 1] = yy;
             }
         }
         const bool dom_bad = __syncthreads_or(nonfinite) != 0;
-        if constexpr (!TWO)
-        if (A.dual) {
+        if constexpr (DUAL) {
             if (dom_bad) {
                 if (tid == 0) {
                     atomicExch(A.dom_bad, 1);
                     atomicOr(A.status, ST_NONFINITE);
                 }
             } else {
-                if (!analyse_dual(ctl, smem, tbase, &ph_mma, d)) break;
+                if (!analyse_dual(A, ctl, smem, tbase, &ph_mma, d)) break;
             }
             __syncthreads();
             if (warp == 0) fetch_item(B, ctl, smem, 1 << 30);
             __syncthreads();
-            continue;
-        }
+        } else {
         // ---- 1. the halo rows of the observed instant and the own rows
         if constexpr (!TWO) {
             if (!wait_all(ctl, &ctl->bar_load, ph_load, A.status)) break;
@@ -2555,9 +2603,10 @@ __global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_con
             __syncthreads();
         }
         tc_fence_after();
+        }
     }
     // a wait that ran out may leave bulk copies in flight: give them a bounded time to land
-    if (!TWO && ctl->abort && tid == 0) mbar_wait_bounded(&ctl->bar_load, ph_load, WAIT_CYCLES);
+    if (MODE == MODE_ONE && ctl->abort && tid == 0) mbar_wait_bounded(&ctl->bar_load, ph_load, WAIT_CYCLES);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -2569,7 +2618,9 @@ __global__ void __launch_bounds__(FT, TWO ? 2 : 1) fused_kernel(const __grid_con
         if (ctl->last) __threadfence();
     }
     __syncthreads();
-    if (ctl->last) finish_batch(B);
+    if (ctl->last) finish_batch<NT>(B);
+    // launched behind another of the same batch (launch_batch): complete only after it
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Self-test of the tensor-core product: D (128 x N) = A (128 x K) * B (N x K)^T, operands
@@ -2705,7 +2756,7 @@ FusedLayout fused_layout(const letkf_ctx* c) {
         const int limit = 227 * 1024 - L.off_big;
         L.off_hs = round_up(gram, 1024);
         if (L.off_hs + hs_bytes > limit) L.off_hs = -1;
-        L.off_hs2 = round_up(8192 + L.NP * (L.NP + 4) * 4, 1024);
+        L.off_hs2 = round_up(DUAL_ZF + L.NP * (L.NP + 4) * 4, 1024);
         if (L.off_hs2 + hs_bytes > limit) L.off_hs2 = -1;
         L.hs_w = hs_bytes <= L.sz_a ? 1 : 0;
         if (L.off_hs >= 0) big = std::max(big, round_up(L.off_hs + hs_bytes, 1024));
@@ -2843,10 +2894,13 @@ int fused_prepare(letkf_ctx* c) {
         c->device_bytes += sb;
     }
     static_assert(sizeof(FusedBatch) < 32000, "kernel parameters too large");
-    if (cudaFuncSetAttribute(fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
+    if (cudaFuncSetAttribute(fused_kernel<MODE_ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TWO_SMEM) != cudaSuccess ||
-        cudaFuncSetAttribute(fused_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        cudaFuncSetAttribute(fused_kernel<MODE_DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(fused_kernel<MODE_TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, TWO_SMEM) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(fused_kernel<MODE_TWO>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared) != cudaSuccess)
         return LETKF_ECUDA;
     // One CTA per SM pulling domains from the work queue: domains differ in cost (edge domains
@@ -2978,62 +3032,91 @@ void fill_desc(const FusedFrame& f, const float* V, bool two, SysDesc* S) {
     S->cap_dom = c->cap_dom;
 }
 
-// Descriptor of system c's next frame; `stream` (the kernel's) waits for its noise block.
-int make_desc(const FusedFrame& f, cudaStream_t stream, bool two, SysDesc* S) {
-    const float* V = nullptr;
-    if (f.with_forecast && (f.c->Lq || f.c->Lt)) {
-        const int rc = noise_ready(f.c, f.c->frame, stream, &V);
-        if (rc) return rc;
-    }
-    fill_desc(f, V, two, S);
-    return LETKF_OK;
-}
-
-// How a launch over n systems' frames runs: two CTAs per SM when every system fits them and there are
-// more domains than SMs, else one (a lone domain per SM is faster with the SM's registers and shared
-// memory to itself).  One system alone runs on its tuned grid (letkf_set_tuning); a batch fills every SM.
+// How a launch over n systems' frames (all dual or none) runs: two CTAs per SM when every system fits
+// them and there are more domains than SMs, else one (a lone domain per SM is faster with the SM's
+// registers and shared memory to itself).  One system alone runs on its tuned grid (letkf_set_tuning); a batch
+// fills every SM.
 struct FusedLaunch {
     bool two;
     int grid, smem;
     const void* fn;
+    int threads;
 };
-FusedLaunch fused_launch(const FusedFrame* f, int n, int sms) {
-    FusedLaunch l{true, 0, 0, nullptr};
+FusedLaunch fused_launch(const FusedFrame* f, const int* order, int n, int sms) {
+    FusedLaunch l{true, 0, 0, nullptr, FT};
     int items = 0, smem1 = 0, smem2 = 0;
     for (int k = 0; k < n; ++k) {
-        const letkf_ctx* c = f[k].c;
+        const letkf_ctx* c = f[order[k]].c;
         items += c->n_dom;
         smem1 = std::max(smem1, c->fused_smem);
         smem2 = std::max(smem2, c->fused_smem2);
         l.two = l.two && c->fused_smem2 > 0;
     }
-    const int per_sm = n == 1 && f[0].c->fused_grid > 0 ? f[0].c->fused_grid : sms;
+    const letkf_ctx* c0 = f[order[0]].c;
+    const int per_sm = n == 1 && c0->fused_grid > 0 ? c0->fused_grid : sms;
     l.two = l.two && items > sms;
     l.grid = std::min(l.two ? 2 * per_sm : per_sm, items);
     l.smem = l.two ? smem2 : smem1;
-    l.fn = l.two ? reinterpret_cast<const void*>(fused_kernel<true>) : reinterpret_cast<const void*>(fused_kernel<false>);
+    l.threads = c0->dual ? FTD : FT;
+    l.fn = c0->dual ? reinterpret_cast<const void*>(fused_kernel<MODE_DUAL>)
+           : l.two  ? reinterpret_cast<const void*>(fused_kernel<MODE_TWO>)
+                    : reinterpret_cast<const void*>(fused_kernel<MODE_ONE>);
     return l;
 }
 
-int launch_batch(const FusedFrame* f, const int* order, int n, int* queue, cudaStream_t stream, int sms) {
+// One launch over n systems of one kind.  behind: the launch follows one that it does not depend on
+// and starts as that one's CTAs leave.
+int launch_kind(const FusedFrame* f, const int* order, int n, int* queue, cudaStream_t stream, int sms, bool behind) {
     thread_local FusedBatch B;   // host staging of the kernel parameters
-    const FusedLaunch L = fused_launch(f, n, sms);
+    const FusedLaunch L = fused_launch(f, order, n, sms);
     int items = 0;
     for (int k = 0; k < n; ++k) {
         SysDesc& S = B.sys[k];
-        const int rc = make_desc(f[order[k]], stream, L.two, &S);
-        if (rc) return rc;
+        const FusedFrame& fr = f[order[k]];
+        fill_desc(fr, static_cast<const float*>(fr.c->Vbuf[fr.c->frame & 1]), L.two, &S);
         S.item0 = items;
         items += S.n_dom;
     }
     B.n_sys = n;
     B.n_items = items;
     B.queue = queue;
-    if (L.two)
-        fused_kernel<true><<<L.grid, FT, L.smem, stream>>>(B);
-    else
-        fused_kernel<false><<<L.grid, FT, L.smem, stream>>>(B);
-    if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
+    void* args[1] = {&B};
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(L.grid);
+    cfg.blockDim = dim3(L.threads);
+    cfg.dynamicSmemBytes = L.smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = behind ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, L.fn, args) == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
+}
+
+// Systems in `order`: those of the observation-space form in one launch, the others in a second behind it.
+int launch_batch(const FusedFrame* f, const int* order, int n, int* queue, cudaStream_t stream, int sms) {
+    int kind[2][FUSED_MAX_BATCH], nk[2] = {0, 0};
+    for (int k = 0; k < n; ++k) {
+        const int j = f[order[k]].c->dual ? 0 : 1;
+        kind[j][nk[j]++] = order[k];
+    }
+    // `stream` waits for every system's noise block before the first launch (an event wait between the
+    // two would keep the second from starting early)
+    for (int k = 0; k < n; ++k) {
+        const FusedFrame& fr = f[order[k]];
+        const float* V = nullptr;
+        if (fr.with_forecast && (fr.c->Lq || fr.c->Lt)) {
+            const int rc = noise_ready(fr.c, fr.c->frame, stream, &V);
+            if (rc) return rc;
+        }
+    }
+    for (int j = 0; j < 2; ++j)
+        if (nk[j]) {
+            const int rc = launch_kind(f, kind[j], nk[j], queue + 4 * j, stream, sms, j == 1 && nk[0] > 0);
+            if (rc) return rc;
+        }
     for (int k = 0; k < n; ++k) {
         letkf_ctx* c = f[order[k]].c;
         if (f[order[k]].with_forecast && (c->Lq || c->Lt)) {
@@ -3087,7 +3170,8 @@ int graph_capture(letkf_ctx* c, int p) {
     const bool dense = c->Lq != nullptr || c->Lt != nullptr;
     thread_local FusedBatch B;
     FusedFrame f{c, nullptr, 0.0, nullptr, 1};
-    const FusedLaunch L = fused_launch(&f, 1, c->sms);
+    const int first = 0;
+    const FusedLaunch L = fused_launch(&f, &first, 1, c->sms);
     fill_desc(f, dense ? static_cast<const float*>(c->Vbuf[p]) : nullptr, L.two, &B.sys[0]);
     B.sys[0].item0 = 0;
     B.n_sys = 1;
@@ -3101,7 +3185,7 @@ int graph_capture(letkf_ctx* c, int p) {
     cudaStream_t cs = c->cap_stream;
     if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LETKF_ECUDA;
     void* fargs[1] = {&B};
-    cudaLaunchKernel(L.fn, dim3(L.grid), dim3(FT), fargs, L.smem, cs);
+    cudaLaunchKernel(L.fn, dim3(L.grid), dim3(L.threads), fargs, L.smem, cs);
     bool ok = cudaGetLastError() == cudaSuccess;
     if (ok && dense) {
         NormalsNode nn;
@@ -3175,7 +3259,8 @@ int graph_step(letkf_ctx* c, const void* y, double sigma, void* xpred) {
     }
     thread_local FusedBatch B;
     FusedFrame f{c, y, sigma, xpred, 1};
-    const FusedLaunch L = fused_launch(&f, 1, c->sms);
+    const int first = 0;
+    const FusedLaunch L = fused_launch(&f, &first, 1, c->sms);
     fill_desc(f, V, L.two, &B.sys[0]);
     B.sys[0].item0 = 0;
     B.n_sys = 1;
@@ -3185,7 +3270,7 @@ int graph_step(letkf_ctx* c, const void* y, double sigma, void* xpred) {
     cudaKernelNodeParams kp;
     kp.func = const_cast<void*>(L.fn);
     kp.gridDim = dim3(L.grid);
-    kp.blockDim = dim3(FT);
+    kp.blockDim = dim3(L.threads);
     kp.sharedMemBytes = L.smem;
     kp.kernelParams = args;
     kp.extra = nullptr;

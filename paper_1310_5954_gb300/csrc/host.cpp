@@ -294,7 +294,7 @@ size_t footprint_bytes(const letkf_params* p, const HostModel& h) {
     const size_t row = m_pad * eb;
     size_t b = 4 * (h.own_off.size() + h.own.size() + h.obs_off.size() + h.obs_sub.size() +
                     h.obs_corner.size() + h.halo_off.size() + h.halo.size() + h.order.size());
-    b += 2 * n * row + na * row + 4 + 4 + 16;
+    b += 2 * n * row + na * row + 4 + 4 + 32;
     if (p->path == LETKF_PATH_GLOBAL) {
         // the common part and the noise buffers only; the path's own buffers are added below
     } else if (p->path == LETKF_PATH_PLAIN) {
@@ -365,7 +365,7 @@ int create_impl(const letkf_params* p, letkf_ctx* c) {
     if ((rc = alloc(c, &c->V, (size_t)c->n_act * row))) return rc;
     if ((rc = alloc(c, (void**)&c->d_status, sizeof(int)))) return rc;
     if ((rc = alloc(c, (void**)&c->d_frame_bad, sizeof(int)))) return rc;
-    if ((rc = alloc(c, (void**)&c->d_queue, 4 * sizeof(int)))) return rc;
+    if ((rc = alloc(c, (void**)&c->d_queue, 8 * sizeof(int)))) return rc;
     if (c->path == LETKF_PATH_GLOBAL) {
         // buffers after the initial ensemble (they need the device noise factor)
     } else if (c->path == LETKF_PATH_PLAIN) {

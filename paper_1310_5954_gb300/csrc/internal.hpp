@@ -91,7 +91,8 @@ struct letkf_ctx {
     // device flags
     int* d_status = nullptr;        // latched status bits
     int* d_frame_bad = nullptr;     // current frame rejected
-    int* d_queue = nullptr;         // fused kernel: [0] work queue, [1] CTAs done, [2] non-finite slope seen
+    int* d_queue = nullptr;         // fused kernel: [0] work queue, [1] CTAs done, [2] non-finite slope seen;
+                                    // [4], [5]: queue and count of a batch's second launch
     size_t device_bytes = 0;
     int fused_smem = 0;             // dynamic shared memory of the fused kernel
     int fused_smem2 = 0;            // the same with two CTAs per SM (0: does not fit)
@@ -274,8 +275,8 @@ int launch_copy_rows(letkf_ctx* c, const void* src, void* dst);
 int fused_plan(letkf_ctx* c);
 int fused_prepare(letkf_ctx* c);
 int fused_step(letkf_ctx* c, const void* y, double sigma, void* xpred, int with_forecast);
-// One launch of the fused kernel over the next frame of n systems (fused path, same device):
-// their domains form one work queue (`queue`: 4 zeroed ints on the device, reset by the kernel).
+// The next frame of n systems (fused path, same device) in one launch per form of the analysis, each
+// with its systems' domains as one work queue (`queue`: 8 zeroed ints on the device, reset by the kernels).
 constexpr int FUSED_MAX_BATCH = 32;
 struct FusedFrame {
     letkf_ctx* c;

@@ -45,7 +45,7 @@ struct Slot {
     cudaStream_t stream = nullptr;
     cudaEvent_t start = nullptr;      // the batch's first operation on the stream (device clock)
     cudaEvent_t done = nullptr;       // its last
-    int* queue = nullptr;             // 4 ints: the fused kernel's work-queue counters
+    int* queue = nullptr;             // 8 ints: the fused kernels' work-queue counters
     bool busy = false;
     long long t_launch = 0;
     std::vector<int> systems;
@@ -232,7 +232,7 @@ int letkf_server_create(const letkf_server_params* p, letkf_server** out) {
             rc = LETKF_ECUDA;
             break;
         }
-        if (cudaMalloc(&sl.queue, 4 * sizeof(int)) != cudaSuccess || cudaMemset(sl.queue, 0, 4 * sizeof(int)) != cudaSuccess) {
+        if (cudaMalloc(&sl.queue, 8 * sizeof(int)) != cudaSuccess || cudaMemset(sl.queue, 0, 8 * sizeof(int)) != cudaSuccess) {
             rc = LETKF_ENOMEM;
             break;
         }
