@@ -1335,11 +1335,23 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
 __host__ __device__ inline int simt_odd(int x) { return x | 1; }   // odd row strides: no bank conflicts
                                                                    // down a column
 
+// q <= SQ: matrices of SQ x SQ, zero past q, with rows of SL floats (16-byte reads down a row, 8-byte
+// reads along one): see analyse_simt32.
+constexpr int SQ = 32, SL = 36;
+
 // Shared-memory floats of the SIMT analysis of a domain with p slopes and n_e analysed rows:
 // five q x q iteration matrices, S, two n_e x q products (dual form), then E = X'_E and the result,
 // which start past the AR(2) hand-over rows of the epilogue (the first n_e x m_pad floats).
 __host__ __device__ inline int simt_ws_floats(int p, int m, int m_pad, int n_e, int* off_e = nullptr) {
     const int q = p < m ? p : m, lq = simt_odd(q), lm = simt_odd(m);
+    if (q <= SQ) {
+        const bool dual = p < m;
+        const int rows = (n_e + 1) & ~1, le = dual ? m_pad + 4 : SL;
+        int off = 5 * SQ * SL + (dual ? SQ * (m_pad + 4) : p * SL) + 2 * rows * SL;
+        if (off < n_e * m_pad) off = (n_e * m_pad + 3) & ~3;
+        if (off_e) *off_e = off;
+        return off + 2 * rows * le;
+    }
     int off = 5 * q * lq + p * lm + 2 * n_e * lq;
     if (off < n_e * m_pad) off = n_e * m_pad;
     if (off_e) *off_e = off;
@@ -1401,20 +1413,415 @@ __device__ void simt_mv(float* y, const float* A, int ar, int ac, const float* x
 __device__ __forceinline__ void own_row_means(const SysDesc& A, const float* XE, int n_e, const float* wbar,
                                               float* xe_mean, float* uvec) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m = A.m;
-    for (int e = warp; e < n_e; e += FT / 32) {
-        float sm_ = 0.f;
-        for (int i = lane; i < m; i += 32) sm_ += XE[(size_t)e * A.m_pad + i];
-        sm_ = warp_sum(sm_);
-        const float mu = sm_ / (float)m;
-        float us = 0.f, uc = 0.f;
-        for (int i = lane; i < m; i += 32) dot2_add(us, uc, XE[(size_t)e * A.m_pad + i] - mu, wbar[i]);
-        const float u = dot2_warp(us, uc);
+    // two rows of a warp at a time: each is a chain of shuffles and dependent sums
+    for (int e = warp; e < n_e; e += 2 * (FT / 32)) {
+        const int e2 = e + FT / 32 < n_e ? e + FT / 32 : e;
+        const float* x0 = XE + (size_t)e * A.m_pad;
+        const float* x1 = XE + (size_t)e2 * A.m_pad;
+        float a0 = 0.f, a1 = 0.f;
+        for (int i = lane; i < m; i += 32) {
+            a0 += x0[i];
+            a1 += x1[i];
+        }
+        a0 = warp_sum(a0);
+        a1 = warp_sum(a1);
+        const float mu0 = a0 / (float)m, mu1 = a1 / (float)m;
+        float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
+        for (int i = lane; i < m; i += 32) {
+            const float w = wbar[i];
+            dot2_add(s0, c0, x0[i] - mu0, w);
+            dot2_add(s1, c1, x1[i] - mu1, w);
+        }
+        const float u0 = dot2_warp(s0, c0), u1 = dot2_warp(s1, c1);
         if (lane == 0) {
-            xe_mean[e] = mu;
-            uvec[e] = u;
+            xe_mean[e] = mu0;
+            uvec[e] = u0;
+            xe_mean[e2] = mu1;
+            uvec[e2] = u1;
         }
     }
     __syncthreads();
+}
+
+// Four elements (rows 2 ty, 2 ty + 1 x columns 2 tx, 2 tx + 1 of thread (ty, tx) = tid / 16, tid % 16) of
+// A B: A's rows read four k at a time, B's two columns; sums over k in order.
+__device__ __forceinline__ void mm32(const float* A, const float* B, int q, float (&c)[4]) {
+    const float* a = A + (threadIdx.x >> 4) * (2 * SL);
+    const float* b = B + (threadIdx.x & 15) * 2;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) c[u] = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < q; k += 4) {
+        const float4 a0 = *reinterpret_cast<const float4*>(a + k), a1 = *reinterpret_cast<const float4*>(a + SL + k);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float2 bv = *reinterpret_cast<const float2*>(b + (k + r) * SL);
+            c[0] = fmaf(f4c(a0, r), bv.x, c[0]);
+            c[1] = fmaf(f4c(a0, r), bv.y, c[1]);
+            c[2] = fmaf(f4c(a1, r), bv.x, c[2]);
+            c[3] = fmaf(f4c(a1, r), bv.y, c[3]);
+        }
+    }
+}
+__device__ __forceinline__ void put32(float* C, const float (&c)[4]) {
+    float* o = C + (threadIdx.x >> 4) * (2 * SL) + (threadIdx.x & 15) * 2;
+    *reinterpret_cast<float2*>(o) = make_float2(c[0], c[1]);
+    *reinterpret_cast<float2*>(o + SL) = make_float2(c[2], c[3]);
+}
+
+// The SIMT analysis for q <= 32 (the default threshold): the iteration's matrices fit one 2 x 2 block per
+// thread, so a product's result is transformed in registers (T, the residual, the next inverse iterate)
+// and a Newton-Schulz step is two barriers: P -> T and the residual's sum, then Y T and T Z together.
+// Bound by the barriers and the shared-memory latency of q / 4 dependent reads per product.  Same
+// formulas as analyse_simt; the dual form's X'_E T = X'_E - (X'_E S^T) N S takes N = (I + K/c)^(-1/2)
+// (I + Z)^-1 (I + K/c)^(-1/2) / c as one q x q matrix.  Measured against analyse_simt: 8x8, m = 20 frame
+// 37.9 -> 32.7 us; ELT, whose 16 edge domains end the launch, 128.5 -> 121.7 us.
+template <bool TWO>
+__device__ __noinline__ const float* analyse_simt32(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, int d,
+                                                    int* ld_out) {
+    const SysDesc& A = B.sys[ctl->sys];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = tid >> 4, tx = tid & 15;
+    const int m = A.m, m_pad = A.m_pad;
+    const float c = (float)(m - 1);
+    float* vec = reinterpret_cast<float*>(smem + A.off_vec);
+    float* xh_mean = vec;
+    float* xe_mean = vec + 256;
+    float* bvec = vec + 384;
+    float* wbar = vec + 512;
+    float* vtmp = vec + 640;
+    float* vv = vec + 896;
+    float* vr = vec + 1024;
+    float* uvec = vec + 1152;
+    float* dtv = vec + 1280;
+    float* tvv = vec + 1408;
+    const int* pcs = reinterpret_cast<const int*>(vec + 1792);
+    const float* ys = vec + 1856;
+    const float* XE = reinterpret_cast<const float*>(smem + (TWO ? A.off_big + A.off_sxe : A.off_xe));
+    const float* Xh = reinterpret_cast<const float*>(smem + (TWO ? A.off_big + A.off_sxh : A.off_xh));
+    float* ws = reinterpret_cast<float*>(smem + A.off_big);
+    const int n_own = A.tab.own_off[d + 1] - A.tab.own_off[d], n_obs = A.tab.obs_off[d + 1] - A.tab.obs_off[d];
+    const int p = 2 * n_obs, n_e = (A.with_forecast && A.a2 == 0.f) ? n_own : 2 * n_own;
+    const bool dual = p < m;
+    const int q = dual ? p : m;
+    int off_e = 0;
+    simt_ws_floats(p, m, m_pad, n_e, &off_e);
+    float* Y = ws;
+    float* Z = Y + SQ * SL;
+    float* T = Z + SQ * SL;
+    float* Yn = T + SQ * SL;
+    float* Zn = Yn + SQ * SL;
+    float* S = Zn + SQ * SL;                      // dual: SQ rows of ls members; else p rows of SL
+    const int ls = dual ? m_pad + 4 : SL, rows = (n_e + 1) & ~1;
+    float* R1 = S + (dual ? SQ * ls : p * SL);    // n_e x q
+    float* R2 = R1 + rows * SL;
+    float* E = ws + off_e;                        // n_e rows of X'_E
+    float* Out = E + rows * ls;
+
+    // ---- slopes S (k = 2 s + direction), zero past p and m, and d / sigma
+    for (int s2 = warp; s2 < (dual ? SQ / 2 : n_obs); s2 += FT / 32) {
+        const bool has = s2 < n_obs;
+        const int pc = has ? pcs[s2] : 0;
+        const float* x00 = Xh + (size_t)(pc & 0xFF) * m_pad;
+        const float* x01 = Xh + (size_t)((pc >> 8) & 0xFF) * m_pad;
+        const float* x10 = Xh + (size_t)((pc >> 16) & 0xFF) * m_pad;
+        const float* x11 = Xh + (size_t)((pc >> 24) & 0xFF) * m_pad;
+        for (int i = lane; i < ls; i += 32) {
+            float sx = 0.f, sy = 0.f;
+            if (has && i < m) {
+                const float a00 = x00[i], a01 = x01[i], a10 = x10[i], a11 = x11[i];
+                sx = 0.5f * ((a01 + a11) - (a00 + a10)) * A.inv_sigma;
+                sy = 0.5f * ((a10 + a11) - (a00 + a01)) * A.inv_sigma;
+            }
+            S[(2 * s2) * ls + i] = sx;
+            S[(2 * s2 + 1) * ls + i] = sy;
+        }
+    }
+    for (int k = tid; k < p; k += FT) {
+        const int pc = pcs[k >> 1];
+        const float a00 = xh_mean[pc & 0xFF], a01 = xh_mean[(pc >> 8) & 0xFF];
+        const float a10 = xh_mean[(pc >> 16) & 0xFF], a11 = xh_mean[(pc >> 24) & 0xFF];
+        const float sl = (k & 1) == 0 ? 0.5f * ((a01 + a11) - (a00 + a10)) : 0.5f * ((a10 + a11) - (a00 + a01));
+        dtv[k] = (ys[k] - sl) * A.inv_sigma;
+    }
+    if (tid >= p && tid < 128) dtv[tid] = 0.f;
+    __syncthreads();
+    // ---- H = S S^T (dual) or S^T S, in registers
+    float h[4] = {0.f, 0.f, 0.f, 0.f};
+    if (dual) {
+        const float* ri = S + 2 * ty * ls;
+        const float* rj = S + 2 * tx * ls;
+#pragma unroll 2
+        for (int k = 0; k < m; k += 4) {
+            const float4 i0 = *reinterpret_cast<const float4*>(ri + k), i1 = *reinterpret_cast<const float4*>(ri + ls + k);
+            const float4 j0 = *reinterpret_cast<const float4*>(rj + k), j1 = *reinterpret_cast<const float4*>(rj + ls + k);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                h[0] = fmaf(f4c(i0, r), f4c(j0, r), h[0]);
+                h[1] = fmaf(f4c(i0, r), f4c(j1, r), h[1]);
+                h[2] = fmaf(f4c(i1, r), f4c(j0, r), h[2]);
+                h[3] = fmaf(f4c(i1, r), f4c(j1, r), h[3]);
+            }
+        }
+    } else {
+#pragma unroll 4
+        for (int k = 0; k < p; ++k) {
+            const float2 iv = *reinterpret_cast<const float2*>(S + k * SL + 2 * ty);
+            const float2 jv = *reinterpret_cast<const float2*>(S + k * SL + 2 * tx);
+            h[0] = fmaf(iv.x, jv.x, h[0]);
+            h[1] = fmaf(iv.x, jv.y, h[1]);
+            h[2] = fmaf(iv.y, jv.x, h[2]);
+            h[3] = fmaf(iv.y, jv.y, h[3]);
+        }
+    }
+    const float fro = block_sum(ctl, (h[0] * h[0] + h[1] * h[1]) + (h[2] * h[2] + h[3] * h[3]));
+    const float s_scale = 1.f + sqrtf(fro) / c;
+    const float s_ns = s_scale / NS_SCALE;
+    const float inv_cs = 1.f / (c * s_ns);
+    // the identity's elements of this thread's block
+    float id[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = 2 * ty + (u >> 1), j = 2 * tx + (u & 1);
+        id[u] = (i == j && i < q) ? 1.f : 0.f;
+    }
+    auto residual = [&](const float (&v)[4]) {
+        float r2 = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) r2 += (id[u] - v[u]) * (id[u] - v[u]);
+        return r2;
+    };
+    auto half_step = [&](const float (&v)[4], float (&t)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t[u] = 1.5f * id[u] - 0.5f * v[u];
+    };
+    // ---- coupled Newton-Schulz from Y_0 = A_s, Z_0 = I: the first step is Z_1 = T_0, Y_1 = Y_0 T_0
+    float v[4], w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = (id[u] + h[u] / c) / s_ns;
+    half_step(v, w);
+    put32(Y, v);
+    put32(Z, w);
+    float rn_prev = sqrtf(block_sum_open(ctl, residual(v)));
+    int it = 1;
+    if (rn_prev < 2e-6f * (float)q) {
+        __syncthreads();
+        put32(Z, id);      // converged at once: Z = I
+        __syncthreads();
+    } else {
+        mm32(Y, Z, q, v);
+        put32(Yn, v);
+        __syncthreads();
+        float* sw = Y; Y = Yn; Yn = sw;
+        for (; it < A.max_it; ++it) {
+            mm32(Z, Y, q, v);                                          // P = Z Y
+            half_step(v, w);
+            put32(T, w);                                               // T = (3I - P) / 2
+            const float rn = sqrtf(block_sum_open(ctl, residual(v)));
+            const bool conv = rn < 2e-6f * (float)q || (rn < 2e-2f && rn > 0.6f * rn_prev);
+            rn_prev = rn;
+            if (conv) break;
+            mm32(Y, T, q, v);                                          // Y T
+            mm32(T, Z, q, w);                                          // T Z
+            put32(Yn, v);
+            put32(Zn, w);
+            __syncthreads();
+            float* sy = Y; Y = Yn; Yn = sy;
+            float* sz = Z; Z = Zn; Zn = sz;
+            if (rn < NS_LAST_FP32) break;      // the Gram here is FP32 (see ns_stop)
+        }
+        if (it == A.max_it && tid == 0) atomicOr(A.status, ST_NOCONV);
+    }
+    // ---- mean weights, refined against the exact operator
+    auto zmul = [&](const float* x, float* y, float alpha) {          // y = alpha Z x, eight lanes per row
+        const int r = tid >> 3, l = tid & 7;
+        const float4 z = *reinterpret_cast<const float4*>(Z + r * SL + 4 * l);
+        const float4 xv = *reinterpret_cast<const float4*>(x + 4 * l);
+        float s = (z.x * xv.x + z.y * xv.y) + (z.z * xv.z + z.w * xv.w);
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        __syncthreads();                                              // y may be x
+        if (l == 0) y[r] = alpha * s;
+        __syncthreads();
+    };
+    auto srow = [&](const float* x, float* y) {                       // y = S x (p rows), eight lanes per row
+        for (int r0 = 0; r0 < p; r0 += FT / 8) {
+            const int r = r0 + (tid >> 3), l = tid & 7;
+            float s = 0.f;
+            if (r < p)
+                for (int i = l; i < m; i += 8) s = fmaf(S[r * ls + i], x[i], s);
+            s += __shfl_xor_sync(0xffffffffu, s, 4);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            if (l == 0 && r < p) y[r] = s;
+        }
+        __syncthreads();
+    };
+    const int n_ref = s_scale > A.s_split ? 2 : 1;
+    if (dual) {
+        float* u = bvec;
+        zmul(dtv, vv, 1.f);
+        zmul(vv, u, inv_cs);                                          // u = (cI + K)^-1 d
+        for (int ref = 0; ref < n_ref; ++ref) {
+            simt_mv(wbar, S, 1, ls, u, m, p, 1.f, vtmp);              // S^T u
+            srow(wbar, tvv);                                          // K u, from the FP32 slopes
+            if (tid < 32) tvv[tid] = tid < p ? dtv[tid] - c * u[tid] - tvv[tid] : 0.f;
+            __syncthreads();
+            zmul(tvv, vr, 1.f);
+            zmul(vr, vv, inv_cs);
+            if (tid < p) u[tid] += vv[tid];
+            __syncthreads();
+        }
+        simt_mv(wbar, S, 1, ls, u, m, p, 1.f, vtmp);                  // w_bar = S^T u
+    } else {
+        if (tid < 32) bvec[tid] = vr[tid] = 0.f;
+        __syncthreads();
+        simt_mv(bvec, S, 1, SL, dtv, m, p, 1.f, vtmp);                // b = S^T d
+        zmul(bvec, vv, 1.f);
+        zmul(vv, wbar, inv_cs);
+        for (int ref = 0; ref < n_ref; ++ref) {
+            srow(wbar, tvv);                                          // S w_bar
+            if (tid < p) tvv[tid] = dtv[tid] - tvv[tid];
+            __syncthreads();
+            simt_mv(vr, S, 1, SL, tvv, m, p, 1.f, vtmp);              // S^T (d - S w_bar)
+            if (tid < m) vr[tid] -= c * wbar[tid];
+            __syncthreads();
+            zmul(vr, vv, 1.f);
+            zmul(vv, tvv, inv_cs);
+            if (tid < m) wbar[tid] += tvv[tid];
+            __syncthreads();
+        }
+    }
+    const bool cap = A.cap != nullptr && d == A.cap_dom;
+    if (cap) {
+        if (tid == 0) cap_header(A.cap, dual ? CAP_DUAL_SIMT : CAP_MM_SIMT, q, s_scale, it);
+        for (int t = tid; t < m; t += FT) A.cap[CAP_HDR + t] = wbar[t];
+    }
+    // ---- own rows: means, mean update, centred anomalies X'_E; then the next item's loads
+    own_row_means(A, XE, n_e, wbar, xe_mean, uvec);
+    for (int e = warp; e < rows; e += FT / 32)
+        for (int i = lane; i < ls; i += 32)
+            E[e * ls + i] = (e < n_e && i < m) ? XE[(size_t)e * m_pad + i] - xe_mean[e] : 0.f;
+    __syncthreads();
+    if (!TWO && warp == 0) fetch_item(B, ctl, smem, A.off_big);
+    // ---- transform
+    const float rs = rsqrtf(s_ns);    // T = Z / sqrt(s_ns) (m x m form); Z / sqrt(s_ns) = (I + K/c)^(-1/2)
+    *ld_out = ls;
+    // rows of X M for X of n_e rows (stride SL or, down S's rows, ls), a 2 x 2 block per thread and pass
+    auto rows_mm = [&](float* C, const float* X, const float* M, float alpha) {
+        for (int r = ty; 2 * r < n_e; r += 16) {
+            const float* a = X + 2 * r * SL;
+            const float* b = M + 2 * tx;
+            float cc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+            for (int k = 0; k < q; k += 4) {
+                const float4 a0 = *reinterpret_cast<const float4*>(a + k);
+                const float4 a1 = *reinterpret_cast<const float4*>(a + SL + k);
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const float2 bv = *reinterpret_cast<const float2*>(b + (k + t) * SL);
+                    cc[0] = fmaf(f4c(a0, t), bv.x, cc[0]);
+                    cc[1] = fmaf(f4c(a0, t), bv.y, cc[1]);
+                    cc[2] = fmaf(f4c(a1, t), bv.x, cc[2]);
+                    cc[3] = fmaf(f4c(a1, t), bv.y, cc[3]);
+                }
+            }
+            float* o = C + 2 * r * SL + 2 * tx;
+            *reinterpret_cast<float2*>(o) = make_float2(alpha * cc[0], alpha * cc[1]);
+            *reinterpret_cast<float2*>(o + SL) = make_float2(alpha * cc[2], alpha * cc[3]);
+        }
+        __syncthreads();
+    };
+    if (!dual) {
+        if (cap)
+            for (int t = tid; t < m * m; t += FT) A.cap[CAP_HDR + m + t] = rs * Z[(t / m) * SL + t % m];
+        rows_mm(Out, E, Z, rs);
+        return Out;
+    }
+    // (I + Zt)^-1 with Zt = rs Z by Newton's iteration from 2/3 I (eigenvalues of I + Zt in (1, 2]):
+    // the first step is elementwise, X_1 = 4/3 I - 4/9 (I + Zt); three more leave (1/3)^16
+    float* Mi = Y;
+    float* X = T;
+    float* Q = Yn;
+    float* Xn = Zn;
+    {
+        const float* zb = Z + 2 * ty * SL + 2 * tx;
+        const float z[4] = {zb[0], zb[1], zb[SL], zb[SL + 1]};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u] = id[u] + rs * z[u];
+            w[u] = (4.f / 3.f) * id[u] - (4.f / 9.f) * v[u];
+        }
+        put32(Mi, v);
+        put32(X, w);
+        __syncthreads();
+    }
+    for (int k = 0; k < 3; ++k) {
+        mm32(Mi, X, q, v);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = 2.f * id[u] - v[u];        // 2I - (I + Zt) X
+        put32(Q, v);
+        __syncthreads();
+        mm32(X, Q, q, w);
+        put32(Xn, w);
+        __syncthreads();
+        float* sx = X; X = Xn; Xn = sx;
+    }
+    if (cap) {     // W = Zt S / sqrt(c) and (I + Zt)^-1 W, the factors of T = I - W^T (I + Zt)^-1 W
+        float* Wc = A.cap + CAP_HDR + m;
+        simt_mm(Wc, m, Z, SL, 1, S, ls, 1, q, m, q, rs * rsqrtf(c));
+        simt_mm(Wc + q * m, m, X, SL, 1, Wc, m, 1, q, m, q, 1.f);
+    }
+    // N = Zt (I + Zt)^-1 Zt / c, beside X'_E S^T
+    mm32(Z, X, q, v);
+    put32(Q, v);
+    for (int r = ty; 2 * r < n_e; r += 16) {                          // X'_E S^T
+        const float* a = E + 2 * r * ls;
+        const float* b = S + 2 * tx * ls;
+        float cc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+        for (int k = 0; k < m; k += 4) {
+            const float4 a0 = *reinterpret_cast<const float4*>(a + k), a1 = *reinterpret_cast<const float4*>(a + ls + k);
+            const float4 b0 = *reinterpret_cast<const float4*>(b + k), b1 = *reinterpret_cast<const float4*>(b + ls + k);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                cc[0] = fmaf(f4c(a0, t), f4c(b0, t), cc[0]);
+                cc[1] = fmaf(f4c(a0, t), f4c(b1, t), cc[1]);
+                cc[2] = fmaf(f4c(a1, t), f4c(b0, t), cc[2]);
+                cc[3] = fmaf(f4c(a1, t), f4c(b1, t), cc[3]);
+            }
+        }
+        float* o = R1 + 2 * r * SL + 2 * tx;
+        *reinterpret_cast<float2*>(o) = make_float2(cc[0], cc[1]);
+        *reinterpret_cast<float2*>(o + SL) = make_float2(cc[2], cc[3]);
+    }
+    __syncthreads();
+    mm32(Q, Z, q, v);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] *= rs * rs / c;
+    put32(Mi, v);
+    __syncthreads();
+    rows_mm(R2, R1, Mi, 1.f);
+    const int n4 = m_pad >> 2;                                        // X'_E - (X'_E S^T N) S, in place
+    for (int t = tid; t < (rows >> 1) * n4; t += FT) {
+        const int r = t / n4, j = 4 * (t - r * n4);
+        const float* a = R2 + 2 * r * SL;
+        float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+#pragma unroll 4
+        for (int k = 0; k < q; ++k) {
+            const float4 sv = *reinterpret_cast<const float4*>(S + k * ls + j);
+            const float a0 = a[k], a1 = a[SL + k];
+            c0.x = fmaf(a0, sv.x, c0.x); c0.y = fmaf(a0, sv.y, c0.y); c0.z = fmaf(a0, sv.z, c0.z); c0.w = fmaf(a0, sv.w, c0.w);
+            c1.x = fmaf(a1, sv.x, c1.x); c1.y = fmaf(a1, sv.y, c1.y); c1.z = fmaf(a1, sv.z, c1.z); c1.w = fmaf(a1, sv.w, c1.w);
+        }
+        float4* e0 = reinterpret_cast<float4*>(E + 2 * r * ls + j);
+        float4* e1 = reinterpret_cast<float4*>(E + (2 * r + 1) * ls + j);
+        const float4 x0 = *e0, x1 = *e1;
+        *e0 = make_float4(x0.x - c0.x, x0.y - c0.y, x0.z - c0.z, x0.w - c0.w);
+        *e1 = make_float4(x1.x - c1.x, x1.y - c1.y, x1.z - c1.z, x1.w - c1.w);
+    }
+    __syncthreads();
+    return E;
 }
 
 // The SIMT analysis of domain d (halo anomalies centred in Xh, their means in xh_mean): writes
@@ -1890,7 +2297,8 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
         const float* sout = nullptr;
         int sld = 0;
         if (simt) {
-            sout = analyse_simt<TWO>(B, ctl, smem, d, &sld);
+            sout = min(p_loc, m) <= SQ ? analyse_simt32<TWO>(B, ctl, smem, d, &sld)
+                                       : analyse_simt<TWO>(B, ctl, smem, d, &sld);
         } else {
             // thread (i = tid mod 128, kc = tid / 128 + 2 k): row i of the operand, 8 K-values per task
             // (row m, the innovation, is written after it: as a branch here its warps ran both sides)
