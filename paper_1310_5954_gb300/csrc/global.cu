@@ -43,10 +43,10 @@ enum { CTL_RUN = 0, CTL_STEPS = NS_MAX + 1, CTL_ZFINAL = NS_MAX + 2, CTL_N = NS_
 struct GlobalState {
     int mr = 0, pk = 0, mp = 0, nr = 0, ka = 0;   // padded sizes: S' rows, slopes, m, state rows, actuators
     uint8_t *st_hi = nullptr, *st_lo = nullptr;   // [S d]^T tiles (mr x pk)
-    float* G = nullptr;                            // (m+1) x (m+1) Gram, row-major
-    float* Gpart = nullptr;                        // gram_split partial Grams of the upper tiles
-    int2* gram_tiles = nullptr;                    // the upper 128 x 128 tiles of the Gram
-    int gram_ntiles = 0, gram_split = 1;
+    float* G = nullptr;                            // m x (m+1) Gram, row-major
+    float* Gpart = nullptr;                        // partial Grams of the upper tiles, one per share
+    int ldg = 0, gram_split = 1;                   // leading dimension of the Gram, shares of its K steps
+    GemmPlan pl_gram, pl_one, pl_two, pl_tr, pl_noise;   // one / two m x m products, transform, noise draw
     uint8_t *as_hi = nullptr, *as_lo = nullptr, *t_hi = nullptr, *t_lo = nullptr;
     uint8_t *y_hi[2] = {}, *y_lo[2] = {}, *z_hi[2] = {}, *z_lo[2] = {};
     uint8_t *xp_hi = nullptr, *xp_lo = nullptr;    // X' tiles (nr x mp)
@@ -69,17 +69,57 @@ constexpr int TILE_B = 128 * 64 * 2;
 
 int rup(int v, int a) { return (v + a - 1) / a * a; }
 
-// Split of the Gram's K steps: enough shares that the upper tiles fill about one wave of SMs,
-// each share at least two steps and none empty.
-int gram_split_for(int m, int p, int sms) {
-    const int rt = rup(m + 1, 128) / 128, ct = (m + 1 + 127) / 128;
-    int tiles = 0;
-    for (int r = 0; r < rt; ++r)
-        for (int c = r; c < ct; ++c) ++tiles;
-    const int nkb = rup(p, 64) / 64;
-    int ks = std::max(1, std::min(nkb / 2, sms / std::max(tiles, 1)));
-    while (ks > 1 && ((nkb + ks - 1) / ks) * (ks - 1) >= nkb) --ks;
-    return ks;
+// Row tiles per cluster of a wide product: they share the 256 columns of B.
+int cluster_rows(int row_tiles) { return row_tiles >= 2 ? 2 : 1; }
+
+// The plans of the analysis's products, and the Gram's shares: as many as make its pieces fill the SMs,
+// against the partial Grams that every share writes and the reduction reads (at 2 KB per cycle).
+struct Plans {
+    GemmPlan gram, one, two, tr, noise;
+    int split = 1;
+};
+Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
+    Plans P;
+    const int mt = rup(m, 128) / 128, rows = rup(2 * n_act, 128) / 128, acts = rup(n_act, 128) / 128;
+    GemmShape g;
+    g.m_tiles = mt;             // row m of the Gram is its column m
+    g.N = m + 1;
+    g.nkb = rup(2 * n_subv, 64) / 64;
+    g.bn = 256;
+    g.cm = cluster_rows(mt);
+    g.upper = 1;
+    long long best = -1;
+    for (g.ksplit = 1; g.ksplit <= std::max(1, std::min(g.nkb / 2, 16)); ++g.ksplit) {
+        GemmPlan p = gemm_plan(g, sms);
+        const long long t = p.cycles + (long long)g.ksplit * m * m * 4 / 2048;
+        if (best >= 0 && t >= best) continue;
+        best = t;
+        P.gram = p;
+        P.split = g.ksplit;
+    }
+    GemmShape q;
+    q.m_tiles = mt;
+    q.N = m;
+    q.mn = 1;
+    q.nkb = rup(m, 128) / 64;
+    P.one = gemm_plan(q, sms);
+    q.batch = 2;
+    P.two = gemm_plan(q, sms);
+    GemmShape t;
+    t.m_tiles = rows;
+    t.N = m;
+    t.nkb = rup(m, 128) / 64;
+    t.bn = 256;
+    t.cm = cluster_rows(rows);
+    P.tr = gemm_plan(t, sms);
+    if (dense) {
+        t.m_tiles = acts;
+        t.nkb = rup(n_act, 64) / 64;
+        t.cm = cluster_rows(acts);
+        t.lower = lower;
+        P.noise = gemm_plan(t, sms);
+    }
+    return P;
 }
 
 __device__ __forceinline__ size_t toff(int row, int col, int nkb) {
@@ -151,7 +191,7 @@ __global__ void gl_slopes_kernel(const float* __restrict__ X, const float* __res
                 v[q] = (i < m ? s : y[col] - s) * inv_sigma;
             }
         }
-        store8(hi, lo, toff(i, c0, pk >> 6), v);
+        store8(hi, lo, umma::slice_offset(i, c0, pk >> 6), v);
     }
 }
 
@@ -287,7 +327,7 @@ __global__ void gl_wt_kernel(const uint8_t* __restrict__ z0_hi, const uint8_t* _
             const int k = k0 + q;
             v[q] = (j < m && k < m) ? wbar[k] + rs * tval(zh, zl, off + 2 * q) : 0.f;
         }
-        store8(hi, lo, off, v);
+        store8(hi, lo, umma::slice_offset(j, k0, nkb), v);
     }
 }
 
@@ -305,7 +345,7 @@ __global__ void gl_xp_kernel(const float* __restrict__ X, const float* __restric
             const int i = i0 + q;
             v[q] = (r < n && i < m) ? X[(size_t)r * m_pad + i] - mu : 0.f;
         }
-        store8(hi, lo, toff(r, i0, mp >> 6), v);
+        store8(hi, lo, umma::slice_offset(r, i0, mp >> 6), v);
     }
 }
 
@@ -330,7 +370,7 @@ __global__ void gl_normals_kernel(unsigned long long seed, uint32_t frame, int n
         __align__(8) __nv_bfloat16 h[4], l[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) split2(4 * q + r < n_act ? z[r] : 0.f, h[r], l[r]);
-        const size_t off = toff(i, 4 * q, ka >> 6);
+        const size_t off = umma::slice_offset(i, 4 * q, ka >> 6);
         *reinterpret_cast<uint2*>(hi + off) = *reinterpret_cast<const uint2*>(h);
         *reinterpret_cast<uint2*>(lo + off) = *reinterpret_cast<const uint2*>(l);
     }
@@ -338,15 +378,15 @@ __global__ void gl_normals_kernel(unsigned long long seed, uint32_t frame, int n
 
 // The Gram from its split-K partials: the upper 128 x 128 tiles were computed, the lower ones
 // are their mirror; the shares are added in order.
-__global__ void gl_gram_reduce_kernel(const float* __restrict__ part, int splits, size_t stride, int m1,
+__global__ void gl_gram_reduce_kernel(const float* __restrict__ part, int splits, size_t stride, int m, int ld,
                                       float* __restrict__ G) {
-    const size_t total = (size_t)m1 * m1;
+    const size_t total = (size_t)m * (m + 1);
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t / m1), j = (int)(t - (size_t)i * m1);
-        const size_t src = (j >> 7) >= (i >> 7) ? t : (size_t)j * m1 + i;
+        const int i = (int)(t / (m + 1)), j = (int)(t - (size_t)i * (m + 1));
+        const size_t src = (j >> 7) >= (i >> 7) ? (size_t)i * ld + j : (size_t)j * ld + i;
         float v = 0.f;
         for (int z = 0; z < splits; ++z) v += part[z * stride + src];
-        G[t] = v;
+        G[(size_t)i * ld + j] = v;
     }
 }
 
@@ -357,12 +397,13 @@ int grid_for(size_t work, int block) {
 GemmArgs gemm_args(const uint8_t* ah, const uint8_t* al, const uint8_t* bh, const uint8_t* bl, int nkb, int M,
                    int N, int* status) {
     GemmArgs g{};
-    g.a_hi = ah;
-    g.a_lo = al;
-    g.b_hi = bh;
-    g.b_lo = bl;
-    g.a_nkb = g.b_nkb = g.nkb = nkb;
+    g.a_hi[0] = ah;
+    g.a_lo[0] = al;
+    g.b_hi[0] = bh;
+    g.b_lo[0] = bl;
+    g.a_nkb = g.b_nkb = nkb;
     g.split = 1;
+    g.m_tiles = (M + 127) / 128;
     g.M = M;
     g.N = N;
     g.alpha = 1.f;
@@ -370,27 +411,32 @@ GemmArgs gemm_args(const uint8_t* ah, const uint8_t* al, const uint8_t* bh, cons
     return g;
 }
 
-// Newton-Schulz step k from buffers a to b: P = Z_a Y_a -> T (max |P - I| into dev[k]),
-// Y_b = Y_a T, Z_b = T Z_a, all gated by run[k]; the Y product sets run[k + 1].
+// Newton-Schulz step k from buffers a to b, all gated by run[k]: P = Z_a Y_a -> T (max |P - I| into
+// dev[k]), then Y_b = Y_a T and Z_b = T Z_a in one launch, which sets run[k + 1].
 int ns_step(letkf_ctx* c, GlobalState* S, int a, int k, cudaStream_t s) {
     const int m = c->m, nkb = S->mp >> 6, b = a ^ 1;
-    const int mt = S->mp / 128, nt = (m + 63) / 64;
     int rc;
     GemmArgs g = gemm_args(S->z_hi[a], S->z_lo[a], S->y_hi[a], S->y_lo[a], nkb, m, m, c->d_status);
     g.mode = GEMM_EPI_TILES;
-    g.o_hi = S->t_hi;
-    g.o_lo = S->t_lo;
+    g.o_hi[0] = S->t_hi;
+    g.o_lo[0] = S->t_lo;
     g.o_nkb = nkb;
     g.alpha = -0.5f;
     g.beta = 1.5f;
     g.dev = S->dev + k;
     g.b_mn = 1;
     g.run = S->ctl + CTL_RUN + k;
-    if ((rc = gemm_launch(g, 64, mt, nt, s))) return rc;
+    if ((rc = gemm_launch(g, S->pl_one, s))) return rc;
     g = gemm_args(S->y_hi[a], S->y_lo[a], S->t_hi, S->t_lo, nkb, m, m, c->d_status);
+    g.a_hi[1] = S->t_hi;
+    g.a_lo[1] = S->t_lo;
+    g.b_hi[1] = S->z_hi[a];
+    g.b_lo[1] = S->z_lo[a];
     g.mode = GEMM_EPI_TILES;
-    g.o_hi = S->y_hi[b];
-    g.o_lo = S->y_lo[b];
+    g.o_hi[0] = S->y_hi[b];
+    g.o_lo[0] = S->y_lo[b];
+    g.o_hi[1] = S->z_hi[b];
+    g.o_lo[1] = S->z_lo[b];
     g.o_nkb = nkb;
     g.b_mn = 1;
     g.run = S->ctl + CTL_RUN + k;
@@ -400,15 +446,7 @@ int ns_step(letkf_ctx* c, GlobalState* S, int a, int k, cudaStream_t s) {
     g.z_final = S->ctl + CTL_ZFINAL;
     g.z_index = b;
     g.steps = S->ctl + CTL_STEPS;
-    if ((rc = gemm_launch(g, 64, mt, nt, s))) return rc;
-    g = gemm_args(S->t_hi, S->t_lo, S->z_hi[a], S->z_lo[a], nkb, m, m, c->d_status);
-    g.mode = GEMM_EPI_TILES;
-    g.o_hi = S->z_hi[b];
-    g.o_lo = S->z_lo[b];
-    g.o_nkb = nkb;
-    g.b_mn = 1;
-    g.run = S->ctl + CTL_RUN + k;
-    return gemm_launch(g, 64, mt, nt, s);
+    return gemm_launch(g, S->pl_two, s);
 }
 
 // Sets the condition of the conditional node holding the later steps: whether step k runs.
@@ -431,12 +469,12 @@ int build_ns_graph(letkf_ctx* c, GlobalState* S) {
         return LETKF_ECUDA;
     GemmArgs g = gemm_args(S->as_hi, S->as_lo, S->z_hi[1], S->z_lo[1], nkb, m, m, c->d_status);
     g.mode = GEMM_EPI_TILES;
-    g.o_hi = S->y_hi[1];
-    g.o_lo = S->y_lo[1];
+    g.o_hi[0] = S->y_hi[1];
+    g.o_lo[0] = S->y_lo[1];
     g.o_nkb = nkb;
     g.b_mn = 1;
     g.run = S->ctl + CTL_RUN + 1;
-    int rc = gemm_launch(g, 64, S->mp / 128, (m + 63) / 64, S->cap);
+    int rc = gemm_launch(g, S->pl_one, S->cap);
     for (int k = 1; k < NS_FLAT && !rc; ++k) rc = ns_step(c, S, k & 1, k, S->cap);
     if (!rc) {
         gl_cond_kernel<<<1, 1, 0, S->cap>>>(S->ctl, NS_FLAT, h);
@@ -478,20 +516,16 @@ int build_ns_graph(letkf_ctx* c, GlobalState* S) {
 
 }  // namespace
 
-size_t global_bytes(int n_act, int n_subv, int m, bool dense, int sms) {
+size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
     const int mr = rup(m + 1, 128), pk = rup(2 * n_subv, 64), mp = rup(m, 128), nr = rup(2 * n_act, 128);
     const int ka = rup(n_act, 64);
-    // [S d]^T, the Gram, A_s, T, Y (2), Z (2), X', W^T (hi and lo tiles each)
-    size_t b = 2 * tiled_bytes(mr, pk) + (size_t)(m + 1) * (m + 1) * 4 + 12 * tiled_bytes(mp, mp) +
-               2 * tiled_bytes(nr, mp) + 2 * tiled_bytes(mp, mp);
+    const size_t gram = (size_t)m * rup(m + 1, 4) * 4;
+    const Plans P = plans_for(n_act, n_subv, m, dense, lower, sms);
+    // [S d]^T, the Gram and its shares, A_s, T, Y (2), Z (2), X', W^T (hi and lo tiles each)
+    size_t b = 2 * tiled_bytes(mr, pk) + gram * (1 + P.split) + 12 * tiled_bytes(mp, mp) + 2 * tiled_bytes(nr, mp) +
+               2 * tiled_bytes(mp, mp);
     if (dense) b += 2 * tiled_bytes(rup(n_act, 128), ka) + 2 * tiled_bytes(mp, ka);
-    {   // split-K partials of the Gram and its tile list
-        const int rt = rup(m + 1, 128) / 128, ct = (m + 1 + 127) / 128;
-        int tiles = 0;
-        for (int r = 0; r < rt; ++r)
-            for (int c = r; c < ct; ++c) ++tiles;
-        b += (size_t)gram_split_for(m, 2 * n_subv, sms) * (m + 1) * (m + 1) * 4 + (size_t)tiles * sizeof(int2);
-    }
+    for (const GemmPlan* p : {&P.gram, &P.one, &P.two, &P.tr, &P.noise}) b += p->bytes();
     b += (size_t)2 * n_act * 4 + (size_t)4 * m * 4 + 16 + CTL_N * 4 + NS_MAX * 4 + (size_t)n_subv * 16;
     return b;
 }
@@ -515,16 +549,23 @@ int global_prepare(letkf_ctx* c) {
     bool ok = true;
     const size_t tst = tiled_bytes(S->mr, S->pk), tsq = tiled_bytes(S->mp, S->mp);
     ok = ok && get(tst, (void**)&S->st_hi) && get(tst, (void**)&S->st_lo);
-    ok = ok && get((size_t)(m + 1) * (m + 1) * 4, (void**)&S->G);
-    std::vector<int2> gt;
-    for (int r = 0; r < S->mr / 128; ++r)
-        for (int cc = r; cc < (m + 1 + 127) / 128; ++cc) gt.push_back(make_int2(r, cc));
-    S->gram_ntiles = (int)gt.size();
-    S->gram_split = gram_split_for(m, c->p, c->sms);
-    ok = ok && get((size_t)S->gram_split * (m + 1) * (m + 1) * 4, (void**)&S->Gpart) &&
-         get(gt.size() * sizeof(int2), (void**)&S->gram_tiles);
-    if (ok && cudaMemcpy(S->gram_tiles, gt.data(), gt.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess)
-        return LETKF_ECUDA;
+    Plans P = plans_for(c->n_act, c->n_subv, m, dense, c->lq_lower != 0, c->sms);
+    S->ldg = rup(m + 1, 4);
+    S->gram_split = P.split;
+    ok = ok && get((size_t)m * S->ldg * 4, (void**)&S->G) &&
+         get((size_t)P.split * m * S->ldg * 4, (void**)&S->Gpart);
+    for (auto& q : {std::make_pair(&P.gram, &S->pl_gram), std::make_pair(&P.one, &S->pl_one),
+                    std::make_pair(&P.two, &S->pl_two), std::make_pair(&P.tr, &S->pl_tr),
+                    std::make_pair(&P.noise, &S->pl_noise)}) {
+        GemmPlan& p = *q.first;
+        if (!p.ncl) continue;
+        const size_t bi = p.items.size() * sizeof(int4), bs = p.start.size() * sizeof(int);
+        ok = ok && get(bi, (void**)&p.d_items) && get(bs, (void**)&p.d_start);
+        if (ok && (cudaMemcpy(p.d_items, p.items.data(), bi, cudaMemcpyHostToDevice) != cudaSuccess ||
+                   cudaMemcpy(p.d_start, p.start.data(), bs, cudaMemcpyHostToDevice) != cudaSuccess))
+            return LETKF_ECUDA;
+        *q.second = std::move(p);
+    }
     ok = ok && get(tsq, (void**)&S->as_hi) && get(tsq, (void**)&S->as_lo) && get(tsq, (void**)&S->t_hi) &&
          get(tsq, (void**)&S->t_lo);
     for (int q = 0; q < 2; ++q)
@@ -557,7 +598,7 @@ int global_prepare(letkf_ctx* c) {
     int rc = gemm_prepare();
     if (rc) return rc;
     // tiles of the process-noise factor, once
-    if (dense && (rc = to_tiles(static_cast<const float*>(c->Lq), c->n_act, c->n_act, c->n_act, S->l_hi, S->l_lo,
+    if (dense && (rc = to_tiles(static_cast<const float*>(c->Lq), c->n_act, c->n_act, c->n_act, S->l_hi, S->l_lo, 1,
                                 c->stream)))
         return rc;
     // zero the square buffers: products write columns up to m rounded to the CTA tile width only,
@@ -604,34 +645,32 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     // Gram [S d]^T [S d]
     prof_begin(c, STAGE_GRAM);
     // the upper tiles only (the Gram is symmetric), K split so that they fill the SMs
-    GemmArgs g = gemm_args(S->st_hi, S->st_lo, S->st_hi, S->st_lo, S->pk >> 6, m + 1, m + 1, c->d_status);
+    GemmArgs g = gemm_args(S->st_hi, S->st_lo, S->st_hi, S->st_lo, S->pk >> 6, m, m + 1, c->d_status);
     g.mode = GEMM_EPI_F32;
     g.c = S->Gpart;
-    g.ldc = m + 1;
-    g.tiles = S->gram_tiles;
-    g.ksplit = S->gram_split;
-    g.c_split_stride = (size_t)(m + 1) * (m + 1);
-    if ((rc = gemm_launch(g, 128, 1, S->gram_ntiles, st))) return rc;
-    gl_gram_reduce_kernel<<<grid_for((size_t)(m + 1) * (m + 1), 256), 256, 0, st>>>(
-        S->Gpart, S->gram_split, (size_t)(m + 1) * (m + 1), m + 1, S->G);
+    g.ldc = S->ldg;
+    g.c_split_stride = (size_t)m * S->ldg;
+    if ((rc = gemm_launch(g, S->pl_gram, st))) return rc;
+    gl_gram_reduce_kernel<<<grid_for((size_t)m * (m + 1), 256), 256, 0, st>>>(S->Gpart, S->gram_split,
+                                                                              (size_t)m * S->ldg, m, S->ldg, S->G);
     prof_end(c);
     // inverse square root
     prof_begin(c, STAGE_EIG);
-    gl_rowsq_kernel<<<grid_for((size_t)m * 32, 256), 256, 0, st>>>(S->G, m + 1, m, S->rowsq);
+    gl_rowsq_kernel<<<grid_for((size_t)m * 32, 256), 256, 0, st>>>(S->G, S->ldg, m, S->rowsq);
     gl_build_kernel<<<grid_for((size_t)S->mp * (S->mp >> 3), 256), 256, 0, st>>>(
-        S->G, m + 1, m, S->mp, S->rowsq, cm, S->as_hi, S->as_lo, S->z_hi[1], S->z_lo[1], S->scal, S->ctl, S->dev,
+        S->G, S->ldg, m, S->mp, S->rowsq, cm, S->as_hi, S->as_lo, S->z_hi[1], S->z_lo[1], S->scal, S->ctl, S->dev,
         c->d_frame_bad);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     if (cudaGraphLaunch(S->exec, st) != cudaSuccess) return LETKF_ECUDA;
     // mean weights, refined once: w = Z^2 b/(cs); w += Z^2 (b - (cI + G) w)/(cs)
     const int nkb = S->mp >> 6, gv = grid_for((size_t)m * 32, 256);
-    gl_bcol_kernel<<<grid_for(m, 256), 256, 0, st>>>(S->G, m + 1, m, S->r);
+    gl_bcol_kernel<<<grid_for(m, 256), 256, 0, st>>>(S->G, S->ldg, m, S->r);
     for (int pass = 0; pass < 2; ++pass) {
         gl_gemv_kernel<<<gv, 256, 0, st>>>(S->z_hi[0], S->z_lo[0], S->z_hi[1], S->z_lo[1], S->ctl + CTL_ZFINAL, nkb, m, S->r,
                                            S->scal, cm, 0, 0, S->u);
         gl_gemv_kernel<<<gv, 256, 0, st>>>(S->z_hi[0], S->z_lo[0], S->z_hi[1], S->z_lo[1], S->ctl + CTL_ZFINAL, nkb, m, S->u,
                                            S->scal, cm, 1, pass, S->wbar);
-        if (pass == 0) gl_resid_kernel<<<gv, 256, 0, st>>>(S->G, m + 1, m, S->wbar, cm, S->r);
+        if (pass == 0) gl_resid_kernel<<<gv, 256, 0, st>>>(S->G, S->ldg, m, S->wbar, cm, S->r);
     }
     gl_wt_kernel<<<grid_for((size_t)S->mp * (S->mp >> 3), 256), 256, 0, st>>>(
         S->z_hi[0], S->z_lo[0], S->z_hi[1], S->z_lo[1], S->ctl + CTL_ZFINAL, m, S->mp, S->wbar, S->scal,
@@ -647,9 +686,7 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     g.c = Xo;
     g.ldc = c->m_pad;
     g.add = S->xbar;
-    // 256-column tiles where the W^T tiles have the rows (m rounded to 256): half the re-reads of X'
-    const int bt = S->mp % 256 == 0 ? 256 : 128;
-    if ((rc = gemm_launch(g, bt, S->nr / 128, (m + bt - 1) / bt, st))) return rc;
+    if ((rc = gemm_launch(g, S->pl_tr, st))) return rc;
     gl_reject_kernel<<<grid_for((size_t)n * c->m_pad, 256), 256, 0, st>>>(X, Xo, (size_t)n * c->m_pad, c->d_frame_bad);
     prof_end(c);
     return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
@@ -664,12 +701,10 @@ int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
         c->seed, (uint32_t)c->frame, c->n_act, c->m, S->mp, S->ka, S->xi_hi, S->xi_lo);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     GemmArgs g = gemm_args(S->l_hi, S->l_lo, S->xi_hi, S->xi_lo, S->ka >> 6, c->n_act, c->m, c->d_status);
-    g.a_lower = c->lq_lower;
     g.mode = GEMM_EPI_F32;
     g.c = static_cast<float*>(c->V);
     g.ldc = c->m;
-    const int bt = S->mp % 256 == 0 ? 256 : 128;
-    const int rc = gemm_launch(g, bt, rup(c->n_act, 128) / 128, (c->m + bt - 1) / bt, c->stream);
+    const int rc = gemm_launch(g, S->pl_noise, c->stream);
     prof_end(c);
     if (rc) return rc;
     return launch_forecast(c, c->V, xpred, in_analysis);

@@ -325,7 +325,8 @@ size_t footprint_bytes(const letkf_params* p, const HostModel& h) {
     if (p->path == LETKF_PATH_GLOBAL) {
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) sms = 0;
-        b += letkf::global_bytes(h.n_act, h.n_subv, p->m, p->q_sqrt != nullptr, sms);
+        b += letkf::global_bytes(h.n_act, h.n_subv, p->m, p->q_sqrt != nullptr,
+                                 p->q_sqrt && letkf::lower_triangular(p->q_sqrt, h.n_act), sms);
     }
     return b;
 }

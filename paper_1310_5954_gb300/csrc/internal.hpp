@@ -195,7 +195,7 @@ struct NormalsNode {
 int normals_node_params(letkf_ctx* c, unsigned long long frame, void* xi, NormalsNode* nn);
 
 // global.cu: the global (single-domain) ETKF at large ensemble sizes
-size_t global_bytes(int n_act, int n_subv, int m, bool dense, int sms);
+size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sms);
 int global_prepare(letkf_ctx* c);
 void global_free(letkf_ctx* c);
 int global_analyze(letkf_ctx* c, const void* y, double sigma);
@@ -203,33 +203,58 @@ int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
 
 // gemm.cu: tiled tensor-core GEMM, C = A B^T with tiled BF16 operands (128 x 64 tiles)
 enum GemmEpilogue { GEMM_EPI_F32 = 0, GEMM_EPI_TILES = 1, GEMM_EPI_ADD_ROW = 2 };
+// How the tiles of a product are dealt to the clusters of one launch.  A piece is `width` columns (64, 128
+// or 256) of cm row tiles (one per CTA of the cluster), over K steps [kb0, kb1); cluster q does
+// items[start[q]] .. items[start[q + 1] - 1].
+struct GemmShape {
+    int m_tiles = 0, N = 0, nkb = 0;    // row tiles, columns, K / 64
+    int bn = 64, mn = 0;                // widest piece; B read MN-major
+    int cm = 1;                         // row tiles (CTAs) per cluster: 1 or 2
+    int lower = 0;                      // A is lower triangular: row tile r needs K steps < 2 (r + 1)
+    int upper = 0;                      // only pieces that reach the diagonal or lie right of it
+    int ksplit = 1;                     // shares of the K steps (partial products)
+    int batch = 1;                      // products of this shape in the launch
+};
+struct GemmPlan {
+    int bn = 64, cm = 1, ncl = 0;
+    long long cycles = 0;               // the model's time of the busiest cluster
+    std::vector<int> start;             // ncl + 1
+    std::vector<int4> items;            // row tile group, first column, kb0 | kb1 << 16,
+                                        // width | share << 10 | product << 28
+    int* d_start = nullptr;
+    int4* d_items = nullptr;
+    size_t bytes() const { return items.size() * sizeof(int4) + start.size() * sizeof(int); }
+};
+GemmPlan gemm_plan(const GemmShape& s, int sms);
+
 struct GemmArgs {
-    const uint8_t* a_hi;
-    const uint8_t* a_lo;        // null: single BF16
-    const uint8_t* b_hi;
-    const uint8_t* b_lo;
+    // product 0 and, where the plan has two, product 1 (operands and tiled output only)
+    const uint8_t* a_hi[2];
+    const uint8_t* a_lo[2];     // null: single BF16
+    const uint8_t* b_hi[2];
+    const uint8_t* b_lo[2];
     int a_nkb, b_nkb;           // column tiles per row tile of A and B
-    int nkb;                    // K / 64 steps to run
     int split;                  // 1: hi hi + hi lo + lo hi
-    int a_lower;                // 1: A is lower triangular (K steps past the row tile skipped)
-    const int2* tiles;          // non-null: blockIdx.x takes output tile (row tile, column tile) tiles[x]
-    int ksplit;                 // > 1: blockIdx.z takes one of ksplit contiguous shares of the K steps,
-    size_t c_split_stride;      //   F32 output of share z at c + z * c_split_stride
+    int m_tiles;                // row tiles of A there are
+    int bn;                     // the plan: its widest piece, and the pieces
+    const int* start;
+    const int4* items;
+    size_t c_split_stride;      // F32 output of share z goes to c + z * c_split_stride
     int b_mn;                   // 1: B is the second factor M itself (tiles of M, rows = K), read
-                                //    MN-major: C = A M (BN = 64 only); 0: C = A B^T
+                                //    MN-major: C = A M (width 64 only); 0: C = A B^T
     int M, N;                   // valid rows / columns of C
     int mode;                   // GemmEpilogue
     float* c;                   // F32 / ADD_ROW: C[row * ldc + col]
     int ldc;
     float alpha;
-    uint8_t* o_hi;              // TILES: alpha C + beta I as a tiled operand with o_nkb column tiles
-    uint8_t* o_lo;
+    uint8_t* o_hi[2];           // TILES: alpha C + beta I as a tiled operand with o_nkb column tiles
+    uint8_t* o_lo[2];
     int o_nkb;
     float beta;
     unsigned int* dev;          // TILES: max |C - I| over valid entries (float bits, atomicMax)
     const float* add;           // ADD_ROW: per-row term
     const int* run;             // non-null: the launch does nothing when *run == 0
-    int* next_flag;             // non-null: CTA (0,0) sets *next_flag = run && (*dev_in >= run_tol),
+    int* next_flag;             // non-null: CTA 0 sets *next_flag = run && (*dev_in >= run_tol),
     unsigned int* dev_in;       //   and, when running, resets *dev_in, sets *z_final = z_index
     float run_tol;              //   and counts one step in *steps
     int* z_final;
@@ -239,8 +264,8 @@ struct GemmArgs {
 };
 size_t tiled_bytes(int rows, int cols);
 int gemm_prepare();
-int gemm_launch(const GemmArgs& g, int bn, int m_tiles, int n_tiles, cudaStream_t stream);
-int to_tiles(const float* src, int R, int K, int ld, void* hi, void* lo, cudaStream_t stream);
+int gemm_launch(const GemmArgs& g, const GemmPlan& p, cudaStream_t stream);
+int to_tiles(const float* src, int R, int K, int ld, void* hi, void* lo, int sliced, cudaStream_t stream);
 
 // piston.cu: differential pistons between domains
 size_t piston_bytes(const HostModel& h, int n_dom, int elem_bytes);

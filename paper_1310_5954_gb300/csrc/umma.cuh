@@ -48,6 +48,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 
 // Poll an mbarrier phase for at most `cycles` SM clocks; false when the limit ran out.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, long long cycles) {
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
         if (clock64() - t0 > cycles) return false;
@@ -82,6 +83,27 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
             smem_u32(dst)),
         "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
+}
+
+// The same bytes to the same offset of every CTA of the cluster named in `mask`; each one's mbarrier at
+// bar's offset counts them.
+__device__ __forceinline__ void bulk_g2s_multicast(void* dst, const void* src, uint32_t bytes, uint64_t* bar,
+                                                   uint16_t mask) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], "
+        "%4;" ::"r"(smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar)), "h"(mask)
+        : "memory");
+}
+
+// ---------------------------------------------------------------- clusters
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // ---------------------------------------------------------------- fences
@@ -222,6 +244,18 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                  : "memory");
 }
 
+// The same arrival on the barrier at bar's offset in every CTA of the cluster named in `mask`.
+__device__ __forceinline__ void mma_commit_multicast(uint64_t* bar, uint16_t mask) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"(mask)
+        : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // A matrix W (K rows x N columns) stored with the same core-matrix layout, row index = k and
 // column index = n, is the MN-major form of the operand B[n][k] = W[k][n]: core matrices
 // adjacent in N are 128 bytes apart (stride byte offset) and core matrices adjacent in K are
@@ -231,6 +265,12 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 // Byte offset of element (row, k) in the canonical layout of an operand with K columns.
 __host__ __device__ __forceinline__ uint32_t op_offset(int row, int k, int K) {
     return (uint32_t)(((row >> 3) * (K >> 3) + (k >> 3)) * 128 + (row & 7) * 16 + (k & 7) * 2);
+}
+
+// Byte offset of element (row, col) in a sliced operand of 64 n64 columns: slices of 128 rows x 16 columns
+// (4 KB, each in the canonical layout), the slices of 128 rows one after another.
+__host__ __device__ __forceinline__ size_t slice_offset(int row, int col, int n64) {
+    return ((size_t)(row >> 7) * n64 * 4 + (col >> 4)) * 4096 + op_offset(row & 127, col & 15, 16);
 }
 
 }  // namespace umma
