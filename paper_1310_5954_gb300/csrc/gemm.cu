@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "../../include/letkf.h"
+#include "gemm_ring.cuh"
 #include "internal.hpp"
 #include "umma.cuh"
 
@@ -43,42 +44,20 @@ using namespace umma;
 namespace {
 
 constexpr int GT = 192;                   // threads per CTA: producer warp, MMA warp, four epilogue warps
-constexpr int TILE_B = 128 * 64 * 2;      // bytes of one operand tile
-constexpr long long GEMM_WAIT = 4000000000LL;
-
-__device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& h, __nv_bfloat16& l) {
-    h = __float2bfloat16_rn(x);
-    l = __float2bfloat16_rn(x - __bfloat162float(h));
-}
-
-// Byte offset of element (row, col) in a tiled operand with nkb column tiles.
-__device__ __forceinline__ size_t tiled_offset(int row, int col, int nkb) {
-    return ((size_t)(row >> 7) * nkb + (col >> 6)) * TILE_B + op_offset(row & 127, col & 63, 64);
-}
-
-// One stage: KC columns of A (128 rows, hi and lo) and of B (bn rows or columns).  MN: a whole tile, B read
-// MN-major; else SL slices of 16 columns.  A unit (tile or slice) is [A hi, A lo, B hi, B lo].
-template <bool MN>
-struct GemmStage {
-    static constexpr int UC = MN ? 64 : 16, SL = MN ? 1 : 2, KC = UC * SL;    // columns of a unit, units, columns
-    static constexpr int A_BYTES = 128 * 2 * UC;
-    static constexpr int RING = 192 * 1024, MOST = MN ? 4 : 8;
-    static constexpr int EPI = 4 * 32 * 36 * 4;        // 32 rows x 32 columns per epilogue warp, padded rows
-    static constexpr int BYTES = 1024 + RING + EPI;
-};
+constexpr int GEMM_EPI = 4 * 32 * 36 * 4;  // 32 rows x 32 columns per epilogue warp, padded rows
+constexpr int GEMM_SMEM = 1024 + 192 * 1024 + GEMM_EPI;
 
 // CM CTAs per cluster, along the rows: they share the columns of B.
 template <int CM, bool MN>
 __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ GemmArgs g) {
     using L = GemmStage<MN>;
     constexpr int BN = MN ? 64 : 256;
-    const uint32_t b_slot = (uint32_t)g.bn * 2 * L::UC, unit = 2 * L::A_BYTES + 2 * b_slot, stage_b = L::SL * unit;
-    const int stages = min(L::MOST, L::RING / (int)stage_b);
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) uint64_t full[L::MOST], empty[L::MOST], tfull[2], tempty[2];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag, issued;        // issued: stages the producer filled (for the drain on abort)
+    __shared__ int abort_flag, filled;
+    const Ring ring = make_ring<MN>(smem, full, empty, g.bn);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, uwarp = uniform_warp();
     const uint32_t rank = CM > 1 ? cluster_rank() : 0u;
     if (tid == 0) {
@@ -90,7 +69,7 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
             mbar_init(&tfull[a], 1);
             mbar_init(&tempty[a], 128);
         }
-        abort_flag = issued = 0;
+        abort_flag = filled = 0;
         fence_mbar_init();
     }
     if (warp == 0) {
@@ -102,22 +81,10 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
     tc_fence_after();
     if (CM > 1) cluster_sync();                    // every barrier is initialised before a peer's copy arrives
     const uint32_t tmem = tmem_slot;
-    const bool on = g.run == nullptr || *g.run != 0;
-    if (g.next_flag && blockIdx.x == 0 && tid == 0) {
-        // this launch decides whether the next step runs (see GemmArgs), also when it does
-        // nothing itself, so that a finished iteration stays finished
-        *g.next_flag = (on && __uint_as_float(*g.dev_in) >= g.run_tol) ? 1 : 0;
-        if (on) {
-            *g.dev_in = 0u;
-            if (g.z_final) *g.z_final = g.z_index;
-            if (g.steps) *g.steps += 1;
-        }
-    }
     const bool split = g.split != 0;
-    const int cid = blockIdx.x / CM;
-    const int i0 = on ? g.start[cid] : 0, i1 = on ? g.start[cid + 1] : 0;
+    const int cid = blockIdx.x / CM, i0 = g.start[cid], i1 = g.start[cid + 1];
     struct Work {
-        int ty, col0, kb0, kb1, width, share, z;
+        int ty, col0, kb0, kb1, width, share;
     };
     auto work = [&](int i) {
         const int4 it = g.items[i];
@@ -127,109 +94,35 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
         w.col0 = it.y;
         w.kb0 = it.z & 0xFFFF;
         w.kb1 = it.z >> 16;
-        w.share = (it.w >> 10) & 0xFFFF;
-        w.z = it.w >> 28;
+        w.share = it.w >> 10;
         return w;
     };
     if (uwarp == 0 && elect_one()) {
-        constexpr uint16_t all = (uint16_t)((1u << CM) - 1u);
-        // Each CTA copies its part of a chunk of B to all of them.
-        // 256 columns are two consecutive 128-row tiles, copied next to each other so that one descriptor
-        // with the same row-group stride spans all 256 rows
-        auto copy_b = [&](uint8_t* dst, const uint8_t* src, uint32_t bytes, size_t next, uint64_t* bar) {
-            if (CM > 1) {
-                const uint32_t part = bytes / CM, off = rank * part;
-                bulk_g2s_multicast(dst + off, src + (off / L::A_BYTES) * next + off % L::A_BYTES, part, bar, all);
-            } else {
-                bulk_g2s(dst, src, min(bytes, (uint32_t)L::A_BYTES), bar);
-                if (bytes > L::A_BYTES) bulk_g2s(dst + L::A_BYTES, src + next, L::A_BYTES, bar);
-            }
-        };
-        int c = 0, s = 0, par = 0;                 // stages filled so far, the next one and its parity
+        RingPos pos;
         bool ok = true;
         for (int i = i0; i < i1 && ok; ++i) {
             const Work w = work(i);
             // a CTA past the last row tile reads that one's operands (its results are dropped)
-            const int ty = min(w.ty, g.m_tiles - 1), col0 = w.col0;
-            const uint32_t b_bytes = (uint32_t)w.width * (MN ? 128u : 32u);
-            const uint32_t stage_bytes = (split ? 2u : 1u) * L::SL * (L::A_BYTES + b_bytes);
-            const size_t a_row = (size_t)ty * g.a_nkb * TILE_B;
-            // K-major B (rows = N): the 128-row tile holding this CTA's columns, from the slice's second half
-            // for odd blocks of 64.  MN-major B (the second factor itself, rows = K; width 64): step kb takes
-            // rows 64 kb .. 64 kb + 63 of column tile col0 / 64, the first or second half of that tile.
-            const size_t b_row = MN ? (size_t)(col0 >> 6) * TILE_B
-                                    : (size_t)(col0 >> 7) * g.b_nkb * TILE_B + ((col0 & 64) ? L::A_BYTES / 2 : 0);
-            const size_t b_next = (size_t)g.b_nkb * TILE_B;
-            const uint8_t *a_hi = g.a_hi[w.z] + a_row, *b_hi = g.b_hi[w.z] + b_row;
-            const uint8_t *a_lo = split ? g.a_lo[w.z] + a_row : nullptr, *b_lo = split ? g.b_lo[w.z] + b_row : nullptr;
-            const int k_end = w.kb1 * 64 / L::KC;
-            for (int k = w.kb0 * 64 / L::KC; k < k_end; ++k, ++c) {
-                if (c >= stages && !mbar_wait_bounded(&empty[s], par ^ 1, GEMM_WAIT)) {
-                    atomicOr(g.status, ST_TIMEOUT);
-                    abort_flag = 1;
-                    ok = false;
-                    break;
-                }
-                mbar_arrive_expect_tx(&full[s], stage_bytes);
-#pragma unroll
-                for (int u = 0; u < L::SL; ++u) {
-                    uint8_t* st = smem + s * stage_b + u * unit;
-                    const size_t ao = (size_t)(k * L::SL + u) * L::A_BYTES;
-                    const size_t bo = MN ? (size_t)(k >> 1) * g.b_nkb * TILE_B + (size_t)(k & 1) * (TILE_B / 2) : ao;
-                    bulk_g2s(st, a_hi + ao, L::A_BYTES, &full[s]);
-                    copy_b(st + 2 * L::A_BYTES, b_hi + bo, b_bytes, b_next, &full[s]);
-                    if (split) {
-                        bulk_g2s(st + L::A_BYTES, a_lo + ao, L::A_BYTES, &full[s]);
-                        copy_b(st + 2 * L::A_BYTES + b_slot, b_lo + bo, b_bytes, b_next, &full[s]);
-                    }
-                }
-                if (++s == stages) s = 0, par ^= 1;
-            }
+            const RingOperands o = ring_operands<MN>(g.a_hi, split ? g.a_lo : nullptr, g.a_nkb, min(w.ty, g.m_tiles - 1),
+                                                     g.b_hi, g.b_lo, g.b_nkb, w.col0, w.width);
+            ok = ring_fill<CM, MN>(ring, pos, o, rank, w.kb0 * 64 / L::KC, w.kb1 * 64 / L::KC);
         }
-        issued = c;
+        filled = pos.c;
+        if (!ok) {
+            atomicOr(g.status, ST_TIMEOUT);
+            abort_flag = 1;
+        }
     } else if (uwarp == 1 && elect_one()) {
-        // A: K-adjacent core matrices 128 B apart, row-adjacent 1024 B in a tile, 256 B in a slice; K-major B
-        // alike.  MN-major B: N-adjacent core matrices 128 B apart, K-adjacent 1024 B, a K step 2048 B
-        constexpr uint32_t a_sbo = MN ? 1024u : 256u, b_lbo = MN ? 1024u : 128u, b_sbo = MN ? 128u : 256u;
-        constexpr uint32_t a_step = 256u, b_step = 2048u;   // within a tile; slices lie a unit apart
-        constexpr uint16_t all = (uint16_t)((1u << CM) - 1u);       // their copies fill this CTA's stages
-        int n = 0, s = 0, par = 0;
+        RingPos pos;
+        int n = 0;
         bool ok = true;
-        for (int i = i0; i < i1 && ok; ++i) {
+        for (int i = i0; i < i1 && ok; ++i, ++n) {
             const Work w = work(i);
-            const uint32_t idesc = idesc_bf16(128, w.width, MN);
             const int acc_i = n & 1;
-            if (n >= 2 && !mbar_wait_bounded(&tempty[acc_i], ((n >> 1) - 1) & 1, GEMM_WAIT)) ok = false;
+            ok = n < 2 || mbar_wait_bounded(&tempty[acc_i], ((n >> 1) - 1) & 1, GEMM_WAIT);
             tc_fence_after();
-            const uint32_t dt = tmem + acc_i * BN;
-            const int k_begin = w.kb0 * 64 / L::KC, k_end = w.kb1 * 64 / L::KC;
-            for (int kc = k_begin; kc < k_end && ok; ++kc) {
-                if (!mbar_wait_bounded(&full[s], par, GEMM_WAIT)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t st = smem_u32(smem + s * stage_b);
-                const uint32_t sa_lo = st + L::A_BYTES, sb_hi = st + 2 * L::A_BYTES, sb_lo = sb_hi + b_slot;
-#pragma unroll
-                for (int k = 0; k < L::KC / 16; ++k) {
-                    const uint32_t acc = (kc > k_begin || k > 0) ? 1u : 0u;
-                    const uint32_t da = MN ? a_step * k : unit * k, db = MN ? b_step * k : unit * k;
-                    const uint64_t ah = sdesc(st + da, 128, a_sbo), bh = sdesc(sb_hi + db, b_lbo, b_sbo);
-                    mma_bf16(dt, ah, bh, idesc, acc);
-                    if (split) {
-                        mma_bf16(dt, ah, sdesc(sb_lo + db, b_lbo, b_sbo), idesc, 1u);
-                        mma_bf16(dt, sdesc(sa_lo + da, 128, a_sbo), bh, idesc, 1u);
-                    }
-                }
-                if (CM > 1)
-                    mma_commit_multicast(&empty[s], all);
-                else
-                    mma_commit(&empty[s]);
-                if (++s == stages) s = 0, par ^= 1;
-            }
+            ok = ok && ring_issue<CM, MN>(ring, pos, tmem + acc_i * BN, w.width, split, (w.kb1 - w.kb0) * 64 / L::KC);
             if (ok) mma_commit(&tfull[acc_i]);
-            ++n;
         }
         if (!ok) {
             atomicOr(g.status, ST_TIMEOUT);
@@ -237,9 +130,8 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
         }
     } else if (warp >= 2) {
         const int quad = warp & 3, trow = 32 * quad + lane;      // TMEM lane = tile row of this thread
-        float* stg = reinterpret_cast<float*>(smem + L::RING) + quad * 32 * 36;
+        float* stg = reinterpret_cast<float*>(smem + 192 * 1024) + quad * 32 * 36;
         const bool vec = ((g.ldc | g.c_split_stride) & 3) == 0 && (reinterpret_cast<uintptr_t>(g.c) & 15) == 0;
-        float dev = 0.f;
         int n = 0;
         for (int i = i0; i < i1; ++i) {
             const Work w = work(i);
@@ -260,59 +152,32 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
                 float v[64];
                 tmem_ld64(tmem + acc_i * BN + ((uint32_t)(quad * 32) << 16) + c0, v);
                 if (!mine) continue;
-                if (g.mode == GEMM_EPI_TILES) {
-                    // out = alpha * acc + beta * I, as a tiled operand (all padded positions written:
-                    // rows and columns beyond M, N get zeros)
+                // ADD_ROW: add[row] + acc; F32: acc; valid rows and columns only.  32 columns at a time
+                // through shared memory, so that a warp writes whole 128-byte row pieces
+                float* cz = g.c + (size_t)w.share * g.c_split_stride;
+                const float base = g.mode == GEMM_EPI_ADD_ROW && row < g.M ? g.add[row] : 0.f;
 #pragma unroll
-                    for (int j = 0; j < 64; j += 8) {
-                        __align__(16) __nv_bfloat16 h[8], l[8];
+                for (int hf = 0; hf < 64; hf += 32) {
+                    __syncwarp();
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const int col = col0 + c0 + j + q;
-                            const bool in = row < g.M && col < g.N;
-                            const float x = in ? g.alpha * v[j + q] + (row == col ? g.beta : 0.f) : 0.f;
-                            if (g.dev && in) dev = fmaxf(dev, fabsf(v[j + q] - (row == col ? 1.f : 0.f)));
-                            split_bf16(x, h[q], l[q]);
-                        }
-                        const size_t off = tiled_offset(row, col0 + c0 + j, g.o_nkb);
-                        *reinterpret_cast<uint4*>(g.o_hi[w.z] + off) = *reinterpret_cast<const uint4*>(h);
-                        if (g.o_lo[w.z]) *reinterpret_cast<uint4*>(g.o_lo[w.z] + off) = *reinterpret_cast<const uint4*>(l);
-                    }
-                } else {
-                    // F32: alpha acc; ADD_ROW: add[row] + acc; valid rows and columns only.  32 columns
-                    // at a time through shared memory, so that a warp writes whole 128-byte row pieces
-                    float* cz = g.c + (size_t)w.share * g.c_split_stride;
-                    const bool add = g.mode == GEMM_EPI_ADD_ROW;
-                    const float base = add && row < g.M ? g.add[row] : 0.f;
-#pragma unroll
-                    for (int hf = 0; hf < 64; hf += 32) {
-                        __syncwarp();
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4) {
-                            float4 o;
-                            o.x = add ? base + v[hf + j] : g.alpha * v[hf + j];
-                            o.y = add ? base + v[hf + j + 1] : g.alpha * v[hf + j + 1];
-                            o.z = add ? base + v[hf + j + 2] : g.alpha * v[hf + j + 2];
-                            o.w = add ? base + v[hf + j + 3] : g.alpha * v[hf + j + 3];
-                            *reinterpret_cast<float4*>(stg + lane * 36 + j) = o;
-                        }
-                        __syncwarp();
+                    for (int j = 0; j < 32; j += 4)
+                        *reinterpret_cast<float4*>(stg + lane * 36 + j) = make_float4(
+                            base + v[hf + j], base + v[hf + j + 1], base + v[hf + j + 2], base + v[hf + j + 3]);
+                    __syncwarp();
 #pragma unroll 2
-                        for (int q = 0; q < 8; ++q) {
-                            const int rr = 4 * q + (lane >> 3), cc = 4 * (lane & 7);
-                            const int gr = row0 + 32 * quad + rr, gc = col0 + c0 + hf + cc;
-                            const float4 o = *reinterpret_cast<const float4*>(stg + rr * 36 + cc);
-                            if (gr < g.M) {
-                                float* dst = cz + (size_t)gr * g.ldc + gc;
-                                if (vec && gc + 4 <= g.N) {
-                                    *reinterpret_cast<float4*>(dst) = o;
-                                } else {
-                                    if (gc + 0 < g.N) dst[0] = o.x;
-                                    if (gc + 1 < g.N) dst[1] = o.y;
-                                    if (gc + 2 < g.N) dst[2] = o.z;
-                                    if (gc + 3 < g.N) dst[3] = o.w;
-                                }
-                            }
+                    for (int q = 0; q < 8; ++q) {
+                        const int rr = 4 * q + (lane >> 3), cc = 4 * (lane & 7);
+                        const int gr = row0 + 32 * quad + rr, gc = col0 + c0 + hf + cc;
+                        const float4 o = *reinterpret_cast<const float4*>(stg + rr * 36 + cc);
+                        if (gr >= g.M) continue;
+                        float* dst = cz + (size_t)gr * g.ldc + gc;
+                        if (vec && gc + 4 <= g.N) {
+                            *reinterpret_cast<float4*>(dst) = o;
+                        } else {
+                            if (gc + 0 < g.N) dst[0] = o.x;
+                            if (gc + 1 < g.N) dst[1] = o.y;
+                            if (gc + 2 < g.N) dst[2] = o.z;
+                            if (gc + 3 < g.N) dst[3] = o.w;
                         }
                     }
                 }
@@ -321,17 +186,11 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
             mbar_arrive(&tempty[acc_i]);
             ++n;
         }
-        if (g.dev) {
-            for (int o = 16; o > 0; o >>= 1) dev = fmaxf(dev, __shfl_xor_sync(0xffffffffu, dev, o));
-            if (lane == 0) atomicMax(g.dev, __float_as_uint(dev));
-        }
     }
     __syncwarp();
     __syncthreads();
     // copies still in flight after a wait gave up land in shared memory before the CTA leaves
-    if (abort_flag && tid == 0)
-        for (int c = max(0, issued - stages); c < issued; ++c)
-            mbar_wait_bounded(&full[c % stages], (c / stages) & 1, GEMM_WAIT);
+    if (abort_flag && tid == 0) ring_drain(ring, filled);
     tc_fence_before();
     __syncthreads();
     if (CM > 1) cluster_sync();                    // no peer's copy or arrival comes after a CTA has left
@@ -361,7 +220,7 @@ __global__ void to_tiles_kernel(const float* __restrict__ src, int R, int K, int
 }  // namespace
 
 size_t tiled_bytes(int rows, int cols) {
-    return (size_t)((rows + 127) / 128) * ((cols + 63) / 64) * TILE_B;
+    return (size_t)((rows + 127) / 128) * ((cols + 63) / 64) * GEMM_TILE_B;
 }
 
 // The pieces are dealt longest first, each to the cluster with the least work so far.  A piece costs the
@@ -381,11 +240,10 @@ GemmPlan gemm_plan(const GemmShape& s, int sms) {
     auto pieces = [&](int row, int col, int width, std::vector<int4>& out) {   // one column group of one row group
         const int last = std::min(s.m_tiles, (row + 1) * s.cm);      // row tiles [row * cm, last)
         const int kend = s.lower ? std::min(s.nkb, 2 * last) : s.nkb;
-        for (int z = 0; z < s.batch; ++z)
-            for (int k = 0; k < s.ksplit; ++k) {
-                const int k0 = (int)((long long)kend * k / s.ksplit), k1 = (int)((long long)kend * (k + 1) / s.ksplit);
-                out.push_back(make_int4(row, col, k0 | (k1 << 16), width | (k << 10) | (z << 28)));
-            }
+        for (int k = 0; k < s.ksplit; ++k) {
+            const int k0 = (int)((long long)kend * k / s.ksplit), k1 = (int)((long long)kend * (k + 1) / s.ksplit);
+            out.push_back(make_int4(row, col, k0 | (k1 << 16), width | (k << 10)));
+        }
     };
     for (int base = s.bn; base >= 64; base /= 2)
         for (int tail = base; tail >= 64; tail /= 2) {
@@ -435,9 +293,9 @@ GemmPlan gemm_plan(const GemmShape& s, int sms) {
 namespace {
 template <typename F>
 int gemm_with(bool mn, int cm, F&& f) {
-    if (mn) return cm == 1 ? f(gemm_kernel<1, true>, GemmStage<true>::BYTES) : LETKF_EINVAL;
-    if (cm == 1) return f(gemm_kernel<1, false>, GemmStage<false>::BYTES);
-    return cm == 2 ? f(gemm_kernel<2, false>, GemmStage<false>::BYTES) : LETKF_EINVAL;
+    if (mn) return cm == 1 ? f(gemm_kernel<1, true>, GEMM_SMEM) : LETKF_EINVAL;
+    if (cm == 1) return f(gemm_kernel<1, false>, GEMM_SMEM);
+    return cm == 2 ? f(gemm_kernel<2, false>, GEMM_SMEM) : LETKF_EINVAL;
 }
 }  // namespace
 
@@ -528,10 +386,10 @@ extern "C" int letkf_gemm_selftest(const float* A, const float* B, float* C, int
     }
     if (!rc) {
         GemmArgs g{};
-        g.a_hi[0] = ah;
-        g.a_lo[0] = split ? al : nullptr;
-        g.b_hi[0] = bh;
-        g.b_lo[0] = split ? bl : nullptr;
+        g.a_hi = ah;
+        g.a_lo = split ? al : nullptr;
+        g.b_hi = bh;
+        g.b_lo = split ? bl : nullptr;
         g.m_tiles = mp / 128;
         g.a_nkb = kp / 64;
         g.b_nkb = b_mn ? (N + 63) / 64 : kp / 64;
@@ -542,7 +400,6 @@ extern "C" int letkf_gemm_selftest(const float* A, const float* B, float* C, int
         g.mode = GEMM_EPI_F32;
         g.c = C;
         g.ldc = N;
-        g.alpha = 1.f;
         g.status = st;
         rc = gemm_launch(g, plan, s);
     }

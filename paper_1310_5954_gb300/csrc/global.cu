@@ -14,10 +14,9 @@
 // (FP32-level, ~2^-16 per element).  The iteration's products are true products (the second
 // factor's tiles read MN-major): the matrices are symmetric in exact arithmetic, but taking
 // A B^T for A B lets the rounding's antisymmetric part grow until the iteration diverges at the
-// conditioning of the first frames (s ~ 1e4).  The iteration runs at most NS_MAX steps and stops
-// once max |P - I| < NS_TOL (the deciding flag is written on the device; the products of a
-// finished iteration return at once; ST_NOCONV when the limit stops it); the steps are one CUDA
-// graph, launched every frame, whose steps past NS_FLAT sit behind a conditional node.
+// conditioning of the first frames (s ~ 1e4).  From the Gram's shares to W^T everything is one
+// cooperative kernel (root.cu); the iteration runs at most ROOT_STEPS steps and stops once
+// max |P - I| < 1e-2 (ST_NOCONV when the limit stops it).
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -34,32 +33,23 @@
 
 namespace letkf {
 
-constexpr int NS_MAX = 24;
-constexpr int NS_FLAT = 12;     // steps launched unconditionally; the rest behind one conditional node
-constexpr float NS_TOL = 1e-2f;   // the last update then lands at ~0.75 NS_TOL^2 ~ 7.5e-5 of max |P - I|
-// device control words: run[k] (step k runs) for k = 0 .. NS_MAX, steps taken, final Z buffer
-enum { CTL_RUN = 0, CTL_STEPS = NS_MAX + 1, CTL_ZFINAL = NS_MAX + 2, CTL_N = NS_MAX + 4 };
-
 struct GlobalState {
     int mr = 0, pk = 0, mp = 0, nr = 0, ka = 0;   // padded sizes: S' rows, slopes, m, state rows, actuators
     uint8_t *st_hi = nullptr, *st_lo = nullptr;   // [S d]^T tiles (mr x pk)
     float* G = nullptr;                            // m x (m+1) Gram, row-major
     float* Gpart = nullptr;                        // partial Grams of the upper tiles, one per share
     int ldg = 0, gram_split = 1;                   // leading dimension of the Gram, shares of its K steps
-    GemmPlan pl_gram, pl_one, pl_two, pl_tr, pl_noise;   // one / two m x m products, transform, noise draw
+    GemmPlan pl_gram, pl_tr, pl_noise;
     uint8_t *as_hi = nullptr, *as_lo = nullptr, *t_hi = nullptr, *t_lo = nullptr;
     uint8_t *y_hi[2] = {}, *y_lo[2] = {}, *z_hi[2] = {}, *z_lo[2] = {};
     uint8_t *xp_hi = nullptr, *xp_lo = nullptr;    // X' tiles (nr x mp)
     uint8_t *wt_hi = nullptr, *wt_lo = nullptr;    // W^T tiles (mp x mp)
     uint8_t *l_hi = nullptr, *l_lo = nullptr;      // L tiles (rup(n_act) x ka)
     uint8_t *xi_hi = nullptr, *xi_lo = nullptr;    // xi^T tiles (mp x ka)
-    float *xbar = nullptr, *rowsq = nullptr, *wbar = nullptr, *u = nullptr, *r = nullptr, *scal = nullptr;
-    int* ctl = nullptr;                            // control words (CTL_*)
-    unsigned int* dev = nullptr;                   // [NS_MAX]: max |P - I| of each step
+    float *xbar = nullptr, *sq = nullptr, *wbar = nullptr, *u = nullptr, *r = nullptr, *b = nullptr;
+    RootStats* stats = nullptr;
+    unsigned *dev = nullptr, *bar = nullptr;       // max |P - I| of each step; the grid barrier of the iteration
     int4* corner = nullptr;                        // per valid subaperture: its four corner actuators
-    cudaStream_t cap = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
     std::vector<void*> allocs;
 };
 
@@ -75,7 +65,7 @@ int cluster_rows(int row_tiles) { return row_tiles >= 2 ? 2 : 1; }
 // The plans of the analysis's products, and the Gram's shares: as many as make its pieces fill the SMs,
 // against the partial Grams that every share writes and the reduction reads (at 2 KB per cycle).
 struct Plans {
-    GemmPlan gram, one, two, tr, noise;
+    GemmPlan gram, tr, noise;
     int split = 1;
 };
 Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
@@ -97,14 +87,6 @@ Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
         P.gram = p;
         P.split = g.ksplit;
     }
-    GemmShape q;
-    q.m_tiles = mt;
-    q.N = m;
-    q.mn = 1;
-    q.nkb = rup(m, 128) / 64;
-    P.one = gemm_plan(q, sms);
-    q.batch = 2;
-    P.two = gemm_plan(q, sms);
     GemmShape t;
     t.m_tiles = rows;
     t.N = m;
@@ -122,18 +104,9 @@ Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
     return P;
 }
 
-__device__ __forceinline__ size_t toff(int row, int col, int nkb) {
-    return ((size_t)(row >> 7) * nkb + (col >> 6)) * TILE_B + umma::op_offset(row & 127, col & 63, 64);
-}
-
 __device__ __forceinline__ void split2(float x, __nv_bfloat16& h, __nv_bfloat16& l) {
     h = __float2bfloat16_rn(x);
     l = __float2bfloat16_rn(x - __bfloat162float(h));
-}
-
-__device__ __forceinline__ float tval(const uint8_t* hi, const uint8_t* lo, size_t off) {
-    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(hi + off)) +
-           __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(lo + off));
 }
 
 __device__ __forceinline__ void store8(uint8_t* hi, uint8_t* lo, size_t off, const float (&v)[8]) {
@@ -144,8 +117,10 @@ __device__ __forceinline__ void store8(uint8_t* hi, uint8_t* lo, size_t off, con
     *reinterpret_cast<uint4*>(lo + off) = *reinterpret_cast<const uint4*>(l);
 }
 
-// member means of every state row (one warp per row)
-__global__ void gl_mean_kernel(const float* __restrict__ X, int n, int m, int m_pad, float* __restrict__ xbar) {
+// member means of every state row (one warp per row); resets the iteration's grid barrier
+__global__ void gl_mean_kernel(const float* __restrict__ X, int n, int m, int m_pad, float* __restrict__ xbar,
+                               unsigned* __restrict__ bar) {
+    if (blockIdx.x == 0 && threadIdx.x < 2) bar[threadIdx.x] = 0u;
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
@@ -195,143 +170,7 @@ __global__ void gl_slopes_kernel(const float* __restrict__ X, const float* __res
     }
 }
 
-// sum of squares of each row of G (i, j < m), one warp per row
-__global__ void gl_rowsq_kernel(const float* __restrict__ G, int ld, int m, float* __restrict__ rowsq) {
-    const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += warps) {
-        float s = 0.f;
-        for (int j = lane; j < m; j += 32) {
-            const float g = G[(size_t)i * ld + j];
-            s += g * g;
-        }
-        s = warp_sum(s);
-        if (lane == 0) rowsq[i] = s;
-    }
-}
-
-// A_s = (I + G/c)/s and T_0 = (3I - A_s)/2 (= Z_1) as tiles; the iteration's flags for the frame.
-__global__ void gl_build_kernel(const float* __restrict__ G, int ld, int m, int mp, const float* __restrict__ rowsq,
-                                float c, uint8_t* __restrict__ as_hi, uint8_t* __restrict__ as_lo,
-                                uint8_t* __restrict__ t_hi, uint8_t* __restrict__ t_lo, float* __restrict__ scal,
-                                int* __restrict__ ctl, unsigned int* __restrict__ dev,
-                                const int* __restrict__ frame_bad) {
-    __shared__ float s_sh;
-    if (threadIdx.x < 32) {
-        float a = 0.f;
-        for (int i = threadIdx.x; i < m; i += 32) a += rowsq[i];
-        a = warp_sum(a);
-        if (threadIdx.x == 0) s_sh = 1.f + sqrtf(a) / c;
-    }
-    __syncthreads();
-    const float s = s_sh;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        scal[0] = s;
-        for (int k = 0; k <= NS_MAX; ++k) ctl[CTL_RUN + k] = 0;
-        ctl[CTL_RUN + 1] = *frame_bad ? 0 : 1;
-        ctl[CTL_STEPS] = 1;      // the product-free first step
-        ctl[CTL_ZFINAL] = 1;     // Z_1 = T_0, in Z buffer 1
-        for (int k = 0; k < NS_MAX; ++k) dev[k] = 0u;
-    }
-    const int g8 = mp >> 3;
-    const size_t total = (size_t)mp * g8;
-    const float inv = 1.f / s, invc = 1.f / (c * s);
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t / g8), j0 = (int)(t - (size_t)i * g8) * 8;
-        float a[8], tt[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int j = j0 + q;
-            a[q] = 0.f;
-            tt[q] = 0.f;
-            if (i < m && j < m) {
-                a[q] = G[(size_t)i * ld + j] * invc + (i == j ? inv : 0.f);
-                tt[q] = (i == j ? 1.5f : 0.f) - 0.5f * a[q];
-            }
-        }
-        const size_t off = toff(i, j0, mp >> 6);
-        store8(as_hi, as_lo, off, a);
-        store8(t_hi, t_lo, off, tt);
-    }
-}
-
-// out[i] (= or +=) scale * sum_j Z[i][j] v[j] for i < m, Z from the final Newton-Schulz buffer;
-// scale = 1, or 1 / (c s) when use_s.  One warp per row.
-__global__ void gl_gemv_kernel(const uint8_t* __restrict__ z0_hi, const uint8_t* __restrict__ z0_lo,
-                               const uint8_t* __restrict__ z1_hi, const uint8_t* __restrict__ z1_lo,
-                               const int* __restrict__ zfinal, int nkb, int m, const float* __restrict__ v,
-                               const float* __restrict__ scal, float c, int use_s, int accumulate,
-                               float* __restrict__ out) {
-    const int odd = *zfinal & 1;
-    const uint8_t* zh = odd ? z1_hi : z0_hi;
-    const uint8_t* zl = odd ? z1_lo : z0_lo;
-    const float scale = use_s ? 1.f / (c * scal[0]) : 1.f;
-    const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += warps) {
-        float s = 0.f;
-        // eight consecutive columns per lane and pass: one 16-byte load from each of hi and lo
-        for (int j0 = 8 * lane; j0 < m; j0 += 256) {
-            const size_t off = toff(i, j0, nkb);
-            const uint4 hv = *reinterpret_cast<const uint4*>(zh + off);
-            const uint4 lv = *reinterpret_cast<const uint4*>(zl + off);
-            const __nv_bfloat16* hb = reinterpret_cast<const __nv_bfloat16*>(&hv);
-            const __nv_bfloat16* lb = reinterpret_cast<const __nv_bfloat16*>(&lv);
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (j0 + q < m) s += (__bfloat162float(hb[q]) + __bfloat162float(lb[q])) * v[j0 + q];
-        }
-        s = warp_sum(s);
-        if (lane == 0) out[i] = (accumulate ? out[i] : 0.f) + scale * s;
-    }
-}
-
-// r = b - (c w + G w), b = column m of the Gram
-__global__ void gl_resid_kernel(const float* __restrict__ G, int ld, int m, const float* __restrict__ w, float c,
-                                float* __restrict__ r) {
-    const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < m; i += warps) {
-        float s = 0.f;
-        for (int j = lane; j < m; j += 32) s += G[(size_t)i * ld + j] * w[j];
-        s = warp_sum(s);
-        if (lane == 0) r[i] = G[(size_t)i * ld + m] - (c * w[i] + s);
-    }
-}
-
-// b = column m of the Gram, into a contiguous vector
-__global__ void gl_bcol_kernel(const float* __restrict__ G, int ld, int m, float* __restrict__ b) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) b[i] = G[(size_t)i * ld + m];
-}
-
-// W^T tiles: element (j, k) = w_bar[k] + Z[j][k] / sqrt(s) for j, k < m (W = w_bar 1^T + T_a; T_a
-// symmetric); latches ST_NOCONV if the step limit stopped the iteration.
-__global__ void gl_wt_kernel(const uint8_t* __restrict__ z0_hi, const uint8_t* __restrict__ z0_lo,
-                             const uint8_t* __restrict__ z1_hi, const uint8_t* __restrict__ z1_lo,
-                             const int* __restrict__ zfinal, int m, int mp, const float* __restrict__ wbar,
-                             const float* __restrict__ scal, const int* __restrict__ noconv, uint8_t* __restrict__ hi,
-                             uint8_t* __restrict__ lo, int* __restrict__ status) {
-    const int odd = *zfinal & 1;
-    const uint8_t* zh = odd ? z1_hi : z0_hi;
-    const uint8_t* zl = odd ? z1_lo : z0_lo;
-    const float rs = rsqrtf(scal[0]);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && *noconv) atomicOr(status, ST_NOCONV);
-    const int nkb = mp >> 6, g8 = mp >> 3;
-    const size_t total = (size_t)mp * g8;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(t / g8), k0 = (int)(t - (size_t)j * g8) * 8;
-        const size_t off = toff(j, k0, nkb);
-        float v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int k = k0 + q;
-            v[q] = (j < m && k < m) ? wbar[k] + rs * tval(zh, zl, off + 2 * q) : 0.f;
-        }
-        store8(hi, lo, umma::slice_offset(j, k0, nkb), v);
-    }
-}
-
-// X' tiles: element (r, i) = X[r][i] - x_bar[r] for r < n, i < m
+// X' slices: element (r, i) = X[r][i] - x_bar[r] for r < n, i < m
 __global__ void gl_xp_kernel(const float* __restrict__ X, const float* __restrict__ xbar, int n, int m, int m_pad,
                              int nr, int mp, uint8_t* __restrict__ hi, uint8_t* __restrict__ lo) {
     const int g8 = mp >> 3;
@@ -376,20 +215,6 @@ __global__ void gl_normals_kernel(unsigned long long seed, uint32_t frame, int n
     }
 }
 
-// The Gram from its split-K partials: the upper 128 x 128 tiles were computed, the lower ones
-// are their mirror; the shares are added in order.
-__global__ void gl_gram_reduce_kernel(const float* __restrict__ part, int splits, size_t stride, int m, int ld,
-                                      float* __restrict__ G) {
-    const size_t total = (size_t)m * (m + 1);
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t / (m + 1)), j = (int)(t - (size_t)i * (m + 1));
-        const size_t src = (j >> 7) >= (i >> 7) ? (size_t)i * ld + j : (size_t)j * ld + i;
-        float v = 0.f;
-        for (int z = 0; z < splits; ++z) v += part[z * stride + src];
-        G[(size_t)i * ld + j] = v;
-    }
-}
-
 int grid_for(size_t work, int block) {
     return (int)std::max<size_t>(1, std::min<size_t>((work + block - 1) / block, 152 * 16));
 }
@@ -397,121 +222,17 @@ int grid_for(size_t work, int block) {
 GemmArgs gemm_args(const uint8_t* ah, const uint8_t* al, const uint8_t* bh, const uint8_t* bl, int nkb, int M,
                    int N, int* status) {
     GemmArgs g{};
-    g.a_hi[0] = ah;
-    g.a_lo[0] = al;
-    g.b_hi[0] = bh;
-    g.b_lo[0] = bl;
+    g.a_hi = ah;
+    g.a_lo = al;
+    g.b_hi = bh;
+    g.b_lo = bl;
     g.a_nkb = g.b_nkb = nkb;
     g.split = 1;
     g.m_tiles = (M + 127) / 128;
     g.M = M;
     g.N = N;
-    g.alpha = 1.f;
     g.status = status;
     return g;
-}
-
-// Newton-Schulz step k from buffers a to b, all gated by run[k]: P = Z_a Y_a -> T (max |P - I| into
-// dev[k]), then Y_b = Y_a T and Z_b = T Z_a in one launch, which sets run[k + 1].
-int ns_step(letkf_ctx* c, GlobalState* S, int a, int k, cudaStream_t s) {
-    const int m = c->m, nkb = S->mp >> 6, b = a ^ 1;
-    int rc;
-    GemmArgs g = gemm_args(S->z_hi[a], S->z_lo[a], S->y_hi[a], S->y_lo[a], nkb, m, m, c->d_status);
-    g.mode = GEMM_EPI_TILES;
-    g.o_hi[0] = S->t_hi;
-    g.o_lo[0] = S->t_lo;
-    g.o_nkb = nkb;
-    g.alpha = -0.5f;
-    g.beta = 1.5f;
-    g.dev = S->dev + k;
-    g.b_mn = 1;
-    g.run = S->ctl + CTL_RUN + k;
-    if ((rc = gemm_launch(g, S->pl_one, s))) return rc;
-    g = gemm_args(S->y_hi[a], S->y_lo[a], S->t_hi, S->t_lo, nkb, m, m, c->d_status);
-    g.a_hi[1] = S->t_hi;
-    g.a_lo[1] = S->t_lo;
-    g.b_hi[1] = S->z_hi[a];
-    g.b_lo[1] = S->z_lo[a];
-    g.mode = GEMM_EPI_TILES;
-    g.o_hi[0] = S->y_hi[b];
-    g.o_lo[0] = S->y_lo[b];
-    g.o_hi[1] = S->z_hi[b];
-    g.o_lo[1] = S->z_lo[b];
-    g.o_nkb = nkb;
-    g.b_mn = 1;
-    g.run = S->ctl + CTL_RUN + k;
-    g.next_flag = S->ctl + CTL_RUN + k + 1;
-    g.dev_in = S->dev + k;
-    g.run_tol = NS_TOL;
-    g.z_final = S->ctl + CTL_ZFINAL;
-    g.z_index = b;
-    g.steps = S->ctl + CTL_STEPS;
-    return gemm_launch(g, S->pl_two, s);
-}
-
-// Sets the condition of the conditional node holding the later steps: whether step k runs.
-__global__ void gl_cond_kernel(const int* __restrict__ ctl, int k, cudaGraphConditionalHandle h) {
-    cudaGraphSetConditional(h, ctl[CTL_RUN + k] ? 1u : 0u);
-}
-
-// The iteration as one graph: Y_1 = A_s T_0 (Z_1 = T_0 was written by the builder), steps
-// 1 .. NS_FLAT - 1 in sequence (launches after convergence return at once), then the steps up to
-// NS_MAX - 1 inside one conditional node that runs only when step NS_FLAT is still needed (the
-// first frames' conditioning).  A conditional node whose condition is not set stays off.
-int build_ns_graph(letkf_ctx* c, GlobalState* S) {
-    const int m = c->m, nkb = S->mp >> 6;
-    cudaGraph_t G = nullptr;
-    if (cudaGraphCreate(&G, 0) != cudaSuccess) return LETKF_ECUDA;
-    S->graph = G;
-    cudaGraphConditionalHandle h;
-    if (cudaGraphConditionalHandleCreate(&h, G, 0u, cudaGraphCondAssignDefault) != cudaSuccess) return LETKF_ECUDA;
-    if (cudaStreamBeginCaptureToGraph(S->cap, G, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-        return LETKF_ECUDA;
-    GemmArgs g = gemm_args(S->as_hi, S->as_lo, S->z_hi[1], S->z_lo[1], nkb, m, m, c->d_status);
-    g.mode = GEMM_EPI_TILES;
-    g.o_hi[0] = S->y_hi[1];
-    g.o_lo[0] = S->y_lo[1];
-    g.o_nkb = nkb;
-    g.b_mn = 1;
-    g.run = S->ctl + CTL_RUN + 1;
-    int rc = gemm_launch(g, S->pl_one, S->cap);
-    for (int k = 1; k < NS_FLAT && !rc; ++k) rc = ns_step(c, S, k & 1, k, S->cap);
-    if (!rc) {
-        gl_cond_kernel<<<1, 1, 0, S->cap>>>(S->ctl, NS_FLAT, h);
-        if (cudaGetLastError() != cudaSuccess) rc = LETKF_ECUDA;
-    }
-    cudaGraph_t cap_out = nullptr;
-    const cudaError_t e1 = cudaStreamEndCapture(S->cap, &cap_out);
-    if (rc || e1 != cudaSuccess) return rc ? rc : LETKF_ECUDA;
-    // the node after the last one captured
-    size_t nn = 0;
-    if (cudaGraphGetNodes(G, nullptr, &nn) != cudaSuccess || nn == 0) return LETKF_ECUDA;
-    std::vector<cudaGraphNode_t> nodes(nn);
-    if (cudaGraphGetNodes(G, nodes.data(), &nn) != cudaSuccess) return LETKF_ECUDA;
-    cudaGraphNode_t last = nullptr;
-    for (cudaGraphNode_t nd : nodes) {
-        size_t out = 0;
-        if (cudaGraphNodeGetDependentNodes(nd, nullptr, nullptr, &out) != cudaSuccess) return LETKF_ECUDA;
-        if (out == 0) last = nd;
-    }
-    if (!last) return LETKF_ECUDA;
-    // the parameter struct holds a union of non-trivial members: built in zeroed storage
-    alignas(cudaGraphNodeParams) unsigned char cp_store[sizeof(cudaGraphNodeParams)];
-    std::memset(cp_store, 0, sizeof(cp_store));
-    cudaGraphNodeParams& cp = *reinterpret_cast<cudaGraphNodeParams*>(cp_store);
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = h;
-    cp.conditional.type = cudaGraphCondTypeIf;
-    cp.conditional.size = 1;
-    cudaGraphNode_t node;
-    if (cudaGraphAddNode(&node, G, &last, nullptr, 1, &cp) != cudaSuccess) return LETKF_ECUDA;
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    if (cudaStreamBeginCaptureToGraph(S->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-        return LETKF_ECUDA;
-    for (int k = NS_FLAT; k < NS_MAX && !rc; ++k) rc = ns_step(c, S, k & 1, k, S->cap);
-    const cudaError_t e2 = cudaStreamEndCapture(S->cap, &cap_out);
-    if (rc || e2 != cudaSuccess) return rc ? rc : LETKF_ECUDA;
-    return cudaGraphInstantiate(&S->exec, G, 0) == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
 
 }  // namespace
@@ -525,8 +246,9 @@ size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sm
     size_t b = 2 * tiled_bytes(mr, pk) + gram * (1 + P.split) + 12 * tiled_bytes(mp, mp) + 2 * tiled_bytes(nr, mp) +
                2 * tiled_bytes(mp, mp);
     if (dense) b += 2 * tiled_bytes(rup(n_act, 128), ka) + 2 * tiled_bytes(mp, ka);
-    for (const GemmPlan* p : {&P.gram, &P.one, &P.two, &P.tr, &P.noise}) b += p->bytes();
-    b += (size_t)2 * n_act * 4 + (size_t)4 * m * 4 + 16 + CTL_N * 4 + NS_MAX * 4 + (size_t)n_subv * 16;
+    for (const GemmPlan* p : {&P.gram, &P.tr, &P.noise}) b += p->bytes();
+    b += (size_t)2 * n_act * 4 + (size_t)4 * m * 4 + (size_t)root_parts(m) * 4 + sizeof(RootStats) + ROOT_STEPS * 4 + 8 +
+         (size_t)n_subv * 16;
     return b;
 }
 
@@ -554,8 +276,7 @@ int global_prepare(letkf_ctx* c) {
     S->gram_split = P.split;
     ok = ok && get((size_t)m * S->ldg * 4, (void**)&S->G) &&
          get((size_t)P.split * m * S->ldg * 4, (void**)&S->Gpart);
-    for (auto& q : {std::make_pair(&P.gram, &S->pl_gram), std::make_pair(&P.one, &S->pl_one),
-                    std::make_pair(&P.two, &S->pl_two), std::make_pair(&P.tr, &S->pl_tr),
+    for (auto& q : {std::make_pair(&P.gram, &S->pl_gram), std::make_pair(&P.tr, &S->pl_tr),
                     std::make_pair(&P.noise, &S->pl_noise)}) {
         GemmPlan& p = *q.first;
         if (!p.ncl) continue;
@@ -579,10 +300,10 @@ int global_prepare(letkf_ctx* c) {
         ok = ok && get(tl, (void**)&S->l_hi) && get(tl, (void**)&S->l_lo) && get(tx, (void**)&S->xi_hi) &&
              get(tx, (void**)&S->xi_lo);
     }
-    ok = ok && get((size_t)c->n * 4, (void**)&S->xbar) && get((size_t)m * 4, (void**)&S->rowsq) &&
+    ok = ok && get((size_t)c->n * 4, (void**)&S->xbar) && get((size_t)root_parts(m) * 4, (void**)&S->sq) &&
          get((size_t)m * 4, (void**)&S->wbar) && get((size_t)m * 4, (void**)&S->u) && get((size_t)m * 4, (void**)&S->r) &&
-         get(16, (void**)&S->scal) && get(CTL_N * 4, (void**)&S->ctl) && get(NS_MAX * 4, (void**)&S->dev) &&
-         get((size_t)c->n_subv * 16, (void**)&S->corner);
+         get((size_t)m * 4, (void**)&S->b) && get(sizeof(RootStats), (void**)&S->stats) &&
+         get(ROOT_STEPS * 4, (void**)&S->dev) && get(8, (void**)&S->bar) && get((size_t)c->n_subv * 16, (void**)&S->corner);
     if (!ok) return LETKF_ENOMEM;
     // corner actuators of every valid subaperture: (r,c) (r,c+1) (r+1,c) (r+1,c+1)
     const HostModel& h = c->host;
@@ -596,7 +317,7 @@ int global_prepare(letkf_ctx* c) {
     if (cudaMemcpy(S->corner, cor.data(), cor.size() * sizeof(int4), cudaMemcpyHostToDevice) != cudaSuccess)
         return LETKF_ECUDA;
     int rc = gemm_prepare();
-    if (rc) return rc;
+    if (rc || (rc = root_prepare())) return rc;
     // tiles of the process-noise factor, once
     if (dense && (rc = to_tiles(static_cast<const float*>(c->Lq), c->n_act, c->n_act, c->n_act, S->l_hi, S->l_lo, 1,
                                 c->stream)))
@@ -607,18 +328,12 @@ int global_prepare(letkf_ctx* c) {
                     (void*)S->y_lo[0], (void*)S->y_hi[1], (void*)S->y_lo[1], (void*)S->z_hi[0], (void*)S->z_lo[0],
                     (void*)S->z_hi[1], (void*)S->z_lo[1], (void*)S->wt_hi, (void*)S->wt_lo})
         if (cudaMemsetAsync(p, 0, tsq, c->stream) != cudaSuccess) return LETKF_ECUDA;
-    // the Newton-Schulz steps as one graph with a device-side loop
-    if (cudaStreamCreateWithFlags(&S->cap, cudaStreamNonBlocking) != cudaSuccess) return LETKF_ECUDA;
-    if ((rc = build_ns_graph(c, S))) return rc;
     return LETKF_OK;
 }
 
 void global_free(letkf_ctx* c) {
     GlobalState* S = c->gstate;
     if (!S) return;
-    if (S->exec) cudaGraphExecDestroy(S->exec);
-    if (S->graph) cudaGraphDestroy(S->graph);
-    if (S->cap) cudaStreamDestroy(S->cap);
     for (void* p : S->allocs) cudaFree(p);
     delete S;
     c->gstate = nullptr;
@@ -636,7 +351,7 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     const int m = c->m, n = c->n;
     const float cm = (float)(m - 1);
     prof_begin(c, STAGE_OBS);
-    gl_mean_kernel<<<grid_for((size_t)n * 32, 256), 256, 0, st>>>(X, n, m, c->m_pad, S->xbar);
+    gl_mean_kernel<<<grid_for((size_t)n * 32, 256), 256, 0, st>>>(X, n, m, c->m_pad, S->xbar, S->bar);
     gl_slopes_kernel<<<grid_for((size_t)S->mr * (S->pk >> 3), 256), 256, 0, st>>>(
         X, S->xbar, static_cast<const float*>(yv), S->corner, c->n_subv, c->obs_block == 1 ? c->n_act : 0, m, c->m_pad,
         S->mr, S->pk, (float)(1.0 / c->sigma), S->st_hi, S->st_lo);
@@ -651,32 +366,43 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     g.ldc = S->ldg;
     g.c_split_stride = (size_t)m * S->ldg;
     if ((rc = gemm_launch(g, S->pl_gram, st))) return rc;
-    gl_gram_reduce_kernel<<<grid_for((size_t)m * (m + 1), 256), 256, 0, st>>>(S->Gpart, S->gram_split,
-                                                                              (size_t)m * S->ldg, m, S->ldg, S->G);
     prof_end(c);
-    // inverse square root
+    // Gram, inverse square root, weights
     prof_begin(c, STAGE_EIG);
-    gl_rowsq_kernel<<<grid_for((size_t)m * 32, 256), 256, 0, st>>>(S->G, S->ldg, m, S->rowsq);
-    gl_build_kernel<<<grid_for((size_t)S->mp * (S->mp >> 3), 256), 256, 0, st>>>(
-        S->G, S->ldg, m, S->mp, S->rowsq, cm, S->as_hi, S->as_lo, S->z_hi[1], S->z_lo[1], S->scal, S->ctl, S->dev,
-        c->d_frame_bad);
-    if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
-    if (cudaGraphLaunch(S->exec, st) != cudaSuccess) return LETKF_ECUDA;
-    // mean weights, refined once: w = Z^2 b/(cs); w += Z^2 (b - (cI + G) w)/(cs)
-    const int nkb = S->mp >> 6, gv = grid_for((size_t)m * 32, 256);
-    gl_bcol_kernel<<<grid_for(m, 256), 256, 0, st>>>(S->G, S->ldg, m, S->r);
-    for (int pass = 0; pass < 2; ++pass) {
-        gl_gemv_kernel<<<gv, 256, 0, st>>>(S->z_hi[0], S->z_lo[0], S->z_hi[1], S->z_lo[1], S->ctl + CTL_ZFINAL, nkb, m, S->r,
-                                           S->scal, cm, 0, 0, S->u);
-        gl_gemv_kernel<<<gv, 256, 0, st>>>(S->z_hi[0], S->z_lo[0], S->z_hi[1], S->z_lo[1], S->ctl + CTL_ZFINAL, nkb, m, S->u,
-                                           S->scal, cm, 1, pass, S->wbar);
-        if (pass == 0) gl_resid_kernel<<<gv, 256, 0, st>>>(S->G, S->ldg, m, S->wbar, cm, S->r);
+    RootArgs ra;
+    std::memset(&ra, 0, sizeof(ra));
+    ra.part = S->Gpart;
+    ra.stride = (size_t)m * S->ldg;
+    ra.splits = S->gram_split;
+    ra.m = m;
+    ra.mp = S->mp;
+    ra.ldg = S->ldg;
+    ra.c = cm;
+    ra.G = S->G;
+    ra.as_hi = S->as_hi;
+    ra.as_lo = S->as_lo;
+    ra.t_hi = S->t_hi;
+    ra.t_lo = S->t_lo;
+    for (int q = 0; q < 2; ++q) {
+        ra.y_hi[q] = S->y_hi[q];
+        ra.y_lo[q] = S->y_lo[q];
+        ra.z_hi[q] = S->z_hi[q];
+        ra.z_lo[q] = S->z_lo[q];
     }
-    gl_wt_kernel<<<grid_for((size_t)S->mp * (S->mp >> 3), 256), 256, 0, st>>>(
-        S->z_hi[0], S->z_lo[0], S->z_hi[1], S->z_lo[1], S->ctl + CTL_ZFINAL, m, S->mp, S->wbar, S->scal,
-        S->ctl + CTL_RUN + NS_MAX, S->wt_hi, S->wt_lo, c->d_status);
+    ra.wt_hi = S->wt_hi;
+    ra.wt_lo = S->wt_lo;
+    ra.sq = S->sq;
+    ra.b = S->b;
+    ra.r = S->r;
+    ra.u = S->u;
+    ra.wbar = S->wbar;
+    ra.dev = S->dev;
+    ra.bar = S->bar;
+    ra.stats = S->stats;
+    ra.frame_bad = c->d_frame_bad;
+    ra.status = c->d_status;
+    if ((rc = root_launch(ra, c->sms, st))) return rc;
     prof_end(c);
-    if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     // transform X_a = x_bar + X' W
     prof_begin(c, STAGE_TRANSFORM);
     gl_xp_kernel<<<grid_for((size_t)S->nr * (S->mp >> 3), 256), 256, 0, st>>>(X, S->xbar, n, m, c->m_pad, S->nr, S->mp,
@@ -719,13 +445,11 @@ extern "C" int letkf_global_stats(letkf_ctx* c, int* ns_steps, double* s_bound) 
     if (!c || !ns_steps || !s_bound) return LETKF_EINVAL;
     GlobalState* S = c->gstate;
     if (!S) return LETKF_ESTATE;
-    int zf = 0;
-    float sv = 0.f;
+    RootStats st;
     if (cudaSetDevice(c->device) != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess ||
-        cudaMemcpy(&zf, S->ctl + CTL_STEPS, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(&sv, S->scal, sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
+        cudaMemcpy(&st, S->stats, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess)
         return LETKF_ECUDA;
-    *ns_steps = zf;
-    *s_bound = sv;
+    *ns_steps = st.steps;
+    *s_bound = st.s;
     return LETKF_OK;
 }

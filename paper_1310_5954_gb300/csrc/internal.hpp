@@ -202,7 +202,7 @@ int global_analyze(letkf_ctx* c, const void* y, double sigma);
 int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis);
 
 // gemm.cu: tiled tensor-core GEMM, C = A B^T with tiled BF16 operands (128 x 64 tiles)
-enum GemmEpilogue { GEMM_EPI_F32 = 0, GEMM_EPI_TILES = 1, GEMM_EPI_ADD_ROW = 2 };
+enum GemmEpilogue { GEMM_EPI_F32 = 0, GEMM_EPI_ADD_ROW = 1 };
 // How the tiles of a product are dealt to the clusters of one launch.  A piece is `width` columns (64, 128
 // or 256) of cm row tiles (one per CTA of the cluster), over K steps [kb0, kb1); cluster q does
 // items[start[q]] .. items[start[q + 1] - 1].
@@ -213,14 +213,13 @@ struct GemmShape {
     int lower = 0;                      // A is lower triangular: row tile r needs K steps < 2 (r + 1)
     int upper = 0;                      // only pieces that reach the diagonal or lie right of it
     int ksplit = 1;                     // shares of the K steps (partial products)
-    int batch = 1;                      // products of this shape in the launch
 };
 struct GemmPlan {
     int bn = 64, cm = 1, ncl = 0;
     long long cycles = 0;               // the model's time of the busiest cluster
     std::vector<int> start;             // ncl + 1
     std::vector<int4> items;            // row tile group, first column, kb0 | kb1 << 16,
-                                        // width | share << 10 | product << 28
+                                        // width | share << 10
     int* d_start = nullptr;
     int4* d_items = nullptr;
     size_t bytes() const { return items.size() * sizeof(int4) + start.size() * sizeof(int); }
@@ -228,13 +227,9 @@ struct GemmPlan {
 GemmPlan gemm_plan(const GemmShape& s, int sms);
 
 struct GemmArgs {
-    // product 0 and, where the plan has two, product 1 (operands and tiled output only)
-    const uint8_t* a_hi[2];
-    const uint8_t* a_lo[2];     // null: single BF16
-    const uint8_t* b_hi[2];
-    const uint8_t* b_lo[2];
+    const uint8_t *a_hi, *a_lo, *b_hi, *b_lo;
     int a_nkb, b_nkb;           // column tiles per row tile of A and B
-    int split;                  // 1: hi hi + hi lo + lo hi
+    int split;                  // 1: hi hi + hi lo + lo hi; 0: single BF16, a_lo and b_lo unused
     int m_tiles;                // row tiles of A there are
     int bn;                     // the plan: its widest piece, and the pieces
     const int* start;
@@ -244,27 +239,39 @@ struct GemmArgs {
                                 //    MN-major: C = A M (width 64 only); 0: C = A B^T
     int M, N;                   // valid rows / columns of C
     int mode;                   // GemmEpilogue
-    float* c;                   // F32 / ADD_ROW: C[row * ldc + col]
+    float* c;                   // C[row * ldc + col]
     int ldc;
-    float alpha;
-    uint8_t* o_hi[2];           // TILES: alpha C + beta I as a tiled operand with o_nkb column tiles
-    uint8_t* o_lo[2];
-    int o_nkb;
-    float beta;
-    unsigned int* dev;          // TILES: max |C - I| over valid entries (float bits, atomicMax)
     const float* add;           // ADD_ROW: per-row term
-    const int* run;             // non-null: the launch does nothing when *run == 0
-    int* next_flag;             // non-null: CTA 0 sets *next_flag = run && (*dev_in >= run_tol),
-    unsigned int* dev_in;       //   and, when running, resets *dev_in, sets *z_final = z_index
-    float run_tol;              //   and counts one step in *steps
-    int* z_final;
-    int z_index;
-    int* steps;
     int* status;
 };
 size_t tiled_bytes(int rows, int cols);
 int gemm_prepare();
 int gemm_launch(const GemmArgs& g, const GemmPlan& p, cudaStream_t stream);
+
+// root.cu: Gram, matrix iteration, mean weights and W^T of the global analysis in one cooperative kernel
+constexpr int ROOT_STEPS = 24;          // limit of Newton-Schulz steps
+struct RootStats {
+    float s;                            // scaling bound
+    int steps;                          // Newton-Schulz steps, the product-free first one included
+};
+struct RootArgs {
+    const float* part;                  // partial Grams (upper tiles), shares `stride` floats apart
+    size_t stride;
+    int splits, m, mp, ldg;             // mp: m rounded to 128; leading dimension of the Grams
+    float c;                            // m - 1
+    float* G;                           // m x ldg
+    uint8_t *as_hi, *as_lo, *t_hi, *t_lo, *y_hi[2], *y_lo[2], *z_hi[2], *z_lo[2];   // mp x mp tiles
+    uint8_t *wt_hi, *wt_lo;             // mp x mp slices
+    float *sq, *b, *r, *u, *wbar;       // parts of |G|_F^2 (root_parts(m)); vectors of m
+    unsigned* dev;                      // [ROOT_STEPS]: max |P - I| of each step
+    unsigned* bar;                      // grid barrier: arrivals and the gave-up flag, zero before the launch
+    RootStats* stats;
+    const int* frame_bad;
+    int* status;
+};
+inline int root_parts(int m) { return ((m + 63) / 64) * ((m + 63) / 64 + 1) / 2; }
+int root_prepare();
+int root_launch(const RootArgs& a, int sms, cudaStream_t stream);
 int to_tiles(const float* src, int R, int K, int ld, void* hi, void* lo, int sliced, cudaStream_t stream);
 
 // piston.cu: differential pistons between domains
