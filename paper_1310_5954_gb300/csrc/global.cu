@@ -2,8 +2,8 @@
 // tensor-core GEMM of gemm.cu.  With S = Y'/sigma (p x m) and d = (y - y_bar)/sigma:
 //
 //   [S d]^T [S d]      one product (K = p) gives G = S^T S, b = S^T d                 (Gram)
-//   A_s = (I + G/c)/s  c = m - 1, s = 1 + ||G||_F / c >= its largest eigenvalue
-//   Z = A_s^(-1/2)     coupled Newton-Schulz: P = Z Y, T = (3I - P)/2, Y <- Y T, Z <- T Z,
+//   A_s = (I + G/c)/s  c = m - 1, s = (1 + ||G||_F / c) / 2.5; eigenvalues in (0, 2.5]
+//   Z = A_s^(-1/2)     coupled Newton-Schulz: P = Z Y, T = a I - b P, Y <- Y T, Z <- T Z,
 //                      from Y = A_s, Z = I (first step without products: P = A_s, Z = T)
 //   T_a = Z / sqrt(s) = (I + G/c)^(-1/2),   w_bar = Z^2 b / (c s), refined once against the
 //                      FP32 operator (c I + G)

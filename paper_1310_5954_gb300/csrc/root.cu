@@ -1,14 +1,15 @@
 // From the Gram's partial products to the weights of a global analysis, in one cooperative kernel: the Gram
-// G and the bound s, A_s = (I + G/c)/s, the Newton-Schulz iteration Z -> A_s^{-1/2}, the mean weights (refined
-// once) and the operand W^T = (w_bar 1^T + Z / sqrt(s))^T of the transform.
+// G and the bound s, A_s = (I + G/c)/s_ns, the Newton-Schulz iteration Z -> A_s^{-1/2}, the mean weights
+// (refined once) and the operand W^T = (w_bar 1^T + Z / sqrt(s_ns))^T of the transform.
 //
-// The iteration is a chain of m x m products (P = Z Y; Y T and T Z, T = (3 I - P) / 2), each a few
+// The iteration is a chain of m x m products (P = Z Y; Y T and T Z, T = a I - b P), each a few
 // microseconds of work even at m = 1024.  As a graph of launches per product, with the passes before and
 // behind it as kernels of their own, most of the time went into starting them, 12 steps' worth of which
 // found the iteration already finished.  Here the CTAs, one per SM, go from phase to phase through a grid
 // barrier (1.9 us), the ring of operand stages and the tensor-memory accumulators stay set up, the decision
-// to stop needs no launch, and the last step leaves out Y, which only a next one would read.  Seven steps,
-// with what is before and behind them: 160 -> 107 us at m = 197, 298 -> 219 us at m = 1024.
+// to stop needs no launch, and the last step leaves out Y, which only a next one would read.  With what
+// is before and behind it: 160 -> 86 us at m = 197, 298 -> 173 us at m = 1024 (107 and 219 us with seven
+// plain steps; five are taken, see NsStep).
 //
 // A product is dealt in tiles of 128 x 64, B read MN-major (see gemm.cu): at m = 1024 that is 128 tiles for
 // P (9 us: 1.4 until the first operands are there, 6.2 of products at 60 cycles each, 1.2 to read out) and
@@ -39,6 +40,41 @@ constexpr float NS_TOL = 1e-2f;   // the last update then lands at ~0.75 NS_TOL^
 constexpr int RT = 320;           // eight epilogue warps, a producer warp, an MMA warp
 constexpr int RW = RT / 32;
 constexpr int ROOT_SMEM = 1024 + GemmStage<true>::RING;
+
+// The coefficients of an iteration step, P = Z Y, T = a I - b P, Y <- Y T, Z <- T Z.  With eigenvalues x^2 of
+// P a step maps x -> x (a - b x^2).  The plain step (a = 3/2, b = 1/2) raises small x by 1.5 only;
+// a = 3 rho / 2, b = rho^3 / 2 raises them by 1.5 rho and keeps [l, 1] in [l', 1], best with
+// rho^2 = 3 / (1 + l + l^2), where l and 1 land on the same l' (J. Chen and E. Chow, "A stable scaling of
+// Newton-Schulz for improving the sign function computation of a Hermitian matrix", 2014).  l is known:
+// (I + G/c)/s has no eigenvalue below 1/s, and has that one (the anomalies of a row add up to zero).  rho^2
+// stays below NS_SCALE, so that what is 1 up to rounding lands at NS_EDGE or above; the first step is a plain
+// one on A_s scaled up by NS_SCALE, which is the same.  From l = NS_PLAIN on the steps are plain, and only
+// those may be taken for the last ones (one of them brings 1 - P from 0.12 to 0.01).
+//
+// Plain steps needed 7 steps at s = 25 (m = 197) and s = 39 (m = 1024), this 5, and the analysis's
+// error against 64 bits, dominated by the rounding of the iterates, is no larger (16 sizes m = 100 .. 700 on
+// 32 x 32 and 40 x 40, frames 1 to 3 of a cold start: anomalies 1.1e-4 against 1.5e-4, mean 4.8e-5 against
+// 4.8e-5, geometric means).  Below s = NS_SCALED_FROM the largest eigenvalue is usually so far below the
+// bound that plain steps are as quick (s = 15: 6 against 5 steps, 10: 5 and 5, 6: 4 and 5).
+constexpr float NS_SCALE = 2.5f, NS_EDGE = 0.395f, NS_PLAIN = 0.94f;   // NS_EDGE: sqrt(2.5) (3 - 2.5) / 2
+constexpr float NS_SCALED_FROM = 16.f;
+struct NsStep {
+    float a, b;
+    bool plain;
+};
+// The bound l after the first step; s_ns = s / NS_SCALE.
+__device__ __forceinline__ float ns_first(float s_ns) {
+    const float l2 = 1.f / s_ns;
+    return fminf(0.5f * sqrtf(l2) * (3.f - l2), NS_EDGE);
+}
+// The next step, and the bound behind it.
+__device__ __forceinline__ NsStep ns_next(float& l) {
+    if (!(l < NS_PLAIN)) return {1.5f, 0.5f, true};
+    const float r2 = fminf(NS_SCALE, 3.f / (1.f + l + l * l)), r = sqrtf(r2);
+    const NsStep t = {1.5f * r, 0.5f * r * r2, false};
+    l = fminf(l * (t.a - t.b * l * l), t.a - t.b);
+    return t;
+}
 
 struct Tiles {
     uint8_t *hi, *lo;
@@ -286,7 +322,7 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
     unsigned target = 0;
     int chunks = 0, acc = 0, steps = 1, zf = 1;
     bool run = *a.frame_bad == 0, ok = true;
-    float s = 1.f;
+    float s = 1.f, sn = 1.f;                   // the bound, and the scale of A_s
 
     // G = sum of the shares, in order: the blocks of 64 x 64 on and above the diagonal, and their mirror;
     // sq = a block's part of the squared Frobenius norm; b = column m
@@ -367,11 +403,12 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         sum = 0.f;
         for (int w = 0; w < RW; ++w) sum += cta.red[w];
         s = 1.f + sqrtf(sum) / a.c;
+        sn = s / NS_SCALE;
     }
 
-    // A_s = (I + G/c)/s and the first step's Z_1 = T_0 = (3I - A_s)/2
+    // A_s = (I + G/c)/s_ns and the first step's Z_1 = T_0 = (3I - A_s)/2
     if (ok) {
-        const float inv = 1.f / s, invc = 1.f / (a.c * s);
+        const float inv = 1.f / sn, invc = 1.f / (a.c * sn);
         for (int u = blockIdx.x * RT + tid; u < units; u += gridDim.x * RT) {
             int i, j0;
             unit_at(u, nkb, i, j0);
@@ -404,13 +441,15 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         products(ring, &cta, chunks, acc, &p, 1, m, mp, 1.f, 0.f, nullptr, a.status);
         ok = grid_sync(a.bar, target, &cta, a.status);
     }
+    float l = s >= NS_SCALED_FROM ? ns_first(sn) : 1.f;
     for (int k = 1; ok && run && k < NS_MAX; ++k) {
+        const NsStep ns = ns_next(l);
         const int from = k & 1, to = from ^ 1;
         const Product p{z[from], y[from], tt};
-        products(ring, &cta, chunks, acc, &p, 1, m, mp, -0.5f, 1.5f, a.dev + k, a.status);
+        products(ring, &cta, chunks, acc, &p, 1, m, mp, -ns.b, ns.a, a.dev + k, a.status);
         ok = grid_sync(a.bar, target, &cta, a.status);
         if (!ok) break;
-        run = __uint_as_float(__ldcg(a.dev + k)) >= NS_TOL;     // whether a step follows, which needs Y
+        run = !ns.plain || __uint_as_float(__ldcg(a.dev + k)) >= NS_TOL;     // whether a step follows, which needs Y
         const Product two[2] = {{tt, z[from], z[to]}, {y[from], tt, y[to]}};
         products(ring, &cta, chunks, acc, two, run ? 2 : 1, m, mp, 1.f, 0.f, nullptr, a.status);
         ok = grid_sync(a.bar, target, &cta, a.status);
@@ -418,8 +457,8 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         ++steps;
     }
 
-    // mean weights, refined once: w = Z^2 b / (c s); w += Z^2 (b - (c I + G) w) / (c s)
-    const float scale = 1.f / (a.c * s);
+    // mean weights, refined once: w = Z^2 b / (c s_ns); w += Z^2 (b - (c I + G) w) / (c s_ns)
+    const float scale = 1.f / (a.c * sn);
     float* sv = reinterpret_cast<float*>(smem);
     for (int pass = 0; ok && pass < 2; ++pass) {
         take(pass ? a.r : a.b, m, sv);
@@ -453,9 +492,9 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         ok = grid_sync(a.bar, target, &cta, a.status);
     }
 
-    // W^T: element (j, k) = w_bar[k] + Z[j][k] / sqrt(s) (W = w_bar 1^T + T_a; T_a symmetric)
+    // W^T: element (j, k) = w_bar[k] + Z[j][k] / sqrt(s_ns) (W = w_bar 1^T + T_a; T_a symmetric)
     if (ok) {
-        const float rs = rsqrtf(s);
+        const float rs = rsqrtf(sn);
         take(a.wbar, m, sv);
         for (int u = blockIdx.x * RT + tid; u < units; u += gridDim.x * RT) {
             int j, k0;
