@@ -28,6 +28,7 @@
 
 #include "../../include/letkf.h"
 #include "common.cuh"
+#include "gemm_ring.cuh"
 #include "internal.hpp"
 #include "umma.cuh"
 
@@ -55,9 +56,11 @@ struct GlobalState {
 
 namespace {
 
-constexpr int TILE_B = 128 * 64 * 2;
 
 int rup(int v, int a) { return (v + a - 1) / a * a; }
+
+// Columns of the slopes' operand: the x and y slopes of eight subapertures to a slice (see gl_slopes_kernel).
+int slope_cols(int n_subv) { return rup(2 * rup(n_subv, 8), 64); }
 
 // Row tiles per cluster of a wide product: they share the 256 columns of B.
 int cluster_rows(int row_tiles) { return row_tiles >= 2 ? 2 : 1; }
@@ -74,7 +77,7 @@ Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
     GemmShape g;
     g.m_tiles = mt;             // row m of the Gram is its column m
     g.N = m + 1;
-    g.nkb = rup(2 * n_subv, 64) / 64;
+    g.nkb = slope_cols(n_subv) / 64;
     g.bn = 256;
     g.cm = cluster_rows(mt);
     g.upper = 1;
@@ -104,87 +107,121 @@ Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
     return P;
 }
 
-__device__ __forceinline__ void split2(float x, __nv_bfloat16& h, __nv_bfloat16& l) {
-    h = __float2bfloat16_rn(x);
-    l = __float2bfloat16_rn(x - __bfloat162float(h));
-}
-
+// Eight consecutive columns of a row as hi and lo, one 16-byte store each.
 __device__ __forceinline__ void store8(uint8_t* hi, uint8_t* lo, size_t off, const float (&v)[8]) {
     __align__(16) __nv_bfloat16 h[8], l[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) split2(v[q], h[q], l[q]);
+    for (int q = 0; q < 8; ++q) split_bf16(v[q], h[q], l[q]);
     *reinterpret_cast<uint4*>(hi + off) = *reinterpret_cast<const uint4*>(h);
     *reinterpret_cast<uint4*>(lo + off) = *reinterpret_cast<const uint4*>(l);
 }
 
-// member means of every state row (one warp per row); resets the iteration's grid barrier
-__global__ void gl_mean_kernel(const float* __restrict__ X, int n, int m, int m_pad, float* __restrict__ xbar,
-                               unsigned* __restrict__ bar) {
+// Member means of the state rows and the X' slices, element (r, i) = X[r][i] - x_bar[r] for r < n, i < m
+// and zero beyond; resets the iteration's grid barrier.  Bound by HBM: X is read once, from HBM for the
+// means, one warp per row, and again, now from L1, by threads that take the eight rows of a core matrix side
+// by side, so that the slices are written in pieces of 256 bytes.  (Two kernels, the second with one thread
+// per row piece and 16-byte stores 2 KB apart, took 11 + 26 us at n = 9666, m = 1024; this 19 us.)
+__global__ void __launch_bounds__(256) gl_center_kernel(const float* __restrict__ X, int n, int m, int m_pad, int mp,
+                                                        float* __restrict__ xbar, uint8_t* __restrict__ hi,
+                                                        uint8_t* __restrict__ lo, unsigned* __restrict__ bar) {
+    __shared__ float mu_sh[8];
     if (blockIdx.x == 0 && threadIdx.x < 2) bar[threadIdx.x] = 0u;
-    const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
+    const int r0 = blockIdx.x * 8, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    {
+        const int r = r0 + warp;
         float s = 0.f;
-        for (int i = lane; i < m; i += 32) s += X[(size_t)r * m_pad + i];
-        s = warp_sum(s);
-        if (lane == 0) xbar[r] = s / (float)m;
-    }
-}
-
-// [S d]^T as tiles: row i < m is member i's observed-anomaly slopes / sigma, row m the innovation
-// (y - D x_bar) / sigma, the rest zero; columns are the slopes (x then y), padded with zeros.
-// One thread per (row, 8 consecutive columns), rows fastest.
-__global__ void gl_slopes_kernel(const float* __restrict__ X, const float* __restrict__ xbar,
-                                 const float* __restrict__ y, const int4* __restrict__ corner, int n_subv,
-                                 int row_obs, int m, int m_pad, int mr, int pk, float inv_sigma,
-                                 uint8_t* __restrict__ hi, uint8_t* __restrict__ lo) {
-    const size_t total = (size_t)mr * (pk >> 3);
-    const int p = 2 * n_subv;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t % mr), c0 = (int)(t / mr) * 8;
-        float v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int col = c0 + q;
-            v[q] = 0.f;
-            if (i <= m && col < p) {
-                const bool is_y = col >= n_subv;
-                const int4 a = corner[is_y ? col - n_subv : col];
-                float a00, a01, a10, a11;
-                if (i < m) {
-                    a00 = X[(size_t)(row_obs + a.x) * m_pad + i] - xbar[row_obs + a.x];
-                    a01 = X[(size_t)(row_obs + a.y) * m_pad + i] - xbar[row_obs + a.y];
-                    a10 = X[(size_t)(row_obs + a.z) * m_pad + i] - xbar[row_obs + a.z];
-                    a11 = X[(size_t)(row_obs + a.w) * m_pad + i] - xbar[row_obs + a.w];
-                } else {
-                    a00 = xbar[row_obs + a.x];
-                    a01 = xbar[row_obs + a.y];
-                    a10 = xbar[row_obs + a.z];
-                    a11 = xbar[row_obs + a.w];
-                }
-                const float s = is_y ? 0.5f * ((a10 + a11) - (a00 + a01)) : 0.5f * ((a01 + a11) - (a00 + a10));
-                v[q] = (i < m ? s : y[col] - s) * inv_sigma;
+        if (r < n) {
+            const float* x = X + (size_t)r * m_pad;
+            const int m4 = m & ~3;
+#pragma unroll 8
+            for (int i = 4 * lane; i < m4; i += 128) {
+                const float4 v = *reinterpret_cast<const float4*>(x + i);
+                s += (v.x + v.y) + (v.z + v.w);
             }
+            if (lane < m - m4) s += x[m4 + lane];
         }
-        store8(hi, lo, umma::slice_offset(i, c0, pk >> 6), v);
+        s = warp_sum(s);
+        if (lane == 0) {
+            mu_sh[warp] = s / (float)m;
+            if (r < n) xbar[r] = s / (float)m;
+        }
     }
-}
-
-// X' slices: element (r, i) = X[r][i] - x_bar[r] for r < n, i < m
-__global__ void gl_xp_kernel(const float* __restrict__ X, const float* __restrict__ xbar, int n, int m, int m_pad,
-                             int nr, int mp, uint8_t* __restrict__ hi, uint8_t* __restrict__ lo) {
-    const int g8 = mp >> 3;
-    const size_t total = (size_t)nr * g8;
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(t / g8), i0 = (int)(t - (size_t)r * g8) * 8;
+    __syncthreads();
+    const int r = r0 + (threadIdx.x & 7);
+    const float mu = mu_sh[threadIdx.x & 7];
+    const float* x = X + (size_t)r * m_pad;
+    for (int i0 = 8 * (threadIdx.x >> 3); i0 < mp; i0 += 256) {
         float v[8];
-        const float mu = r < n ? xbar[r] : 0.f;
+        if (r < n && i0 + 8 <= m) {
+            const float4 a = *reinterpret_cast<const float4*>(x + i0), b = *reinterpret_cast<const float4*>(x + i0 + 4);
+            v[0] = a.x - mu;
+            v[1] = a.y - mu;
+            v[2] = a.z - mu;
+            v[3] = a.w - mu;
+            v[4] = b.x - mu;
+            v[5] = b.y - mu;
+            v[6] = b.z - mu;
+            v[7] = b.w - mu;
+        } else {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int i = i0 + q;
-            v[q] = (r < n && i < m) ? X[(size_t)r * m_pad + i] - mu : 0.f;
+            for (int q = 0; q < 8; ++q) v[q] = (r < n && i0 + q < m) ? x[i0 + q] - mu : 0.f;
         }
         store8(hi, lo, umma::slice_offset(r, i0, mp >> 6), v);
+    }
+}
+
+// [S d]^T as slices: row i < m is member i's observed-anomaly slopes / sigma, row m the innovation
+// (y - D x_bar) / sigma, the rest zero.  The order of the slopes is free (the Gram sums over them): columns
+// 16 g .. 16 g + 7 are the x slopes of subapertures 8 g .. 8 g + 7, the next eight their y slopes, padded
+// with zeros, so that a thread (one row, one group) takes both from the same corners, and a corner that two
+// neighbouring subapertures share once: 16 to 18 loads for 16 slopes, where one thread per 8 slopes of one
+// kind loaded 32 (34 us at n_subv = 4632, m = 1024; this 22).
+__global__ void __launch_bounds__(256) gl_slopes_kernel(const float* __restrict__ X, const float* __restrict__ xbar,
+                                                        const float* __restrict__ y, const int4* __restrict__ corner,
+                                                        int n_subv, int row_obs, int m, int m_pad, int mr, int pk,
+                                                        float inv_sigma, uint8_t* __restrict__ hi,
+                                                        uint8_t* __restrict__ lo) {
+    const size_t total = (size_t)mr * (pk >> 4);
+    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
+        const int i = (int)(t % mr), g = (int)(t / mr), k0 = 8 * g;
+        float sx[8], sy[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sx[q] = sy[q] = 0.f;
+        if (i <= m && k0 < n_subv) {
+            const float* x = i < m ? X + (size_t)row_obs * m_pad + i : nullptr;
+            auto at = [&](int act) {
+                const float b = xbar[row_obs + act];
+                return i < m ? x[(size_t)act * m_pad] - b : b;
+            };
+            int4 c[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) c[q] = corner[min(k0 + q, n_subv - 1)];
+            float r0[8], r1[8];               // the right-hand corners
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                r0[q] = at(c[q].y);
+                r1[q] = at(c[q].w);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                float l0, l1;                 // the left-hand ones: usually the neighbour's right
+                if (q > 0 && c[q].x == c[q > 0 ? q - 1 : 0].y && c[q].z == c[q > 0 ? q - 1 : 0].w) {
+                    l0 = r0[q > 0 ? q - 1 : 0];
+                    l1 = r1[q > 0 ? q - 1 : 0];
+                } else {
+                    l0 = at(c[q].x);
+                    l1 = at(c[q].z);
+                }
+                const float dx = 0.5f * ((r0[q] + r1[q]) - (l0 + l1)), dy = 0.5f * ((l1 + r1[q]) - (l0 + r0[q]));
+                if (k0 + q < n_subv) {
+                    sx[q] = (i < m ? dx : y[k0 + q] - dx) * inv_sigma;
+                    sy[q] = (i < m ? dy : y[n_subv + k0 + q] - dy) * inv_sigma;
+                }
+            }
+        }
+        const size_t off = umma::slice_offset(i, 16 * g, pk >> 6);
+        store8(hi, lo, off, sx);
+        store8(hi, lo, off + 128, sy);
     }
 }
 
@@ -196,22 +233,23 @@ __global__ void gl_reject_kernel(const float* __restrict__ X, float* __restrict_
         Xo[t] = X[t];
 }
 
-// xi^T tiles for the noise product: element (member i, actuator j) = Philox normal (stream 1,
-// frame, counter (j / 4, i)), the same draws as the plain forecast's white-noise path.
-__global__ void gl_normals_kernel(unsigned long long seed, uint32_t frame, int n_act, int m, int mp, int ka,
-                                  uint8_t* __restrict__ hi, uint8_t* __restrict__ lo) {
-    const int nq = ka >> 2;
-    const size_t total = (size_t)mp * nq;
+// xi^T slices for the noise product: element (member i, actuator j) = Philox normal (stream 1,
+// frame, counter (j / 4, i)), the same draws as the plain forecast's white-noise path.  One thread per
+// member and eight actuators: a warp writes pieces of 128 bytes.
+__global__ void __launch_bounds__(256) gl_normals_kernel(unsigned long long seed, uint32_t frame, int n_act, int m, int mp,
+                                                         int ka, uint8_t* __restrict__ hi, uint8_t* __restrict__ lo) {
+    const size_t total = (size_t)mp * (ka >> 3);
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < total; t += (size_t)gridDim.x * blockDim.x) {
-        const int q = (int)(t / mp), i = (int)(t - (size_t)q * mp);
-        float z[4] = {0.f, 0.f, 0.f, 0.f};
-        if (i < m && 4 * q < n_act) normals4<float>(seed, 1u, frame, (uint32_t)i, (uint32_t)q, z);
-        __align__(8) __nv_bfloat16 h[4], l[4];
+        const int g = (int)(t / mp), i = (int)(t - (size_t)g * mp);
+        float z[8];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) split2(4 * q + r < n_act ? z[r] : 0.f, h[r], l[r]);
-        const size_t off = umma::slice_offset(i, 4 * q, ka >> 6);
-        *reinterpret_cast<uint2*>(hi + off) = *reinterpret_cast<const uint2*>(h);
-        *reinterpret_cast<uint2*>(lo + off) = *reinterpret_cast<const uint2*>(l);
+        for (int h = 0; h < 2; ++h) {
+            float w[4] = {0.f, 0.f, 0.f, 0.f};
+            if (i < m && 8 * g + 4 * h < n_act) normals4<float>(seed, 1u, frame, (uint32_t)i, (uint32_t)(2 * g + h), w);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) z[4 * h + r] = 8 * g + 4 * h + r < n_act ? w[r] : 0.f;
+        }
+        store8(hi, lo, umma::slice_offset(i, 8 * g, ka >> 6), z);
     }
 }
 
@@ -238,7 +276,7 @@ GemmArgs gemm_args(const uint8_t* ah, const uint8_t* al, const uint8_t* bh, cons
 }  // namespace
 
 size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
-    const int mr = rup(m + 1, 128), pk = rup(2 * n_subv, 64), mp = rup(m, 128), nr = rup(2 * n_act, 128);
+    const int mr = rup(m + 1, 128), pk = slope_cols(n_subv), mp = rup(m, 128), nr = rup(2 * n_act, 128);
     const int ka = rup(n_act, 64);
     const size_t gram = (size_t)m * rup(m + 1, 4) * 4;
     const Plans P = plans_for(n_act, n_subv, m, dense, lower, sms);
@@ -257,7 +295,7 @@ int global_prepare(letkf_ctx* c) {
     c->gstate = S;
     const int m = c->m;
     S->mr = rup(m + 1, 128);
-    S->pk = rup(c->p, 64);
+    S->pk = slope_cols(c->n_subv);
     S->mp = rup(m, 128);
     S->nr = rup(c->n, 128);
     S->ka = rup(c->n_act, 64);
@@ -351,8 +389,8 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     const int m = c->m, n = c->n;
     const float cm = (float)(m - 1);
     prof_begin(c, STAGE_OBS);
-    gl_mean_kernel<<<grid_for((size_t)n * 32, 256), 256, 0, st>>>(X, n, m, c->m_pad, S->xbar, S->bar);
-    gl_slopes_kernel<<<grid_for((size_t)S->mr * (S->pk >> 3), 256), 256, 0, st>>>(
+    gl_center_kernel<<<S->nr / 8, 256, 0, st>>>(X, n, m, c->m_pad, S->mp, S->xbar, S->xp_hi, S->xp_lo, S->bar);
+    gl_slopes_kernel<<<grid_for((size_t)S->mr * (S->pk >> 4), 256), 256, 0, st>>>(
         X, S->xbar, static_cast<const float*>(yv), S->corner, c->n_subv, c->obs_block == 1 ? c->n_act : 0, m, c->m_pad,
         S->mr, S->pk, (float)(1.0 / c->sigma), S->st_hi, S->st_lo);
     prof_end(c);
@@ -405,15 +443,13 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     prof_end(c);
     // transform X_a = x_bar + X' W
     prof_begin(c, STAGE_TRANSFORM);
-    gl_xp_kernel<<<grid_for((size_t)S->nr * (S->mp >> 3), 256), 256, 0, st>>>(X, S->xbar, n, m, c->m_pad, S->nr, S->mp,
-                                                                               S->xp_hi, S->xp_lo);
     g = gemm_args(S->xp_hi, S->xp_lo, S->wt_hi, S->wt_lo, S->mp >> 6, n, m, c->d_status);
     g.mode = GEMM_EPI_ADD_ROW;
     g.c = Xo;
     g.ldc = c->m_pad;
     g.add = S->xbar;
     if ((rc = gemm_launch(g, S->pl_tr, st))) return rc;
-    gl_reject_kernel<<<grid_for((size_t)n * c->m_pad, 256), 256, 0, st>>>(X, Xo, (size_t)n * c->m_pad, c->d_frame_bad);
+    gl_reject_kernel<<<152, 256, 0, st>>>(X, Xo, (size_t)n * c->m_pad, c->d_frame_bad);
     prof_end(c);
     return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
@@ -423,7 +459,7 @@ int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
     if (v_user || !c->Lq || !S) return launch_forecast(c, v_user, xpred, in_analysis);
     // V = L xi on the tensor cores (FP32-level), into c->V with leading dimension m
     prof_begin(c, STAGE_NOISE);
-    gl_normals_kernel<<<grid_for((size_t)S->mp * (S->ka >> 2), 256), 256, 0, c->stream>>>(
+    gl_normals_kernel<<<grid_for((size_t)S->mp * (S->ka >> 3), 256), 256, 0, c->stream>>>(
         c->seed, (uint32_t)c->frame, c->n_act, c->m, S->mp, S->ka, S->xi_hi, S->xi_lo);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     GemmArgs g = gemm_args(S->l_hi, S->l_lo, S->xi_hi, S->xi_lo, S->ka >> 6, c->n_act, c->m, c->d_status);
