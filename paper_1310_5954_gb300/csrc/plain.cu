@@ -23,14 +23,90 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// Observed anomalies of one domain: the halo actuators of the observed instant are staged
-// in shared memory, centred on their member mean, and differenced at the corners of each
-// observed subaperture (Fried geometry, Sect. 3).
+// These kernels run one small problem per domain, a hundred domains at most at once, so latency bounds
+// them, not bandwidth: rows go through registers (loaded, averaged over the lanes and centred in one pass),
+// tables that one warp needs one after another are loaded together, and short sums are split over lanes.  In
+// FP64 (2 operations per cycle and SM, measured) the operations count as well: no padding, half of the
+// symmetric Gram, and the blocks of a domain are shared by several CTAs where the domains leave SMs idle.
+// Per frame, FP64 8 x 8 pupil with m = 20 / FP32 40 x 40 pupil with m = 50, launch included: plain_obs
+// 15 -> 12 / 20 -> 10 us, plain_gram 43 -> 12 / 36 -> 17, plain_transform 25 -> 12 / 18 -> 13.
+
+// Members per lane of a row in registers (plain_limits_ok ends at m = 168 in FP32, 118 in FP64).
+template <typename T>
+constexpr int kRowLanes = sizeof(T) == 4 ? 6 : 4;
+
+// Rows warp, warp + 8, ... below n of a matrix whose row j starts at src(j), `cols` columns each, to
+// dst (leading dimension ld): the loads of four rows are issued before their stores.
+template <typename T, typename F>
+__device__ __forceinline__ void copy_rows(int cols, int n, T* dst, int ld, F&& src) {
+    constexpr int U = kRowLanes<T>, B = 4, W = kThreads / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int j0 = warp; j0 < n; j0 += B * W) {
+        T v[B][U];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const T* x = src(min(j0 + b * W, n - 1));
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[b][u] = lane + 32 * u < cols ? x[lane + 32 * u] : (T)0;
+        }
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 + b * W < n && lane + 32 * u < cols) dst[(j0 + b * W) * ld + lane + 32 * u] = v[b][u];
+    }
+}
+
+// The same for rows of the ensemble, centred on their member mean (ld = m + 1, the mean behind the
+// members).  The four means are summed together: 6 additions in place of 20.
+template <typename T, typename F>
+__device__ __forceinline__ void centred_rows(int m, T inv_m, int n, T* dst, F&& src) {
+    constexpr int U = kRowLanes<T>, B = 4, W = kThreads / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mp1 = m + 1;
+    for (int j0 = warp; j0 < n; j0 += B * W) {
+        T v[B][U], s[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const T* x = src(min(j0 + b * W, n - 1));
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[b][u] = lane + 32 * u < m ? x[lane + 32 * u] : (T)0;
+        }
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            s[b] = v[b][0];
+#pragma unroll
+            for (int u = 1; u < U; ++u)
+                if (32 * u < m) s[b] += v[b][u];
+        }
+        // lanes with bit 4 set go on with rows 2 and 3, with bit 3 set with the odd one of the two
+        const bool hi = lane & 16, odd = lane & 8;
+        T a = (hi ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[2], 16);
+        T b = (hi ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, hi ? s[1] : s[3], 16);
+        a = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        a *= inv_m;
+#pragma unroll
+        for (int b4 = 0; b4 < B; ++b4) {
+            const int j = j0 + b4 * W;
+            const T mean = __shfl_sync(0xffffffffu, a, 8 * b4);
+            if (j >= n) break;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (lane + 32 * u < m) dst[j * mp1 + lane + 32 * u] = v[b4][u] - mean;
+            if (lane == 0) dst[j * mp1 + m] = mean;
+        }
+    }
+}
+
+// Observed anomalies of one domain: the halo actuators of the observed instant, centred on their
+// member mean in shared memory, and differenced at the corners of each observed subaperture
+// (Fried geometry, Sect. 3).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) plain_obs(const T* __restrict__ X, const T* __restrict__ y,
                                                       DomainTables tab, const int* __restrict__ so_off,
                                                       T* __restrict__ S, T* __restrict__ dt, int m, int m_pad,
-                                                      int row0, int n_subv, T inv_sigma,
+                                                      int row0, int n_subv, T inv_sigma, T inv_m,
                                                       const int* __restrict__ frame_bad) {
     extern __shared__ unsigned char smem_raw[];
     T* Xh = reinterpret_cast<T*>(smem_raw);
@@ -40,44 +116,90 @@ __global__ void __launch_bounds__(kThreads) plain_obs(const T* __restrict__ X, c
     const int o0 = tab.obs_off[d], no = tab.obs_off[d + 1] - o0;
     if (no == 0) return;
     const int mp1 = m + 1;  // smem row: m members, then the mean
-    for (int idx = threadIdx.x; idx < nh * m; idx += blockDim.x) {
-        const int j = idx / m, i = idx - j * m;
-        Xh[j * mp1 + i] = X[(size_t)(row0 + tab.halo[h0 + j]) * m_pad + i];
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int j = warp; j < nh; j += blockDim.x / 32) {
-        T s = 0;
-        for (int i = lane; i < m; i += 32) s += Xh[j * mp1 + i];
-        s = warp_sum(s);
-        if (lane == 0) Xh[j * mp1 + m] = s / (T)m;
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nh * m; idx += blockDim.x) {
-        const int j = idx / m, i = idx - j * m;
-        Xh[j * mp1 + i] -= Xh[j * mp1 + m];
-    }
-    __syncthreads();
+    centred_rows(m, inv_m, nh, Xh, [&](int j) { return X + (size_t)(row0 + tab.halo[h0 + j]) * m_pad; });
     const int base = so_off[d];
-    for (int idx = threadIdx.x; idx < no * mp1; idx += blockDim.x) {
-        const int s = idx / mp1, i = idx - s * mp1;
-        const int pc = tab.obs_corner[o0 + s];
-        const T a00 = Xh[(pc & 0xFF) * mp1 + i], a01 = Xh[((pc >> 8) & 0xFF) * mp1 + i];
-        const T a10 = Xh[((pc >> 16) & 0xFF) * mp1 + i], a11 = Xh[((pc >> 24) & 0xFF) * mp1 + i];
-        const T sx = (T)0.5 * ((a01 + a11) - (a00 + a10));
-        const T sy = (T)0.5 * ((a10 + a11) - (a00 + a01));
-        if (i < m) {
-            S[(size_t)(base + s) * m_pad + i] = sx * inv_sigma;
-            S[(size_t)(base + no + s) * m_pad + i] = sy * inv_sigma;
-        } else {  // i == m: the mean column gives the slopes of the ensemble mean
-            const int k = tab.obs_sub[o0 + s];
-            dt[base + s] = (y[k] - sx) * inv_sigma;
-            dt[base + no + s] = (y[n_subv + k] - sy) * inv_sigma;
+    // the corners of this warp's subapertures, one per lane (warp, warp + 8, ...), up to 256 at a time
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto corners = [&](int s0) {
+        const int s = s0 + warp + 8 * lane;
+        return s < no ? tab.obs_corner[o0 + s] : 0;
+    };
+    int pcs = corners(0);
+    __syncthreads();
+    const T half = (T)0.5 * inv_sigma;
+    for (int s = warp; s < no; s += 8) {
+        if (s >= 256 && (s >> 3 & 31) == 0) pcs = corners(s - warp);
+        const int pc = __shfl_sync(0xffffffffu, pcs, s >> 3 & 31);
+        const T *r00 = Xh + (pc & 0xFF) * mp1, *r01 = Xh + ((pc >> 8) & 0xFF) * mp1;
+        const T *r10 = Xh + ((pc >> 16) & 0xFF) * mp1, *r11 = Xh + ((pc >> 24) & 0xFF) * mp1;
+        for (int i = lane; i < m; i += 32) {
+            const T u = r11[i] - r00[i], v = r01[i] - r10[i];
+            S[(size_t)(base + s) * m_pad + i] = half * (u + v);
+            S[(size_t)(base + no + s) * m_pad + i] = half * (u - v);
         }
+    }
+    // the mean's slopes against the measured ones
+    for (int s = threadIdx.x; s < no; s += kThreads) {
+        const int pc = tab.obs_corner[o0 + s], k = tab.obs_sub[o0 + s];
+        const T yx = y[k], yy = y[n_subv + k];
+        const T a00 = Xh[(pc & 0xFF) * mp1 + m], a01 = Xh[((pc >> 8) & 0xFF) * mp1 + m];
+        const T a10 = Xh[((pc >> 16) & 0xFF) * mp1 + m], a11 = Xh[((pc >> 24) & 0xFF) * mp1 + m];
+        dt[base + s] = (yx - (T)0.5 * ((a01 + a11) - (a00 + a10))) * inv_sigma;
+        dt[base + no + s] = (yy - (T)0.5 * ((a10 + a11) - (a00 + a01))) * inv_sigma;
     }
 }
 
-// G = S^T S and b = S^T dt for one domain; S staged in shared memory.
+// Blocks of 4 x 4 of S^T S on and above the diagonal, 2^LK lanes to a block with every 2^LK-th row of S
+// each: blocks [first, last) of this CTA, in passes of kThreads >> LK.
+template <typename T, int LK>
+__device__ __forceinline__ void gram_blocks(const T* __restrict__ Ss, int ld, int pl, T* __restrict__ Gd, int m, int m_pad,
+                                            int first, int last) {
+    constexpr int KS = 1 << LK, CAP = kThreads >> LK;
+    const int nb = (m + 3) >> 2, ks = threadIdx.x & (KS - 1);
+    for (int b0 = first; b0 < last; b0 += CAP) {
+        const int t = b0 + (threadIdx.x >> LK);
+        int rem = min(t, last - 1), bi = 0;
+        while (rem >= nb - bi) rem -= nb - bi++;
+        const int i0 = 4 * bi, j0 = 4 * (bi + rem);
+        // past m: the last column again (not stored)
+        const int i1 = min(i0 + 1, m - 1), i2 = min(i0 + 2, m - 1), i3 = min(i0 + 3, m - 1);
+        const int j1 = min(j0 + 1, m - 1), j2 = min(j0 + 2, m - 1), j3 = min(j0 + 3, m - 1);
+        T acc[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] = 0;
+#pragma unroll 2
+        for (int k = ks; k < pl; k += KS) {
+            const T* row = Ss + k * ld;
+            const T a[4] = {row[i0], row[i1], row[i2], row[i3]}, b[4] = {row[j0], row[j1], row[j2], row[j3]};
+#pragma unroll
+            for (int e = 0; e < 16; ++e) acc[e] += a[e >> 2] * b[e & 3];
+        }
+        // the lanes' sums: each step halves what a lane keeps
+        int e0 = 0;
+#pragma unroll
+        for (int q = 0; q < LK; ++q) {
+            const int half = 8 >> q;
+            const bool up = (ks >> q) & 1;
+            e0 += up ? half : 0;
+#pragma unroll
+            for (int e = 0; e < half; ++e) {
+                const T give = up ? acc[e] : acc[e + half], keep = up ? acc[e + half] : acc[e];
+                acc[e] = keep + __shfl_xor_sync(0xffffffffu, give, 1 << q);
+            }
+        }
+        if (t < last)
+#pragma unroll
+            for (int e = 0; e < (16 >> LK); ++e) {
+                const int i = i0 + ((e0 + e) >> 2), j = j0 + ((e0 + e) & 3);
+                if (i < m && j < m) {
+                    Gd[(size_t)i * m_pad + j] = acc[e];
+                    if (j0 > i0) Gd[(size_t)j * m_pad + i] = acc[e];
+                }
+            }
+    }
+}
+
+// G = S^T S and b = S^T dt for one domain; S staged in shared memory.  gridDim.y CTAs share the blocks.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) plain_gram(const T* __restrict__ S, const T* __restrict__ dt,
                                                        DomainTables tab, const int* __restrict__ so_off,
@@ -92,53 +214,30 @@ __global__ void __launch_bounds__(kThreads) plain_gram(const T* __restrict__ S, 
     const int base = so_off[d];
     T* Gd = G + (size_t)d * m * m_pad;
     const int ld = m + 1;  // rows of m members plus dt
-    for (int idx = threadIdx.x; idx < pl * ld; idx += blockDim.x) {
-        const int k = idx / ld, i = idx - k * ld;
-        Ss[k * ld + i] = (i < m) ? S[(size_t)(base + k) * m_pad + i] : dt[base + k];
-    }
+    copy_rows<T>(m, pl, Ss, ld, [&](int k) { return S + (size_t)(base + k) * m_pad; });
+    for (int k = threadIdx.x; k < pl; k += kThreads) Ss[k * ld + m] = dt[base + k];
     __syncthreads();
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    constexpr int CH = 4;       // row chunk per thread
-    constexpr int MAXC = 16;    // columns per thread (m <= 256)
-    for (int ib = 0; ib < m; ib += 16 * CH) {
-        T acc[CH][MAXC];
-#pragma unroll
-        for (int a = 0; a < CH; ++a)
-#pragma unroll
-            for (int bb = 0; bb < MAXC; ++bb) acc[a][bb] = 0;
-        for (int k = 0; k < pl; ++k) {
-            const T* row = Ss + k * ld;
-            T ri[CH];
-#pragma unroll
-            for (int a = 0; a < CH; ++a) {
-                const int i = ib + ty + 16 * a;
-                ri[a] = (i < m) ? row[i] : (T)0;
-            }
-#pragma unroll
-            for (int bb = 0; bb < MAXC; ++bb) {
-                const int j = tx + 16 * bb;
-                if (j < m) {
-                    const T rj = row[j];
-#pragma unroll
-                    for (int a = 0; a < CH; ++a) acc[a][bb] += ri[a] * rj;
-                }
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < CH; ++a) {
-            const int i = ib + ty + 16 * a;
-            if (i >= m) continue;
-#pragma unroll
-            for (int bb = 0; bb < MAXC; ++bb) {
-                const int j = tx + 16 * bb;
-                if (j < m) Gd[(size_t)i * m_pad + j] = acc[a][bb];
-            }
-        }
-    }
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    const int nb = (m + 3) >> 2, blocks = nb * (nb + 1) / 2, per = (blocks + gridDim.y - 1) / gridDim.y;
+    const int first = min((int)blockIdx.y * per, blocks), last = min(first + per, blocks);
+    // as many lanes to a block as leave every block a place in the first pass
+    if (per * 16 <= kThreads)
+        gram_blocks<T, 4>(Ss, ld, pl, Gd, m, m_pad, first, last);
+    else if (per * 8 <= kThreads)
+        gram_blocks<T, 3>(Ss, ld, pl, Gd, m, m_pad, first, last);
+    else if (per * 4 <= kThreads)
+        gram_blocks<T, 2>(Ss, ld, pl, Gd, m, m_pad, first, last);
+    else if (per * 2 <= kThreads)
+        gram_blocks<T, 1>(Ss, ld, pl, Gd, m, m_pad, first, last);
+    else
+        gram_blocks<T, 0>(Ss, ld, pl, Gd, m, m_pad, first, last);
+    if (blockIdx.y != gridDim.y - 1) return;
+    for (int i0 = 0; i0 < m; i0 += kThreads / 8) {      // eight lanes to a member
+        const int i = i0 + (threadIdx.x >> 3), c = min(i, m - 1);
         T s = 0;
-        for (int k = 0; k < pl; ++k) s += Ss[k * ld + i] * Ss[k * ld + m];
-        bvec[(size_t)d * m_pad + i] = s;
+        for (int k = threadIdx.x & 7; k < pl; k += 8) s += Ss[k * ld + c] * Ss[k * ld + m];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (i < m && (threadIdx.x & 7) == 0) bvec[(size_t)d * m_pad + i] = s;
     }
 }
 
@@ -489,54 +588,57 @@ void launch_eig(int n_dom, cudaStream_t st, const T* G, const T* b, T* W, int m,
         plain_eig<T, 6><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, bad);
 }
 
-// X_out[E] = x_bar[E] 1^T + X'[E] W for the domain's own rows E (both instants).
+// X_out[E] = x_bar[E] 1^T + X'[E] W for the domain's own rows E (both instants), the rows shared by
+// gridDim.y CTAs; blocks of 2 x 2 results per thread.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) plain_transform(const T* __restrict__ X, T* __restrict__ Xo,
                                                             const T* __restrict__ W, DomainTables tab, int m,
-                                                            int m_pad, int n_act,
+                                                            int m_pad, int n_act, T inv_m,
                                                             const int* __restrict__ frame_bad) {
     extern __shared__ unsigned char smem_raw[];
     const int d = blockIdx.x;
     const int e0 = tab.own_off[d], ne = tab.own_off[d + 1] - e0;
-    const int nl = 2 * ne;
+    const int per = (2 * ne + gridDim.y - 1) / gridDim.y, r0 = blockIdx.y * per, nl = min(per, 2 * ne - r0);
+    if (nl <= 0) return;
     const int ld = m + 1;
     T* Ws = reinterpret_cast<T*>(smem_raw);
     T* Xe = Ws + m * m;
-    // a domain without observations keeps its forecast exactly (G = 0: w_bar = 0, T = I)
-    const bool bad = *frame_bad != 0 || tab.obs_off[d + 1] == tab.obs_off[d];
-    const T* Wd = W + (size_t)d * m * m_pad;
-    if (!bad)
-        for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-            const int k = idx / m, l = idx - k * m;
-            Ws[idx] = Wd[(size_t)k * m_pad + l];
-        }
-    for (int idx = threadIdx.x; idx < nl * m; idx += blockDim.x) {
-        const int e = idx / m, i = idx - e * m;
-        const int row = (e < ne) ? tab.own[e0 + e] : n_act + tab.own[e0 + e - ne];
-        Xe[e * ld + i] = X[(size_t)row * m_pad + i];
-    }
-    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int e = warp; e < nl; e += blockDim.x / 32) {
-        T s = 0;
-        for (int i = lane; i < m; i += 32) s += Xe[e * ld + i];
-        s = warp_sum(s);
-        if (lane == 0) Xe[e * ld + m] = s / (T)m;
+    auto row = [&](int q) {
+        const int e = r0 + q;
+        return (e < ne) ? tab.own[e0 + e] : n_act + tab.own[e0 + e - ne];
+    };
+    // a domain without observations keeps its forecast exactly (G = 0: w_bar = 0, T = I)
+    if (*frame_bad != 0 || tab.obs_off[d + 1] == tab.obs_off[d]) {
+        for (int q = warp; q < nl; q += kThreads / 32)
+            for (int i = lane; i < m; i += 32) Xo[(size_t)row(q) * m_pad + i] = X[(size_t)row(q) * m_pad + i];
+        return;
     }
+    const T* Wd = W + (size_t)d * m * m_pad;
+    copy_rows<T>(m, m, Ws, m, [&](int k) { return Wd + (size_t)k * m_pad; });
+    centred_rows(m, inv_m, nl, Xe, [&](int q) { return X + (size_t)row(q) * m_pad; });
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nl * m; idx += blockDim.x) {
-        const int e = idx / m, l = idx - e * m;
-        const int row = (e < ne) ? tab.own[e0 + e] : n_act + tab.own[e0 + e - ne];
-        T out;
-        if (bad) {
-            out = Xe[e * ld + l];
-        } else {
-            const T xb = Xe[e * ld + m];
-            T s = 0;
-            for (int k = 0; k < m; ++k) s += (Xe[e * ld + k] - xb) * Ws[k * m + l];
-            out = xb + s;
+    const int cb = (m + 1) >> 1, rb = (nl + 1) >> 1;
+    for (int t = threadIdx.x; t < cb * rb; t += kThreads) {
+        const int b = t / cb, l0 = 2 * (t - b * cb), l1 = min(l0 + 1, m - 1), q0 = 2 * b, q1 = min(q0 + 1, nl - 1);
+        const T *xa = Xe + q0 * ld, *xb = Xe + q1 * ld;
+        T s00 = 0, s01 = 0, s10 = 0, s11 = 0;
+#pragma unroll 4
+        for (int k = 0; k < m; ++k) {
+            const T u = xa[k], v = xb[k], w0 = Ws[k * m + l0], w1 = Ws[k * m + l1];
+            s00 += u * w0;
+            s01 += u * w1;
+            s10 += v * w0;
+            s11 += v * w1;
         }
-        Xo[(size_t)row * m_pad + l] = out;
+        T* oa = Xo + (size_t)row(q0) * m_pad;
+        T* ob = Xo + (size_t)row(q1) * m_pad;
+        oa[l0] = xa[m] + s00;
+        if (l0 + 1 < m) oa[l1] = xa[m] + s01;
+        if (q0 + 1 < nl) {
+            ob[l0] = xb[m] + s10;
+            if (l0 + 1 < m) ob[l1] = xb[m] + s11;
+        }
     }
 }
 
@@ -578,6 +680,8 @@ int plain_analyze_t(letkf_ctx* c, const T* y, double sigma) {
     T* Xo = static_cast<T*>(c->X[c->cur ^ 1]);
     const int m = c->m, mp = c->m_pad, nd = c->n_dom;
     const int row0 = c->obs_block == 1 ? c->n_act : 0;
+    // CTAs per domain: where the domains leave SMs idle, up to eight
+    const dim3 shared_by(nd, std::max(1, std::min(8, c->sms / std::max(nd, 1))));
     const size_t sm_obs = (size_t)c->host.n_h_max * (m + 1) * sizeof(T);
     const size_t sm_gram = (size_t)std::max(c->host.p_loc_max, 1) * (m + 1) * sizeof(T);
     const size_t sm_tr = ((size_t)m * m + (size_t)c->host.n_loc_max * (m + 1)) * sizeof(T);
@@ -585,10 +689,10 @@ int plain_analyze_t(letkf_ctx* c, const T* y, double sigma) {
     prof_begin(c, STAGE_OBS);
     plain_obs<T><<<nd, kThreads, sm_obs, c->stream>>>(X, y, c->tab, c->so_off, static_cast<T*>(c->S),
                                                       static_cast<T*>(c->dt), m, mp, row0, c->n_subv,
-                                                      (T)(1.0 / c->sigma), c->d_frame_bad);
+                                                      (T)(1.0 / c->sigma), (T)(1.0 / m), c->d_frame_bad);
     prof_end(c);
     prof_begin(c, STAGE_GRAM);
-    plain_gram<T><<<nd, kThreads, sm_gram, c->stream>>>(static_cast<const T*>(c->S), static_cast<const T*>(c->dt),
+    plain_gram<T><<<shared_by, kThreads, sm_gram, c->stream>>>(static_cast<const T*>(c->S), static_cast<const T*>(c->dt),
                                                         c->tab, c->so_off, static_cast<T*>(c->G),
                                                         static_cast<T*>(c->b), m, mp, c->d_frame_bad);
     prof_end(c);
@@ -597,8 +701,8 @@ int plain_analyze_t(letkf_ctx* c, const T* y, double sigma) {
                   c->d_frame_bad);
     prof_end(c);
     prof_begin(c, STAGE_TRANSFORM);
-    plain_transform<T><<<nd, kThreads, sm_tr, c->stream>>>(X, Xo, static_cast<const T*>(c->W), c->tab, m, mp,
-                                                           c->n_act, c->d_frame_bad);
+    plain_transform<T><<<shared_by, kThreads, sm_tr, c->stream>>>(X, Xo, static_cast<const T*>(c->W), c->tab, m, mp,
+                                                           c->n_act, (T)(1.0 / m), c->d_frame_bad);
     prof_end(c);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     return LETKF_OK;
@@ -703,16 +807,18 @@ int analyze_static_t(letkf_ctx* c, const T* y, double sigma, T* out) {
     const T* X = static_cast<const T*>(c->X[c->cur]);
     const double sg = sigma > 0 ? sigma : c->sigma;
     const int row0 = c->obs_block == 1 ? c->n_act : 0;
+    // CTAs per domain: where the domains leave SMs idle, up to eight
+    const dim3 shared_by(nd, std::max(1, std::min(8, c->sms / std::max(nd, 1))));
     const size_t sm_obs = (size_t)c->host.n_h_max * (m + 1) * sizeof(T);
     const size_t sm_gram = (size_t)std::max(c->host.p_loc_max, 1) * (m + 1) * sizeof(T);
     const size_t sm_tr = ((size_t)m * m + (size_t)c->host.n_loc_max * (m + 1)) * sizeof(T);
     if ((rc = plain_kernels_ready<T>(c->device))) return rc;
     static_check_kernel<T><<<1, 1024, 0, c->stream>>>(y, c->p, flag, c->d_status);
     plain_obs<T><<<nd, kThreads, sm_obs, c->stream>>>(X, y, c->tab, c->so_off, S, dt, m, mp, row0, c->n_subv,
-                                                      (T)(1.0 / sg), flag);
-    plain_gram<T><<<nd, kThreads, sm_gram, c->stream>>>(S, dt, c->tab, c->so_off, G, bv, m, mp, flag);
+                                                      (T)(1.0 / sg), (T)(1.0 / m), flag);
+    plain_gram<T><<<shared_by, kThreads, sm_gram, c->stream>>>(S, dt, c->tab, c->so_off, G, bv, m, mp, flag);
     launch_eig<T>(nd, c->stream, G, bv, W, m, mp, flag);
-    plain_transform<T><<<nd, kThreads, sm_tr, c->stream>>>(X, Xo, W, c->tab, m, mp, c->n_act, flag);
+    plain_transform<T><<<shared_by, kThreads, sm_tr, c->stream>>>(X, Xo, W, c->tab, m, mp, c->n_act, (T)(1.0 / m), flag);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     if (cudaMemcpy2DAsync(out, (size_t)m * eb, Xo, (size_t)mp * eb, (size_t)m * eb, c->n, cudaMemcpyDeviceToDevice,
                           c->stream) != cudaSuccess)
