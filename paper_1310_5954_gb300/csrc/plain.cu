@@ -241,8 +241,11 @@ __global__ void __launch_bounds__(kThreads) plain_gram(const T* __restrict__ S, 
     }
 }
 
-// Quadrature nodes per pass over the tridiagonal function (their recursions live in shared memory).
-constexpr int kNodes = 8;
+// Quadrature nodes per pass over the tridiagonal function (their recursions live in shared memory): one
+// lane each for the serial recursions, whose divisions (FP64: about 1000 cycles) bound a pass, so that
+// all nodes of a usual kappa go in one (kappa = 100: 17 in FP64, 10 in FP32).
+template <typename T>
+constexpr int kNodes = sizeof(T) == 8 ? 32 : 16;
 
 template <typename T>
 __device__ __forceinline__ void sincos_halfpi(T a, T& s, T& c);   // sin and cos of (pi/2) a
@@ -268,7 +271,7 @@ __device__ __forceinline__ void sincos_halfpi<double>(double a, double& s, doubl
 // matrix-vector product and rank-2 update between them); the reflectors are then applied to J's
 // function column by column, 8 lanes and two columns per thread group, in registers and without a
 // barrier.  Measured, whole stage: 92 domains of m = 50 in FP32 522 -> 110 us, 4 domains of m = 20 in
-// FP64 499 -> 183 us (before: Jacobi).
+// FP64 499 -> 148 us (before: Jacobi; 183 with the nodes eight at a time).
 template <typename T, int UM>   // m <= 32 UM members; 4 threads per member, at most 640
 __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __restrict__ G,
                                                                      const T* __restrict__ bvec, T* __restrict__ W,
@@ -278,7 +281,8 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
     const int ld = m | 1;                  // odd row stride: no bank conflicts down a column
     T* A = reinterpret_cast<T*>(smem_raw);   // B, then (row k, columns > k) the reflector v_k
     T* F = A + m * ld;                     // the function of J, then T
-    const int mv = max(m, 2 * kNodes);
+    constexpr int NK = kNodes<T>;
+    const int mv = max(m, 2 * NK);
     T* dd = F + m * ld;                    // J's diagonal and (ee) off-diagonal
     T* ee = dd + mv;
     T* bt = ee + mv;                       // 2 / v_k^T v_k
@@ -382,25 +386,33 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
     // k_(s+1)' = 2 sqrt(k_s')/(1 + k_s'); K' = (pi/2) prod (1 + k_s)
     constexpr int LS = sizeof(T) == 8 ? 9 : 7;
     T lk[LS], kprod = (T)1;
-    {
+    if (tid < 2 * NK) {
+        // until k_s no longer counts (a few steps: k_(s+1) ~ (k_s / 2)^2)
         T kc = (T)1 / sqrt(hi);
+        bool more = true;
 #pragma unroll
         for (int s = 0; s < LS; ++s) {
-            lk[s] = ((T)1 - kc) / ((T)1 + kc);
-            kprod *= (T)1 + lk[s];
-            kc = (T)2 * sqrt(kc) / ((T)1 + kc);
+            lk[s] = 0;
+            if (more) {
+                const T q = (T)1 / ((T)1 + kc);
+                lk[s] = ((T)1 - kc) * q;
+                kprod *= (T)1 + lk[s];
+                kc = (T)2 * sqrt(kc) * q;
+                more = lk[s] > (sizeof(T) == 8 ? (T)1e-17 : (T)1e-9);
+            }
         }
     }
     for (int n0 = 0; n0 < N; n0 += kb) {
         const int nn = min(kb, N - n0);
-        if (tid < 2 * kNodes && (tid & (kNodes - 1)) < nn) {
+        if (tid < 2 * NK && (tid & (NK - 1)) < nn) {
             // thread (node, direction): the pivots of cn^2 J + sn^2 I from the top (into gn) or from
             // the bottom (into rn)
-            const int n = tid & (kNodes - 1);
+            const int n = tid & (NK - 1);
             T sn, cn, dn = (T)1;
             sincos_halfpi<T>((T)(2 * (n0 + n) + 1) / (T)(2 * N), sn, cn);
 #pragma unroll
             for (int s = LS - 1; s >= 0; --s) {
+                if (lk[s] == (T)0) continue;
                 const T s2 = lk[s] * sn * sn, q = (T)1 / ((T)1 + s2);
                 const T cd = cn * dn * q;
                 dn = ((T)1 - s2) * q;
@@ -408,7 +420,7 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
                 cn = cd;
             }
             const T c2 = cn * cn, s2 = sn * sn;
-            if (tid < kNodes) {
+            if (tid < NK) {
                 T pv = c2 * dd[0] + s2;
                 gn[n * m] = pv;
                 for (int i = 1; i < m; ++i) {
@@ -417,7 +429,7 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
                     gn[n * m + i] = pv;
                 }
                 vs[n] = c2;                // the node's parameters, for the pass below
-                vs[kNodes + n] = s2;
+                vs[NK + n] = s2;
                 ps[n] = dn * kprod / (T)N;
             } else {
                 T pv = c2 * dd[m - 1] + s2;
@@ -433,7 +445,7 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
         // the inverse's diagonal 1 / (top + bottom pivot - diagonal), weighted, and the ratios
         // inv(i, j + 1) / inv(i, j) = -e_j / (bottom pivot j + 1), j >= i
         for (int n = warp; n < nn; n += nw) {
-            const T c2 = vs[n], s2 = vs[kNodes + n], wt = ps[n];
+            const T c2 = vs[n], s2 = vs[NK + n], wt = ps[n];
             T nx[UM];
 #pragma unroll
             for (int u = 0; u < UM; ++u) {
@@ -450,27 +462,29 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
                 if (lane + 32 * u < m) rn[n * m + lane + 32 * u] = nx[u];
         }
         __syncthreads();
-        // rows of the sum: two lanes per row, half the nodes each, walking right from the diagonal
-        for (int t = tid; t < 2 * ((m + 15) & ~15); t += nt) {     // whole warps
-            const int i = t >> 1, h = t & 1, i_lo = (t & ~31) >> 1;
-            T r[kNodes / 2];
+        // rows of the sum: four lanes per row, a quarter of the nodes each, walking right from the diagonal
+        for (int t = tid; t < 4 * ((m + 7) & ~7); t += nt) {       // whole warps
+            const int i = t >> 2, h = t & 3, i_lo = (t & ~31) >> 2;
+            T r[NK / 4];
 #pragma unroll
-            for (int q = 0; q < kNodes / 2; ++q) {
-                const int n = 2 * q + h;
+            for (int q = 0; q < NK / 4; ++q) {
+                const int n = 4 * q + h;
                 r[q] = (i < m && n < nn) ? gn[n * m + i] : (T)0;
             }
             for (int st = 0; st < m - i_lo; ++st) {
                 const int j = i + st;
-                T sum = 0;
+                T sum = r[0];
 #pragma unroll
-                for (int q = 0; q < kNodes / 2; ++q) sum += r[q];
+                for (int q = 1; q < NK / 4; ++q)
+                    if (4 * q < nn) sum += r[q];
                 sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                sum += __shfl_xor_sync(0xffffffffu, sum, 2);
                 if (j < m) {
-                    T* f = h ? F + j * ld + i : F + i * ld + j;    // the lanes write the two triangles
-                    if (h == 0 || j > i) *f = n0 ? *f + sum : sum;
+                    T* f = h ? F + j * ld + i : F + i * ld + j;    // two lanes write the two triangles
+                    if (h == 0 || (h == 1 && j > i)) *f = n0 ? *f + sum : sum;
 #pragma unroll
-                    for (int q = 0; q < kNodes / 2; ++q)
-                        if (2 * q + h < nn) r[q] *= rn[(2 * q + h) * m + j];
+                    for (int q = 0; q < NK / 4; ++q)
+                        if (4 * q + h < nn) r[q] *= rn[(4 * q + h) * m + j];
                 }
             }
         }
@@ -566,16 +580,16 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
 // Dynamic shared memory of plain_eig: B and F (m x m, odd row stride), vectors, kb nodes' recursions.
 template <typename T>
 size_t eig_smem(int m, int kb) {
-    return ((size_t)2 * m * (m | 1) + (size_t)5 * std::max(m, 2 * kNodes) + (size_t)2 * kb * m) * sizeof(T);
+    return ((size_t)2 * m * (m | 1) + (size_t)5 * std::max(m, 2 * kNodes<T>) + (size_t)2 * kb * m) * sizeof(T);
 }
 
 // Four threads per member (two columns per group of eight lanes in the back-transformation), at
 // least four warps; as many nodes per pass, up to kNodes, as shared memory leaves room for (all of
-// them up to m = 160 in FP32 and 114 in FP64).
+// them up to m = 161 in FP32 and 104 in FP64).
 template <typename T>
 void launch_eig(int n_dom, cudaStream_t st, const T* G, const T* b, T* W, int m, int m_pad, const int* bad) {
     const int nt = std::min(640, std::max(128, (4 * m + 31) / 32 * 32));
-    int kb = kNodes;
+    int kb = kNodes<T>;
     while (kb > 1 && eig_smem<T>(m, kb) > 227 * 1024) --kb;
     const size_t sm = eig_smem<T>(m, kb);
     if (m <= 32)
