@@ -454,11 +454,13 @@ __device__ __forceinline__ void issue_loads(const SysDesc& A, int d, float* Xh, 
 
 // Warp 0, all 32 lanes: take the next work item of the batch.  Its loads are issued at once when
 // they cannot overwrite shared memory still in use (everything at or above busy_from).
-__device__ void fetch_item(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, int busy_from) {
+__device__ void fetch_item(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, int busy_from, bool first = false) {
     const int lane = threadIdx.x & 31;
-    int g = 0;
-    if (lane == 0) g = atomicAdd(B.queue, 1);
-    g = __shfl_sync(0xffffffffu, g, 0);
+    int g = blockIdx.x;              // a CTA's first item needs no queue
+    if (!first) {
+        if (lane == 0) g = atomicAdd(B.queue, 1) + (int)gridDim.x;
+        g = __shfl_sync(0xffffffffu, g, 0);
+    }
     if (lane == 0) {
         ctl->item = g;
         ctl->loaded = 0;
@@ -2076,7 +2078,13 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
         ctl->abort = 0;
         fence_mbar_init();
     }
+    // the first item's tables and rows are under way while another warp takes the tensor memory: one round
+    // trip to the tables is a microsecond here, of 19 for the whole 8 x 8 pupil
+    constexpr int fetch_all = TWO ? -1 : 1 << 30;    // TWO: an item's rows are copied when its turn comes
     if (warp == 0) {
+        __syncwarp();
+        fetch_item(B, ctl, smem, fetch_all, true);
+    } else if (warp == 1) {
         tmem_alloc(&ctl->tmem_base, tmem_cols);
         tmem_relinquish();
     }
@@ -2088,10 +2096,6 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
     // a launch that follows this kernel through a programmatic edge may start now (it does not
     // read what this kernel writes)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-    constexpr int fetch_all = TWO ? -1 : 1 << 30;    // TWO: an item's rows are copied when its turn comes
-    if (warp == 0) fetch_item(B, ctl, smem, fetch_all);
-    __syncthreads();
 
     while (ctl->item < B.n_items && !ctl->abort) {
         // ONE: by value, fields stay in registers across barriers; the others, with half the registers per
@@ -3018,7 +3022,7 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) tmem_dealloc(tbase, tmem_cols);
+    if (warp == 1) tmem_dealloc(tbase, tmem_cols);
     // the last CTA to finish (all work items taken and done) closes the launch
     if (tid == 0) {
         __threadfence();
