@@ -40,7 +40,7 @@ struct GlobalState {
     float* G = nullptr;                            // m x (m+1) Gram, row-major
     float* Gpart = nullptr;                        // partial Grams of the upper tiles, one per share
     int ldg = 0, gram_split = 1;                   // leading dimension of the Gram, shares of its K steps
-    GemmPlan pl_gram, pl_tr, pl_noise;
+    GemmPlan pl_gram, pl_tr, pl_tr1, pl_noise;     // Gram, transform (both instants / the first), noise draw
     uint8_t *as_hi = nullptr, *as_lo = nullptr, *t_hi = nullptr, *t_lo = nullptr;
     uint8_t *y_hi[2] = {}, *y_lo[2] = {}, *z_hi[2] = {}, *z_lo[2] = {};
     uint8_t *xp_hi = nullptr, *xp_lo = nullptr;    // X' tiles (nr x mp)
@@ -68,7 +68,7 @@ int cluster_rows(int row_tiles) { return row_tiles >= 2 ? 2 : 1; }
 // The plans of the analysis's products, and the Gram's shares: as many as make its pieces fill the SMs,
 // against the partial Grams that every share writes and the reduction reads (at 2 KB per cycle).
 struct Plans {
-    GemmPlan gram, tr, noise;
+    GemmPlan gram, tr, tr1, noise;
     int split = 1;
 };
 Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
@@ -97,10 +97,11 @@ Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
     t.bn = 256;
     t.cm = cluster_rows(rows);
     P.tr = gemm_plan(t, sms);
+    t.m_tiles = acts;
+    t.cm = cluster_rows(acts);
+    P.tr1 = gemm_plan(t, sms);
     if (dense) {
-        t.m_tiles = acts;
         t.nkb = rup(n_act, 64) / 64;
-        t.cm = cluster_rows(acts);
         t.lower = lower;
         P.noise = gemm_plan(t, sms);
     }
@@ -117,11 +118,11 @@ __device__ __forceinline__ void store8(uint8_t* hi, uint8_t* lo, size_t off, con
 }
 
 // Member means of the state rows and the X' slices, element (r, i) = X[r][i] - x_bar[r] for r < n, i < m
-// and zero beyond; resets the iteration's grid barrier.  Bound by HBM: X is read once, from HBM for the
+// and zero beyond (for the rows below n_x rounded up to eight); resets the iteration's grid barrier.  Bound by HBM: X is read once, from HBM for the
 // means, one warp per row, and again, now from L1, by threads that take the eight rows of a core matrix side
 // by side, so that the slices are written in pieces of 256 bytes.  (Two kernels, the second with one thread
 // per row piece and 16-byte stores 2 KB apart, took 11 + 26 us at n = 9666, m = 1024; this 19 us.)
-__global__ void __launch_bounds__(256) gl_center_kernel(const float* __restrict__ X, int n, int m, int m_pad, int mp,
+__global__ void __launch_bounds__(256) gl_center_kernel(const float* __restrict__ X, int n, int n_x, int m, int m_pad, int mp,
                                                         float* __restrict__ xbar, uint8_t* __restrict__ hi,
                                                         uint8_t* __restrict__ lo, unsigned* __restrict__ bar) {
     __shared__ float mu_sh[8];
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(256) gl_center_kernel(const float* __restrict_
         }
     }
     __syncthreads();
+    if (r0 >= n_x) return;
     const int r = r0 + (threadIdx.x & 7);
     const float mu = mu_sh[threadIdx.x & 7];
     const float* x = X + (size_t)r * m_pad;
@@ -284,7 +286,7 @@ size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sm
     size_t b = 2 * tiled_bytes(mr, pk) + gram * (1 + P.split) + 12 * tiled_bytes(mp, mp) + 2 * tiled_bytes(nr, mp) +
                2 * tiled_bytes(mp, mp);
     if (dense) b += 2 * tiled_bytes(rup(n_act, 128), ka) + 2 * tiled_bytes(mp, ka);
-    for (const GemmPlan* p : {&P.gram, &P.tr, &P.noise}) b += p->bytes();
+    for (const GemmPlan* p : {&P.gram, &P.tr, &P.tr1, &P.noise}) b += p->bytes();
     b += (size_t)2 * n_act * 4 + (size_t)4 * m * 4 + (size_t)root_parts(m) * 4 + sizeof(RootStats) + ROOT_STEPS * 4 + 8 +
          (size_t)n_subv * 16;
     return b;
@@ -315,6 +317,7 @@ int global_prepare(letkf_ctx* c) {
     ok = ok && get((size_t)m * S->ldg * 4, (void**)&S->G) &&
          get((size_t)P.split * m * S->ldg * 4, (void**)&S->Gpart);
     for (auto& q : {std::make_pair(&P.gram, &S->pl_gram), std::make_pair(&P.tr, &S->pl_tr),
+                    std::make_pair(&P.tr1, &S->pl_tr1),
                     std::make_pair(&P.noise, &S->pl_noise)}) {
         GemmPlan& p = *q.first;
         if (!p.ncl) continue;
@@ -377,7 +380,7 @@ void global_free(letkf_ctx* c) {
     c->gstate = nullptr;
 }
 
-int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
+int global_analyze(letkf_ctx* c, const void* yv, double sigma, bool first_only) {
     GlobalState* S = c->gstate;
     if (!S) return LETKF_ESTATE;
     if (sigma > 0) c->sigma = sigma;
@@ -389,7 +392,9 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     const int m = c->m, n = c->n;
     const float cm = (float)(m - 1);
     prof_begin(c, STAGE_OBS);
-    gl_center_kernel<<<S->nr / 8, 256, 0, st>>>(X, n, m, c->m_pad, S->mp, S->xbar, S->xp_hi, S->xp_lo, S->bar);
+    // rows of the analysis: both instants, or the first, which the AR(1) forecast makes both from
+    const int rows = first_only ? c->n_act : n;
+    gl_center_kernel<<<S->nr / 8, 256, 0, st>>>(X, n, rup(rows, 128), m, c->m_pad, S->mp, S->xbar, S->xp_hi, S->xp_lo, S->bar);
     gl_slopes_kernel<<<grid_for((size_t)S->mr * (S->pk >> 4), 256), 256, 0, st>>>(
         X, S->xbar, static_cast<const float*>(yv), S->corner, c->n_subv, c->obs_block == 1 ? c->n_act : 0, m, c->m_pad,
         S->mr, S->pk, (float)(1.0 / c->sigma), S->st_hi, S->st_lo);
@@ -443,20 +448,20 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma) {
     prof_end(c);
     // transform X_a = x_bar + X' W
     prof_begin(c, STAGE_TRANSFORM);
-    g = gemm_args(S->xp_hi, S->xp_lo, S->wt_hi, S->wt_lo, S->mp >> 6, n, m, c->d_status);
+    g = gemm_args(S->xp_hi, S->xp_lo, S->wt_hi, S->wt_lo, S->mp >> 6, rows, m, c->d_status);
     g.mode = GEMM_EPI_ADD_ROW;
     g.c = Xo;
     g.ldc = c->m_pad;
     g.add = S->xbar;
-    if ((rc = gemm_launch(g, S->pl_tr, st))) return rc;
+    if ((rc = gemm_launch(g, first_only ? S->pl_tr1 : S->pl_tr, st))) return rc;
     gl_reject_kernel<<<152, 256, 0, st>>>(X, Xo, (size_t)n * c->m_pad, c->d_frame_bad);
     prof_end(c);
     return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
 
-int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis) {
+int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool first_only) {
     GlobalState* S = c->gstate;
-    if (v_user || !c->Lq || !S) return launch_forecast(c, v_user, xpred, in_analysis);
+    if (v_user || !c->Lq || !S) return launch_forecast(c, v_user, xpred, in_analysis, first_only);
     // V = L xi on the tensor cores (FP32-level), into c->V with leading dimension m
     prof_begin(c, STAGE_NOISE);
     gl_normals_kernel<<<grid_for((size_t)S->mp * (S->ka >> 3), 256), 256, 0, c->stream>>>(
@@ -469,7 +474,7 @@ int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
     const int rc = gemm_launch(g, S->pl_noise, c->stream);
     prof_end(c);
     if (rc) return rc;
-    return launch_forecast(c, c->V, xpred, in_analysis);
+    return launch_forecast(c, c->V, xpred, in_analysis, first_only);
 }
 
 }  // namespace letkf

@@ -168,7 +168,7 @@ size_t plain_smem_bytes(const letkf_ctx* c, int which);
 
 // misc.cu
 int launch_precheck(letkf_ctx* c, const void* y);
-int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis);
+int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool first_only = false);
 int draw_perturbations(letkf_ctx* c, unsigned long long frame);
 // Normals of `frame` into xi, then V = L xi into v_out, on `stream`.
 int draw_perturbations_on(letkf_ctx* c, unsigned long long frame, void* xi, void* v_out, cudaStream_t stream);
@@ -198,8 +198,10 @@ int normals_node_params(letkf_ctx* c, unsigned long long frame, void* xi, Normal
 size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sms);
 int global_prepare(letkf_ctx* c);
 void global_free(letkf_ctx* c);
-int global_analyze(letkf_ctx* c, const void* y, double sigma);
-int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis);
+// first_only: the forecast that follows (global_forecast, in the same call) needs only the first instant's
+// analysis (AR(1)); the second instant's rows of the analysis are then not written, unless the frame is bad.
+int global_analyze(letkf_ctx* c, const void* y, double sigma, bool first_only = false);
+int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool first_only = false);
 
 // gemm.cu: tiled tensor-core GEMM, C = A B^T with tiled BF16 operands (128 x 64 tiles)
 enum GemmEpilogue { GEMM_EPI_F32 = 0, GEMM_EPI_ADD_ROW = 1 };

@@ -70,12 +70,13 @@ __global__ void normals_kernel(O* __restrict__ out, int ld, int n_act, int m, un
 }
 
 // In-place forecast of the ensemble X (n x m_pad) and the mean of the new first instant.
+// first_only: the second instant takes no part (AR(1)) and need not hold an analysis.
 // vmode 0: v from V (ld vld); 1: white noise q * xi drawn inline; 2: no perturbation.
 template <typename T>
 __global__ void forecast_kernel(T* __restrict__ X, const T* __restrict__ V, int vld, int vmode, T q_white,
                                 T a, T a2, int n_act, int m, int m_pad, T* __restrict__ xpred,
                                 const int* __restrict__ frame_bad, int check_bad, unsigned long long seed,
-                                uint32_t frame) {
+                                uint32_t frame, int first_only) {
     const bool skip = check_bad && *frame_bad;
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -90,7 +91,7 @@ __global__ void forecast_kernel(T* __restrict__ X, const T* __restrict__ V, int 
             for (int u = 0; u < 4; ++u) {
                 const int i = i0 + 32 * u;
                 v1[u] = i < m ? x1[i] : (T)0;
-                v2[u] = (i < m && !skip) ? x2[i] : (T)0;
+                v2[u] = (i < m && !skip && !first_only) ? x2[i] : (T)0;
                 v[u] = (i < m && !skip && vmode == 0) ? V[(size_t)j * vld + i] : (T)0;
             }
 #pragma unroll
@@ -543,7 +544,7 @@ int normals_node_params(letkf_ctx* c, unsigned long long frame, void* xi, Normal
     return LETKF_OK;
 }
 
-int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis) {
+int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool first_only) {
     int vmode, vld;
     const void* Vp;
     if (v_user) {
@@ -567,13 +568,13 @@ int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
         forecast_kernel<double><<<g, 256, 0, c->stream>>>((double*)c->X[c->cur], (const double*)Vp, vld, vmode,
                                                           c->q_white, c->a, c->a2, c->n_act, c->m, c->m_pad,
                                                           (double*)xpred, c->d_frame_bad, in_analysis, c->seed,
-                                                          (uint32_t)c->frame);
+                                                          (uint32_t)c->frame, first_only ? 1 : 0);
     else
         forecast_kernel<float><<<g, 256, 0, c->stream>>>((float*)c->X[c->cur], (const float*)Vp, vld, vmode,
                                                          (float)c->q_white, (float)c->a, (float)c->a2, c->n_act, c->m,
                                                          c->m_pad,
                                                          (float*)xpred, c->d_frame_bad, in_analysis, c->seed,
-                                                         (uint32_t)c->frame);
+                                                         (uint32_t)c->frame, first_only ? 1 : 0);
     prof_end(c);
     return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }

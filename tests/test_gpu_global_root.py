@@ -63,3 +63,31 @@ def test_two_filters_on_two_streams():
         for a, b in zip(outs[q], serial[q]):
             assert torch.equal(a, b)
         fs[q].close()
+
+
+@pytest.mark.parametrize("ar2", [False, True])
+def test_step_with_a_rejected_frame(ar2):
+    """A step whose frame is rejected keeps both instants, also where an AR(1) step otherwise writes the first
+    instant's analysis only, and the next step goes on from there as the split calls do."""
+    over = dict(ar1_a=1.2, ar2_a=-0.3) if ar2 else {}
+    y, _ = slopes("tiny-8x8", 3)
+    a, b = LETKF(**_kw("tiny-8x8", 150, **over)), LETKF(**_kw("tiny-8x8", 150, **over))
+    bad = y[1].copy()
+    bad[3] = np.inf
+    a.step(_t(y[0]))
+    s0 = a.get_state()[0].clone()
+    p = a.step(_t(bad))
+    assert a.sync() == _lib.LETKF_ENONFINITE
+    s1 = a.get_state()[0]
+    assert torch.equal(s1, s0)
+    n_act = s0.shape[0] // 2
+    assert rel(p.cpu().numpy(), s0[:n_act].double().mean(dim=1).cpu().numpy()) < 1e-6
+    b.step(_t(y[0]))
+    b.analyze(_t(bad))
+    b.forecast()
+    a.step(_t(y[2]))
+    b.analyze(_t(y[2]))
+    b.forecast()
+    assert torch.equal(a.get_state()[0], b.get_state()[0])
+    a.close()
+    b.close()
