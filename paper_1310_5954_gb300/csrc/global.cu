@@ -51,6 +51,9 @@ struct GlobalState {
     RootStats* stats = nullptr;
     unsigned *dev = nullptr, *bar = nullptr;       // max |P - I| of each step; the grid barrier of the iteration
     int4* corner = nullptr;                        // per valid subaperture: its four corner actuators
+    cudaStream_t side = nullptr;                   // a step's normals, beside its analysis
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    bool forked = false;                           // normals on the side stream that no product has waited for
     std::vector<void*> allocs;
 };
 
@@ -369,22 +372,49 @@ int global_prepare(letkf_ctx* c) {
                     (void*)S->y_lo[0], (void*)S->y_hi[1], (void*)S->y_lo[1], (void*)S->z_hi[0], (void*)S->z_lo[0],
                     (void*)S->z_hi[1], (void*)S->z_lo[1], (void*)S->wt_hi, (void*)S->wt_lo})
         if (cudaMemsetAsync(p, 0, tsq, c->stream) != cudaSuccess) return LETKF_ECUDA;
+    if (dense && (cudaStreamCreateWithFlags(&S->side, cudaStreamNonBlocking) != cudaSuccess ||
+                  cudaEventCreateWithFlags(&S->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+                  cudaEventCreateWithFlags(&S->ev_join, cudaEventDisableTiming) != cudaSuccess))
+        return LETKF_ECUDA;
     return LETKF_OK;
 }
 
 void global_free(letkf_ctx* c) {
     GlobalState* S = c->gstate;
     if (!S) return;
+    if (S->side) {
+        cudaStreamSynchronize(S->side);
+        cudaStreamDestroy(S->side);
+    }
+    if (S->ev_fork) cudaEventDestroy(S->ev_fork);
+    if (S->ev_join) cudaEventDestroy(S->ev_join);
     for (void* p : S->allocs) cudaFree(p);
     delete S;
     c->gstate = nullptr;
 }
 
-int global_analyze(letkf_ctx* c, const void* yv, double sigma, bool first_only) {
+namespace {
+int draw_normals(letkf_ctx* c, GlobalState* S, cudaStream_t stream) {
+    gl_normals_kernel<<<grid_for((size_t)S->mp * (S->ka >> 3), 256), 256, 0, stream>>>(
+        c->seed, (uint32_t)c->frame, c->n_act, c->m, S->mp, S->ka, S->xi_hi, S->xi_lo);
+    return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
+}
+}  // namespace
+
+int global_analyze(letkf_ctx* c, const void* yv, double sigma, bool step) {
     GlobalState* S = c->gstate;
     if (!S) return LETKF_ESTATE;
     if (sigma > 0) c->sigma = sigma;
     cudaStream_t st = c->stream;
+    const bool first_only = step && c->a2 == 0.0;
+    // a step's normals (18 us at n_act = 4833, m = 1024) beside its analysis, most of which waits for memory
+    // or at barriers; the product that reads them comes after it
+    if (step && S->side) {
+        if (cudaEventRecord(S->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(S->side, S->ev_fork, 0) != cudaSuccess ||
+            draw_normals(c, S, S->side) != LETKF_OK || cudaEventRecord(S->ev_join, S->side) != cudaSuccess)
+            return LETKF_ECUDA;
+        S->forked = true;
+    }
     int rc = launch_precheck(c, yv);
     if (rc) return rc;
     const float* X = static_cast<const float*>(c->X[c->cur]);
@@ -459,14 +489,21 @@ int global_analyze(letkf_ctx* c, const void* yv, double sigma, bool first_only) 
     return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
 
-int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool first_only) {
+int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool step) {
     GlobalState* S = c->gstate;
+    const bool first_only = step && c->a2 == 0.0;
     if (v_user || !c->Lq || !S) return launch_forecast(c, v_user, xpred, in_analysis, first_only);
     // V = L xi on the tensor cores (FP32-level), into c->V with leading dimension m
     prof_begin(c, STAGE_NOISE);
-    gl_normals_kernel<<<grid_for((size_t)S->mp * (S->ka >> 3), 256), 256, 0, c->stream>>>(
-        c->seed, (uint32_t)c->frame, c->n_act, c->m, S->mp, S->ka, S->xi_hi, S->xi_lo);
-    if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
+    // (outside a step there is only something to wait for when one failed between its halves)
+    if (S->forked) {
+        if (cudaStreamWaitEvent(c->stream, S->ev_join, 0) != cudaSuccess) return LETKF_ECUDA;
+        S->forked = false;
+    }
+    if (!step) {
+        const int rd = draw_normals(c, S, c->stream);
+        if (rd) return rd;
+    }
     GemmArgs g = gemm_args(S->l_hi, S->l_lo, S->xi_hi, S->xi_lo, S->ka >> 6, c->n_act, c->m, c->d_status);
     g.mode = GEMM_EPI_F32;
     g.c = static_cast<float*>(c->V);

@@ -641,10 +641,9 @@ int letkf_step(letkf_ctx* c, const void* y, double sigma, void* xpred) {
         c->cur ^= 1;
         if ((rc = letkf::launch_forecast(c, nullptr, xp, 1))) return rc;
     } else if (c->path == LETKF_PATH_GLOBAL) {
-        const bool ar1 = c->a2 == 0.0;
-        if ((rc = letkf::global_analyze(c, y, sigma, ar1))) return rc;
+        if ((rc = letkf::global_analyze(c, y, sigma, true))) return rc;
         c->cur ^= 1;
-        if ((rc = letkf::global_forecast(c, nullptr, xp, 1, ar1))) return rc;
+        if ((rc = letkf::global_forecast(c, nullptr, xp, 1, true))) return rc;
     } else {
         if ((rc = letkf::fused_step(c, y, sigma, xp, 1))) return rc;
         c->cur ^= 1;

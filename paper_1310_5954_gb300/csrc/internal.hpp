@@ -198,10 +198,11 @@ int normals_node_params(letkf_ctx* c, unsigned long long frame, void* xi, Normal
 size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sms);
 int global_prepare(letkf_ctx* c);
 void global_free(letkf_ctx* c);
-// first_only: the forecast that follows (global_forecast, in the same call) needs only the first instant's
-// analysis (AR(1)); the second instant's rows of the analysis are then not written, unless the frame is bad.
-int global_analyze(letkf_ctx* c, const void* y, double sigma, bool first_only = false);
-int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool first_only = false);
+// step: global_forecast follows in the same call, with the same `step`.  The frame's normals are then drawn
+// beside the analysis, and for AR(1), whose forecast needs only the first instant's analysis, the second
+// instant's rows of the analysis are not written, unless the frame is bad.
+int global_analyze(letkf_ctx* c, const void* y, double sigma, bool step = false);
+int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool step = false);
 
 // gemm.cu: tiled tensor-core GEMM, C = A B^T with tiled BF16 operands (128 x 64 tiles)
 enum GemmEpilogue { GEMM_EPI_F32 = 0, GEMM_EPI_ADD_ROW = 1 };
