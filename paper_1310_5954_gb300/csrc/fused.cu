@@ -301,22 +301,46 @@ __device__ __forceinline__ float block_sum(Ctrl* ctl, float v) {
 // This thread's half-row of a tensor-memory matrix (from taddr, nq chunks of 8 columns) passed to
 // f(q8, v) chunk by chunk, the next chunk's load in flight while f runs.  f must issue no tensor-
 // memory load of its own.
-template <typename F>
+// PAIRS: two chunks per turn of the loop, without the moves between the two sets of registers.  The
+// passes over tensor memory are bound by their instructions where several warps share a scheduler: two CTAs
+// per SM and the dual form's 512 threads gain (80 x 80 pupil, frame: m = 100 mixed 121.1 -> 118.8 us, m = 200
+// 235.2 -> 232.4), one CTA of 256 threads loses (40 x 40, m = 50: 44.1 -> 44.6 us), its code being fetched for
+// one pass of one domain.
+template <bool PAIRS, typename F>
 __device__ __forceinline__ void tmem_rows(uint32_t taddr, int nq, F&& f) {
     uint32_t rc[8], rn[8];
     tmem_ld8_async(taddr, rc);
     tmem_wait_ld(rc);
+    if constexpr (PAIRS) {
+        auto give = [&](int q8, const uint32_t (&r)[8]) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(r[u]);
+            f(q8, v);
+        };
 #pragma unroll 1
-    for (int q8 = 0; q8 < nq; ++q8) {
-        if (q8 + 1 < nq) tmem_ld8_async(taddr + 8 * (q8 + 1), rn);
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(rc[u]);
-        f(q8, v);
-        if (q8 + 1 < nq) {
+        for (int q8 = 0; q8 < nq; q8 += 2) {
+            if (q8 + 1 < nq) tmem_ld8_async(taddr + 8 * (q8 + 1), rn);
+            give(q8, rc);
+            if (q8 + 1 >= nq) break;
             tmem_wait_ld(rn);
+            if (q8 + 2 < nq) tmem_ld8_async(taddr + 8 * (q8 + 2), rc);
+            give(q8 + 1, rn);
+            if (q8 + 2 < nq) tmem_wait_ld(rc);
+        }
+    } else {
+#pragma unroll 1
+        for (int q8 = 0; q8 < nq; ++q8) {
+            if (q8 + 1 < nq) tmem_ld8_async(taddr + 8 * (q8 + 1), rn);
+            float v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) rc[u] = rn[u];
+            for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(rc[u]);
+            f(q8, v);
+            if (q8 + 1 < nq) {
+                tmem_wait_ld(rn);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) rc[u] = rn[u];
+            }
         }
     }
 }
@@ -801,7 +825,7 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
             if (!mma_wait()) return false;
             it = 1;
             more = true;
-            tmem_rows(tl + TM_Y, nq, [&](int q8, const float (&yv)[8]) {
+            tmem_rows<true>(tl + TM_Y, nq, [&](int q8, const float (&yv)[8]) {
                 if (row < NP) store8_at(Yh, Yl, off0 + 128u * q8, yv, true);
             });
             to_mma();
@@ -816,7 +840,7 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
         }
         if (!mma_wait()) return false;
         float r2 = 0.f;
-        tmem_rows(tl + TM_P, nq, [&](int q8, const float (&pv)[8]) {
+        tmem_rows<true>(tl + TM_P, nq, [&](int q8, const float (&pv)[8]) {
             float tv[8];
             if (!on_diag(q8)) {
 #pragma unroll
@@ -1067,7 +1091,7 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
         }
         if (!mma_wait()) return false;
         float r2 = 0.f;
-        tmem_rows(tl + TM_P, nq, [&](int q8, const float (&qv)[8]) {
+        tmem_rows<true>(tl + TM_P, nq, [&](int q8, const float (&qv)[8]) {
             float rv[8];
             if (!on_diag(q8)) {
 #pragma unroll
@@ -1096,7 +1120,7 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
         }
         if (!mma_wait()) return false;
         if (last) break;                            // X stays in tensor memory
-        tmem_rows(tl + TM_G, nq, [&](int q8, const float (&xv)[8]) {
+        tmem_rows<true>(tl + TM_G, nq, [&](int q8, const float (&xv)[8]) {
             if (row < NP) store8_at(Th, Tl, off0 + 128u * q8, xv, true);
         });
         to_mma();
@@ -1166,7 +1190,7 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
     const int mc0 = ((MP >> 3) * hh >> 2), mq = ((MP >> 3) * (hh + 1) >> 2) - mc0, mcol0 = 8 * mc0;
     const uint32_t moff0 = op_offset(row, mcol0, MP);
     const uint32_t tlm = tbase + lane_off + (uint32_t)mcol0;
-    tmem_rows(tlm + TM_Y, mq, [&](int q8, const float (&wv)[8]) {   // W -> operand over S (zero past P and m)
+    tmem_rows<true>(tlm + TM_Y, mq, [&](int q8, const float (&wv)[8]) {   // W -> operand over S (zero past P and m)
         if (row < NP) store8_at(Wh, Wl, moff0 + 128u * q8, wv, true);
         if (cap && row < P)
 #pragma unroll
@@ -1199,7 +1223,7 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
     if (!mma_wait()) return false;
     unsigned char* Xh_op = big;                     // (I + Z)^-1 operand over A1
     unsigned char* Xl_op = big + A.sz_op;
-    tmem_rows(tl + TM_G, nq, [&](int q8, const float (&xv)[8]) {    // (zero past P)
+    tmem_rows<true>(tl + TM_G, nq, [&](int q8, const float (&xv)[8]) {    // (zero past P)
         if (row < NP) store8_at(Xh_op, Xl_op, off0 + 128u * q8, xv, true);
     });
     to_mma();
@@ -1211,10 +1235,10 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
     if (!mma_wait()) return false;
     unsigned char* A2h = big;                       // P1 (RA x NP) over X's operand
     unsigned char* A2l = big + RA * NP * 2;
-    tmem_rows(tl + TM_P, nq, [&](int q8, const float (&pv)[8]) {    // (columns past P are zero: W's rows are)
+    tmem_rows<true>(tl + TM_P, nq, [&](int q8, const float (&pv)[8]) {    // (columns past P are zero: W's rows are)
         if (row < n_e) store8_at(A2h, A2l, off0 + 128u * q8, pv, A.tr_terms > 1);
     });
-    tmem_rows(tlm + TM_Y, mq, [&](int q8, const float (&wv)[8]) {   // XW -> operand over W (zero past P and m)
+    tmem_rows<true>(tlm + TM_Y, mq, [&](int q8, const float (&wv)[8]) {   // XW -> operand over W (zero past P and m)
         if (row < NP) store8_at(Wh, Wl, moff0 + 128u * q8, wv, true);
         if (cap && row < P)
 #pragma unroll
@@ -1237,7 +1261,7 @@ __device__ __forceinline__ bool analyse_dual(const SysDesc& A, Ctrl* ctl, unsign
     const int pld = MP + 4;
     {
         float part = 0.f;
-        tmem_rows(tlm + TM_Y, mq, [&](int q8, const float (&dv)[8]) {
+        tmem_rows<true>(tlm + TM_Y, mq, [&](int q8, const float (&dv)[8]) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) part += dv[u];          // (zero past m)
             if (mine) {
@@ -2373,7 +2397,7 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
             // ---- 3a. G and b; scale s = 1 + ||G||_F / c, an upper bound of cond((m-1)I + G)
             auto read_gram = [&]() -> float {
                 float fr = 0.f;
-                tmem_rows(tl + tG, nq, [&](int q8, const float (&g)[8]) {
+                tmem_rows<TWO>(tl + tG, nq, [&](int q8, const float (&g)[8]) {
                     if (col0 + 8 * q8 + 8 <= m) {
     #pragma unroll
                         for (int u = 0; u < 8; ++u) fr += g[u] * g[u];
@@ -2443,7 +2467,7 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
             auto on_diag = [&](int q8) { return col0 + 8 * q8 < rw0 + 32 && col0 + 8 * q8 + 8 > rw0; };
             {
                 float r2 = 0.f;
-                tmem_rows(tl + tG, nq, [&](int q8, const float (&g)[8]) {
+                tmem_rows<TWO>(tl + tG, nq, [&](int q8, const float (&g)[8]) {
                     float yv[8], tv[8];
                     if (!on_diag(q8) && rw0 + 32 <= m && col0 + 8 * q8 + 8 <= m) {
     #pragma unroll
@@ -2486,7 +2510,7 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
                 if (!wait_all(ctl, &ctl->bar_mma, ph_mma, A.status)) break;
                 ph_mma ^= 1;
                 tc_fence_after();
-                tmem_rows(tl + tY, nq, [&](int q8, const float (&yv)[8]) { put_y(q8, yv); });
+                tmem_rows<TWO>(tl + tY, nq, [&](int q8, const float (&yv)[8]) { put_y(q8, yv); });
                 if constexpr (TWO) tmem_wait_st();
                 fence_async_smem();
                 tc_fence_before();
@@ -2503,7 +2527,7 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
                 ph_mma ^= 1;
                 tc_fence_after();
                 float r2 = 0.f;
-                tmem_rows(tl + tP, nq, [&](int q8, const float (&pv)[8]) {
+                tmem_rows<TWO>(tl + tP, nq, [&](int q8, const float (&pv)[8]) {
                     float tv[8];
                     if (!on_diag(q8)) {
     #pragma unroll
@@ -2579,14 +2603,14 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
                 ph_mma2 ^= 1;
                 tc_fence_after();
                 if constexpr (TWO) {
-                    tmem_rows(tl + tZ, nq, [&](int q8, const float (&zv)[8]) {
+                    tmem_rows<TWO>(tl + tZ, nq, [&](int q8, const float (&zv)[8]) {
                         if (row < NP) store8_at(Zh, Zl, off0 + 128u * q8, zv, true);
                     });
                     // Y's left operand goes over Z's accumulator: both warps of these lanes have read it
                     tc_fence_before();
                     asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 3)) : "memory");
                     tc_fence_after();
-                    tmem_rows(tl + tY, nq, [&](int q8, const float (&yv)[8]) { put_y(q8, yv); });
+                    tmem_rows<TWO>(tl + tY, nq, [&](int q8, const float (&yv)[8]) { put_y(q8, yv); });
                     tmem_wait_st();
                 } else {
     #pragma unroll 1
@@ -2704,7 +2728,7 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
                 dst[1] = make_float4(zv[4], zv[5], zv[6], zv[7]);
             };
             if (TWO || z_state == 2) {
-                tmem_rows(tl + tZ, nq, zf_put);
+                tmem_rows<TWO>(tl + tZ, nq, zf_put);
             } else {
     #pragma unroll 1
                 for (int q8 = 0; q8 < nq; ++q8) {
@@ -2881,7 +2905,7 @@ __global__ void __launch_bounds__(MODE == MODE_DUAL ? FTD : FT, MODE == MODE_TWO
                     f(q8, dv);
                 }
             } else {
-                tmem_rows(tl + tP, nq, f);
+                tmem_rows<TWO>(tl + tP, nq, f);
             }
         };
         const bool mine = row < n_e;
