@@ -398,8 +398,9 @@ def global_leg(steps, warmup, flush, torch, workers=16):
     status = f.sync()
     m, n, p, na = f.info.m, f.info.n, f.info.p, f.info.n_act
     lower = bool(np.allclose(L, np.tril(L)))
-    work = {"gram": 2.0 * (m + 1) ** 2 * p, "newton_schulz": 2.0 * m ** 3 * (1 + 3 * max(ns_steps - 1, 0)),
-            "transform": 2.0 * n * m * m, "noise": 2.0 * na * na * m / (2.0 if lower else 1.0)}
+    # the first step takes one product, the last one two, an AR(1) step transforms the first instant
+    work = {"gram": 2.0 * (m + 1) ** 2 * p, "newton_schulz": 2.0 * m ** 3 * 3 * max(ns_steps - 1, 0),
+            "transform": 2.0 * (n if w.ar2_a else na) * m * m, "noise": 2.0 * na * na * m / (2.0 if lower else 1.0)}
     tot = sum(work.values())
     t_med = float(np.median(ms)) / 1e3
     f.close()

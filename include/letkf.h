@@ -229,8 +229,8 @@ int letkf_gemm_selftest(const float* A, const float* B, float* C, int M, int N, 
 
 /*
  * letkf_global_stats (LETKF_PATH_GLOBAL): Newton-Schulz steps taken by the last analysis (the
- * first, product-free step included; each further step is three products) and the spectral bound
- * s = 1 + ||G||_F / (m-1) the iteration was scaled by.  Synchronises the context's stream;
+ * first, product-free step included; each further step is three products, the last one two) and the
+ * spectral bound s = 1 + ||G||_F / (m-1) the iteration was scaled by.  Synchronises the context's stream;
  * LETKF_ESTATE on other paths.
  */
 int letkf_global_stats(letkf_ctx* ctx, int* ns_steps, double* s_bound);
@@ -332,8 +332,9 @@ int letkf_get_graph(const letkf_ctx* ctx, int* enabled);
 
 /*
  * Launch tuning of the fused path (the paper has no counterpart).  Neither knob changes any
- * result: fused_grid is the number of CTAs of the fused kernel for this context (0: one per SM,
- * capped at the number of domains; at most the SM count), graph is letkf_set_graph's mode.
+ * result: fused_grid is the number of SMs the fused kernel takes for this context (0: all,
+ * capped at the number of domains; at most the SM count; one CTA on each, or two where the kernel
+ * runs two domains side by side), graph is letkf_set_graph's mode.
  * letkf_autotune times `frames` letkf_step calls with the slopes y_dev (p elements) for each
  * candidate (one CTA per SM, or the fewest CTAs taking the same number of rounds of domains;
  * graph off or on), keeps the fastest and reports it and its milliseconds per frame (either
