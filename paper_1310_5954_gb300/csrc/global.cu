@@ -36,17 +36,17 @@ namespace letkf {
 
 struct GlobalState {
     int mr = 0, pk = 0, mp = 0, nr = 0, ka = 0;   // padded sizes: S' rows, slopes, m, state rows, actuators
-    uint8_t *st_hi = nullptr, *st_lo = nullptr;   // [S d]^T tiles (mr x pk)
+    uint8_t *st_hi = nullptr, *st_lo = nullptr;   // [S d]^T slices (mr x pk)
     float* G = nullptr;                            // m x (m+1) Gram, row-major
     float* Gpart = nullptr;                        // partial Grams of the upper tiles, one per share
     int ldg = 0, gram_split = 1;                   // leading dimension of the Gram, shares of its K steps
     GemmPlan pl_gram, pl_tr, pl_tr1, pl_noise;     // Gram, transform (both instants / the first), noise draw
     uint8_t *as_hi = nullptr, *as_lo = nullptr, *t_hi = nullptr, *t_lo = nullptr;
     uint8_t *y_hi[2] = {}, *y_lo[2] = {}, *z_hi[2] = {}, *z_lo[2] = {};
-    uint8_t *xp_hi = nullptr, *xp_lo = nullptr;    // X' tiles (nr x mp)
-    uint8_t *wt_hi = nullptr, *wt_lo = nullptr;    // W^T tiles (mp x mp)
-    uint8_t *l_hi = nullptr, *l_lo = nullptr;      // L tiles (rup(n_act) x ka)
-    uint8_t *xi_hi = nullptr, *xi_lo = nullptr;    // xi^T tiles (mp x ka)
+    uint8_t *xp_hi = nullptr, *xp_lo = nullptr;    // X' slices (nr x mp)
+    uint8_t *wt_hi = nullptr, *wt_lo = nullptr;    // W^T slices (mp x mp)
+    uint8_t *l_hi = nullptr, *l_lo = nullptr;      // L slices (rup(n_act) x ka)
+    uint8_t *xi_hi = nullptr, *xi_lo = nullptr;    // xi^T slices (mp x ka)
     float *xbar = nullptr, *sq = nullptr, *wbar = nullptr, *u = nullptr, *r = nullptr, *b = nullptr;
     RootStats* stats = nullptr;
     unsigned *dev = nullptr, *bar = nullptr;       // max |P - I| of each step; the grid barrier of the iteration
@@ -58,7 +58,6 @@ struct GlobalState {
 };
 
 namespace {
-
 
 int rup(int v, int a) { return (v + a - 1) / a * a; }
 
@@ -285,7 +284,7 @@ size_t global_bytes(int n_act, int n_subv, int m, bool dense, bool lower, int sm
     const int ka = rup(n_act, 64);
     const size_t gram = (size_t)m * rup(m + 1, 4) * 4;
     const Plans P = plans_for(n_act, n_subv, m, dense, lower, sms);
-    // [S d]^T, the Gram and its shares, A_s, T, Y (2), Z (2), X', W^T (hi and lo tiles each)
+    // [S d]^T, the Gram and its shares, A_s, T, Y (2), Z (2), X', W^T (hi and lo each)
     size_t b = 2 * tiled_bytes(mr, pk) + gram * (1 + P.split) + 12 * tiled_bytes(mp, mp) + 2 * tiled_bytes(nr, mp) +
                2 * tiled_bytes(mp, mp);
     if (dense) b += 2 * tiled_bytes(rup(n_act, 128), ka) + 2 * tiled_bytes(mp, ka);
@@ -362,7 +361,7 @@ int global_prepare(letkf_ctx* c) {
         return LETKF_ECUDA;
     int rc = gemm_prepare();
     if (rc || (rc = root_prepare())) return rc;
-    // tiles of the process-noise factor, once
+    // slices of the process-noise factor, once
     if (dense && (rc = to_tiles(static_cast<const float*>(c->Lq), c->n_act, c->n_act, c->n_act, S->l_hi, S->l_lo, 1,
                                 c->stream)))
         return rc;

@@ -204,7 +204,7 @@ void global_free(letkf_ctx* c);
 int global_analyze(letkf_ctx* c, const void* y, double sigma, bool step = false);
 int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool step = false);
 
-// gemm.cu: tiled tensor-core GEMM, C = A B^T with tiled BF16 operands (128 x 64 tiles)
+// gemm.cu: tensor-core GEMM, C = A B^T with sliced BF16 operands (or C = A M with tiled ones)
 enum GemmEpilogue { GEMM_EPI_F32 = 0, GEMM_EPI_ADD_ROW = 1 };
 // How the tiles of a product are dealt to the clusters of one launch.  A piece is `width` columns (64, 128
 // or 256) of cm row tiles (one per CTA of the cluster), over K steps [kb0, kb1); cluster q does
