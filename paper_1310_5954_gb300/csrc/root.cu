@@ -6,9 +6,9 @@
 // microseconds of work even at m = 1024.  As a graph of launches per product, with the passes before and
 // behind it as kernels of their own, most of the time went into starting them, 12 steps' worth of which
 // found the iteration already finished.  Here the CTAs, one per SM, go from phase to phase through a grid
-// barrier (1.9 us), the ring of operand stages and the tensor-memory accumulators stay set up, the decision
+// barrier (1.6 us), the ring of operand stages and the tensor-memory accumulators stay set up, the decision
 // to stop needs no launch, and the last step leaves out Y, which only a next one would read.  With what
-// is before and behind it: 160 -> 86 us at m = 197, 298 -> 173 us at m = 1024 (107 and 219 us with seven
+// is before and behind it: 160 -> 80 us at m = 197, 298 -> 168 us at m = 1024 (with a slower barrier 86 and 173 us, 107 and 219 with seven
 // plain steps; five are taken, see NsStep).
 //
 // A product is dealt in tiles of 128 x 64, B read MN-major (see gemm.cu): at m = 1024 that is 128 tiles for
@@ -96,17 +96,20 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, unsigned& target, Cta* 
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
         const long long t0 = clock64();
-        while (!cta->abort) {
+        // the load acquires, so that no fence follows the last one; the flag and the clock are looked at now
+        // and then (a second load per turn would delay the first)
+        for (unsigned polls = 1; !cta->abort; ++polls) {
             unsigned seen, gave_up;
-            asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(seen), "=r"(gave_up) : "l"(bar) : "memory");
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
             if (seen >= target) break;
+            if (polls & 63) continue;
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(gave_up) : "l"(bar + 1) : "memory");
             if (gave_up || clock64() - t0 > GEMM_WAIT) cta->abort = 1;
         }
         if (cta->abort) {
             asm volatile("st.relaxed.gpu.global.u32 [%0], 1;" ::"l"(bar + 1) : "memory");
             atomicOr(status, ST_TIMEOUT);
         }
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
     }
     __syncthreads();
     return cta->abort == 0;
