@@ -8,8 +8,8 @@
 // found the iteration already finished.  Here the CTAs, one per SM, go from phase to phase through a grid
 // barrier (1.6 us), the ring of operand stages and the tensor-memory accumulators stay set up, the decision
 // to stop needs no launch, and the last step leaves out Y, which only a next one would read.  With what
-// is before and behind it: 160 -> 80 us at m = 197, 298 -> 168 us at m = 1024 (with a slower barrier 86 and 173 us, 107 and 219 with seven
-// plain steps; five are taken, see NsStep).
+// is before and behind it: 160 -> 80 us at m = 197, 298 -> 168 us at m = 1024 (86 and 173 us with a slower
+// barrier, before that 107 and 219 with seven plain steps; five are taken, see NsStep).
 //
 // A product is dealt in tiles of 128 x 64, B read MN-major (see gemm.cu): at m = 1024 that is 128 tiles for
 // P (9 us: 1.4 until the first operands are there, 6.2 of products at 60 cycles each, 1.2 to read out) and
