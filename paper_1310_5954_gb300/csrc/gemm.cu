@@ -17,12 +17,11 @@
 //
 // What bounds a split product is the time from a stage's refill to its use, about 2500 cycles: a ring of S
 // stages, each M cycles of products, takes (2500 + M) / S per stage.  Per 64 columns of K a 128 x 256 piece
-// has 1548 cycles of products; two whole-tile stages of 96 KB took 2050, four of two slices take 1645.  (One
+// has 1548 cycles of products; two whole-tile stages of 96 KB took 2050, four of two slices take 1674.  (One
 // slice per stage costs more again, 2500: the producer's waits and copies come to 600 cycles per stage.)
-// Narrower pieces take 1410 (128 columns) and 1395 (64).  Two CTAs of a cluster take the two row tiles of a
-// piece and copy half of the B chunk each to both (multicast): 64 KB instead of 96 KB per step from L2, 1645
-// against 1674 cycles alone, and less when all SMs read at once; clusters of four (2 x 2 CTAs, 1555 cycles)
-// leave 8 of 152 SMs idle and lose that again (transform 44 us, noise draw 56 us).
+// Narrower pieces take 1410 (128 columns) and 1395 (64).  Every CTA copies its own operands:
+// pairs of CTAs that shared the columns of B took 55 / 37 us for the noise draw and the Gram, this 53 / 36 (row
+// tiles dealt one by one come out more even).
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -47,8 +46,7 @@ constexpr int GT = 192;                   // threads per CTA: producer warp, MMA
 constexpr int GEMM_EPI = 4 * 32 * 36 * 4;  // 32 rows x 32 columns per epilogue warp, padded rows
 constexpr int GEMM_SMEM = 1024 + 192 * 1024 + GEMM_EPI;
 
-// CM CTAs per cluster, along the rows: they share the columns of B.
-template <int CM, bool MN>
+template <bool MN>
 __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ GemmArgs g) {
     using L = GemmStage<MN>;
     constexpr int BN = MN ? 64 : 256;
@@ -59,11 +57,10 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
     __shared__ int abort_flag, filled;
     const Ring ring = make_ring<MN>(smem, full, empty, g.bn);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, uwarp = uniform_warp();
-    const uint32_t rank = CM > 1 ? cluster_rank() : 0u;
     if (tid == 0) {
         for (int s = 0; s < L::MOST; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], CM);              // every CTA this one's copies reach
+            mbar_init(&empty[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&tfull[a], 1);
@@ -79,17 +76,16 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (CM > 1) cluster_sync();                    // every barrier is initialised before a peer's copy arrives
     const uint32_t tmem = tmem_slot;
     const bool split = g.split != 0;
-    const int cid = blockIdx.x / CM, i0 = g.start[cid], i1 = g.start[cid + 1];
+    const int i0 = g.start[blockIdx.x], i1 = g.start[blockIdx.x + 1];
     struct Work {
         int ty, col0, kb0, kb1, width, share;
     };
     auto work = [&](int i) {
         const int4 it = g.items[i];
         Work w;
-        w.ty = it.x * CM + rank;
+        w.ty = it.x;
         w.width = it.w & 0x3FF;
         w.col0 = it.y;
         w.kb0 = it.z & 0xFFFF;
@@ -102,10 +98,9 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
         bool ok = true;
         for (int i = i0; i < i1 && ok; ++i) {
             const Work w = work(i);
-            // a CTA past the last row tile reads that one's operands (its results are dropped)
-            const RingOperands o = ring_operands<MN>(g.a_hi, split ? g.a_lo : nullptr, g.a_nkb, min(w.ty, g.m_tiles - 1),
-                                                     g.b_hi, g.b_lo, g.b_nkb, w.col0, w.width);
-            ok = ring_fill<CM, MN>(ring, pos, o, rank, w.kb0 * 64 / L::KC, w.kb1 * 64 / L::KC);
+            const RingOperands o = ring_operands<MN>(g.a_hi, split ? g.a_lo : nullptr, g.a_nkb, w.ty, g.b_hi, g.b_lo,
+                                                     g.b_nkb, w.col0, w.width);
+            ok = ring_fill<MN>(ring, pos, o, w.kb0 * 64 / L::KC, w.kb1 * 64 / L::KC);
         }
         filled = pos.c;
         if (!ok) {
@@ -121,7 +116,7 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
             const int acc_i = n & 1;
             ok = n < 2 || mbar_wait_bounded(&tempty[acc_i], ((n >> 1) - 1) & 1, GEMM_WAIT);
             tc_fence_after();
-            ok = ok && ring_issue<CM, MN>(ring, pos, tmem + acc_i * BN, w.width, split, (w.kb1 - w.kb0) * 64 / L::KC);
+            ok = ok && ring_issue<MN>(ring, pos, tmem + acc_i * BN, w.width, split, (w.kb1 - w.kb0) * 64 / L::KC);
             if (ok) mma_commit(&tfull[acc_i]);
         }
         if (!ok) {
@@ -146,12 +141,10 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
             }
             tc_fence_after();
             const int row0 = w.ty * 128, col0 = w.col0, row = row0 + trow;
-            const bool mine = w.ty < g.m_tiles;
 #pragma unroll 1
             for (int c0 = 0; c0 < w.width; c0 += 64) {
                 float v[64];
                 tmem_ld64(tmem + acc_i * BN + ((uint32_t)(quad * 32) << 16) + c0, v);
-                if (!mine) continue;
                 // ADD_ROW: add[row] + acc; F32: acc; valid rows and columns only.  32 columns at a time
                 // through shared memory, so that a warp writes whole 128-byte row pieces
                 float* cz = g.c + (size_t)w.share * g.c_split_stride;
@@ -193,7 +186,6 @@ __global__ void __launch_bounds__(GT, 1) gemm_kernel(const __grid_constant__ Gem
     if (abort_flag && tid == 0) ring_drain(ring, filled);
     tc_fence_before();
     __syncthreads();
-    if (CM > 1) cluster_sync();                    // no peer's copy or arrival comes after a CTA has left
     if (warp == 0) tmem_dealloc(tmem, 2 * BN);
 }
 
@@ -223,23 +215,22 @@ size_t tiled_bytes(int rows, int cols) {
     return (size_t)((rows + 127) / 128) * ((cols + 63) / 64) * GEMM_TILE_B;
 }
 
-// The pieces are dealt longest first, each to the cluster with the least work so far.  A piece costs the
+// The pieces are dealt longest first, each to the CTA with the least work so far.  A piece costs the
 // measured cycles per K step at its width, and its read-out.  Narrow pieces cost more per column but come
 // out more even: every width is tried, also with only the last, uneven round cut up, and the plan whose
-// busiest cluster is done first is taken.  (Noise draw at n_act = 4833, m = 1024, a triangular factor whose
+// busiest CTA is done first is taken.  (Noise draw at n_act = 4833, m = 1024, a triangular factor whose
 // row tiles take 2 to 76 steps: 128 columns, 53 us; with 256 the longest piece alone is 68 us.)
 GemmPlan gemm_plan(const GemmShape& s, int sms) {
     GemmPlan best;
     best.cycles = -1;
-    const int fit = std::max(1, sms / s.cm);
+    const int fit = std::max(1, sms);
     auto cost = [&](const int4& p) -> long long {
         const int w = p.w & 0x3FF, steps = (p.z >> 16) - (p.z & 0xFFFF);
-        const int c = s.mn ? 768 : w == 64 ? 1395 : w == 128 ? 1410 : 1645;
+        const int c = s.mn ? 768 : w == 64 ? 1395 : w == 128 ? 1410 : 1674;
         return (long long)steps * c + 1000 + 8 * w;
     };
-    auto pieces = [&](int row, int col, int width, std::vector<int4>& out) {   // one column group of one row group
-        const int last = std::min(s.m_tiles, (row + 1) * s.cm);      // row tiles [row * cm, last)
-        const int kend = s.lower ? std::min(s.nkb, 2 * last) : s.nkb;
+    auto pieces = [&](int row, int col, int width, std::vector<int4>& out) {   // one column group of one row tile
+        const int kend = s.lower ? std::min(s.nkb, 2 * (row + 1)) : s.nkb;
         for (int k = 0; k < s.ksplit; ++k) {
             const int k0 = (int)((long long)kend * k / s.ksplit), k1 = (int)((long long)kend * (k + 1) / s.ksplit);
             out.push_back(make_int4(row, col, k0 | (k1 << 16), width | (k << 10)));
@@ -248,11 +239,11 @@ GemmPlan gemm_plan(const GemmShape& s, int sms) {
     for (int base = s.bn; base >= 64; base /= 2)
         for (int tail = base; tail >= 64; tail /= 2) {
             std::vector<int4> all;
-            for (int r = 0; r * s.cm < s.m_tiles; ++r)
+            for (int r = 0; r < s.m_tiles; ++r)
                 for (int c = 0; c < s.N;) {
                     int w = base;
                     while (w > 64 && (c % w || c + w > (s.N + 63) / 64 * 64)) w /= 2;
-                    if (!s.upper || c + w > r * s.cm * 128) pieces(r, c, w, all);
+                    if (!s.upper || c + w > r * 128) pieces(r, c, w, all);
                     c += w;
                 }
             auto longer = [&](const int4& a, const int4& b) { return cost(a) > cost(b); };
@@ -270,10 +261,9 @@ GemmPlan gemm_plan(const GemmShape& s, int sms) {
             }
             GemmPlan p;
             p.bn = base;
-            p.cm = s.cm;
-            p.ncl = (int)std::min<size_t>(fit, all.size());
-            std::vector<std::vector<int4>> mine(p.ncl);
-            std::vector<long long> load(p.ncl, 0);
+            p.ncta = (int)std::min<size_t>(fit, all.size());
+            std::vector<std::vector<int4>> mine(p.ncta);
+            std::vector<long long> load(p.ncta, 0);
             for (const int4& it : all) {
                 const int q = (int)(std::min_element(load.begin(), load.end()) - load.begin());
                 mine[q].push_back(it);
@@ -290,48 +280,24 @@ GemmPlan gemm_plan(const GemmShape& s, int sms) {
     return best;
 }
 
-namespace {
-template <typename F>
-int gemm_with(bool mn, int cm, F&& f) {
-    if (mn) return cm == 1 ? f(gemm_kernel<1, true>, GEMM_SMEM) : LETKF_EINVAL;
-    if (cm == 1) return f(gemm_kernel<1, false>, GEMM_SMEM);
-    return cm == 2 ? f(gemm_kernel<2, false>, GEMM_SMEM) : LETKF_EINVAL;
-}
-}  // namespace
-
 int gemm_prepare() {
-    for (int k = 0; k < 3; ++k) {
-        const int rc = gemm_with(k == 2, k == 1 ? 2 : 1, [](auto* fn, int smem) -> int {
-            return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess
-                       ? LETKF_OK
-                       : LETKF_ECUDA;
-        });
-        if (rc) return rc;
-    }
+    for (auto* fn : {gemm_kernel<false>, gemm_kernel<true>})
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM) != cudaSuccess)
+            return LETKF_ECUDA;
     return LETKF_OK;
 }
 
 int gemm_launch(const GemmArgs& g, const GemmPlan& p, cudaStream_t stream) {
-    if ((g.b_mn && p.bn != 64) ||  p.ncl < 1 || !p.d_start || !p.d_items) return LETKF_EINVAL;
+    if ((g.b_mn && p.bn != 64) || p.ncta < 1 || !p.d_start || !p.d_items) return LETKF_EINVAL;
     GemmArgs a = g;
     a.start = p.d_start;
     a.items = p.d_items;
     a.bn = p.bn;
-    return gemm_with(g.b_mn != 0, p.cm, [&](auto* fn, int smem) -> int {
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = p.cm;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg;
-        std::memset(&cfg, 0, sizeof(cfg));
-        cfg.gridDim = dim3(p.cm * p.ncl);
-        cfg.blockDim = dim3(GT);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = stream;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, fn, a) == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
-    });
+    if (g.b_mn)
+        gemm_kernel<true><<<p.ncta, GT, GEMM_SMEM, stream>>>(a);
+    else
+        gemm_kernel<false><<<p.ncta, GT, GEMM_SMEM, stream>>>(a);
+    return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
 
 int to_tiles(const float* src, int R, int K, int ld, void* hi, void* lo, int sliced, cudaStream_t stream) {
@@ -366,7 +332,6 @@ extern "C" int letkf_gemm_selftest(const float* A, const float* B, float* C, int
     shape.nkb = kp / 64;
     shape.bn = bn;
     shape.mn = b_mn;
-    shape.cm = !b_mn && mp > 128 ? 2 : 1;       // as the analysis has it
     GemmPlan plan = gemm_plan(shape, 152);
     // B as tiles of B (N x K) itself, or (b_mn) of B given as K x N, rows padded to 128
     const size_t ab = tiled_bytes(mp, kp), bb = b_mn ? tiled_bytes((K + 127) / 128 * 128, (N + 63) / 64 * 64)
@@ -390,7 +355,6 @@ extern "C" int letkf_gemm_selftest(const float* A, const float* B, float* C, int
         g.a_lo = split ? al : nullptr;
         g.b_hi = bh;
         g.b_lo = split ? bl : nullptr;
-        g.m_tiles = mp / 128;
         g.a_nkb = kp / 64;
         g.b_nkb = b_mn ? (N + 63) / 64 : kp / 64;
         g.b_mn = b_mn;

@@ -72,13 +72,11 @@ __device__ __forceinline__ RingOperands ring_operands(const uint8_t* a_hi, const
     return {a_hi + a, a_lo ? a_lo + a : nullptr, b_hi + b, a_lo ? b_lo + b : nullptr, b_nkb, width};
 }
 
-// Copies steps [k0, k1) (of KC columns) of a piece into the ring; one thread.  CM: CTAs of the cluster, which
-// take the same columns of B; each copies its part of a chunk of B to all of them.  False: a wait ran out.
-template <int CM, bool MN>
-__device__ __forceinline__ bool ring_fill(const Ring& r, RingPos& p, const RingOperands& o, uint32_t rank, int k0, int k1) {
+// Copies steps [k0, k1) (of KC columns) of a piece into the ring; one thread.  False: a wait ran out.
+template <bool MN>
+__device__ __forceinline__ bool ring_fill(const Ring& r, RingPos& p, const RingOperands& o, int k0, int k1) {
     using namespace umma;
     using L = GemmStage<MN>;
-    constexpr uint16_t all = (uint16_t)((1u << CM) - 1u);
     const bool split = o.a_lo != nullptr;
     const uint32_t b_bytes = (uint32_t)o.width * 2 * L::UC;
     const uint32_t stage_bytes = (split ? 2u : 1u) * L::SL * (L::A_BYTES + b_bytes);
@@ -86,13 +84,8 @@ __device__ __forceinline__ bool ring_fill(const Ring& r, RingPos& p, const RingO
     // 256 columns are two consecutive 128-row tiles, copied next to each other so that one descriptor
     // with the same row-group stride spans all 256 rows
     auto copy_b = [&](uint8_t* dst, const uint8_t* src, uint64_t* bar) {
-        if (CM > 1) {
-            const uint32_t part = b_bytes / CM, off = rank * part;
-            bulk_g2s_multicast(dst + off, src + (off / L::A_BYTES) * b_next + off % L::A_BYTES, part, bar, all);
-        } else {
-            bulk_g2s(dst, src, min(b_bytes, (uint32_t)L::A_BYTES), bar);
-            if (b_bytes > L::A_BYTES) bulk_g2s(dst + L::A_BYTES, src + b_next, L::A_BYTES, bar);
-        }
+        bulk_g2s(dst, src, min(b_bytes, (uint32_t)L::A_BYTES), bar);
+        if (b_bytes > L::A_BYTES) bulk_g2s(dst + L::A_BYTES, src + b_next, L::A_BYTES, bar);
     };
     for (int k = k0; k < k1; ++k) {
         uint64_t* full = &r.full[p.s];
@@ -116,11 +109,10 @@ __device__ __forceinline__ bool ring_fill(const Ring& r, RingPos& p, const RingO
 }
 
 // Issues the products of `steps` stages into the accumulator at TMEM column address dt; one elected thread.
-template <int CM, bool MN>
+template <bool MN>
 __device__ __forceinline__ bool ring_issue(const Ring& r, RingPos& p, uint32_t dt, int width, bool split, int steps) {
     using namespace umma;
     using L = GemmStage<MN>;
-    constexpr uint16_t all = (uint16_t)((1u << CM) - 1u);       // their copies fill this CTA's stages
     // A: K-adjacent core matrices 128 B apart, row-adjacent 1024 B in a tile, 256 B in a slice; K-major B
     // alike.  MN-major B: N-adjacent core matrices 128 B apart, K-adjacent 1024 B, a K step 2048 B
     constexpr uint32_t a_sbo = MN ? 1024u : 256u, b_lbo = MN ? 1024u : 128u, b_sbo = MN ? 128u : 256u;
@@ -140,10 +132,7 @@ __device__ __forceinline__ bool ring_issue(const Ring& r, RingPos& p, uint32_t d
                 mma_bf16(dt, sdesc(sa_lo + da, 128, a_sbo), bh, idesc, 1u);
             }
         }
-        if (CM > 1)
-            mma_commit_multicast(&r.empty[p.s], all);
-        else
-            mma_commit(&r.empty[p.s]);
+        mma_commit(&r.empty[p.s]);
         p.next(r.stages);
     }
     return true;

@@ -64,9 +64,6 @@ int rup(int v, int a) { return (v + a - 1) / a * a; }
 // Columns of the slopes' operand: the x and y slopes of eight subapertures to a slice (see gl_slopes_kernel).
 int slope_cols(int n_subv) { return rup(2 * rup(n_subv, 8), 64); }
 
-// Row tiles per cluster of a wide product: they share the 256 columns of B.
-int cluster_rows(int row_tiles) { return row_tiles >= 2 ? 2 : 1; }
-
 // The plans of the analysis's products, and the Gram's shares: as many as make its pieces fill the SMs,
 // against the partial Grams that every share writes and the reduction reads (at 2 KB per cycle).
 struct Plans {
@@ -81,7 +78,6 @@ Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
     g.N = m + 1;
     g.nkb = slope_cols(n_subv) / 64;
     g.bn = 256;
-    g.cm = cluster_rows(mt);
     g.upper = 1;
     long long best = -1;
     for (g.ksplit = 1; g.ksplit <= std::max(1, std::min(g.nkb / 2, 16)); ++g.ksplit) {
@@ -97,10 +93,8 @@ Plans plans_for(int n_act, int n_subv, int m, bool dense, bool lower, int sms) {
     t.N = m;
     t.nkb = rup(m, 128) / 64;
     t.bn = 256;
-    t.cm = cluster_rows(rows);
     P.tr = gemm_plan(t, sms);
     t.m_tiles = acts;
-    t.cm = cluster_rows(acts);
     P.tr1 = gemm_plan(t, sms);
     if (dense) {
         t.nkb = rup(n_act, 64) / 64;
@@ -270,7 +264,6 @@ GemmArgs gemm_args(const uint8_t* ah, const uint8_t* al, const uint8_t* bh, cons
     g.b_lo = bl;
     g.a_nkb = g.b_nkb = nkb;
     g.split = 1;
-    g.m_tiles = (M + 127) / 128;
     g.M = M;
     g.N = N;
     g.status = status;
@@ -322,7 +315,7 @@ int global_prepare(letkf_ctx* c) {
                     std::make_pair(&P.tr1, &S->pl_tr1),
                     std::make_pair(&P.noise, &S->pl_noise)}) {
         GemmPlan& p = *q.first;
-        if (!p.ncl) continue;
+        if (!p.ncta) continue;
         const size_t bi = p.items.size() * sizeof(int4), bs = p.start.size() * sizeof(int);
         ok = ok && get(bi, (void**)&p.d_items) && get(bs, (void**)&p.d_start);
         if (ok && (cudaMemcpy(p.d_items, p.items.data(), bi, cudaMemcpyHostToDevice) != cudaSuccess ||

@@ -206,22 +206,20 @@ int global_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
 
 // gemm.cu: tensor-core GEMM, C = A B^T with sliced BF16 operands (or C = A M with tiled ones)
 enum GemmEpilogue { GEMM_EPI_F32 = 0, GEMM_EPI_ADD_ROW = 1 };
-// How the tiles of a product are dealt to the clusters of one launch.  A piece is `width` columns (64, 128
-// or 256) of cm row tiles (one per CTA of the cluster), over K steps [kb0, kb1); cluster q does
-// items[start[q]] .. items[start[q + 1] - 1].
+// How the tiles of a product are dealt to the CTAs of one launch.  A piece is `width` columns (64, 128 or
+// 256) of one row tile, over K steps [kb0, kb1); CTA q does items[start[q]] .. items[start[q + 1] - 1].
 struct GemmShape {
     int m_tiles = 0, N = 0, nkb = 0;    // row tiles, columns, K / 64
     int bn = 64, mn = 0;                // widest piece; B read MN-major
-    int cm = 1;                         // row tiles (CTAs) per cluster: 1 or 2
     int lower = 0;                      // A is lower triangular: row tile r needs K steps < 2 (r + 1)
     int upper = 0;                      // only pieces that reach the diagonal or lie right of it
     int ksplit = 1;                     // shares of the K steps (partial products)
 };
 struct GemmPlan {
-    int bn = 64, cm = 1, ncl = 0;
-    long long cycles = 0;               // the model's time of the busiest cluster
-    std::vector<int> start;             // ncl + 1
-    std::vector<int4> items;            // row tile group, first column, kb0 | kb1 << 16,
+    int bn = 64, ncta = 0;
+    long long cycles = 0;               // the model's time of the busiest CTA
+    std::vector<int> start;             // ncta + 1
+    std::vector<int4> items;            // row tile, first column, kb0 | kb1 << 16,
                                         // width | share << 10
     int* d_start = nullptr;
     int4* d_items = nullptr;
@@ -233,7 +231,6 @@ struct GemmArgs {
     const uint8_t *a_hi, *a_lo, *b_hi, *b_lo;
     int a_nkb, b_nkb;           // column tiles per row tile of A and B
     int split;                  // 1: hi hi + hi lo + lo hi; 0: single BF16, a_lo and b_lo unused
-    int m_tiles;                // row tiles of A there are
     int bn;                     // the plan: its widest piece, and the pieces
     const int* start;
     const int4* items;

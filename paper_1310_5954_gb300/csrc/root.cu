@@ -156,8 +156,8 @@ __device__ __forceinline__ void products(const Ring& ring, Cta* cta, int& chunks
         for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
             const Product& q = p[t / per];
             const int u = t % per;
-            ok = ring_fill<1, true>(ring, pos, ring_operands<true>(q.a.hi, q.a.lo, nkb, u / ct, q.b.hi, q.b.lo, nkb,
-                                                                   (u % ct) * 64, 64), 0, 0, steps);
+            ok = ring_fill<true>(ring, pos, ring_operands<true>(q.a.hi, q.a.lo, nkb, u / ct, q.b.hi, q.b.lo, nkb,
+                                                                (u % ct) * 64, 64), 0, steps);
         }
         cta->filled = pos.c;
         if (!ok) cta->abort = 1;
@@ -170,7 +170,7 @@ __device__ __forceinline__ void products(const Ring& ring, Cta* cta, int& chunks
         for (int t = blockIdx.x, n = acc; t < total && ok; t += gridDim.x, ++n) {
             ok = n < 2 || mbar_wait_bounded(&cta->tempty[n & 1], ((n >> 1) - 1) & 1, GEMM_WAIT);
             tc_fence_after();
-            ok = ok && ring_issue<1, true>(ring, pos, cta->tmem + (n & 1) * 64, 64, true, steps);
+            ok = ok && ring_issue<true>(ring, pos, cta->tmem + (n & 1) * 64, 64, true, steps);
             if (ok) mma_commit(&cta->tfull[n & 1]);
         }
         if (!ok) cta->abort = 1;
