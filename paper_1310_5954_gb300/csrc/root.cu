@@ -140,7 +140,7 @@ struct Product {
 };
 
 // out = alpha A B + beta I for `count` products of m x m operands in tiles, this CTA's pieces of them; with
-// dev, max |A B - I| over valid entries as well.  Positions beyond m get zeros.  Threads keep the ring's
+// dev, max |A B - I| over valid entries as well (infinite when one is not finite).  Positions beyond m get zeros.  Threads keep the ring's
 // position (chunks) and the number of accumulators used (acc) in step.
 __device__ __forceinline__ void products(const Ring& ring, Cta* cta, int& chunks, int& acc, const Product* p, int count,
                                          int m, int mp, float alpha, float beta, unsigned* dev, int* status) {
@@ -176,7 +176,7 @@ __device__ __forceinline__ void products(const Ring& ring, Cta* cta, int& chunks
         if (!ok) cta->abort = 1;
     } else if (warp < 8) {
         const int quad = warp & 3, half = warp >> 2;      // TMEM lanes and columns of this warp
-        float worst = 0.f;
+        float worst = 0.f, finite = 0.f;     // (fmaxf drops a NaN; 0 x keeps it)
         for (int t = blockIdx.x, n = acc; t < total; t += gridDim.x, ++n) {
             const bool ok = mbar_wait_bounded(&cta->tfull[n & 1], (n >> 1) & 1, GEMM_WAIT);
             if (__any_sync(0xffffffffu, !ok)) {
@@ -203,6 +203,7 @@ __device__ __forceinline__ void products(const Ring& ring, Cta* cta, int& chunks
                     for (int q = 0; q < 8; ++q) {
                         x[q] = __uint_as_float(v[j][q]);
                         worst = fmaxf(worst, fabsf(x[q]));
+                        finite = fmaf(x[q], 0.f, finite);
                         x[q] *= alpha;
                     }
                     store_split(hi + 128 * j, lo + 128 * j, x);
@@ -216,7 +217,10 @@ __device__ __forceinline__ void products(const Ring& ring, Cta* cta, int& chunks
                         const int col = c0 + 8 * j + q;
                         const bool in = row < m && col < m;
                         x[q] = __uint_as_float(v[j][q]);
-                        if (in) worst = fmaxf(worst, fabsf(x[q] - (row == col ? 1.f : 0.f)));
+                        if (in) {
+                            worst = fmaxf(worst, fabsf(x[q] - (row == col ? 1.f : 0.f)));
+                            finite = fmaf(x[q], 0.f, finite);
+                        }
                         x[q] = in ? alpha * x[q] + (row == col ? beta : 0.f) : 0.f;
                     }
                     store_split(hi + 128 * j, lo + 128 * j, x);
@@ -224,7 +228,7 @@ __device__ __forceinline__ void products(const Ring& ring, Cta* cta, int& chunks
             }
         }
         if (dev) {
-            worst = warp_max(worst);
+            worst = warp_max(finite == 0.f ? worst : INFINITY);
             if (lane == 0) cta->red[warp] = worst;
             asm volatile("bar.sync 1, 256;" ::: "memory");
             if (threadIdx.x == 0) {
