@@ -56,8 +56,13 @@ constexpr int ROOT_SMEM = 1024 + GemmStage<true>::RING;
 // 32 x 32 and 40 x 40, frames 1 to 3 of a cold start: anomalies 1.1e-4 against 1.5e-4, mean 4.8e-5 against
 // 4.8e-5, geometric means).  Below s = NS_SCALED_FROM the largest eigenvalue is usually so far below the
 // bound that plain steps are as quick (s = 15: 6 against 5 steps, 10: 5 and 5, 6: 4 and 5).
+//
+// Above s = NS_SCALED_TO the scaled steps are wrong: they raise the rounding along the smallest eigenvalues
+// by up to 2.4 a step, and an ensemble of fewer members than slopes has none there but the constant one.
+// m = 197, 1400 slopes, mean's error against 64 bits, scaled / plain: s = 2e3 7e-5 / 7e-5, 2e4 1.2e-4 /
+// 1.1e-4, 2e6 2.1e-4 / 9e-5, from 2e7 NaN / 7e-5.  Plain steps on A scaled into (0, 1] take over.
 constexpr float NS_SCALE = 2.5f, NS_EDGE = 0.395f, NS_PLAIN = 0.94f;   // NS_EDGE: sqrt(2.5) (3 - 2.5) / 2
-constexpr float NS_SCALED_FROM = 16.f;
+constexpr float NS_SCALED_FROM = 16.f, NS_SCALED_TO = 1e4f;
 struct NsStep {
     float a, b;
     bool plain;
@@ -410,7 +415,7 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         sum = 0.f;
         for (int w = 0; w < RW; ++w) sum += cta.red[w];
         s = 1.f + sqrtf(sum) / a.c;
-        sn = s / NS_SCALE;
+        sn = s <= NS_SCALED_TO ? s / NS_SCALE : s;
     }
 
     // A_s = (I + G/c)/s_ns and the first step's Z_1 = T_0 = (3I - A_s)/2
@@ -448,7 +453,7 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         products(ring, &cta, chunks, acc, &p, 1, m, mp, 1.f, 0.f, nullptr, a.status);
         ok = grid_sync(a.bar, target, &cta, a.status);
     }
-    float l = s >= NS_SCALED_FROM ? ns_first(sn) : 1.f;
+    float l = s >= NS_SCALED_FROM && s <= NS_SCALED_TO ? ns_first(sn) : 1.f;
     for (int k = 1; ok && run && k < NS_MAX; ++k) {
         const NsStep ns = ns_next(l);
         const int from = k & 1, to = from ^ 1;

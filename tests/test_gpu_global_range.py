@@ -55,3 +55,13 @@ def test_a_result_that_is_not_finite_is_reported(n_sub, m, spread):
     # past s ~ 1e7 the iterates of a rank-deficient system overflow the split operands' precision
     xa, _, _, status, _ = _analysis(n_sub, m, spread)
     assert np.isfinite(xa).all() or status == _lib.LETKF_ENOCONV
+
+
+@pytest.mark.parametrize("n_sub,m", [(32, 197), (40, 300)])
+@pytest.mark.parametrize("spread", [30.0, 300.0, 1e3, 1e4])
+def test_high_conditioning(n_sub, m, spread):
+    # s from 1e5 to 4e10; more slopes than members, so that G has full rank
+    xa, xo, kappa, status, _ = _analysis(n_sub, m, spread)
+    assert status == 0
+    e = _errors(xa, xo)
+    assert max(e) <= max(1e-4, 4.0 * np.sqrt(kappa) * 2.0 ** -16), (kappa, e)
