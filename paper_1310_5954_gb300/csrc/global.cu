@@ -2,7 +2,7 @@
 // tensor-core GEMM of gemm.cu.  With S = Y'/sigma (p x m) and d = (y - y_bar)/sigma:
 //
 //   [S d]^T [S d]      one product (K = p) gives G = S^T S, b = S^T d                 (Gram)
-//   A_s = (I + G/c)/s  c = m - 1, s = (1 + ||G||_F / c) / 2.5; eigenvalues in (0, 2.5]
+//   A_s = (I + G/c)/s  c = m - 1, s = 1 + ||G||_F / c, or less by up to 2.5 (root.cu); eigenvalues in (0, 2.5]
 //   Z = A_s^(-1/2)     coupled Newton-Schulz: P = Z Y, T = a I - b P, Y <- Y T, Z <- T Z,
 //                      from Y = A_s, Z = I (first step without products: P = A_s, Z = T)
 //   T_a = Z / sqrt(s) = (I + G/c)^(-1/2),   w_bar = Z^2 b / (c s), refined once against the
@@ -15,8 +15,8 @@
 // factor's tiles read MN-major): the matrices are symmetric in exact arithmetic, but taking
 // A B^T for A B lets the rounding's antisymmetric part grow until the iteration diverges at the
 // conditioning of the first frames (s ~ 1e4).  From the Gram's shares to W^T everything is one
-// cooperative kernel (root.cu); the iteration runs at most ROOT_STEPS steps and stops once
-// max |P - I| < 1e-2 (ST_NOCONV when the limit stops it).
+// cooperative kernel (root.cu); the iteration runs at most ROOT_STEPS steps and stops by the spectrum's known
+// bound and max |P - I| < 1e-2 (ST_NOCONV when the limit stops it).
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

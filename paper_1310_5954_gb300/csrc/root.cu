@@ -36,7 +36,7 @@ using namespace umma;
 namespace {
 
 constexpr int NS_MAX = ROOT_STEPS;
-constexpr float NS_TOL = 1e-2f;   // the last update then lands at ~0.75 NS_TOL^2 ~ 7.5e-5 of max |P - I|
+constexpr float NS_TOL = 1e-2f;   // of max |P - I| at the last step (see NsStep)
 constexpr int RT = 320;           // eight epilogue warps, a producer warp, an MMA warp
 constexpr int RW = RT / 32;
 constexpr int ROOT_SMEM = 1024 + GemmStage<true>::RING;
@@ -47,37 +47,51 @@ constexpr int ROOT_SMEM = 1024 + GemmStage<true>::RING;
 // rho^2 = 3 / (1 + l + l^2), where l and 1 land on the same l' (J. Chen and E. Chow, "A stable scaling of
 // Newton-Schulz for improving the sign function computation of a Hermitian matrix", 2014).  l is known:
 // (I + G/c)/s has no eigenvalue below 1/s, and has that one (the anomalies of a row add up to zero).  rho^2
-// stays below NS_SCALE, so that what is 1 up to rounding lands at NS_EDGE or above; the first step is a plain
-// one on A_s scaled up by NS_SCALE, which is the same.  From l = NS_PLAIN on the steps are plain, and only
-// those may be taken for the last ones (one of them brings 1 - P from 0.12 to 0.01).
+// stays below NS_SCALE, so that what is 1 up to rounding lands at NS_EDGE or above.  The first step is a plain
+// one, from s = NS_WIDE_FROM on A_s scaled up by NS_SCALE, which is the same as that rho (below, l is the
+// larger without: s = 14 0.395 and 0.387, 6 0.395 and 0.578).  From l = NS_PLAIN on the steps are plain.
 //
-// Plain steps needed 7 steps at s = 25 (m = 197) and s = 39 (m = 1024), this 5, and the analysis's
-// error against 64 bits, dominated by the rounding of the iterates, is no larger (16 sizes m = 100 .. 700 on
-// 32 x 32 and 40 x 40, frames 1 to 3 of a cold start: anomalies 1.1e-4 against 1.5e-4, mean 4.8e-5 against
-// 4.8e-5, geometric means).  Below s = NS_SCALED_FROM the largest eigenvalue is usually so far below the
-// bound that plain steps are as quick (s = 15: 6 against 5 steps, 10: 5 and 5, 6: 4 and 5).
+// When to stop is known from l as well: the update from l >= NS_DONE is the last, and leaves every x within
+// 1.5 (1 - NS_DONE)^2 = 3e-5 of 1.  max |P - I| < NS_TOL must hold as well, which rounding can break; alone it
+// does not do, since an element of v v^T shows 1/m of what is left along a direction v (with it alone, and plain
+// steps up to s = 16: anomalies off by 7e-3 at s = 2.5, m = 300, by 6e-4 at s = 25; now 1e-5 and 2e-5).
+//
+// Unscaled plain steps, stopped by max |P - I| alone, needed 7 steps at s = 25 (m = 197) and s = 39 (m = 1024),
+// this 5; at s = 1 / 2 / 4 / 10 they need 2 / 4 / 5 / 6, this 2 / 3 / 4 / 5.  The error against 64 bits, dominated
+// by the rounding of the iterates, is no larger (geometric means, s = 1 .. 60, m = 64 .. 240: 7.1e-6 to 1.1e-5
+// against 7.6e-6 to 1.8e-5; 16 sizes m = 100 .. 700 on 32 x 32 and 40 x 40, frames 1 to 3 of a cold start:
+// anomalies 1.1e-4 against 1.5e-4, mean 4.8e-5 against 4.8e-5).
 //
 // Above s = NS_SCALED_TO the scaled steps are wrong: they raise the rounding along the smallest eigenvalues
 // by up to 2.4 a step, and an ensemble of fewer members than slopes has none there but the constant one.
 // m = 197, 1400 slopes, mean's error against 64 bits, scaled / plain: s = 2e3 7e-5 / 7e-5, 2e4 1.2e-4 /
-// 1.1e-4, 2e6 2.1e-4 / 9e-5, from 2e7 NaN / 7e-5.  Plain steps on A scaled into (0, 1] take over.
-constexpr float NS_SCALE = 2.5f, NS_EDGE = 0.395f, NS_PLAIN = 0.94f;   // NS_EDGE: sqrt(2.5) (3 - 2.5) / 2
-constexpr float NS_SCALED_FROM = 16.f, NS_SCALED_TO = 1e4f;
+// 1.1e-4, 2e6 2.1e-4 / 9e-5, from 2e7 NaN / 7e-5.  Unscaled plain steps take over (l = 1), stopped by
+// max |P - I| alone: the bulk of the spectrum, at its low end there, comes last, and is on the diagonal.
+constexpr float NS_SCALE = 2.5f, NS_EDGE = 0.395f;   // NS_EDGE: sqrt(2.5) (3 - 2.5) / 2
+constexpr float NS_PLAIN = 0.94f, NS_DONE = 0.9955f;
+constexpr float NS_WIDE_FROM = 14.f, NS_SCALED_TO = 1e4f;
 struct NsStep {
     float a, b;
-    bool plain;
+    bool last;          // as far as l tells
 };
-// The bound l after the first step; s_ns = s / NS_SCALE.
-__device__ __forceinline__ float ns_first(float s_ns) {
-    const float l2 = 1.f / s_ns;
-    return fminf(0.5f * sqrtf(l2) * (3.f - l2), NS_EDGE);
+// The scale of A_s, and the bound l after the first step.
+__device__ __forceinline__ float ns_scale(float s) { return s >= NS_WIDE_FROM && s <= NS_SCALED_TO ? s / NS_SCALE : s; }
+__device__ __forceinline__ float ns_first(float s) {
+    if (!(s <= NS_SCALED_TO)) return 1.f;
+    const float l2 = 1.f / ns_scale(s), l = 0.5f * sqrtf(l2) * (3.f - l2);
+    return s >= NS_WIDE_FROM ? fminf(l, NS_EDGE) : l;
 }
 // The next step, and the bound behind it.
 __device__ __forceinline__ NsStep ns_next(float& l) {
-    if (!(l < NS_PLAIN)) return {1.5f, 0.5f, true};
-    const float r2 = fminf(NS_SCALE, 3.f / (1.f + l + l * l)), r = sqrtf(r2);
-    const NsStep t = {1.5f * r, 0.5f * r * r2, false};
-    l = fminf(l * (t.a - t.b * l * l), t.a - t.b);
+    NsStep t = {1.5f, 0.5f, l >= NS_DONE};
+    if (l < NS_PLAIN) {
+        const float r2 = fminf(NS_SCALE, 3.f / (1.f + l + l * l)), r = sqrtf(r2);
+        t.a = 1.5f * r;
+        t.b = 0.5f * r * r2;
+        l = fminf(l * (t.a - t.b * l * l), t.a - t.b);
+    } else {
+        l *= t.a - t.b * l * l;
+    }
     return t;
 }
 
@@ -415,7 +429,7 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         sum = 0.f;
         for (int w = 0; w < RW; ++w) sum += cta.red[w];
         s = 1.f + sqrtf(sum) / a.c;
-        sn = s <= NS_SCALED_TO ? s / NS_SCALE : s;
+        sn = ns_scale(s);
     }
 
     // A_s = (I + G/c)/s_ns and the first step's Z_1 = T_0 = (3I - A_s)/2
@@ -453,7 +467,7 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         products(ring, &cta, chunks, acc, &p, 1, m, mp, 1.f, 0.f, nullptr, a.status);
         ok = grid_sync(a.bar, target, &cta, a.status);
     }
-    float l = s >= NS_SCALED_FROM && s <= NS_SCALED_TO ? ns_first(sn) : 1.f;
+    float l = ns_first(s);
     for (int k = 1; ok && run && k < NS_MAX; ++k) {
         const NsStep ns = ns_next(l);
         const int from = k & 1, to = from ^ 1;
@@ -461,7 +475,7 @@ __global__ void __launch_bounds__(RT, 1) root_kernel(const __grid_constant__ Roo
         products(ring, &cta, chunks, acc, &p, 1, m, mp, -ns.b, ns.a, a.dev + k, a.status);
         ok = grid_sync(a.bar, target, &cta, a.status);
         if (!ok) break;
-        run = !ns.plain || __uint_as_float(__ldcg(a.dev + k)) >= NS_TOL;     // whether a step follows, which needs Y
+        run = !ns.last || __uint_as_float(__ldcg(a.dev + k)) >= NS_TOL;      // whether a step follows, which needs Y
         const Product two[2] = {{tt, z[from], z[to]}, {y[from], tt, y[to]}};
         products(ring, &cta, chunks, acc, two, run ? 2 : 1, m, mp, 1.f, 0.f, nullptr, a.status);
         ok = grid_sync(a.bar, target, &cta, a.status);

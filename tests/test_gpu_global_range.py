@@ -65,3 +65,17 @@ def test_high_conditioning(n_sub, m, spread):
     assert status == 0
     e = _errors(xa, xo)
     assert max(e) <= max(1e-4, 4.0 * np.sqrt(kappa) * 2.0 ** -16), (kappa, e)
+
+
+# what max |I - P| < 1e-2 on the diagonal leaves of a uniform deviation, 3/8 of its square, and the rounding
+# of the iterates: 4 sqrt(kappa) 2^-16 at least 1e-4 covers both at these kappa
+@pytest.mark.parametrize("n_sub,m", [(16, 64), (24, 300), (32, 197)])
+@pytest.mark.parametrize("spread", [1e-6, 0.01, 0.05, 0.1, 0.126, 0.158, 0.2, 0.25, 0.3, 0.4, 0.5, 0.63])
+def test_low_conditioning(n_sub, m, spread):
+    for seed in range(3):
+        xa, xo, kappa, status, (steps, s) = _analysis(n_sub, m, spread, seed)
+        assert status == 0
+        e = _errors(xa, xo)
+        assert max(e) <= max(1e-4, 4.0 * np.sqrt(kappa) * 2.0 ** -16), (s, steps, kappa, e)
+        if spread < 1e-3:
+            assert steps == 2, (s, steps)     # G = 0 but for rounding: the first step is exact
