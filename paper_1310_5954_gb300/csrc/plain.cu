@@ -312,9 +312,12 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
         }
         sg = warp_sum(sg);                 // every warp forms the reflector itself: no barrier
         const T x0 = __shfl_sync(0xffffffffu, v[0], 0), nrm = sqrt(sg);
-        const T al = x0 >= (T)0 ? -nrm : nrm;
+        // a row as small as that beside the unit diagonal of B is left alone: its square, or 1 / vv, may be
+        // out of range (FP32: an ensemble's spread below 1e-10 sigma)
+        const bool flat = sg <= (sizeof(T) == 8 ? (T)1e-40 : (T)1e-24);
+        const T al = flat ? x0 : x0 >= (T)0 ? -nrm : nrm;
         const T vv = sg + fabs(x0) * nrm;  // v^T v / 2
-        const T beta = vv > (T)0 ? (T)1 / vv : (T)0;
+        const T beta = flat ? (T)0 : (T)1 / vv;
         if (lane == 0) v[0] = x0 - al;
         for (int r = k1 + warp; r < m; r += 2 * nw) {   // p = beta S v, two rows in flight
             const int r2 = r + nw < m ? r + nw : r;
