@@ -57,9 +57,10 @@ typedef enum letkf_status {
     LETKF_ETIMEOUT = -4,    /* a bounded device-side wait gave up */
     LETKF_ENONFINITE = -5,  /* non-finite slopes: that frame was rejected, state unchanged */
     LETKF_ESTATE = -6,      /* call out of order (e.g. analyze twice without a forecast) */
-    LETKF_ENOCONV = -7,     /* an inverse square root (fused and global paths: Newton-Schulz steps) hit
-                               its iteration limit (result still written); the plain path's is a
-                               direct method */
+    LETKF_ENOCONV = -7,     /* an inverse square root (fused and global paths: Newton-Schulz steps;
+                               plain path: Jacobi sweeps, in ill-conditioned domains) hit its iteration
+                               limit or met a matrix that is not numerically positive definite (result
+                               still written) */
     LETKF_ESCRATCH = -8,    /* the problem does not fit letkf_analyze_static's fixed scratch */
     LETKF_EBUSY = -9        /* refused for now (letkf_serve.h): HBM budget or frame queue full */
 } letkf_status;

@@ -3,7 +3,8 @@
 //
 //   plain_obs        halo anomalies -> Fried slopes S = Y'/sigma (p_loc x m), d/sigma
 //   plain_gram       G = S^T S (m x m), b = S^T d/sigma
-//   plain_eig        T = (I + G/(m-1))^(-1/2) through its tridiagonal form in shared memory;
+//   plain_eig        T = (I + G/(m-1))^(-1/2) through its tridiagonal form in shared memory, or by
+//                    two-sided Jacobi where it is ill conditioned;
 //                    W = T + w_bar 1^T with w_bar = T (T b) / (m-1), refined
 //   plain_transform  X_a[E] = x_bar[E] 1^T + X'[E] W on the domain's own rows
 //
@@ -254,6 +255,153 @@ __device__ __forceinline__ void sincos_halfpi<float>(float a, float& s, float& c
 template <>
 __device__ __forceinline__ void sincos_halfpi<double>(double a, double& s, double& c) { sincospi(0.5 * a, &s, &c); }
 
+// ---- ill-conditioned domains: cyclic two-sided Jacobi
+//
+// A rotation is skipped when |a_pq| <= jacobi_tol sqrt(a_pp a_qq), the relative test that gives eigenvalues
+// and eigenvectors to working relative accuracy for positive definite matrices.  In FP32 the off-diagonal
+// rounding floor after a rotation is a few units of roundoff of the larger diagonal, so the threshold sits a
+// little above it and the sweeps end.
+template <typename T>
+constexpr T jacobi_tol = sizeof(T) == 8 ? (T)1e-14 : (T)3e-6;
+constexpr int JACOBI_SWEEPS = 40;
+
+// Round-robin pairing of M (even) indices: step s, pair k.
+__device__ __forceinline__ void rr_pair(int M, int s, int k, int& p, int& q) {
+    const int a = k == 0 ? s : (s + k) % (M - 1), b = k == 0 ? M - 1 : (s - k + M - 1) % (M - 1);
+    p = min(a, b);
+    q = max(a, b);
+}
+
+// Weights of one domain from the eigendecomposition (m-1)I + G = U diag(lambda) U^T:
+// W = U diag(sqrt((m-1)/lambda)) U^T + w_bar 1^T, w_bar = U diag(1/lambda) U^T b, refined once with the
+// residual in FP64.  A (padded to even order M with a zero row and column) and U in shared memory.  In exact
+// arithmetic no lambda is below m - 1; rounding can take one there, and ST_NOCONV tells that the matrix was not
+// numerically positive definite.
+template <typename T>
+__device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* __restrict__ bd, T* __restrict__ Wd, int m,
+                                            int m_pad, unsigned char* smem, int* status) {
+    const int M = m + (m & 1), ld = M + 1, half = M / 2, tid = threadIdx.x, nt = blockDim.x;
+    const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
+    T* A = reinterpret_cast<T*>(smem);
+    T* V = A + M * ld;
+    T* cs = V + M * ld;                        // M/2 (c, s) pairs
+    int* pq = reinterpret_cast<int*>(cs + M);  // M/2 (p, q) pairs
+    T* rv = reinterpret_cast<T*>(pq + M);      // refinement: residual, then U^T r / lambda
+    T* tv = rv + M;
+    __shared__ int nrot;
+    const T c0 = (T)(m - 1);
+    __syncthreads();                           // the caller's reads are done
+    for (int i = warp; i < M; i += nw)
+        for (int j = lane; j < M; j += 32) {
+            A[i * ld + j] = (i < m && j < m ? Gd[(size_t)i * m_pad + j] : (T)0) + (i == j && i < m ? c0 : (T)0);
+            V[i * ld + j] = i == j ? (T)1 : (T)0;
+        }
+    int sweep = 0;
+    for (; sweep < JACOBI_SWEEPS; ++sweep) {
+        if (tid == 0) nrot = 0;
+        __syncthreads();
+        for (int s = 0; s < M - 1; ++s) {
+            for (int k = tid; k < half; k += nt) {
+                int p, q;
+                rr_pair(M, s, k, p, q);
+                const T apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
+                T c = 1, sn = 0;
+                if (fabs(apq) > jacobi_tol<T> * sqrt(fabs(app * aqq))) {
+                    const T tau = (aqq - app) / ((T)2 * apq);
+                    const T t = (tau >= (T)0 ? (T)1 : (T)-1) / (fabs(tau) + sqrt((T)1 + tau * tau));
+                    c = (T)1 / sqrt((T)1 + t * t);
+                    sn = t * c;
+                    atomicAdd(&nrot, 1);
+                }
+                cs[2 * k] = c;
+                cs[2 * k + 1] = sn;
+                pq[2 * k] = p;
+                pq[2 * k + 1] = q;
+            }
+            __syncthreads();
+            // A <- J^T A J on the 2 x 2 blocks of paired rows P x paired columns Q, P <= Q; A stays symmetric, so
+            // the blocks above the diagonal also write their transposes.  Rows r and half - 1 - r of the
+            // triangle have half + 1 blocks together
+            for (int blk = tid; blk < half * (half + 1) / 2; blk += nt) {
+                const int r = blk / (half + 1), c = blk - r * (half + 1);
+                const int P = c < half - r ? r : half - 1 - r, Q = c < half - r ? r + c : c - 1;
+                const int pP = pq[2 * P], qP = pq[2 * P + 1], pQ = pq[2 * Q], qQ = pq[2 * Q + 1];
+                const T cP = cs[2 * P], sP = cs[2 * P + 1], cQ = cs[2 * Q], sQ = cs[2 * Q + 1];
+                const T b00 = A[pP * ld + pQ], b01 = A[pP * ld + qQ];
+                const T b10 = A[qP * ld + pQ], b11 = A[qP * ld + qQ];
+                const T r00 = cP * b00 - sP * b10, r01 = cP * b01 - sP * b11;
+                const T r10 = sP * b00 + cP * b10, r11 = sP * b01 + cP * b11;
+                const T n00 = cQ * r00 - sQ * r01, n01 = sQ * r00 + cQ * r01;
+                const T n10 = cQ * r10 - sQ * r11, n11 = sQ * r10 + cQ * r11;
+                A[pP * ld + pQ] = n00;
+                A[pP * ld + qQ] = n01;
+                A[qP * ld + pQ] = n10;
+                A[qP * ld + qQ] = n11;
+                if (P != Q) {
+                    A[pQ * ld + pP] = n00;
+                    A[qQ * ld + pP] = n01;
+                    A[pQ * ld + qP] = n10;
+                    A[qQ * ld + qP] = n11;
+                }
+            }
+            for (int e = tid; e < half * M; e += nt) {     // V <- V J
+                const int P = e / M, i = e - P * M, p = pq[2 * P], q = pq[2 * P + 1];
+                const T c = cs[2 * P], sn = cs[2 * P + 1], vp = V[i * ld + p], vq = V[i * ld + q];
+                V[i * ld + p] = c * vp - sn * vq;
+                V[i * ld + q] = sn * vp + c * vq;
+            }
+            __syncthreads();
+        }
+        const int nr = nrot;
+        __syncthreads();                       // every thread has read nrot before thread 0 resets it
+        if (nr == 0) break;
+    }
+    // f_i = sqrt((m-1)/lambda_i) in A's padding column M, w_bar in V's
+    T* z = cs;
+    bool bad = sweep == JACOBI_SWEEPS;
+    for (int i = tid; i < m; i += nt) {
+        T lam = A[i * ld + i];
+        bad = bad || !(lam > (T)0);
+        lam = lam < c0 ? c0 : lam;
+        T s = 0;
+        for (int k = 0; k < m; ++k) s += V[k * ld + i] * bd[k];
+        z[i] = s / lam;
+        A[i * ld + i] = lam;
+        A[i * ld + M] = sqrt(c0 / lam);
+    }
+    if (__syncthreads_or(bad) && tid == 0) atomicOr(status, ST_NOCONV);
+    for (int k = tid; k < m; k += nt) {
+        T s = 0;
+        for (int i = 0; i < m; ++i) s += V[k * ld + i] * z[i];
+        V[k * ld + M] = s;
+    }
+    __syncthreads();
+    for (int k = tid; k < m; k += nt) {
+        double acc = (double)bd[k] - (double)c0 * (double)V[k * ld + M];
+        for (int j = 0; j < m; ++j) acc -= (double)Gd[(size_t)k * m_pad + j] * (double)V[j * ld + M];
+        rv[k] = (T)acc;
+    }
+    __syncthreads();
+    for (int i = tid; i < m; i += nt) {
+        T s = 0;
+        for (int k = 0; k < m; ++k) s += V[k * ld + i] * rv[k];
+        tv[i] = s / A[i * ld + i];
+    }
+    __syncthreads();
+    for (int k = tid; k < m; k += nt) {
+        T s = 0;
+        for (int i = 0; i < m; ++i) s += V[k * ld + i] * tv[i];
+        V[k * ld + M] += s;
+    }
+    __syncthreads();
+    for (int k = warp; k < m; k += nw)
+        for (int l = lane; l < m; l += 32) {
+            T t = 0;
+            for (int i = 0; i < m; ++i) t += V[k * ld + i] * A[i * ld + M] * V[l * ld + i];
+            Wd[(size_t)k * m_pad + l] = t + V[k * ld + M];
+        }
+}
+
 // The inverse square root needs no eigenvectors.  With B = I + G/(m-1) = Q J Q^T (J tridiagonal,
 // Q a product of m - 2 Householder reflectors; Golub and Van Loan, Matrix Computations, 8.3.1),
 //   T = B^(-1/2) = Q J^(-1/2) Q^T,
@@ -262,20 +410,28 @@ __device__ __forceinline__ void sincos_halfpi<double>(double a, double& s, doubl
 // spectrum [1, kappa]: sn, cn, dn at (n - 1/2) K' / N for the parameter 1 - 1/kappa.  Every term is
 // positive definite, and N = 0.88 (ln kappa + 3) + 2 (FP32) or 1.82 (ln kappa + 3) + 2 (FP64) nodes
 // leave less than the rounding (the rule's error is exp(-2 pi^2 N / (ln kappa + 3)); kappa is bounded
-// by J's Gershgorin circles).  The inverse of a tridiagonal matrix costs O(m) divisions (the pivots
-// from both ends) and one multiplication per entry, so the work is that of the reflectors: 4/3 m^3
-// multiply-adds to reduce, 4 m^3 in all, against 9 sweeps of m^3 by two-sided Jacobi, which this
-// replaces, and 2 barriers per column instead of 2 per rotation step and sweep.
+// by J's Gershgorin circles).  That holds while kappa times the unit roundoff is small, since the reduction
+// moves J's smallest eigenvalues, 1, by that much, where Jacobi's rotations keep them.  Where the bound is above
+// DIRECT_TO the domain is done by Jacobi.  72 slopes, anomalies' error of Jacobi / direct, geometric means: FP32,
+// m = 16: kappa 3e2 2.0e-6 / 1.6e-6, 1e3 2.1e-6 / 2.3e-6, 3.5e3 2.3e-6 / 3.1e-6; m = 20: 3.5e3 6.1e-6 / 5.8e-6,
+// 6e5 7.5e-6 / 1.6e-4, 4e7 2.7e-5 / 0.2; FP64, m = 20: 6e4 1.5e-14 / 2.0e-14, 6e5 2.8e-14 / 3.1e-13.  (In a running
+// loop kappa is 5 to 20, in its first two frames 1e3 to 1e4.)
+//
+// The inverse of a tridiagonal matrix costs O(m) divisions (the pivots from both ends) and one multiplication
+// per entry, so the work is that of the reflectors: 4/3 m^3 multiply-adds to reduce, 4 m^3 in all, against 9
+// sweeps of m^3 by Jacobi, which takes 4 to 9 times as long, and 2 barriers per column instead of 2 per rotation
+// step and sweep.
 //
 // What bounds it: the m - 2 dependent reduction steps (two barriers each, the trailing matrix's
 // matrix-vector product and rank-2 update between them); the reflectors are then applied to J's
 // function column by column, 8 lanes and two columns per thread group, in registers and without a
-// barrier.  Measured, whole stage: 92 domains of m = 50 in FP32 522 -> 110 us, 4 domains of m = 20 in
-// FP64 499 -> 148 us (before: Jacobi; 183 with the nodes eight at a time).
+// barrier.  Measured, whole stage: 92 domains of m = 50 in FP32 522 -> 112 us, 4 domains of m = 20 in
+// FP64 499 -> 149 us (before: Jacobi; 183 with the nodes eight at a time).
+constexpr float DIRECT_TO = 2048.f;
 template <typename T, int UM>   // m <= 32 UM members; 4 threads per member, at most 640
 __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __restrict__ G,
                                                                      const T* __restrict__ bvec, T* __restrict__ W,
-                                                                     int m, int m_pad, int kb,
+                                                                     int m, int m_pad, int kb, int* status,
                                                                      const int* __restrict__ frame_bad) {
     extern __shared__ unsigned char smem_raw[];
     const int ld = m | 1;                  // odd row stride: no bank conflicts down a column
@@ -383,6 +539,10 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
     for (int i = lane; i < m; i += 32) hi = fmax(hi, fabs(dd[i]) + fabs(ee[i]) + (i > 0 ? fabs(ee[i - 1]) : (T)0));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    if (!(hi <= DIRECT_TO)) {              // (a NaN as well)
+        jacobi_weights(Gd, bvec + (size_t)d * m_pad, W + (size_t)d * m * m_pad, m, m_pad, smem_raw, status);
+        return;
+    }
     const float rate = sizeof(T) == 8 ? 1.83f : 0.88f;
     const int N = max(1, min(128, (int)(rate * (logf((float)hi) + 3.f)) + 3));
     // descending Landen chain of the modulus: k_0' = kappa^(-1/2), k_(s+1) = (1 - k_s')/(1 + k_s'),
@@ -580,6 +740,12 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
     }
 }
 
+// Dynamic shared memory of jacobi_weights: A and U of even order, the rotations, two vectors.
+size_t jacobi_smem(int m, size_t eb) {
+    const size_t M = m + (m & 1);
+    return 2 * M * (M + 1) * eb + M * (3 * eb + 4);
+}
+
 // Dynamic shared memory of plain_eig: B and F (m x m, odd row stride), vectors, kb nodes' recursions.
 template <typename T>
 size_t eig_smem(int m, int kb) {
@@ -590,19 +756,19 @@ size_t eig_smem(int m, int kb) {
 // least four warps; as many nodes per pass, up to kNodes, as shared memory leaves room for (all of
 // them up to m = 161 in FP32 and 104 in FP64).
 template <typename T>
-void launch_eig(int n_dom, cudaStream_t st, const T* G, const T* b, T* W, int m, int m_pad, const int* bad) {
+void launch_eig(int n_dom, cudaStream_t st, const T* G, const T* b, T* W, int m, int m_pad, int* status, const int* bad) {
     const int nt = std::min(640, std::max(128, (4 * m + 31) / 32 * 32));
     int kb = kNodes<T>;
-    while (kb > 1 && eig_smem<T>(m, kb) > 227 * 1024) --kb;
-    const size_t sm = eig_smem<T>(m, kb);
+    while (kb > 1 && eig_smem<T>(m, kb) > 227 * 1024 - 64) --kb;   // (64: jacobi_weights' own variable)
+    const size_t sm = std::max(eig_smem<T>(m, kb), jacobi_smem(m, sizeof(T)));
     if (m <= 32)
-        plain_eig<T, 1><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, bad);
+        plain_eig<T, 1><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, status, bad);
     else if (m <= 64)
-        plain_eig<T, 2><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, bad);
+        plain_eig<T, 2><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, status, bad);
     else if (m <= 128)
-        plain_eig<T, 4><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, bad);
+        plain_eig<T, 4><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, status, bad);
     else if constexpr (sizeof(T) == 4)     // FP64 ends at m = 118 (plain_limits_ok)
-        plain_eig<T, 6><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, bad);
+        plain_eig<T, 6><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, status, bad);
 }
 
 // X_out[E] = x_bar[E] 1^T + X'[E] W for the domain's own rows E (both instants), the rows shared by
@@ -715,7 +881,7 @@ int plain_analyze_t(letkf_ctx* c, const T* y, double sigma) {
     prof_end(c);
     prof_begin(c, STAGE_EIG);
     launch_eig<T>(nd, c->stream, static_cast<const T*>(c->G), static_cast<const T*>(c->b), static_cast<T*>(c->W), m, mp,
-                  c->d_frame_bad);
+                  c->d_status, c->d_frame_bad);
     prof_end(c);
     prof_begin(c, STAGE_TRANSFORM);
     plain_transform<T><<<shared_by, kThreads, sm_tr, c->stream>>>(X, Xo, static_cast<const T*>(c->W), c->tab, m, mp,
@@ -728,12 +894,9 @@ int plain_analyze_t(letkf_ctx* c, const T* y, double sigma) {
 }  // namespace
 
 int plain_limits_ok(int precision, int m) {
-    // plain_eig keeps two matrices of order m and its vectors in shared memory (<= 227 KB; the bound
-    // below, on two matrices of even order, is the tighter one)
-    const size_t eb = precision == LETKF_PREC_FP64 ? 8 : 4;
-    const int M = m + (m & 1);
-    const size_t bytes = 2 * (size_t)M * (M + 1) * eb + (size_t)M * (3 * eb + 4);
-    return bytes <= 227 * 1024 && m <= 256;
+    // plain_eig keeps two matrices of order m and its vectors in shared memory (<= 227 KB; Jacobi's, of even
+    // order, is the tighter bound)
+    return jacobi_smem(m, precision == LETKF_PREC_FP64 ? 8 : 4) <= 227 * 1024 && m <= 256;
 }
 
 int plain_analyze(letkf_ctx* c, const void* y, double sigma) {
@@ -834,7 +997,7 @@ int analyze_static_t(letkf_ctx* c, const T* y, double sigma, T* out) {
     plain_obs<T><<<nd, kThreads, sm_obs, c->stream>>>(X, y, c->tab, c->so_off, S, dt, m, mp, row0, c->n_subv,
                                                       (T)(1.0 / sg), (T)(1.0 / m), flag);
     plain_gram<T><<<shared_by, kThreads, sm_gram, c->stream>>>(S, dt, c->tab, c->so_off, G, bv, m, mp, flag);
-    launch_eig<T>(nd, c->stream, G, bv, W, m, mp, flag);
+    launch_eig<T>(nd, c->stream, G, bv, W, m, mp, c->d_status, flag);
     plain_transform<T><<<shared_by, kThreads, sm_tr, c->stream>>>(X, Xo, W, c->tab, m, mp, c->n_act, (T)(1.0 / m), flag);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     if (cudaMemcpy2DAsync(out, (size_t)m * eb, Xo, (size_t)mp * eb, (size_t)m * eb, c->n, cudaMemcpyDeviceToDevice,

@@ -60,3 +60,38 @@ def test_narrow_ensembles(prec, m, e):
     err, _, _, status, _ = _analysis(prec, m, 10.0 ** e)
     assert status == 0
     assert max(max(q) for q in err) <= 31.0 * 2.0 ** (-53 if prec == "fp64" else -24)
+
+
+# More slopes than members: G has full rank but for the constant direction, which no anomaly has a part in.
+# Rounding G moves its smallest eigenvalue by p u |G|, T along its eigenvector by half of that relative to it
+# (kappa_eff: the ratio of the largest to the smallest eigenvalue away from the constant direction), and
+# rotations that keep small eigenvalues to working accuracy add their own m u; a reduction accurate only beside
+# |G| would lose kappa u.
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("m", [16, 20])
+@pytest.mark.parametrize("e", [1.5, 2.5, 3, 3.5])
+def test_wide_ensembles_of_full_rank(prec, m, e):
+    u = 2.0 ** (-53 if prec == "fp64" else -24)
+    for seed in range(2):
+        err, lam, _, status, _ = _analysis(prec, m, 10.0 ** e, seed)
+        assert status == 0
+        for q, l in zip(err, lam):
+            if l.size >= m:                                   # m - 1 eigenvalues away from the constant direction
+                assert max(q) <= (72.0 + 30.0) * u * l[0] / l[m - 2], (l[0], l[m - 2], q)
+
+
+# Fewer slopes than members: the eigenvalue 1 belongs to the anomalies as well, and rounding G loses kappa u of it.
+@pytest.mark.parametrize("m", [50, 100])
+@pytest.mark.parametrize("e", [2, 2.5, 3])
+def test_wide_ensembles_of_low_rank(m, e):
+    err, lam, _, status, _ = _analysis("fp32", m, 10.0 ** e)
+    assert status == 0
+    for q, l in zip(err, lam):
+        assert max(q) <= (l[0] + 30.0) * 2.0 ** -24, (l[0], q)
+
+
+@pytest.mark.parametrize("m", [20, 50, 100])
+@pytest.mark.parametrize("e", [3.5, 4, 4.5, 6])
+def test_past_the_range_is_finite_or_reported(m, e):
+    _, _, xa, status, _ = _analysis("fp32", m, 10.0 ** e)
+    assert np.isfinite(xa).all() or status == _lib.LETKF_ENOCONV
