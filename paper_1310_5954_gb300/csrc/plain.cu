@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
                                                                      const int* __restrict__ frame_bad) {
     extern __shared__ unsigned char smem_raw[];
     const int ld = m | 1;                  // odd row stride: no bank conflicts down a column
-    T* A = reinterpret_cast<T*>(smem_raw);   // B, then (row k, columns > k) the reflector v_k
+    T* A = reinterpret_cast<T*>(smem_raw);   // G/(m-1), then (row k, columns > k) the reflector v_k
     T* F = A + m * ld;                     // the function of J, then T
     constexpr int NK = kNodes<T>;
     const int mv = max(m, 2 * NK);
@@ -453,9 +453,10 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
     const T* Gd = G + (size_t)d * m * m_pad;
     const T c0 = (T)(m - 1), ic0 = (T)1 / c0;
     for (int i = warp; i < m; i += nw)
-        for (int j = lane; j < m; j += 32) A[i * ld + j] = Gd[(size_t)i * m_pad + j] * ic0 + (i == j ? (T)1 : (T)0);
+        for (int j = lane; j < m; j += 32) A[i * ld + j] = Gd[(size_t)i * m_pad + j] * ic0;
     __syncthreads();
-    // ---- reduction: step k maps row k (columns > k) onto e_k times the first unit vector
+    // ---- reduction of G/(m-1), to which J adds the identity: step k maps row k (columns > k) onto e_k times the
+    // first unit vector
     for (int k = 0; k < m - 2; ++k) {
         const int k1 = k + 1, nk = m - k1;
         T v[UM];
@@ -520,7 +521,7 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
             for (int u = 0; u < UM; ++u)
                 if (lane + 32 * u < nk) A[k * ld + k1 + lane + 32 * u] = v[u];
             if (lane == 0) {
-                dd[k] = A[k * ld + k];
+                dd[k] = (T)1 + A[k * ld + k];
                 ee[k] = al;
                 bt[k] = beta;
             }
@@ -528,8 +529,8 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
         __syncthreads();
     }
     if (tid == 0) {
-        dd[m - 2] = A[(m - 2) * ld + m - 2];
-        dd[m - 1] = A[(m - 1) * ld + m - 1];
+        dd[m - 2] = (T)1 + A[(m - 2) * ld + m - 2];
+        dd[m - 1] = (T)1 + A[(m - 1) * ld + m - 1];
         ee[m - 2] = A[(m - 2) * ld + m - 1];
         ee[m - 1] = 0;
     }
@@ -642,6 +643,7 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
                     if (4 * q < nn) sum += r[q];
                 sum += __shfl_xor_sync(0xffffffffu, sum, 1);
                 sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                if (st == 0 && n0 == 0) sum -= (T)1;               // F - I (see below)
                 if (j < m) {
                     T* f = h ? F + j * ld + i : F + i * ld + j;    // two lanes write the two triangles
                     if (h == 0 || (h == 1 && j > i)) *f = n0 ? *f + sum : sum;
@@ -653,7 +655,9 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
         }
         __syncthreads();
     }
-    // ---- T = Q F Q^T: the reflectors on every column of F, then on every row of the result
+    // ---- T = I + Q (F - I) Q^T: the reflectors on every column of F - I, then on every row of the result.
+    // (Where the ensemble's spread is small beside the noise, B and F are close to the identity, and would take
+    // the reflectors' rounding here and in the reduction: 2.5e-7 .. 4e-7 in FP32, now 9e-8 .. 1.8e-7.)
     const int grp = tid >> 3, l8 = tid & 7;
     auto reflect = [&](int rs, int cs) {   // vectors x_j[i] = F[j rs + i cs], two per group of 8 lanes
         for (int j0 = 2 * grp; j0 - 2 * (grp & 3) < m; j0 += nt >> 2) {   // whole warps
@@ -718,7 +722,10 @@ __global__ void __launch_bounds__(UM < 5 ? 128 * UM : 640) plain_eig(const T* __
         __syncthreads();
     };
     T* wb = dd;            // the tridiagonal matrix is no longer needed
-    for (int i = tid; i < m; i += nt) bs[i] = bvec[(size_t)d * m_pad + i];
+    for (int i = tid; i < m; i += nt) {
+        F[i * ld + i] += (T)1;             // T
+        bs[i] = bvec[(size_t)d * m_pad + i];
+    }
     __syncthreads();
     tmul(bs, vs, (T)1);
     tmul(vs, wb, ic0);

@@ -95,3 +95,16 @@ def test_wide_ensembles_of_low_rank(m, e):
 def test_past_the_range_is_finite_or_reported(m, e):
     _, _, xa, status, _ = _analysis("fp32", m, 10.0 ** e)
     assert np.isfinite(xa).all() or status == _lib.LETKF_ENOCONV
+
+
+# T is the identity to 1e-8 or better and w_bar zero, so that a row whose anomalies are e_j - 1/m reads T's column j:
+# one product that counts, and the rounding of T's entry, of the centring and of the sum with the mean, each at most
+# u = 2^-24 of the row's one large entry.
+@pytest.mark.parametrize("m", [20, 50, 100, 160])
+@pytest.mark.parametrize("e", [-9, -7, -6, -5, -4.5])
+def test_muted_slopes_leave_the_identity(m, e):
+    _, _, xa, status, xo = _analysis("fp32", m, 10.0 ** e, read_t=True)
+    assert status == 0
+    n = xa.shape[0] // 2
+    a, o = xa[:n] - xa[:n].mean(axis=1, keepdims=True), xo[:n] - xo[:n].mean(axis=1, keepdims=True)
+    assert (np.linalg.norm(a - o, axis=1) <= 4.0 * 2.0 ** -24 * np.linalg.norm(o, axis=1)).all()
