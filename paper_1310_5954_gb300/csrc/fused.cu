@@ -1499,8 +1499,10 @@ __device__ __forceinline__ void put32(float* C, const float (&c)[4]) {
 // thread, so a product's result is transformed in registers (T, the residual, the next inverse iterate)
 // and a Newton-Schulz step is two barriers: P -> T and the residual's sum, then Y T and T Z together.
 // Bound by the barriers and the shared-memory latency of q / 4 dependent reads per product.  Same
-// formulas as analyse_simt; the dual form's X'_E T = X'_E - (X'_E S^T) N S takes N = (I + K/c)^(-1/2)
-// (I + Z)^-1 (I + K/c)^(-1/2) / c as one q x q matrix.  Measured against analyse_simt: 8x8, m = 20 frame
+// formulas as analyse_simt, in the same association: the dual form's X'_E T = X'_E - (X'_E S^T) Z (I + Z)^-1 Z S / c
+// from the left, since the product of the three q x q matrices formed first carries the rounding of its largest
+// entries, which S amplifies by kappa instead of its root (anomalies' error, m = 100: kappa 1e3 1.2e-6 / 2.0e-6, 1e4
+// 2.3e-6 / 6.2e-6, 1e5 3.8e-6 / 1.8e-5).  Measured against analyse_simt: 8x8, m = 20 frame
 // 37.9 -> 32.7 us; ELT, whose 16 edge domains end the launch, 128.5 -> 121.7 us.
 template <bool TWO>
 __device__ __noinline__ const float* analyse_simt32(const FusedBatch& B, Ctrl* ctl, unsigned char* smem, int d,
@@ -1798,9 +1800,6 @@ __device__ __noinline__ const float* analyse_simt32(const FusedBatch& B, Ctrl* c
         simt_mm(Wc, m, Z, SL, 1, S, ls, 1, q, m, q, rs * rsqrtf(c));
         simt_mm(Wc + q * m, m, X, SL, 1, Wc, m, 1, q, m, q, 1.f);
     }
-    // N = Zt (I + Zt)^-1 Zt / c, beside X'_E S^T
-    mm32(Z, X, q, v);
-    put32(Q, v);
     for (int r = ty; 2 * r < n_e; r += 16) {                          // X'_E S^T
         const float* a = E + 2 * r * ls;
         const float* b = S + 2 * tx * ls;
@@ -1822,13 +1821,10 @@ __device__ __noinline__ const float* analyse_simt32(const FusedBatch& B, Ctrl* c
         *reinterpret_cast<float2*>(o + SL) = make_float2(cc[2], cc[3]);
     }
     __syncthreads();
-    mm32(Q, Z, q, v);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] *= rs * rs / c;
-    put32(Mi, v);
-    __syncthreads();
-    rows_mm(R2, R1, Mi, 1.f);
-    const int n4 = m_pad >> 2;                                        // X'_E - (X'_E S^T N) S, in place
+    rows_mm(R2, R1, Z, rs * rsqrtf(c));
+    rows_mm(R1, R2, X, 1.f);
+    rows_mm(R2, R1, Z, rs * rsqrtf(c));
+    const int n4 = m_pad >> 2;                                        // X'_E - (...) S, in place
     for (int t = tid; t < (rows >> 1) * n4; t += FT) {
         const int r = t / n4, j = 4 * (t - r * n4);
         const float* a = R2 + 2 * r * SL;
