@@ -246,7 +246,6 @@ void free_all(letkf_ctx* c) {
         if (c->ev_v_used[b]) cudaEventDestroy(c->ev_v_used[b]);
     }
     if (c->Xi_side) cudaFree(c->Xi_side);
-    if (c->part_side) cudaFree(c->part_side);
     if (c->pair_pred) cudaFree(c->pair_pred);
     for (void* q : {c->rg_items, c->rg_tiles, c->rg_part})
         if (q) cudaFree(q);
@@ -320,8 +319,7 @@ size_t footprint_bytes(const letkf_params* p, const HostModel& h) {
     } else if (p->q_sqrt) {
         b += p->path == LETKF_PATH_GLOBAL
                  ? na * na * eb
-                 : letkf::rg_bytes(h.n_act, p->m, letkf::lower_triangular(p->q_sqrt, h.n_act), eb,
-                                   p->path == LETKF_PATH_FUSED);
+                 : letkf::rg_bytes(h.n_act, p->m, letkf::lower_triangular(p->q_sqrt, h.n_act), eb);
     }
     if (p->piston != LETKF_PISTON_OFF) b += letkf::piston_bytes(h, (int)nd, (int)eb);
     if (p->path == LETKF_PATH_GLOBAL) {

@@ -107,8 +107,6 @@ struct letkf_ctx {
     cudaEvent_t ev_v_used[2] = {nullptr, nullptr};
     void* Vbuf[2] = {nullptr, nullptr};
     void* Xi_side = nullptr;
-    void* part_side = nullptr;      // the side stream's draws' partial sums (letkf_forecast draws on the
-                                    // context's stream meanwhile, into noise_part or rg_part)
     unsigned long long v_frame[2] = {~0ull, ~0ull};
     // fused step as a CUDA graph (one per frame parity): the fused kernel and, on a forked branch,
     // the next frame's noise draw; captured for the ensemble buffer in use (gcur)
@@ -177,14 +175,13 @@ int draw_perturbations_on(letkf_ctx* c, unsigned long long frame, void* xi, void
 int init_ensemble(letkf_ctx* c, const double* L_host, const double* P0_host);
 // Work plan of the FP32 / FP64 per-frame draw V = L xi (n x n factor, m members, eb bytes per
 // element): items and tiles (4 ints each, filled when not null), elements of the factor's and the
-// normals' layouts and of the partial tiles; rg_bytes: its device bytes (side: with partial tiles for a second stream's
-// draws); rg_xi_bytes: the normals'.
+// normals' layouts and of the partial tiles; rg_bytes: its device bytes; rg_xi_bytes: the normals'.
 struct RowGemmPlan {
     int n_items = 0, n_tiles = 0, n_slots = 0;
     size_t part_elems = 0, l_elems = 0, xi_elems = 0;
 };
 RowGemmPlan rg_plan(int n, int m, bool lower, size_t eb, int* items, int* tiles);
-size_t rg_bytes(int n, int m, bool lower, size_t eb, bool side);
+size_t rg_bytes(int n, int m, bool lower, size_t eb);
 size_t rg_xi_bytes(int n, int m, size_t eb);
 // Node parameters of the normals kernel draw_perturbations_on launches (arguments held in *nn).
 struct NormalsNode {

@@ -433,17 +433,15 @@ template <typename T>
 int rg_product(letkf_ctx* c, const void* xi, void* V, cudaStream_t stream) {
     const int n = c->n_act, m = c->m;
     const RkShape s = rk_shape(n, m, sizeof(T));
-    // the side stream's normals go with partial tiles of their own
-    T* part = static_cast<T*>(c->Xi_side && xi == c->Xi_side ? c->part_side : c->rg_part);
     const int rc = rk_with<T>(s, [&](auto* k) -> int {
         k<<<c->rg_n_items, RK_THREADS, rk_smem_bytes(s, sizeof(T)), stream>>>(
             (const T*)c->Lq, (const T*)xi, (T*)V, n, m, c->m_pad, c->lq_lower, (const int4*)c->rg_items,
-            (const int4*)c->rg_tiles, part, c->d_status);
+            (const int4*)c->rg_tiles, (T*)c->rg_part, c->d_status);
         return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
     });
-    if (rc || !part) return rc;
+    if (rc || !c->rg_part) return rc;
     rg_reduce_kernel<T><<<dim3((s.bm * (s.bn >> 2) + 255) / 256, s.nrb * s.ncb), 256, 0, stream>>>(
-        part, (const int4*)c->rg_tiles, s.bm, s.bn, (T*)V, n, m, c->m_pad);
+        (const T*)c->rg_part, (const int4*)c->rg_tiles, s.bm, s.bn, (T*)V, n, m, c->m_pad);
     return cudaGetLastError() == cudaSuccess ? LETKF_OK : LETKF_ECUDA;
 }
 
@@ -617,9 +615,9 @@ RowGemmPlan rg_plan(int n, int m, bool lower, size_t eb, int* items, int* tiles)
     return P;
 }
 
-size_t rg_bytes(int n, int m, bool lower, size_t eb, bool side) {
+size_t rg_bytes(int n, int m, bool lower, size_t eb) {
     const RowGemmPlan P = rg_plan(n, m, lower, eb, nullptr, nullptr);
-    return 16 * (size_t)P.n_items + 16 * (size_t)P.n_tiles + eb * ((side ? 2 : 1) * P.part_elems + P.l_elems + P.xi_elems);
+    return 16 * (size_t)P.n_items + 16 * (size_t)P.n_tiles + eb * (P.part_elems + P.l_elems + P.xi_elems);
 }
 
 size_t rg_xi_bytes(int n, int m, size_t eb) {
@@ -642,10 +640,7 @@ int rg_prepare(letkf_ctx* c, const double* L64) {
         cudaMalloc(&c->rg_items, items.size() * 4) != cudaSuccess ||
         cudaMalloc(&c->rg_tiles, tiles.size() * 4) != cudaSuccess)
         return LETKF_ENOMEM;
-    const bool side = c->path == LETKF_PATH_FUSED;
-    if (P.part_elems && (cudaMalloc(&c->rg_part, P.part_elems * sizeof(T)) != cudaSuccess ||
-                         (side && cudaMalloc(&c->part_side, P.part_elems * sizeof(T)) != cudaSuccess)))
-        return LETKF_ENOMEM;
+    if (P.part_elems && cudaMalloc(&c->rg_part, P.part_elems * sizeof(T)) != cudaSuccess) return LETKF_ENOMEM;
     if (cudaMemset(c->Xi, 0, P.xi_elems * sizeof(T)) != cudaSuccess ||
         cudaMemcpy(c->rg_items, items.data(), items.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->rg_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess)
@@ -653,7 +648,7 @@ int rg_prepare(letkf_ctx* c, const double* L64) {
     rg_pack_kernel<T><<<dim3(64, s.nrb), 256, 0, c->stream>>>(L64, (T*)c->Lq, n, s.bm, lower ? 1 : 0);
     if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
     c->rg_n_items = P.n_items;
-    c->device_bytes += rg_bytes(n, m, lower, sizeof(T), side);
+    c->device_bytes += rg_bytes(n, m, lower, sizeof(T));
     // (the attribute belongs to the kernel: every context with this shape sets the same value)
     return rk_with<T>(s, [&](auto* k) -> int {
         return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, rk_smem_bytes(s, sizeof(T))) == cudaSuccess

@@ -268,7 +268,7 @@ NoisePlan noise_plan(int n_act, int m, bool lower) {
     P.n_items = (int)items.size();
     P.bytes = (size_t)P.n_tiles * TILE_A                       // L tiles
               + (size_t)P.n_items * 16 + (size_t)P.nb * 4 * 4  // items; prefix, jn, jslot, split blocks
-              + (size_t)2 * P.n_slots * NBM * P.np * 4;        // partial sums, the side stream's draws' as well
+              + (size_t)P.n_slots * NBM * P.np * 4;            // partial sums
     return P;
 }
 
@@ -317,9 +317,8 @@ int noise_prepare(letkf_ctx* c, const double* L) {
     if ((rc = up((void**)&c->noise_tabs, tabs.data(), tabs.size() * 4))) return rc;
     const size_t pb = (size_t)P.n_slots * NBM * P.np * 4;
     if (pb) {
-        if (cudaMalloc(&c->noise_part, pb) != cudaSuccess || cudaMalloc(&c->part_side, pb) != cudaSuccess)
-            return LETKF_ENOMEM;
-        c->device_bytes += 2 * pb;
+        if (cudaMalloc(&c->noise_part, pb) != cudaSuccess) return LETKF_ENOMEM;
+        c->device_bytes += pb;
     }
     c->noise_nb = P.nb;
     c->noise_np = P.np;
@@ -383,8 +382,7 @@ int noise_product(letkf_ctx* c, const void* xi, void* v_out, cudaStream_t stream
     a.Lt = static_cast<const unsigned char*>(c->Lt);
     a.Xi = static_cast<const unsigned char*>(xi);
     a.V = static_cast<float*>(v_out);
-    // the side stream's normals go with partial sums of their own
-    a.part = static_cast<float*>(c->Xi_side && xi == c->Xi_side ? c->part_side : c->noise_part);
+    a.part = static_cast<float*>(c->noise_part);
     a.items = reinterpret_cast<const int4*>(c->noise_items);
     a.prefix = c->noise_tabs;
     a.status = c->d_status;
@@ -399,7 +397,7 @@ int noise_product(letkf_ctx* c, const void* xi, void* v_out, cudaStream_t stream
     if (c->noise_n_rb > 0) {
         const int nb = c->noise_nb, per = NBM * (c->noise_np >> 2);
         const int g = std::min(8192, (c->noise_n_rb * per + 255) / 256);
-        noise_reduce_kernel<<<g, 256, 0, stream>>>(a.part, c->noise_tabs + 3 * nb,
+        noise_reduce_kernel<<<g, 256, 0, stream>>>(static_cast<const float*>(c->noise_part), c->noise_tabs + 3 * nb,
                                                    c->noise_n_rb, c->noise_tabs + nb, c->noise_tabs + 2 * nb,
                                                    static_cast<float*>(v_out), c->m_pad, c->n_act, c->m, c->noise_np);
         if (cudaGetLastError() != cudaSuccess) return LETKF_ECUDA;
