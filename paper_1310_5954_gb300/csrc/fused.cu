@@ -3351,6 +3351,7 @@ int fused_prepare(letkf_ctx* c) {
         if (cudaMalloc(&c->Vbuf[b], vbytes) != cudaSuccess) return LETKF_ENOMEM;
         c->device_bytes += vbytes;
     }
+    if (cudaEventCreateWithFlags(&c->ev_draw, cudaEventDisableTiming) != cudaSuccess) return LETKF_ECUDA;
     if (cudaMalloc(&c->pair_pred, (size_t)c->n_act * 4) != cudaSuccess) return LETKF_ENOMEM;
     c->device_bytes += (size_t)c->n_act * 4;
     if (cudaMalloc(&c->Xi_side, xbytes) != cudaSuccess) return LETKF_ENOMEM;
@@ -3366,16 +3367,29 @@ int fused_prepare(letkf_ctx* c) {
 
 namespace {
 
-// The process-noise block of `frame` in buffer frame & 1, drawn on the side stream (after the
-// kernel that last read that buffer) unless it is there already; `stream` waits for it.
+// Draws the process-noise block of `frame` into buffer frame & 1 on the side stream: after the kernel that last
+// read that buffer, and after letkf_forecast's draws, which use the same partial sums.
+int noise_side(letkf_ctx* c, unsigned long long frame) {
+    const int b = (int)(frame & 1);
+    if (cudaStreamWaitEvent(c->side, c->ev_v_used[b], 0) != cudaSuccess) return LETKF_ECUDA;
+    if (c->draw_wait) {
+        if (cudaStreamWaitEvent(c->side, c->ev_draw, 0) != cudaSuccess) return LETKF_ECUDA;
+        if (c->draw_wait == 1) c->draw_wait = 0;
+    }
+    const int rc = draw_perturbations_on(c, frame, c->Xi_side, c->Vbuf[b], c->side);
+    if (rc) return rc;
+    if (cudaEventRecord(c->ev_v_ready[b], c->side) != cudaSuccess) return LETKF_ECUDA;
+    c->v_frame[b] = frame;
+    return LETKF_OK;
+}
+
+// The process-noise block of `frame` in buffer frame & 1, drawn on the side stream unless it is there already;
+// `stream` waits for it.
 int noise_ready(letkf_ctx* c, unsigned long long frame, cudaStream_t stream, const float** v) {
     const int b = (int)(frame & 1);
     if (c->v_frame[b] != frame) {
-        if (cudaStreamWaitEvent(c->side, c->ev_v_used[b], 0) != cudaSuccess) return LETKF_ECUDA;
-        const int rc = draw_perturbations_on(c, frame, c->Xi_side, c->Vbuf[b], c->side);
+        const int rc = noise_side(c, frame);
         if (rc) return rc;
-        if (cudaEventRecord(c->ev_v_ready[b], c->side) != cudaSuccess) return LETKF_ECUDA;
-        c->v_frame[b] = frame;
     }
     if (cudaStreamWaitEvent(stream, c->ev_v_ready[b], 0) != cudaSuccess) return LETKF_ECUDA;
     *v = static_cast<const float*>(c->Vbuf[b]);
@@ -3388,12 +3402,7 @@ int noise_prefetch(letkf_ctx* c, unsigned long long frame, cudaStream_t stream) 
     const int b = (int)(frame & 1), nb = b ^ 1;
     if (cudaEventRecord(c->ev_v_used[b], stream) != cudaSuccess) return LETKF_ECUDA;
     if (c->v_frame[nb] == frame + 1) return LETKF_OK;
-    if (cudaStreamWaitEvent(c->side, c->ev_v_used[nb], 0) != cudaSuccess) return LETKF_ECUDA;
-    const int rc = draw_perturbations_on(c, frame + 1, c->Xi_side, c->Vbuf[nb], c->side);
-    if (rc) return rc;
-    if (cudaEventRecord(c->ev_v_ready[nb], c->side) != cudaSuccess) return LETKF_ECUDA;
-    c->v_frame[nb] = frame + 1;
-    return LETKF_OK;
+    return noise_side(c, frame + 1);
 }
 
 // Descriptor of system c's next frame, with the process-noise block V (dense noise) given.

@@ -246,6 +246,7 @@ void free_all(letkf_ctx* c) {
         if (c->ev_v_used[b]) cudaEventDestroy(c->ev_v_used[b]);
     }
     if (c->Xi_side) cudaFree(c->Xi_side);
+    if (c->ev_draw) cudaEventDestroy(c->ev_draw);
     if (c->pair_pred) cudaFree(c->pair_pred);
     for (void* q : {c->rg_items, c->rg_tiles, c->rg_part})
         if (q) cudaFree(q);

@@ -108,6 +108,12 @@ struct letkf_ctx {
     void* Vbuf[2] = {nullptr, nullptr};
     void* Xi_side = nullptr;
     unsigned long long v_frame[2] = {~0ull, ~0ull};
+    // Draws on the side stream (or in a step's graph) and letkf_forecast's on the context's stream share the
+    // draw's partial sums and wait for each other: ev_v_ready, and ev_draw after one of the latter.
+    // draw_wait: the side stream has not waited for ev_draw since it was recorded; 2: it is recorded by a
+    // graph of the caller's as well, whenever that is launched
+    cudaEvent_t ev_draw = nullptr;
+    int draw_wait = 0;
     // fused step as a CUDA graph (one per frame parity): the fused kernel and, on a forked branch,
     // the next frame's noise draw; captured for the ensemble buffer in use (gcur)
     int graph_on = 0;

@@ -544,6 +544,37 @@ int normals_node_params(letkf_ctx* c, unsigned long long frame, void* xi, Normal
     return LETKF_OK;
 }
 
+namespace {
+
+// Around a draw on the context's stream where there is a side stream that draws as well: the draws made there
+// so far are done before it, and noise_side (fused.cu) has the later ones wait for it.  In a stream capture of the
+// caller's the events are external ones: they count as they stand when the caller's graph runs.
+bool capturing(letkf_ctx* c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) == cudaSuccess) return st == cudaStreamCaptureStatusActive;
+    cudaGetLastError();    // the legacy stream while another one is captured
+    return false;
+}
+
+int draws_join(letkf_ctx* c) {
+    if (!c->side) return LETKF_OK;
+    const unsigned flag = capturing(c) ? cudaEventWaitExternal : cudaEventWaitDefault;
+    for (cudaEvent_t ev : c->ev_v_ready)
+        if (cudaStreamWaitEvent(c->stream, ev, flag) != cudaSuccess) return LETKF_ECUDA;
+    return LETKF_OK;
+}
+
+int draws_fork(letkf_ctx* c) {
+    if (!c->side) return LETKF_OK;
+    const bool cap = capturing(c);
+    if (cudaEventRecordWithFlags(c->ev_draw, c->stream, cap ? cudaEventRecordExternal : cudaEventRecordDefault) != cudaSuccess)
+        return LETKF_ECUDA;
+    c->draw_wait = cap ? 2 : std::max(c->draw_wait, 1);
+    return LETKF_OK;
+}
+
+}  // namespace
+
 int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analysis, bool first_only) {
     int vmode, vld;
     const void* Vp;
@@ -552,8 +583,8 @@ int launch_forecast(letkf_ctx* c, const void* v_user, void* xpred, int in_analys
         Vp = v_user;
         vld = c->m;
     } else if (c->Lq || c->Lt) {
-        int rc = draw_perturbations(c, c->frame);
-        if (rc) return rc;
+        int rc = draws_join(c);
+        if (rc || (rc = draw_perturbations(c, c->frame)) || (rc = draws_fork(c))) return rc;
         vmode = 0;
         Vp = c->V;
         vld = c->m_pad;
