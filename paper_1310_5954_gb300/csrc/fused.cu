@@ -3368,7 +3368,8 @@ int fused_prepare(letkf_ctx* c) {
 namespace {
 
 // Draws the process-noise block of `frame` into buffer frame & 1 on the side stream: after the kernel that last
-// read that buffer, and after letkf_forecast's draws, which use the same partial sums.
+// read that buffer, and after the draws that use the same normals or partial sums: letkf_forecast's, and a step's
+// graph's, whose frame set_state can leave unused (ev_v_ready follows it).
 int noise_side(letkf_ctx* c, unsigned long long frame) {
     const int b = (int)(frame & 1);
     if (cudaStreamWaitEvent(c->side, c->ev_v_used[b], 0) != cudaSuccess) return LETKF_ECUDA;
@@ -3376,6 +3377,9 @@ int noise_side(letkf_ctx* c, unsigned long long frame) {
         if (cudaStreamWaitEvent(c->side, c->ev_draw, 0) != cudaSuccess) return LETKF_ECUDA;
         if (c->draw_wait == 1) c->draw_wait = 0;
     }
+    if (c->graph_on)
+        for (cudaEvent_t ev : c->ev_v_ready)
+            if (cudaStreamWaitEvent(c->side, ev, 0) != cudaSuccess) return LETKF_ECUDA;
     const int rc = draw_perturbations_on(c, frame, c->Xi_side, c->Vbuf[b], c->side);
     if (rc) return rc;
     if (cudaEventRecord(c->ev_v_ready[b], c->side) != cudaSuccess) return LETKF_ECUDA;

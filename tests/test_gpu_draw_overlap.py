@@ -69,3 +69,28 @@ def test_captured_forecast(prec):
             assert f.sync() == 0
             f.close()
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("name,prec", [("vlt-40x40", "mixed"), ("elt-80x80", "fp32")])
+@pytest.mark.parametrize("back", [1, 2, 5])
+def test_another_frame_behind_a_graph_step(name, prec, back):
+    """Steps as graphs draw the next frame's block; set_state to another frame has it drawn on the side stream."""
+    y, _ = slopes(name, 4)
+    ys = [torch.as_tensor(v, dtype=torch.float32, device="cuda") for v in y]
+    out = []
+    for idle in (lambda: None, torch.cuda.synchronize):
+        f = gpu_filter(name, prec, "fused")
+        f.set_graph(True)
+        x0 = f.get_state()[0].clone()
+        for k in range(4):
+            f.step(ys[k % 3])
+            f.step(ys[k % 3])
+            f.set_state(x0, 10 * k + back)
+            idle()
+            f.step(ys[3])
+            f.step(ys[0])
+            idle()
+        out.append(f.get_state()[0].clone())
+        assert f.sync() == 0
+        f.close()
+    assert torch.equal(out[0], out[1])
