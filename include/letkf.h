@@ -333,11 +333,12 @@ int letkf_get_graph(const letkf_ctx* ctx, int* enabled);
 
 /*
  * Launch tuning of the fused path (the paper has no counterpart).  Neither knob changes any
- * result: fused_grid is the number of SMs the fused kernel takes for this context (0: all,
- * capped at the number of domains; at most the SM count; one CTA on each, or two where the kernel
- * runs two domains side by side), graph is letkf_set_graph's mode.
+ * result: fused_grid sets the number of CTAs of the fused kernel for this context (0: the SM count,
+ * capped at the number of domains; at most the SM count): that many, or twice as many where two fit
+ * an SM and there are more domains than SMs.  Which SMs they run on is up to the device.  graph is
+ * letkf_set_graph's mode.
  * letkf_autotune times `frames` letkf_step calls with the slopes y_dev (p elements) for each
- * candidate (one CTA per SM, or the fewest CTAs taking the same number of rounds of domains;
+ * candidate (every SM full, or the fewest CTAs that take the same number of rounds of domains;
  * graph off or on), keeps the fastest and reports it and its milliseconds per frame (either
  * pointer may be NULL).  The context's ensemble, frame counter, noise std and latched status
  * are restored afterwards.  Plain-path contexts: tuning is fixed at {0, 0}.

@@ -3315,6 +3315,8 @@ int fused_plan(letkf_ctx* c) {
     return LETKF_OK;
 }
 
+int fused_ctas_per_sm(const letkf_ctx* c) { return c->fused_smem2 > 0 && c->n_dom > c->sms ? 2 : 1; }
+
 int fused_prepare(letkf_ctx* c) {
     const HostModel& h = c->host;
     const int rc = fused_plan(c);

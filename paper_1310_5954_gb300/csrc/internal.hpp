@@ -312,6 +312,7 @@ int launch_copy_rows(letkf_ctx* c, const void* src, void* dst);
 // (c->simt_q, c->simt_ws) from the geometry, m, m_pad and simt_q_max; LETKF_EINVAL if it does not fit.
 int fused_plan(letkf_ctx* c);
 int fused_prepare(letkf_ctx* c);
+int fused_ctas_per_sm(const letkf_ctx* c);    // of the context's own launches
 int fused_step(letkf_ctx* c, const void* y, double sigma, void* xpred, int with_forecast);
 // The next frame of n systems (fused path, same device) in one launch per form of the analysis, each
 // with its systems' domains as one work queue (`queue`: 8 zeroed ints on the device, reset by the kernels).

@@ -11,10 +11,11 @@
 
 namespace {
 
-// The grid with the fewest CTAs that still takes ceil(n_dom / SMs) rounds of domains.
+// The grid with the fewest CTAs that takes as many rounds of domains as all SMs full of CTAs (one or two each).
 int balanced_grid(const letkf_ctx* c) {
-    const int rounds = (c->n_dom + c->sms - 1) / c->sms;
-    return (c->n_dom + rounds - 1) / rounds;
+    const int per = letkf::fused_ctas_per_sm(c), rounds = (c->n_dom + per * c->sms - 1) / (per * c->sms);
+    const int ctas = (c->n_dom + rounds - 1) / rounds;
+    return (ctas + per - 1) / per;
 }
 
 }  // namespace
