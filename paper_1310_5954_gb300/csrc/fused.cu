@@ -1,6 +1,6 @@
 // Fused per-frame local ETKF kernel on the tensor cores (Sect. 2.3 analysis + Sect. 2.1 forecast).
 //
-// One persistent CTA per SM takes domains from a work queue (most expensive first).  Per
+// Persistent CTAs, one or two per SM, take domains from a work queue (most expensive first).  Per
 // domain, every product runs as a 128-row tcgen05 BF16 MMA with FP32 accumulation in
 // tensor memory:
 //
@@ -3228,7 +3228,7 @@ FusedLayout fused_layout(const letkf_ctx* c) {
 // Shared memory of a CTA when two share an SM (228 KB per SM, 1 KB of it reserved per CTA).
 constexpr int TWO_SMEM = 113 * 1024;
 
-// The layout of fused_kernel<true> (offsets within the big region unless they are off_vec or
+// The layout of fused_kernel<MODE_TWO> (offsets within the big region unless they are off_vec or
 // off_big); total = 0 when the system does not fit or takes the dual form.
 FusedLayout fused_layout2(const letkf_ctx* c) {
     const HostModel& h = c->host;
@@ -3337,7 +3337,7 @@ int fused_prepare(letkf_ctx* c) {
         cudaFuncSetAttribute(fused_kernel<MODE_TWO>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared) != cudaSuccess)
         return LETKF_ECUDA;
-    // One CTA per SM pulling domains from the work queue: domains differ in cost (edge domains
+    // Every SM pulling domains from the work queue: domains differ in cost (edge domains
     // see fewer subapertures), so the full grid balances better than fewer, evenly loaded CTAs.
     c->fused_grid = std::min(c->sms, c->n_dom);
     // lowest priority: the side stream's blocks never take an SM that the frame's kernel is waiting for

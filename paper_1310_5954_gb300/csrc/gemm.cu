@@ -13,7 +13,7 @@
 // tcgen05.mma into one of two accumulators in tensor memory, and four warps read the other back for the
 // epilogue, so that a piece's read-out runs under the next one's products (one CTA per piece, 128 threads
 // doing all three in turn and 8-byte row-strided stores, took 103 / 90 / 43 us for the noise draw, the
-// transform and the Gram at n_act = 4833, m = 1024; this takes 53 / 39 / 35 us).
+// transform and the Gram at n_act = 4833, m = 1024; this takes 53 / 39 / 36 us).
 //
 // What bounds a split product is the time from a stage's refill to its use, about 2500 cycles: a ring of S
 // stages, each M cycles of products, takes (2500 + M) / S per stage.  Per 64 columns of K a 128 x 256 piece

@@ -33,7 +33,7 @@ struct DomainTables {
     int* order = nullptr;       // [n_dom] processing order, most expensive first
 };
 
-struct GlobalState;   // global.cu: buffers and graph of the global path
+struct GlobalState;   // global.cu: buffers and plans of the global path
 
 // Host copy of the geometry and domains.
 struct HostModel {
@@ -170,7 +170,6 @@ void prof_end(letkf_ctx* c);
 // plain.cu
 int plain_analyze(letkf_ctx* c, const void* y, double sigma);
 int plain_limits_ok(int precision, int m);
-size_t plain_smem_bytes(const letkf_ctx* c, int which);
 
 // misc.cu
 int launch_precheck(letkf_ctx* c, const void* y);
