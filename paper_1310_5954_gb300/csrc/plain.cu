@@ -277,6 +277,9 @@ __device__ __forceinline__ void rr_pair(int M, int s, int k, int& p, int& q) {
 // residual in FP64.  A (padded to even order M with a zero row and column) and U in shared memory.  In exact
 // arithmetic no lambda is below m - 1; rounding can take one there, and ST_NOCONV tells that the matrix was not
 // numerically positive definite.
+// Latency bounds it: two barriers per step of half-M rotations, of which the last sweeps have few, so that steps
+// and blocks without one are passed over and V's rows need no division per element (FP32, m = 20 / 50 / 100: 159 /
+// 980 / 3870 -> 145 / 898 / 3260 us; FP64, m = 20 / 50: 651 / 4510 -> 623 / 4290).
 template <typename T>
 __device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* __restrict__ bd, T* __restrict__ Wd, int m,
                                             int m_pad, unsigned char* smem, int* status) {
@@ -288,7 +291,6 @@ __device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* _
     int* pq = reinterpret_cast<int*>(cs + M);  // M/2 (p, q) pairs
     T* rv = reinterpret_cast<T*>(pq + M);      // refinement: residual, then U^T r / lambda
     T* tv = rv + M;
-    __shared__ int nrot;
     const T c0 = (T)(m - 1);
     __syncthreads();                           // the caller's reads are done
     for (int i = warp; i < M; i += nw)
@@ -296,11 +298,15 @@ __device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* _
             A[i * ld + j] = (i < m && j < m ? Gd[(size_t)i * m_pad + j] : (T)0) + (i == j && i < m ? c0 : (T)0);
             V[i * ld + j] = i == j ? (T)1 : (T)0;
         }
+    __syncthreads();
+    // columns of V: thread (group vg of M threads, row tid mod M) takes pairs vg, vg + groups, ...
+    const int groups = nt / M, vg = tid / M;                 // (launch_eig: three groups or more)
+    T* Vr = V + (tid - vg * M) * ld;
     int sweep = 0;
     for (; sweep < JACOBI_SWEEPS; ++sweep) {
-        if (tid == 0) nrot = 0;
-        __syncthreads();
+        bool rotated = false;
         for (int s = 0; s < M - 1; ++s) {
+            bool rot = false;
             for (int k = tid; k < half; k += nt) {
                 int p, q;
                 rr_pair(M, s, k, p, q);
@@ -311,14 +317,15 @@ __device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* _
                     const T t = (tau >= (T)0 ? (T)1 : (T)-1) / (fabs(tau) + sqrt((T)1 + tau * tau));
                     c = (T)1 / sqrt((T)1 + t * t);
                     sn = t * c;
-                    atomicAdd(&nrot, 1);
+                    rot = true;
                 }
                 cs[2 * k] = c;
                 cs[2 * k + 1] = sn;
                 pq[2 * k] = p;
                 pq[2 * k + 1] = q;
             }
-            __syncthreads();
+            if (!__syncthreads_or(rot)) continue;      // (most steps of the last sweeps)
+            rotated = true;
             // A <- J^T A J on the 2 x 2 blocks of paired rows P x paired columns Q, P <= Q; A stays symmetric, so
             // the blocks above the diagonal also write their transposes.  Rows r and half - 1 - r of the
             // triangle have half + 1 blocks together
@@ -327,6 +334,7 @@ __device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* _
                 const int P = c < half - r ? r : half - 1 - r, Q = c < half - r ? r + c : c - 1;
                 const int pP = pq[2 * P], qP = pq[2 * P + 1], pQ = pq[2 * Q], qQ = pq[2 * Q + 1];
                 const T cP = cs[2 * P], sP = cs[2 * P + 1], cQ = cs[2 * Q], sQ = cs[2 * Q + 1];
+                if (sP == (T)0 && sQ == (T)0) continue;
                 const T b00 = A[pP * ld + pQ], b01 = A[pP * ld + qQ];
                 const T b10 = A[qP * ld + pQ], b11 = A[qP * ld + qQ];
                 const T r00 = cP * b00 - sP * b10, r01 = cP * b01 - sP * b11;
@@ -344,17 +352,18 @@ __device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* _
                     A[qQ * ld + qP] = n11;
                 }
             }
-            for (int e = tid; e < half * M; e += nt) {     // V <- V J
-                const int P = e / M, i = e - P * M, p = pq[2 * P], q = pq[2 * P + 1];
-                const T c = cs[2 * P], sn = cs[2 * P + 1], vp = V[i * ld + p], vq = V[i * ld + q];
-                V[i * ld + p] = c * vp - sn * vq;
-                V[i * ld + q] = sn * vp + c * vq;
-            }
+            if (vg < groups)                                 // V <- V J
+                for (int P = vg; P < half; P += groups) {
+                    const T c = cs[2 * P], sn = cs[2 * P + 1];
+                    if (sn == (T)0) continue;
+                    const int p = pq[2 * P], q = pq[2 * P + 1];
+                    const T vp = Vr[p], vq = Vr[q];
+                    Vr[p] = c * vp - sn * vq;
+                    Vr[q] = sn * vp + c * vq;
+                }
             __syncthreads();
         }
-        const int nr = nrot;
-        __syncthreads();                       // every thread has read nrot before thread 0 resets it
-        if (nr == 0) break;
+        if (!rotated) break;
     }
     // f_i = sqrt((m-1)/lambda_i) in A's padding column M, w_bar in V's
     T* z = cs;
@@ -419,7 +428,7 @@ __device__ __noinline__ void jacobi_weights(const T* __restrict__ Gd, const T* _
 //
 // The inverse of a tridiagonal matrix costs O(m) divisions (the pivots from both ends) and one multiplication
 // per entry, so the work is that of the reflectors: 4/3 m^3 multiply-adds to reduce, 4 m^3 in all, against 9
-// sweeps of m^3 by Jacobi, which takes 4 to 9 times as long, and 2 barriers per column instead of 2 per rotation
+// sweeps of m^3 by Jacobi, which takes 4 to 10 times as long, and 2 barriers per column instead of 2 per rotation
 // step and sweep.
 //
 // What bounds it: the m - 2 dependent reduction steps (two barriers each, the trailing matrix's
@@ -766,7 +775,7 @@ template <typename T>
 void launch_eig(int n_dom, cudaStream_t st, const T* G, const T* b, T* W, int m, int m_pad, int* status, const int* bad) {
     const int nt = std::min(640, std::max(128, (4 * m + 31) / 32 * 32));
     int kb = kNodes<T>;
-    while (kb > 1 && eig_smem<T>(m, kb) > 227 * 1024 - 64) --kb;   // (64: jacobi_weights' own variable)
+    while (kb > 1 && eig_smem<T>(m, kb) > 227 * 1024) --kb;
     const size_t sm = std::max(eig_smem<T>(m, kb), jacobi_smem(m, sizeof(T)));
     if (m <= 32)
         plain_eig<T, 1><<<n_dom, nt, sm, st>>>(G, b, W, m, m_pad, kb, status, bad);
